@@ -363,10 +363,10 @@ __global__ void k_kepler_all(p3t_particles p, double dt, KepConst K, DevStatus *
 }
 
 // ---- Hermite-4 with block steps (+ collisions), one block per cluster ------
-// Clusters of up to 32 members (nearly all) run one warp each, so that the
-// FP64 instructions of their few work items are not spread over idle lanes
-// of several warps; clusters of 33 to 128 members run one 128-thread block
-// each, their work items (member components, or (active member, source)
+// Clusters of up to hermite_warp_max members (8 by default) run one warp each,
+// so that the FP64 instructions of their few work items are not spread over
+// idle lanes of several warps (two to five members: integrate_five below);
+// larger ones up to 128 members run one 128-thread block each, their work items (member components, or (active member, source)
 // terms) dealt round-robin over the four warps so that one long cluster keeps
 // the FP64 pipes of all four SM sub-partitions busy.  Each active member's
 // force is the sum, in the fixed order star term first then sources in
@@ -405,6 +405,19 @@ struct HSmall {  // a cluster of <= KM members
   double T[kT][6];
   int64_t t[KM];
   int32_t lvl[KM], act[KM], set[KM], nset[KM], partner[KM], chg[KM];
+};
+
+// what the block steps take from (dt, parameters), formed once on the host in
+// the same IEEE operations
+struct HConst {
+  double unit, unit6;       // dt / 2^40, 6 unit
+  double m52u;              // -2^52 unit
+  double c3u, c4u, c5u;     // unit^3 / 6, unit^4 / 24, unit^5 / 120
+  double idt2, idt3;        // 1 / dt^2, 1 / dt^3
+  double i1mg, gms;         // 1 / (1 - gamma), G M_*
+  float etaf, eta0f;
+  float gin2;               // (y r_out)^2 below this in FP32: y < gamma in FP64
+  int fast;                 // the constants stay normal at every level
 };
 
 static_assert(sizeof(HSmall<kHMax>) <= 48 * 1024,
@@ -838,56 +851,51 @@ __device__ void emit_composites(const V &S, const HCtl &C, int nc, int64_t off,
   }
 }
 
-// block-step integration of one cluster (the whole block takes part)
+// block-step integration of one cluster (the whole block takes part); with
+// `resume` S holds the state after the evaluation at tn that found a contact
 template <int NT, class V>
 __device__ void integrate_cluster(const V &S, HCtl &C, double (*Tb)[6], int64_t off, int nc,
                                   const int32_t *cl_mem, const p3t_particles &p,
-                                  const p3t_params &prm, double dt, bool coll,
+                                  const p3t_params &prm, const HConst &hc, double dt, bool coll,
                                   const CollOut &co, unsigned long long &steps,
                                   bool &underflow, DevStatus *st, int64_t iter_limit,
-                                  int32_t *rec) {
+                                  int32_t *rec, bool resume, int64_t tn, int64_t iter) {
   const int tid = threadIdx.x;
   const int item = (tid & 31) * (NT / 32) + (tid >> 5);  // consecutive items -> different warps
   bool uf = false;  // a step of this cluster fell below dt / 2^40
   const int64_t T = ((int64_t)1) << P3T_KMAX;
-  const double unit = ldexp(dt, -P3T_KMAX);
-  const double idt = 1.0 / dt;
-  const double i1mg = 1.0 / (1.0 - prm.gamma);
-  // a step of level l is D = unit 2^(40 - l) exactly, so D^n = RN(unit^n)
-  // 2^(n (40 - l)) and RN(D^n c) = RN(unit^n c) 2^(n (40 - l)) with unit^n
-  // formed by the same successive products: the corrector's powers of D and
-  // of 1/D are these constants shifted in the exponent (the same bits as the
-  // products, no FP64 instruction)
-  const double u2 = unit * unit, u3 = u2 * unit, u4 = u3 * unit, u5 = u4 * unit;
-  const double c3u = u3 * (1.0 / 6.0), c4u = u4 * (1.0 / 24.0), c5u = u5 * (1.0 / 120.0);
-  const double idt2 = idt * idt, idt3 = idt2 * idt;
-  for (int k = item; k < nc; k += NT) {
-    const int32_t i = cl_mem[off + k];
-    S.x(0, k) = p.x[i]; S.x(1, k) = p.y[i]; S.x(2, k) = p.z[i];
-    S.v(0, k) = p.vx[i]; S.v(1, k) = p.vy[i]; S.v(2, k) = p.vz[i];
-    for (int q = 0; q < 3; ++q) { S.p(q, k) = S.x(q, k); S.pv(q, k) = S.v(q, k); }
-    S.m(k) = p.m[i];
-    S.iro(k) = 1.0 / p.r_out[i];
-    S.rp(k) = coll ? p.r_phys[i] : 0.0;
-    S.set(k) = k;
-    S.partner(k) = kNone;
-    if (rec) rec[i] = 0;
+  const double i1mg = hc.i1mg, unit = hc.unit;
+  int nact = 0;
+  if (tid == 0) { C.any = resume ? 1 : 0; C.ncomp = 0; C.stop = 0; C.edisp = 0.0; }
+  if (!resume) {
+    for (int k = item; k < nc; k += NT) {
+      const int32_t i = cl_mem[off + k];
+      S.x(0, k) = p.x[i]; S.x(1, k) = p.y[i]; S.x(2, k) = p.z[i];
+      S.v(0, k) = p.vx[i]; S.v(1, k) = p.vy[i]; S.v(2, k) = p.vz[i];
+      for (int q = 0; q < 3; ++q) { S.p(q, k) = S.x(q, k); S.pv(q, k) = S.v(q, k); }
+      S.m(k) = p.m[i];
+      S.iro(k) = 1.0 / p.r_out[i];
+      S.rp(k) = coll ? p.r_phys[i] : 0.0;
+      S.set(k) = k;
+      S.partner(k) = kNone;
+      if (rec) rec[i] = 0;
+    }
   }
-  if (tid == 0) { C.any = 0; C.ncomp = 0; C.stop = 0; C.edisp = 0.0; }
   __syncthreads();
-  // initial forces of every member (the block-time state is the initial
-  // state), first steps
-  int nact = build_list<NT>(S, C, nc, [](int) { return true; });
-  block_forces<NT>(S, C, Tb, nc, nact, item, prm, i1mg, coll);
-  for (int k = item; k < nc; k += NT) {
-    for (int q = 0; q < 3; ++q) { S.a(q, k) = S.a1(q, k); S.j(q, k) = S.j1(q, k); }
-    S.t(k) = 0;
-    S.lvl(k) = first_level(S, k, prm, dt, 0, uf);
-    if (S.partner(k) != kNone) C.any = 1;
+  if (!resume) {
+    // initial forces of every member (the block-time state is the initial
+    // state), first steps
+    nact = build_list<NT>(S, C, nc, [](int) { return true; });
+    block_forces<NT>(S, C, Tb, nc, nact, item, prm, i1mg, coll);
+    for (int k = item; k < nc; k += NT) {
+      for (int q = 0; q < 3; ++q) { S.a(q, k) = S.a1(q, k); S.j(q, k) = S.j1(q, k); }
+      S.t(k) = 0;
+      S.lvl(k) = first_level(S, k, prm, dt, 0, uf);
+      if (S.partner(k) != kNone) C.any = 1;
+    }
+    if (uf) C.stop = 1;
+    __syncthreads();
   }
-  if (uf) C.stop = 1;
-  __syncthreads();
-  int64_t tn = 0, iter = 0;
   for (;;) {
     // a step below dt / 2^40 ends the cluster's integration (the error is
     // recorded when the block finishes): every thread reads the flag after
@@ -950,15 +958,15 @@ __device__ void integrate_cluster(const V &S, HCtl &C, double (*Tb)[6], int64_t 
       const int lv = S.lvl(k), sh = P3T_KMAX - lv;
       const double D = ldexp_fast(unit, sh);
       // 1 / D = 2^lvl (1 / dt) exactly (D = dt 2^-lvl): a product, not a division
-      const double iD2 = ldexp_fast(idt2, 2 * lv), iD3 = ldexp_fast(idt3, 3 * lv);
+      const double iD2 = ldexp_fast(hc.idt2, 2 * lv), iD3 = ldexp_fast(hc.idt3, 3 * lv);
       const double da = S.a(q, k) - S.a1(q, k);
       const double j0 = S.j(q, k), j1 = S.j1(q, k);
       const double A2 = __fma_rn(-D, __fma_rn(2.0, j1, 4.0 * j0), -6.0 * da) * iD2;
       const double A3 = __fma_rn(6.0 * D, j0 + j1, 12.0 * da) * iD3;
       S.a2e(q, k) = __fma_rn(D, A3, A2);
       S.a3(q, k) = A3;
-      const double c3 = ldexp_fast(c3u, 3 * sh), c4 = ldexp_fast(c4u, 4 * sh),
-                   c5 = ldexp_fast(c5u, 5 * sh);
+      const double c3 = ldexp_fast(hc.c3u, 3 * sh), c4 = ldexp_fast(hc.c4u, 4 * sh),
+                   c5 = ldexp_fast(hc.c5u, 5 * sh);
       S.x(q, k) = __fma_rn(A3, c5, __fma_rn(A2, c4, S.p(q, k)));
       S.v(q, k) = __fma_rn(A3, c4, __fma_rn(A2, c3, S.pv(q, k)));
       S.a(q, k) = S.a1(q, k);
@@ -996,14 +1004,426 @@ __device__ void integrate_cluster(const V &S, HCtl &C, double (*Tb)[6], int64_t 
   __syncthreads();
 }
 
+// ---- one warp per cluster of two to five: FP64 slots shared by the lanes -------
+// On this part an FP64 warp instruction holds its sub-partition's pipe for 64
+// cycles whatever its mask (measured: 64.2 cycles a DFMA with 1 to 32 active
+// lanes, in one chain or eight), so a block step of a small cluster costs its
+// number of FP64 warp instructions and the latency of what stands between
+// them, not its arithmetic.  Clusters of at most five members (nearly all)
+// therefore keep a member in six lanes (three positions, three velocities;
+// state, forces and times in registers), and independent operations sit in
+// different lanes of one instruction: every FP64 slot is one fma(A, B, C) with
+// operands chosen per lane, a product A B + 0, a difference fma(-1, B, C).
+// Factors of two are moved between operands (exact), so every value has the
+// bits of hard_term and integrate_cluster:
+//  - predictor, 4 slots: D = RN(n unit) from one fma on 2^52 + n (beside j/3),
+//    then positions and velocities side by side;
+//  - pair terms, six lanes a term, five terms a round: r.r beside r.u; with
+//    every term inside gamma r_out (decided on the leading bits, with a
+//    margin: K = 0) the changeover is left out, otherwise its two polynomials
+//    run side by side: 14 or 30 slots a round against 55 or 75 for hard_term's
+//    one lane a term;
+//  - corrector, 8 slots: A2 beside A3, then x beside v.
+//  - step criterion: approximate FP32 norms decide the level unless they are
+//    within 2^-14 of a power of two (then the criterion as written), so no
+//    conversion, root or division of full precision is on the path.
+// What bounds it: the FP64 pipe of one sub-partition, 27 to 44 slots of the
+// 4,000-5,500 cycles of a block step.  Measured (one cluster, both members
+// active): 6.5 -> 2.3 us a block step inside gamma r_out, 6.8 -> 3.0 us in the
+// changeover; triples 5.8 -> 2.7 us; 20,000 pairs of 15 block steps at once
+// 1,844 -> 641 us.  Clusters of 6 and more keep integrate_cluster's one lane a
+// term (eight members: 25 rounds here against 3 batches there).
+constexpr int kFive = 5;
+
+struct HFive {
+  double P[kFive + 1][6];   // positions and velocities at the block time; the star's row is zero
+  double D[kFive][6];       // a round's r and u
+  double T[kFive * kFive][6];
+  double gm[kFive + 1], iro[kFive + 1];  // G m, 1 / r_out; the star: G M_*, 0
+  double sr2[kFive * kFive];             // (f (R_k + R_j))^2
+  float irf2[kFive + 1];                 // 1 / r_out^2 in FP32
+  int32_t partner[kFive];
+};
+
+__device__ __forceinline__ double shfl_d(double v, int src) {
+  return __shfl_sync(0xffffffffu, v, src);
+}
+// a > b and a >= b for a >= 0 or NaN and b >= 0 from the bit patterns (an FP64
+// comparison takes an FP64 slot); false for NaN
+__device__ __forceinline__ bool gt_pos(double a, double b) {
+  const long long x = __double_as_longlong(a);
+  return x > __double_as_longlong(b) && x <= 0x7ff0000000000000LL;
+}
+__device__ __forceinline__ bool ge_pos(double a, double b) {
+  const long long x = __double_as_longlong(a);
+  return x >= __double_as_longlong(b) && x <= 0x7ff0000000000000LL;
+}
+// x 2^k for x and x 2^k normal
+__device__ __forceinline__ double shift_exp(double x, int k) {
+  return __hiloint2double(__double2hiint(x) + (k << 20), __double2loint(x));
+}
+// (float)(x 2^k)
+__device__ __forceinline__ float scaled_float(double x, int k) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  const bool plain = (unsigned)(e - 1) < 2046u && (unsigned)(e + k - 1) < 2046u;
+  return (float)(plain || k == 0 ? __hiloint2double(hi + (k << 20), __double2loint(x))
+                                 : ldexp(x, k));
+}
+
+// quantise_level for a normal positive dt (with every dt / 2^k normal), from
+// the bit patterns: dt / 2^l <= dt_des iff bits(dt) - (l << 52) <= bits(dt_des)
+__device__ __forceinline__ int level_bits(double dt_des, long long bd, int prev, int64_t t,
+                                          bool &underflow) {
+  const long long bs = __double_as_longlong(dt_des);
+  int lvl = 0;
+  if (bs < bd && (bs & 0x7fffffffffffffffLL) <= 0x7ff0000000000000LL) {
+    const long long l = bs > 0 ? (bd - bs + 0xfffffffffffffLL) >> 52 : P3T_KMAX + 1;
+    underflow = underflow || l > P3T_KMAX;
+    lvl = l > P3T_KMAX ? P3T_KMAX : (int)l;
+  }
+  lvl = max(lvl, prev - 1);
+  if (t != 0) lvl = max(lvl, P3T_KMAX - __ffsll((long long)t) + 1);
+  return min(lvl, P3T_KMAX);
+}
+
+// the terms of the listed members (act: four bits each) at the block-time
+// state F.P, five a round, into F.T[b nc + jj] (jj: the other members by
+// index, then the star)
+__device__ __forceinline__ void five_terms(HFive &F, int nc, int nact, unsigned act,
+                                           const p3t_params &prm, const HConst &hc, bool coll) {
+  const int lane = threadIdx.x & 31, g = lane / 6, c = lane - 6 * g, g0 = lane - c;
+  const bool jerk = c >= 3, hlp = c == 1;
+  const int terms = nact * nc;
+  const unsigned inc = 65536u / (unsigned)nc + 1u;  // x / nc = x inc >> 16 for x <= 25
+  for (int t0 = 0; t0 < terms; t0 += kFive) {
+    const int ti = t0 + g;
+    const bool in = g < kFive && ti < terms;
+    const int tc = in ? ti : 0;
+    const int b = (int)(((unsigned)tc * inc) >> 16), jj = tc - b * nc;
+    const int k = (int)(act >> (4 * b)) & 7;
+    const int j = jj == nc - 1 ? kFive : (jj < k ? jj : jj + 1);
+    const double d = F.P[k][c] - F.P[j][c];
+    const int gd = g < kFive ? g : 0;
+    if (g < kFive) F.D[g][c] = d;
+    const double Gm = F.gm[j], ik = F.iro[k], ij = F.iro[j];
+    const double irot = __double_as_longlong(ik) < __double_as_longlong(ij) ? ik : ij;
+    const float irf2 = fminf(F.irf2[k], F.irf2[j]);
+    __syncwarp();
+    const double rx = F.D[gd][0], ry = F.D[gd][1], rz = F.D[gd][2];
+    const int o = jerk ? 3 : 0;
+    // r.r in lanes 0-2, r.u in lanes 3-5
+    const double s = __fma_rn(rx, F.D[gd][o], __fma_rn(ry, F.D[gd][o + 1], rz * F.D[gd][o + 2]));
+    double r2 = shfl_d(s, g0);
+    const int hi = __double2hiint(r2);
+    if (coll && in && c == 0 && j < kFive && gt_pos(F.sr2[k * kFive + j], r2))
+      atomicMin(&F.partner[k], j);
+    const bool on = in && __double_as_longlong(r2) != 0;
+    if (!on) r2 = 1.0;
+    const double rinv = rsqrt(r2);
+    // r^2 from its leading 20 bits (FP32 range checked by the exponent)
+    const int e = hi >> 20;
+    const float r2f = __uint_as_float(((unsigned)(e - 896) << 23) | ((unsigned)(hi & 0xfffff) << 3));
+    const bool inner = !on || j == kFive || (e > 900 && e < 1100 && r2f * irf2 < hc.gin2);
+    double w = 1.0, dK = 0.0;
+    bool dead = false, any_mid = false;
+    if (!__all_sync(0xffffffffu, inner)) {
+      const double yv = (r2 * rinv) * irot;
+      dead = ge_pos(yv, 1.0);
+      const bool mid = on && !dead && gt_pos(yv, prm.gamma);
+      any_mid = __any_sync(0xffffffffu, mid);
+      if (any_mid) {
+        // lanes 0, 2: w = 1 - x^4 P; lanes 3-5: dK; lane 1: P's first terms
+        const double xs = (yv - prm.gamma) * hc.i1mg;
+        const double v1 = __fma_rn(hlp ? 84.0 : xs, xs, 0.0);                          // x^2 | 84 x
+        const double v2 = __fma_rn(hlp ? -1.0 : v1, hlp ? v1 : xs, hlp ? 35.0 : 0.0);  // x^3
+        const double x2 = shfl_d(v1, g0);
+        // x^4 | 1 - x | 70 x^2
+        const double v3 = __fma_rn(hlp ? 70.0 : (jerk ? -1.0 : x2), jerk ? xs : x2,
+                                   jerk ? 1.0 : 0.0);
+        // 20 x^3 | u^2 | 35 - 84 x + 70 x^2
+        const double v4 = __fma_rn(hlp ? 1.0 : (jerk ? v3 : 20.0), hlp ? v2 : (jerk ? v3 : v2),
+                                   hlp ? v3 : 0.0);
+        const double m4 = shfl_d(v4, g0 + 1);
+        // P | u^3
+        const double v5 = __fma_rn(jerk ? v4 : -1.0, jerk ? v3 : v4, jerk ? 0.0 : m4);
+        // x^4 P | 140 x^3
+        const double v6 = __fma_rn(jerk ? 140.0 : v3, jerk ? v2 : v5, 0.0);
+        // w | 140 x^3 u^3
+        const double v7 = __fma_rn(jerk ? v6 : -1.0, jerk ? v5 : v6, jerk ? 0.0 : 1.0);
+        const double ww = shfl_d(v7, g0);
+        const double dk = v7 * hc.i1mg;
+        if (mid) {
+          w = ww;
+          dK = dk;  // read by the jerk lanes only
+        }
+      }
+    }
+    const double rq = F.D[gd][jerk ? c - 3 : c];
+    const double m1 = (jerk ? 3.0 : rinv) * (jerk ? w : rinv);       // 3 w | rinv^2
+    const double rinv2 = shfl_d(m1, g0);
+    const double m2 = m1 * (jerk ? s : rinv);                        // 3 w r.u | rinv^3
+    const double m3 = (jerk ? m2 : Gm) * (jerk ? rinv2 : m2);        // 3 w r.u rinv^2 | g3
+    const double g3 = shfl_d(m3, g0);
+    double out;
+    if (!any_mid) {  // w = 1, dK = 0: f = g3, c = 3 r.u rinv^2
+      out = g3 * (jerk ? __fma_rn(-m3, rq, d) : rq);
+    } else {
+      const double e1 = (jerk ? dK : g3) * (jerk ? s : w);           // dK r.u | f
+      const double e2 = e1 * (jerk ? rinv : rq);                     // dK r.u rinv | f r
+      const double t = __fma_rn(-__fma_rn(e2, irot, m3), rq, w * d);
+      out = jerk ? g3 * t : e2;
+    }
+    if (in) F.T[ti][c] = on && !dead ? out : 0.0;
+    __syncwarp();
+  }
+}
+
+// x 2^k in FP32 from the leading 20 bits of x (relative error below 2^-20);
+// zero below and infinity above FP32's normal range
+__device__ __forceinline__ float lead_float(double x, int k) {
+  const int hi = __double2hiint(x), ef = ((hi >> 20) & 0x7ff) - 896 + k;
+  const unsigned u = ef <= 0 ? 0u : (ef >= 255 ? 0x7f800000u
+                                               : (unsigned)ef << 23 | (unsigned)(hi & 0xfffff) << 3);
+  return __uint_as_float(u);
+}
+// sum of the squares held by the three lanes from l0 on
+__device__ __forceinline__ float norm_lanes(float x, int l0) {
+  const float s = x * x;
+  return __shfl_sync(0xffffffffu, s, l0 & 31) + __shfl_sync(0xffffffffu, s, (l0 + 1) & 31) +
+         __shfl_sync(0xffffffffu, s, (l0 + 2) & 31);
+}
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// the step criterion as first_level and integrate_cluster evaluate it: x1 = a
+// and x2 = a2 in a member's position lanes, j and a3 in its velocity lanes
+__device__ __forceinline__ double exact_step(double x1, double x2, bool vel, int other, int gq, int e,
+                                          bool later, const HConst &hc, double dt) {
+  const float n1 = sqrtf(norm_lanes(scaled_float(x1, vel ? e : 0), gq));
+  const float n2 = sqrtf(norm_lanes(scaled_float(x2, vel ? 3 * e : 2 * e), gq));
+  const float o1 = __shfl_sync(0xffffffffu, n1, other), o2 = __shfl_sync(0xffffffffu, n2, other);
+  const float an = vel ? o1 : n1, jn = vel ? n1 : o1;
+  const float a2n = vel ? o2 : n2, a3n = vel ? n2 : o2;
+  const float num = an * a2n + jn * jn, den = later ? jn * a3n + a2n * a2n : jn;
+  if (!(den > 0.0f)) return dt;
+  return ldexp((double)(later ? sqrtf(hc.etaf * num / den) : hc.eta0f * an / jn), e);
+}
+
+// block-step integration of a cluster of 2..5 members by one warp: the values
+// of integrate_cluster.  Returns true when done; when members touch (a
+// composite is to be formed, rare) the state goes to S and *tn, and
+// integrate_cluster carries on from there.
+template <class V>
+__device__ bool integrate_five(const V &S, HFive &F, int64_t off, int nc, const int32_t *cl_mem,
+                               const p3t_particles &p, const p3t_params &prm, const HConst &hc,
+                               double dt, bool coll, unsigned long long &steps, bool &underflow,
+                               DevStatus *st, int64_t iter_limit, int32_t *rec, int64_t *tn_out,
+                               int64_t *iter_out) {
+  const int lane = threadIdx.x & 31, g = lane / 6, c = lane - 6 * g, q = c >= 3 ? c - 3 : c;
+  const bool vel = c >= 3;
+  const int other = g < kFive ? (vel ? lane - 3 : lane + 3) : lane;
+  const int g0 = lane - c, gq = g0 + (vel ? 3 : 0);  // first lane of the member, of this half
+  const bool mine = g < nc;
+  const int64_t T = ((int64_t)1) << P3T_KMAX;
+  const long long bd = __double_as_longlong(dt);
+  const int e_unit = ((__double2hiint(hc.unit) >> 20) & 0x7ff) - 1023;
+  // per-lane constants of the slots: positions | velocities
+  const double b1 = vel ? 2.0 / 6.0 : hc.unit, o1 = vel ? -0.0 : hc.m52u;
+  const double kap = vel ? 1.0 : 2.0, del = vel ? 12.0 : -6.0;
+  const double gD0 = vel ? hc.unit6 : -2.0 * hc.unit, iD0 = vel ? hc.idt3 : hc.idt2;
+  const double h0 = vel ? hc.c3u : hc.c4u, h1c = vel ? hc.c4u : hc.c5u;
+  const int ni = vel ? 3 : 2, nh0 = vel ? 3 : 4, nh1 = vel ? 4 : 5;
+  int32_t i = 0;
+  double s0 = 0.0, vq = 0.0, a = 0.0, j = 0.0;
+  if (mine) {
+    i = cl_mem[off + g];
+    const double *X = q == 0 ? p.x : (q == 1 ? p.y : p.z);
+    const double *W = q == 0 ? p.vx : (q == 1 ? p.vy : p.vz);
+    vq = W[i];
+    s0 = vel ? vq : X[i];
+    F.P[g][c] = s0;
+    if (c == 0) {
+      F.gm[g] = prm.G * p.m[i];
+      F.partner[g] = kNone;
+      if (rec) rec[i] = 0;
+    }
+    if (c == 1) {
+      const double iro = 1.0 / p.r_out[i];
+      const float f = (float)iro;
+      F.iro[g] = iro;
+      F.irf2[g] = f * f;
+    }
+  }
+  if (lane < 6) F.P[kFive][lane] = 0.0;
+  if (lane == 6) { F.gm[kFive] = hc.gms; F.iro[kFive] = 0.0; F.irf2[kFive] = 0.0f; }
+  if (coll && lane < kFive * kFive) {
+    const int k = lane / kFive, l = lane - kFive * k;
+    if (k < nc && l < nc) {
+      const double sr = prm.f_radius * (p.r_phys[cl_mem[off + k]] + p.r_phys[cl_mem[off + l]]);
+      F.sr2[lane] = sr * sr;
+    }
+  }
+  __syncwarp();
+  bool uf = false, hit = false, done = true;
+  int64_t t = 0, tn = 0, iter = 0;
+  int lvl = 0, nact = nc;
+  unsigned act = 0x43210;  // the active members, four bits each
+  double pred = s0;
+  int64_t e_end = 0;       // end of the member's step; the initial evaluation is at 0
+  for (;;) {
+    const bool on = mine && e_end == tn;
+    five_terms(F, nc, nact, act, prm, hc, coll);
+    // the fixed order: star, then the sources by index
+    double a1 = 0.0, j1 = 0.0;
+    {
+      const unsigned bal = __ballot_sync(0xffffffffu, on && c == 0);
+      const int b = on ? __popc(bal & ((1u << g0) - 1u)) : 0;
+      const double *t = F.T[b * nc] + c;
+      double acc = -t[6 * (nc - 1)] - t[0];
+      if (nc > 2) acc -= t[6];
+      if (nc > 3) acc -= t[12];
+      if (nc > 4) acc -= t[18];
+      const double oa = shfl_d(acc, other);
+      a1 = vel ? oa : acc;
+      j1 = vel ? acc : oa;
+    }
+    double A2 = 0.0, A3 = 0.0, a2e = 0.0;
+    int e;  // the step criterion's scale 2^e
+    if (iter > 0) {
+      const int sh = P3T_KMAX - lvl;
+      // A2 = (-D (2 j1 + 4 j0) - 6 da) / D^2, A3 = (6 D (j0 + j1) + 12 da) /
+      // D^3 (the factor 2 of A2's sum moved to D, exactly)
+      const double da = a - a1;
+      const double sj = __fma_rn(kap, j, j1);
+      const double A = __fma_rn(shift_exp(gD0, sh), sj, del * da) * shift_exp(iD0, ni * lvl);
+      const double oA = shfl_d(A, other);
+      A2 = vel ? oA : A;
+      A3 = vel ? A : oA;
+      const double h = __fma_rn(A2, shift_exp(h0, nh0 * sh), pred);
+      const double sn = __fma_rn(A3, shift_exp(h1c, nh1 * sh), h);
+      a2e = __fma_rn(shift_exp(hc.unit, sh), A3, A2);
+      const double on_v = shfl_d(sn, other);
+      if (on) {
+        s0 = sn;
+        vq = vel ? sn : on_v;
+      }
+      e = e_unit + sh;
+    } else {
+      e = e_unit + P3T_KMAX;
+    }
+    // the new step, first from norms good to 1e-5 (components by their leading
+    // 20 bits, approximate roots): |a| and |a2| in the position lanes, |j| and
+    // |a3| in the velocity lanes.  Its level is the exact one's unless it lies
+    // within 2^-14 of a power of two times dt (or out of range): then the
+    // criterion is evaluated as written
+    double dtd;
+    {
+      const float x1 = lead_float(vel ? j1 : a1, vel ? e : 0);
+      const float x2 = lead_float(vel ? A3 : a2e, vel ? 3 * e : 2 * e);
+      const float n1 = norm_lanes(x1, gq), n2 = norm_lanes(x2, gq);
+      const float o1 = __shfl_sync(0xffffffffu, n1, other),
+                  o2 = __shfl_sync(0xffffffffu, n2, other);
+      const float an = vel ? o1 : n1, jn = vel ? n1 : o1;  // squared
+      const float a2n = vel ? o2 : n2, a3n = vel ? n2 : o2;
+      float r;
+      if (iter > 0) {
+        r = sqrt_approx(__fdividef(hc.etaf * (sqrt_approx(an * a2n) + jn),
+                                   sqrt_approx(jn * a3n) + a2n));
+      } else {  // first step eta0 |a| / |j|
+        r = hc.eta0f * sqrt_approx(__fdividef(an, jn));
+      }
+      const unsigned u = __float_as_uint(r);
+      const int er = (int)(u >> 23) - 127 + 1023 + e;
+      const bool fine = an > 1e-30f && an < 1e30f && jn > 1e-30f && jn < 1e30f &&
+                        (iter == 0 || (a2n > 1e-30f && a2n < 1e30f && a3n > 1e-30f && a3n < 1e30f)) &&
+                        r > 1e-30f && r < 1e30f && er > 0 && er < 2047;
+      const long long bs = (long long)er << 52 | (long long)(u & 0x7fffffu) << 29;
+      const long long frac = (bs - bd) & 0xfffffffffffffLL, lim = 1LL << 38;
+      dtd = __longlong_as_double(bs);
+      if (__any_sync(0xffffffffu, on && (!fine || frac < lim || frac > (1LL << 52) - lim)))
+        dtd = exact_step(vel ? j1 : a1, vel ? A3 : a2e, vel, other, gq, e, iter > 0, hc, dt);
+    }
+    if (on) {
+      lvl = level_bits(dtd, bd, iter > 0 ? lvl : 0, tn, uf);
+      a = a1;
+      j = j1;
+      t = tn;
+      if (iter > 0 && rec && c == 0) rec[i] += 1;
+      if (coll) hit = F.partner[g] != kNone;
+    }
+    if (iter > 0) steps += lane == 0 ? (unsigned long long)nact : 0ull;
+    if (__any_sync(0xffffffffu, uf || hit)) {
+      if (__any_sync(0xffffffffu, uf)) break;  // a step below dt / 2^40 ends the integration
+      done = false;
+      break;
+    }
+    // every step ends at or before T, so all members are at T once a block
+    // time was T
+    if (tn >= T) break;
+    e_end = mine ? t + (T >> lvl) : T;
+    tn = warp_min64(e_end < T ? e_end : T);
+    if (++iter > iter_limit) {
+      if (lane == 0) dev_fail(st, P3T_ERR_TIMEOUT, 61, 0);
+      break;
+    }
+    // predict: x + D (v + D (a/2 + D j/6)), v + D (a + D j/2), with D = RN(n
+    // unit) = fma(2^52 + n, unit, -2^52 unit) for the n units since t, and
+    // the halves moved to D (exact)
+    const long long n = tn - t;
+    const double mg = __longlong_as_double(0x4330000000000000LL + n);
+    const double s1 = __fma_rn(vel ? j : mg, b1, o1);
+    const double os = shfl_d(s1, other);
+    const double D = vel ? os : s1, Dh = shift_exp(D, -1);
+    const double s2 = __fma_rn(vel ? j : os, vel ? Dh : D, a);
+    const double s3 = __fma_rn(s2, vel ? D : Dh, vq);
+    const double s4 = __fma_rn(s3, D, s0);
+    pred = vel ? s3 : s4;
+    if (mine) F.P[g][c] = pred;
+    const unsigned bal = __ballot_sync(0xffffffffu, mine && e_end == tn && c == 0);
+    act = 0;
+    nact = 0;
+#pragma unroll
+    for (int m = 0; m < kFive; ++m)
+      if ((bal >> (6 * m)) & 1u) { act |= (unsigned)m << (4 * nact); ++nact; }
+    __syncwarp();
+  }
+  if (done) {
+    if (mine) {
+      double *X = q == 0 ? p.x : (q == 1 ? p.y : p.z);
+      double *W = q == 0 ? p.vx : (q == 1 ? p.vy : p.vz);
+      (vel ? W : X)[i] = s0;
+    }
+  } else if (mine) {
+    (vel ? S.v(q, g) : S.x(q, g)) = s0;
+    (vel ? S.pv(q, g) : S.p(q, g)) = pred;
+    (vel ? S.j(q, g) : S.a(q, g)) = vel ? j : a;
+    if (c == 0) {
+      S.m(g) = p.m[i];
+      S.iro(g) = F.iro[g];
+      S.rp(g) = p.r_phys[i];
+      S.set(g) = g;
+      S.partner(g) = F.partner[g];
+      S.t(g) = t;
+      S.lvl(g) = lvl;
+    }
+  }
+  *tn_out = tn;
+  *iter_out = iter;
+  if (uf) underflow = true;
+  __syncwarp();
+  return done;
+}
+
 // clusters of nc_lo..nc_hi members; NT threads per block; state in shared
 // memory for up to KM members or (BIG) in the global workspace.  One block
 // per cluster, clusters handed out dynamically (a long encounter keeps its
 // block while the others move on).
 template <int NT, int KM, bool BIG>
-__global__ void __launch_bounds__(NT) k_hermite_block(
+__global__ void __launch_bounds__(NT, NT == 32 ? 20 : 1) k_hermite_block(
     const int64_t *d_ncl, const int64_t *cl_off, const int32_t *cl_mem, p3t_particles p,
-    p3t_params prm, double dt, int nc_lo, int nc_hi, unsigned long long *steps_out,
+    p3t_params prm, HConst hc, double dt, int nc_lo, int nc_hi, unsigned long long *steps_out,
     int64_t *cursor, const int32_t *list, const int64_t *d_nlist, HBig big, CollOut co,
     DevStatus *st, int64_t iter_limit, int32_t *rec) {
   pdl_wait();
@@ -1022,7 +1442,11 @@ __global__ void __launch_bounds__(NT) k_hermite_block(
     // encounter keeps its block while the others move on); the rare larger
     // ones are dealt statically
     int64_t c = k;
-    if constexpr (!BIG) {
+    if constexpr (NT == 32) {
+      unsigned long long u = 0;
+      if (tid == 0) u = atomicAdd(reinterpret_cast<unsigned long long *>(cursor), 1ull);
+      c = (int64_t)__shfl_sync(0xffffffffu, u, 0);
+    } else if constexpr (!BIG) {
       if (tid == 0) C.cluster = atomicAdd(reinterpret_cast<unsigned long long *>(cursor), 1ull);
       __syncthreads();
       c = C.cluster;
@@ -1035,12 +1459,23 @@ __global__ void __launch_bounds__(NT) k_hermite_block(
     if (nc < nc_lo || nc > nc_hi) continue;
     if constexpr (BIG) {
       const BigView S{big.d, big.t, big.i, big.cap, off};
-      integrate_cluster<NT>(S, C, nullptr, off, nc, cl_mem, p, prm, dt, coll, co, steps,
-                            underflow, st, iter_limit, rec);
+      integrate_cluster<NT>(S, C, nullptr, off, nc, cl_mem, p, prm, hc, dt, coll, co, steps,
+                            underflow, st, iter_limit, rec, false, 0, 0);
     } else {
       const SmallView<KM> S{Sm};
-      integrate_cluster<NT>(S, C, Sm->T, off, nc, cl_mem, p, prm, dt, coll, co, steps,
-                            underflow, st, iter_limit, rec);
+      bool resume = false;
+      int64_t tn = 0, iter = 0;
+      if constexpr (NT == 32) {
+        __shared__ HFive F;
+        if (nc <= kFive && hc.fast) {
+          if (integrate_five(S, F, off, nc, cl_mem, p, prm, hc, dt, coll, steps, underflow, st,
+                             iter_limit, rec, &tn, &iter))
+            continue;
+          resume = true;
+        }
+      }
+      integrate_cluster<NT>(S, C, Sm->T, off, nc, cl_mem, p, prm, hc, dt, coll, co, steps,
+                            underflow, st, iter_limit, rec, resume, tn, iter);
     }
   }
   if (underflow) dev_fail(st, P3T_ERR_DT_UNDERFLOW, 62, 0);
@@ -1265,6 +1700,32 @@ __global__ void k_iota(int64_t n, int32_t *a) {
     a[i] = (int32_t)i;
 }
 
+// a step of level l is D = unit 2^(40 - l) exactly, so D^n = RN(unit^n)
+// 2^(n (40 - l)) and RN(D^n c) = RN(unit^n c) 2^(n (40 - l)) with unit^n
+// formed by successive products: the corrector's powers of D and of 1/D are
+// these constants shifted in the exponent (the same bits as the products, no
+// FP64 instruction)
+HConst hermite_const(const p3t_params &prm, double dt) {
+  HConst h;
+  h.unit = ldexp(dt, -P3T_KMAX);
+  h.unit6 = 6.0 * h.unit;
+  h.m52u = -4503599627370496.0 * h.unit;
+  const double u2 = h.unit * h.unit, u3 = u2 * h.unit, u4 = u3 * h.unit, u5 = u4 * h.unit;
+  h.c3u = u3 * (1.0 / 6.0);
+  h.c4u = u4 * (1.0 / 24.0);
+  h.c5u = u5 * (1.0 / 120.0);
+  const double idt = 1.0 / dt;
+  h.idt2 = idt * idt;
+  h.idt3 = h.idt2 * idt;
+  h.i1mg = 1.0 / (1.0 - prm.gamma);
+  h.gms = prm.G * prm.m_star;
+  h.etaf = (float)prm.eta;
+  h.eta0f = (float)prm.eta0;
+  h.gin2 = (float)(prm.gamma * prm.gamma * (1.0 - 1e-5));
+  h.fast = dt >= 1e-30 && dt <= 1e30;
+  return h;
+}
+
 CollOut coll_out(p3t_ctx *c) {
   CollOut co;
   co.ctr = c->coll_ctr;
@@ -1313,6 +1774,7 @@ int p3t_run_hard_step(p3t_ctx *c, p3t_particles *p, const p3t_clusters *cl,
   P3T_CUDA_TRY(cudaStreamWaitEvent(c->aux[0], c->ev_fork, 0));
   P3T_CUDA_TRY(cudaStreamWaitEvent(c->aux[1], c->ev_fork, 0));
   const int64_t ncl_max = (n / 2) > 0 ? n / 2 : 1;
+  const HConst hc = hermite_const(c->prm, dt);
   const int64_t nbig = c->num_sms < 32 ? c->num_sms : 32;
   // clusters of 2..hw members: a warp each (stream aux[0]), up to 32 such
   // one-warp blocks an SM (the FP64 latency of their block steps, not the
@@ -1321,25 +1783,25 @@ int p3t_run_hard_step(p3t_ctx *c, p3t_particles *p, const p3t_clusters *cl,
   const unsigned gw = (unsigned)p3t_grid(ncl_max * 32, 32, (int64_t)c->num_sms * 32);
   if (hw <= 8)
     pdl_launch(k_hermite_block<32, 8, false>, dim3(gw), dim3(32), sizeof(HSmall<8>), c->aux[0], 
-        &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, dt, 2, hw, steps, c->hcursor,
+        &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, hc, dt, 2, hw, steps, c->hcursor,
         (const int32_t *)nullptr, (const int64_t *)nullptr, big, co, c->status, c->hermite_limit,
         c->hermite_rec);
   else if (hw <= 16)
     pdl_launch(k_hermite_block<32, 16, false>, dim3(gw), dim3(32), sizeof(HSmall<16>), c->aux[0], 
-        &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, dt, 2, hw, steps, c->hcursor,
+        &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, hc, dt, 2, hw, steps, c->hcursor,
         (const int32_t *)nullptr, (const int64_t *)nullptr, big, co, c->status, c->hermite_limit,
         c->hermite_rec);
   else
     pdl_launch(k_hermite_block<32, 32, false>, dim3(gw), dim3(32), sizeof(HSmall<32>), c->aux[0], 
-        &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, dt, 2, hw, steps, c->hcursor,
+        &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, hc, dt, 2, hw, steps, c->hcursor,
         (const int32_t *)nullptr, (const int64_t *)nullptr, big, co, c->status, c->hermite_limit,
         c->hermite_rec);
   pdl_launch(k_hermite_block<128, kHMax, false>, dim3((unsigned)p3t_grid(ncl_max * 128, 128, (int64_t)c->num_sms * 2)), dim3(128), sizeof(HSmall<kHMax>), c->aux[1], 
-      &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, dt, hw + 1, kHMax, steps,
+      &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, hc, dt, hw + 1, kHMax, steps,
       c->hcursor + 1, (const int32_t *)c->hlist, (const int64_t *)(c->hcursor + 3),
       big, co, c->status, c->hermite_limit, c->hermite_rec);
   pdl_launch(k_hermite_block<128, 1, true>, dim3((unsigned)p3t_grid(ncl_max, 1, nbig)), dim3(128), 0, c->aux[1], 
-      &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, dt, kHMax + 1, 0x7fffffff, steps,
+      &cl->counts[1], cl->cl_off, cl->cl_mem, *p, c->prm, hc, dt, kHMax + 1, 0x7fffffff, steps,
       c->hcursor + 2, (const int32_t *)(c->hlist + c->hlist_cap),
       (const int64_t *)(c->hcursor + 4), big, co, c->status, c->hermite_limit, c->hermite_rec);
   KepConst kc;
