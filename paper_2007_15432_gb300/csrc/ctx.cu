@@ -116,7 +116,7 @@ int reserve(p3t_ctx *c, int64_t n, int64_t cand_cap) {
   c->node_cap = NC;
   c->cand_cap = cand_cap;
   c->walk_warps = p3t_walk_warps(c->num_sms, N);
-  c->stack_cap = kStackCap;
+  c->stack_cap = kStackCap < NC ? kStackCap : NC;  // a walk pushes a node at most once
   c->radix_hist_cap = p3t_radix_hist_entries(N > NC ? N : NC);
   bool ok = true;
   ok &= dalloc(c->keys, N) && dalloc(c->keys_alt, N) && dalloc(c->idx, N) && dalloc(c->idx_alt, N);

@@ -1178,14 +1178,6 @@ __device__ __forceinline__ void five_terms(HFive &F, int nc, int nact, unsigned 
   }
 }
 
-// x 2^k in FP32 from the leading 20 bits of x (relative error below 2^-20);
-// zero below and infinity above FP32's normal range
-__device__ __forceinline__ float lead_float(double x, int k) {
-  const int hi = __double2hiint(x), ef = ((hi >> 20) & 0x7ff) - 896 + k;
-  const unsigned u = ef <= 0 ? 0u : (ef >= 255 ? 0x7f800000u
-                                               : (unsigned)ef << 23 | (unsigned)(hi & 0xfffff) << 3);
-  return __uint_as_float(u);
-}
 // sum of the squares held by the three lanes from l0 on
 __device__ __forceinline__ float norm_lanes(float x, int l0) {
   const float s = x * x;

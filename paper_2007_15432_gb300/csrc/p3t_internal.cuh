@@ -59,6 +59,32 @@ __device__ __forceinline__ FF ff_rsqrt(FF r2) {
   return ff_fast(y, 0.5f * y * d);
 }
 
+// ---- inverse powers of a distance in FP64 -----------------------------------------
+// On this part an FP64 warp instruction costs 64 cycles of its sub-partition
+// (76 with all four busy), the 20-bit reciprocal square root seed 8 on
+// another pipe.  With y the seed and e = 1 - x y^2 (|e| <= 2^-19, measured
+// over all leading mantissas), x^(-3/2) = y^3 (1 - e)^(-3/2) = y^3 (1 + 3/2 e +
+// 15/8 e^2 + O(2.2 e^3)): the rest is below 2^-55, so the result carries only
+// its last rounding and y^3's, and takes 6 FP64 instructions where rsqrt()
+// cubed takes 7 to 8 and three more roundings.  Valid for x well inside the
+// normal range (rsqrt_seed_ok); x = 0 must be excluded by the caller.
+__device__ __forceinline__ double rsqrt_seed(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ bool rsqrt_seed_ok(double x) {  // 2^-511 <= x < 2^513
+  return (unsigned)((__double2hiint(x) >> 20) - 512) < 1024u;
+}
+// x 2^k in FP32 from the leading 20 bits of x (relative error below 2^-20,
+// towards zero); zero below and infinity above FP32's normal range
+__device__ __forceinline__ float lead_float(double x, int k) {
+  const int hi = __double2hiint(x), ef = ((hi >> 20) & 0x7ff) - 896 + k;
+  const unsigned u = ef <= 0 ? 0u : (ef >= 255 ? 0x7f800000u
+                                               : (unsigned)ef << 23 | (unsigned)(hi & 0xfffff) << 3);
+  return __uint_as_float(u | ((unsigned)hi & 0x80000000u));
+}
+
 // ---- packed FP32 pairs ----------------------------------------------------------
 // a pair of floats in one 64-bit register (low half: the first value); the
 // .f32x2 instructions round each half as the scalar instruction would

@@ -3,8 +3,8 @@
 // One warp per target group (the highest tree node holding <= group_size
 // particles, or a leaf), 32 targets per walk (larger groups are taken 32
 // targets at a time; the warps take a group's first 32 targets and its rest
-// as separate units of work, each walking with the whole group's box).  A walk of k < 32 targets gives each target r =
-// floor(32 / k) lanes, each of which takes every r-th entry of a batch; the
+// as separate units of work, each walking with the whole group's box).  A walk
+// of k < 32 targets gives each target r = floor(32 / k) lanes, each of which takes every r-th entry of a batch; the
 // r partial sums are added at the end, so that lanes are not left idle.  The
 // walk pops up to 32 nodes at a time from a per-warp stack, decides opening
 // for all of them at once on the integer grid, and compacts accepted nodes,
@@ -23,8 +23,8 @@
 // one issue for two lanes' worth of FP32 work per thread), the batch staged
 // so that one 16-byte shared load gives one coordinate of both entries;
 // replicas split a batch by pairs, and each pair slot keeps its own partial
-// sum (even and odd entries) until the batch is folded.  FP64 path:
-// everything in FP64.
+// sum (even and odd entries) until the batch is folded.  The FP64 path
+// (k_walk64) shares the traversal and has a layout of its own.
 #include "p3t_internal.cuh"
 
 namespace {
@@ -58,6 +58,7 @@ struct WalkArgs {
   int64_t *cursor;
   DevStatus *st;
   SegView seg;                     // segments: the root of segment d is node d
+  int group_max;                   // largest target group but for oversized leaves
   double G, gamma;
   double inv1mg;                   // 1 / (1 - gamma)
   float inv1mg_f, mgi_f;           // 1 / (1 - gamma), -gamma / (1 - gamma)
@@ -102,9 +103,7 @@ constexpr int kPairUnroll = P3T_PAIR_UNROLL;
 
 
 // ---- per-target state (one lane per target) ---------------------------------
-template <bool MIXED> struct Target;
-
-template <> struct Target<true> {
+struct Target {
   f2 X, Y, Z, XL, YL, ZL;              // (hi, hi) and (lo, lo) of each coordinate
   float inv_ro, rs2;                   // rs2: r_search^2 with the FP32 margin
   float ahx, ahy, ahz, alx, aly, alz;  // float-float accumulators
@@ -155,36 +154,6 @@ template <> struct Target<true> {
   }
 };
 
-template <> struct Target<false> {
-  double x, y, z, iro, rs;  // iro = 1 / r_out
-  double ax, ay, az;
-  int32_t self;
-  int rep, nrep;
-  bool valid;
-  __device__ void load(const WalkArgs &a, int32_t ti, bool v, int r, int nr) {
-    valid = v;
-    self = ti;
-    rep = r;
-    nrep = nr;
-    ax = ay = az = 0.0;
-    if (v) {
-      x = a.sx[ti]; y = a.sy[ti]; z = a.sz[ti]; iro = 1.0 / a.sro[ti]; rs = a.srs[ti];
-    } else {
-      x = y = z = 1.0e300; iro = 1.0; rs = 0.0;
-    }
-  }
-  __device__ void reduce(int k) {
-    const int lane = threadIdx.x & 31;
-    for (int q = 1; q < nrep; ++q) {
-      const int src = lane < k ? lane + q * k : lane;
-      const double x2 = __shfl_sync(0xffffffffu, ax, src);
-      const double y2 = __shfl_sync(0xffffffffu, ay, src);
-      const double z2 = __shfl_sync(0xffffffffu, az, src);
-      if (lane < k) { ax += x2; ay += y2; az += z2; }
-    }
-  }
-};
-
 __device__ __forceinline__ void record_candidate(const WalkArgs &a, int32_t i,
                                                  int32_t j) {
   const unsigned long long slot = atomicAdd(a.cand_count, 1ull);
@@ -209,9 +178,7 @@ struct StagePP32 {
 struct StageND32 {
   ulonglong2 hxy[16], hzw[16], lxy[16], lzw[16], q0xy[16], q0zw[16], q1xy[16];
 };
-struct StagePP64 { double x[32], y[32], z[32], m[32], iro[32], rs[32]; int32_t idx[32]; };
-static_assert(sizeof(StagePP32) <= kStageBytes && sizeof(StagePP64) <= kStageBytes &&
-              sizeof(StageND32) <= kStageBytes && sizeof(Mom64) * 32 <= kStageBytes,
+static_assert(sizeof(StagePP32) <= kStageBytes && sizeof(StageND32) <= kStageBytes,
               "stage area");
 
 // entry s of a pair-staged batch: component c (0..3) of word w
@@ -230,7 +197,7 @@ __device__ __forceinline__ void stage_put(ulonglong2 *w, int s, float v0, float 
 // max(r_search^2) (squared and widened in the gather); far-away dummy targets
 // and the massless dummy entry that pads an odd batch never pass it.  The
 // batch sums are kept negated (B = -sum f dx), which is exact.
-__device__ __forceinline__ void pp_pair(const WalkArgs &a, Target<true> &t,
+__device__ __forceinline__ void pp_pair(const WalkArgs &a, Target &t,
                                         const StagePP32 &S, int p, f2 &BX, f2 &BY, f2 &BZ,
                                         f2 &TB, unsigned &npp) {
   const ulonglong2 axy = S.axy[p], azw = S.azw[p], bxy = S.bxy[p], bzw = S.bzw[p];
@@ -291,31 +258,9 @@ __device__ __forceinline__ bool far_from(const FarBox &b, const float4 A, const 
   return d2 > 0.f && d2 >= R2;
 }
 
-// The FP64 walk's counterpart: the targets' box in FP64 and the largest
-// max(r_search, r_out)^2 of its targets.  A source whose distance to the box
-// exceeds max(r_search, r_out) of the source and of every target by a
-// relative 1e-9 (far above the rounding of the pair's r and y) has y >= 1
-// (K = 1 exactly) and r^2 >= r_search,max^2 for every target: the far
-// evaluation below then gives the bits of the full one.
-struct FarBox64 {
-  double lo[3], hi[3], R2;
-};
-template <bool MIXED> struct BoxOf { using type = FarBox; };
-template <> struct BoxOf<false> { using type = FarBox64; };
-
-__device__ __forceinline__ bool far_from64(const FarBox64 &b, double x, double y, double z,
-                                           double ro, double rs) {
-  const double gx = fmax(fmax(b.lo[0] - x, x - b.hi[0]), 0.0);
-  const double gy = fmax(fmax(b.lo[1] - y, y - b.hi[1]), 0.0);
-  const double gz = fmax(fmax(b.lo[2] - z, z - b.hi[2]), 0.0);
-  const double d2 = gx * gx + gy * gy + gz * gz;
-  const double R2 = fmax(b.R2, fmax(rs * rs, ro * ro));
-  return d2 > 0.0 && d2 >= R2 * (1.0 + 1e-9);
-}
-
 // pair terms with K = 1 and no candidate test (the batch is far, see above):
 // the same operations as pp_pair's K = 1 case, so the same bits
-__device__ __forceinline__ void pp_pair_far(Target<true> &t, const StagePP32 &S, int p, f2 &BX,
+__device__ __forceinline__ void pp_pair_far(Target &t, const StagePP32 &S, int p, f2 &BX,
                                             f2 &BY, f2 &BZ, f2 &TB) {
   const ulonglong2 axy = S.axy[p], azw = S.azw[p], bxy = S.bxy[p], bzw = S.bzw[p];
   const f2 dx = add2(sub2(t.X, axy.x), sub2(t.XL, bxy.x));
@@ -333,12 +278,12 @@ __device__ __forceinline__ void pp_pair_far(Target<true> &t, const StagePP32 &S,
 
 // the batch sums of the even and odd slots into the target: the force sums
 // negated back (B = -sum), the magnitude sum as it is
-__device__ __forceinline__ void fold_pairs(Target<true> &t, f2 BX, f2 BY, f2 BZ, f2 TB) {
+__device__ __forceinline__ void fold_pairs(Target &t, f2 BX, f2 BY, f2 BZ, f2 TB) {
   t.fold(-(f2_lo(BX) + f2_hi(BX)), -(f2_lo(BY) + f2_hi(BY)), -(f2_lo(BZ) + f2_hi(BZ)));
   t.tabs += f2_lo(TB) + f2_hi(TB);
 }
 
-__device__ __forceinline__ void eval_pp(const WalkArgs &a, Target<true> &t, const int32_t *list,
+__device__ __forceinline__ void eval_pp(const WalkArgs &a, Target &t, const int32_t *list,
                                         int nsrc, void *stage, const FarBox &box,
                                         unsigned &npp) {
   StagePP32 &S = *reinterpret_cast<StagePP32 *>(stage);
@@ -377,64 +322,10 @@ __device__ __forceinline__ void eval_pp(const WalkArgs &a, Target<true> &t, cons
   fold_pairs(t, BX, BY, BZ, TB);
 }
 
-__device__ __forceinline__ void eval_pp(const WalkArgs &a, Target<false> &t, const int32_t *list,
-                                        int nsrc, void *stage, const FarBox64 &box,
-                                        unsigned &npp) {
-  StagePP64 &S = *reinterpret_cast<StagePP64 *>(stage);
-  const int lane = threadIdx.x & 31;
-  bool near = false;
-  if (lane < nsrc) {
-    const int32_t j = list[lane];
-    const double x = a.sx[j], y = a.sy[j], z = a.sz[j], ro = a.sro[j], rs = a.srs[j];
-    S.x[lane] = x; S.y[lane] = y; S.z[lane] = z;
-    S.m[lane] = a.sm[j]; S.iro[lane] = 1.0 / ro; S.rs[lane] = rs;
-    S.idx[lane] = j;
-    near = !far_from64(box, x, y, z, ro, rs);
-  }
-  const bool any_near = __any_sync(0xffffffffu, near);
-  __syncwarp();
-  npp += (t.valid && t.rep == 0) ? (unsigned)nsrc : 0u;
-  if (!any_near) {
-    // K = 1 for every pair and no candidate: the full loop's operations with
-    // K = 1 (m K = m exactly)
-    for (int s = t.rep; s < nsrc; s += t.nrep) {
-      const double dx = t.x - S.x[s], dy = t.y - S.y[s], dz = t.z - S.z[s];
-      const double r2 = dx * dx + dy * dy + dz * dz;
-      const double rinv = r2 > 0.0 ? rsqrt(r2) : 0.0;
-      const double f = S.m[s] * (rinv * rinv * rinv);
-      t.ax -= f * dx; t.ay -= f * dy; t.az -= f * dz;
-    }
-    __syncwarp();
-    return;
-  }
-  for (int s = t.rep; s < nsrc; s += t.nrep) {
-    const double dx = t.x - S.x[s], dy = t.y - S.y[s], dz = t.z - S.z[s];
-    const double r2 = dx * dx + dy * dy + dz * dz;
-    const double rinv = r2 > 0.0 ? rsqrt(r2) : 0.0;
-    const double r = r2 * rinv;
-    // y = r / max(r_out,i, r_out,j) as r min(1 / r_out): one reciprocal a
-    // staged source, not a division a pair
-    const double y = r * fmin(t.iro, S.iro[s]);
-    double x = (y - a.gamma) * a.inv1mg;
-    x = x < 0.0 ? 0.0 : (x > 1.0 ? 1.0 : x);
-    const double x2 = x * x;
-    const double K = (x2 * x2) * (((-20.0 * x + 70.0) * x - 84.0) * x + 35.0);
-    const double f = S.m[s] * K * (rinv * rinv * rinv);
-    t.ax -= f * dx; t.ay -= f * dy; t.az -= f * dz;
-    const double rsj = fmax(t.rs, S.rs[s]);
-    if (r2 < rsj * rsj && t.valid) {
-      const int32_t j = S.idx[s];
-      if (j != t.self) record_candidate(a, t.self, j);
-      else --npp;
-    }
-  }
-  __syncwarp();
-}
-
 // ---- particle-node batch (monopole + traceless quadrupole) ---------------
 // a += -M r/r^3 + Q.r/r^5 - (5/2)(r.Q.r) r/r^7, r = x_i - com, for the two
 // nodes of pair slot p (the stage holds -M)
-__device__ __forceinline__ void node_pair(Target<true> &t, const StageND32 &S, int p, f2 &BX,
+__device__ __forceinline__ void node_pair(Target &t, const StageND32 &S, int p, f2 &BX,
                                           f2 &BY, f2 &BZ, f2 &TB) {
   const ulonglong2 hxy = S.hxy[p], hzw = S.hzw[p], lxy = S.lxy[p], lzw = S.lzw[p];
   const ulonglong2 q0xy = S.q0xy[p], q0zw = S.q0zw[p], q1xy = S.q1xy[p];
@@ -458,7 +349,7 @@ __device__ __forceinline__ void node_pair(Target<true> &t, const StageND32 &S, i
   TB = fma2(hzw.y, rinv2, TB);  // -M / r^2
 }
 
-__device__ __forceinline__ void eval_nodes(const WalkArgs &a, Target<true> &t,
+__device__ __forceinline__ void eval_nodes(const WalkArgs &a, Target &t,
                                            const int32_t *list, int nnd, void *stage,
                                            unsigned &npn) {
   StageND32 &S = *reinterpret_cast<StageND32 *>(stage);
@@ -490,39 +381,9 @@ __device__ __forceinline__ void eval_nodes(const WalkArgs &a, Target<true> &t,
   t.tabs -= f2_lo(TB) + f2_hi(TB);
 }
 
-__device__ __forceinline__ void eval_nodes(const WalkArgs &a, Target<false> &t,
-                                           const int32_t *list, int nnd, void *stage,
-                                           unsigned &npn) {
-  Mom64 *S = reinterpret_cast<Mom64 *>(stage);
-  const int lane = threadIdx.x & 31;
-  if (lane < nnd) S[lane] = a.mom64[list[lane]];
-  __syncwarp();
-  npn += (t.valid && t.rep == 0) ? (unsigned)nnd : 0u;
-  for (int s = t.rep; s < nnd; s += t.nrep) {
-    const Mom64 &m = S[s];
-    const double dx = t.x - m.cx, dy = t.y - m.cy, dz = t.z - m.cz;
-    const double r2 = dx * dx + dy * dy + dz * dz;
-    const double rinv = r2 > 0.0 ? rsqrt(r2) : 0.0;
-    const double rinv2 = rinv * rinv, rinv3 = rinv2 * rinv, rinv5 = rinv3 * rinv2;
-    const double qx = m.qxx * dx + m.qxy * dy + m.qxz * dz;
-    const double qy = m.qxy * dx + m.qyy * dy + m.qyz * dz;
-    const double qz = m.qxz * dx + m.qyz * dy + m.qzz * dz;
-    const double rqr = dx * qx + dy * qy + dz * qz;
-    const double c = -m.M * rinv3 - 2.5 * rqr * rinv5 * rinv2;
-    t.ax += c * dx + qx * rinv5;
-    t.ay += c * dy + qy * rinv5;
-    t.az += c * dz + qz * rinv5;
-  }
-  __syncwarp();
-}
-
 // writes the target's acceleration; returns whether the target is to be
-// redone in float-float (mixed path)
-template <bool MIXED>
-__device__ __forceinline__ bool write_result(const WalkArgs &a, Target<MIXED> &t);
-
-template <>
-__device__ __forceinline__ bool write_result<true>(const WalkArgs &a, Target<true> &t) {
+// redone in float-float
+__device__ __forceinline__ bool write_result(const WalkArgs &a, Target &t) {
   if (!t.valid || t.rep != 0) return false;
   const double x = (double)t.ahx + (double)t.alx;
   const double y = (double)t.ahy + (double)t.aly;
@@ -533,14 +394,6 @@ __device__ __forceinline__ bool write_result<true>(const WalkArgs &a, Target<tru
   // much smaller than their magnitudes the target is redone in float-float
   const float amag = sqrtf((float)(x * x + y * y + z * z));
   return t.tabs > a.refine_cf * amag;
-}
-
-template <>
-__device__ __forceinline__ bool write_result<false>(const WalkArgs &a, Target<false> &t) {
-  if (!t.valid || t.rep != 0) return false;
-  const int32_t i = a.idx[t.self];
-  a.ax[i] = a.G * t.ax; a.ay[i] = a.G * t.ay; a.az[i] = a.G * t.az;
-  return false;
 }
 
 // ---- the traversal, shared by the group walk and the float-float redo ------
@@ -696,18 +549,18 @@ __device__ bool traverse(const WalkArgs &a, const GroupBox &gb, int32_t first, i
 
 // up to 32 targets of a group (each on nrep lanes), batches staged in shared
 // memory
-template <bool MIXED> struct GroupEval {
+struct GroupEval {
   const WalkArgs &a;
-  Target<MIXED> &t;
+  Target &t;
   void *stage;
-  const typename BoxOf<MIXED>::type &box;
+  const FarBox &box;
   unsigned &npp, &npn;
   __device__ void nodes(const int32_t *list, int n) { eval_nodes(a, t, list, n, stage, npn); }
   __device__ void pp(const int32_t *list, int n) { eval_pp(a, t, list, n, stage, box, npp); }
 };
 
 // the walk's FarBox from its (valid) targets, written by lane 0
-__device__ __forceinline__ void far_box(const Target<true> &t, FarBox &b) {
+__device__ __forceinline__ void far_box(const Target &t, FarBox &b) {
   const float x = f2_lo(t.X) + f2_lo(t.XL), y = f2_lo(t.Y) + f2_lo(t.YL),
               z = f2_lo(t.Z) + f2_lo(t.ZL);
   const float inf = __int_as_float(0x7f800000);
@@ -732,31 +585,6 @@ __device__ __forceinline__ void far_box(const Target<true> &t, FarBox &b) {
     b.hi[0] = hi0; b.hi[1] = hi1; b.hi[2] = hi2;
     b.R2 = R2;
     b.amax = am;
-  }
-  __syncwarp();
-}
-
-// the FP64 walk's FarBox64 from its (valid) targets, written by lane 0
-__device__ __forceinline__ void far_box64(const Target<false> &t, FarBox64 &b) {
-  const double inf = __longlong_as_double(0x7ff0000000000000ll);
-  double lo0 = t.valid ? t.x : inf, lo1 = t.valid ? t.y : inf, lo2 = t.valid ? t.z : inf;
-  double hi0 = t.valid ? t.x : -inf, hi1 = t.valid ? t.y : -inf, hi2 = t.valid ? t.z : -inf;
-  const double ro = 1.0 / t.iro;
-  double R2 = t.valid ? fmax(t.rs * t.rs, ro * ro) : 0.0;
-  for (int o = 16; o > 0; o >>= 1) {
-    lo0 = fmin(lo0, __shfl_xor_sync(0xffffffffu, lo0, o));
-    lo1 = fmin(lo1, __shfl_xor_sync(0xffffffffu, lo1, o));
-    lo2 = fmin(lo2, __shfl_xor_sync(0xffffffffu, lo2, o));
-    hi0 = fmax(hi0, __shfl_xor_sync(0xffffffffu, hi0, o));
-    hi1 = fmax(hi1, __shfl_xor_sync(0xffffffffu, hi1, o));
-    hi2 = fmax(hi2, __shfl_xor_sync(0xffffffffu, hi2, o));
-    R2 = fmax(R2, __shfl_xor_sync(0xffffffffu, R2, o));
-  }
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) {
-    b.lo[0] = lo0; b.lo[1] = lo1; b.lo[2] = lo2;
-    b.hi[0] = hi0; b.hi[1] = hi1; b.hi[2] = hi2;
-    b.R2 = R2;
   }
   __syncwarp();
 }
@@ -874,8 +702,20 @@ __device__ bool refine_group(const WalkArgs &a, const GroupBox &gb, bool redo, i
 #define P3T_WALK_MINB_MIXED 6  // resident blocks per SM asked of the mixed walk
 #endif
 
-template <bool MIXED>
-__global__ void __launch_bounds__(kWarps * 32, MIXED ? P3T_WALK_MINB_MIXED : 1)
+// the warp's interaction counts to the caller's: a lane that met its target's
+// own entry holds npp below zero, the warp sum is taken modulo 2^32, where a
+// warp's true count fits
+__device__ __forceinline__ void add_counts(const WalkArgs &a, unsigned p, unsigned q) {
+  if (!a.counts) return;
+  p = __reduce_add_sync(0xffffffffu, p);
+  q = __reduce_add_sync(0xffffffffu, q);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&a.counts[0], (unsigned long long)p);
+    atomicAdd(&a.counts[1], (unsigned long long)q);
+  }
+}
+
+__global__ void __launch_bounds__(kWarps * 32, P3T_WALK_MINB_MIXED)
     k_walk(const WalkArgs a) {
   pdl_wait();
   __shared__ int32_t s_pp[kWarps][kPPCap];
@@ -883,7 +723,7 @@ __global__ void __launch_bounds__(kWarps * 32, MIXED ? P3T_WALK_MINB_MIXED : 1)
   __shared__ int32_t s_big[kWarps][kBigCap];
   __shared__ __align__(16) unsigned char s_stage[kWarps][kStageBytes];
   __shared__ int64_t s_bh[P3T_BITS + 1];
-  __shared__ typename BoxOf<MIXED>::type s_box[kWarps];
+  __shared__ FarBox s_box[kWarps];
   if (threadIdx.x <= P3T_BITS) s_bh[threadIdx.x] = a.bh[threadIdx.x];
   __syncthreads();
 
@@ -914,34 +754,279 @@ __global__ void __launch_bounds__(kWarps * 32, MIXED ? P3T_WALK_MINB_MIXED : 1)
     for (int32_t tb = t0; tb < t1 && ok; tb += 32) {
       const int k = min(32, t1 - tb);
       const int nrep = 32 / k, rep = lane / k;
-      Target<MIXED> t;
+      Target t;
       t.load(a, tb + (lane - rep * k), rep < nrep, rep < nrep ? rep : 0, nrep);
-      if constexpr (MIXED) far_box(t, s_box[w]); else far_box64(t, s_box[w]);
-      GroupEval<MIXED> ev{a, t, s_stage[w], s_box[w], npp, npn};
+      far_box(t, s_box[w]);
+      GroupEval ev{a, t, s_stage[w], s_box[w], npp, npn};
       ok = traverse(a, gb, gfirst, stack, s_pp[w], s_nd[w], s_big[w], s_bh, round_limit, ev);
       if (ok) {
         t.reduce(k);
-        const bool redo = write_result<MIXED>(a, t);
-        if constexpr (MIXED)
-          ok = refine_group(a, gb, redo, t.self, gfirst, stack, s_pp[w], s_nd[w], s_big[w],
-                            s_bh, round_limit);
+        const bool redo = write_result(a, t);
+        ok = refine_group(a, gb, redo, t.self, gfirst, stack, s_pp[w], s_nd[w], s_big[w], s_bh,
+                          round_limit);
       }
     }
     if (!ok) break;
   }
-  if (a.counts) {
-    // a replica lane that met its target's own entry holds npp below zero:
-    // the warp sum is taken modulo 2^32, where a warp's true count fits
-    unsigned p = npp, q = npn;
-    for (int o = 16; o > 0; o >>= 1) {
-      p += __shfl_xor_sync(0xffffffffu, p, o);
-      q += __shfl_xor_sync(0xffffffffu, q, o);
+  add_counts(a, npp, npn);
+}
+
+// ---- the FP64 walk ------------------------------------------------------------
+// Bound by the FP64 pipe (a warp instruction per 19 cycles of an SM), with
+// issue slots to spare.  A chunk of up to kChunk targets of a group is walked
+// at a time; a batch of 32 list entries stands in the lanes' registers, one
+// entry a lane, and the chunk's targets (in shared memory, read by broadcast)
+// are taken in turn, each lane adding its entry's term to its own partial sum
+// of that target in shared memory.  Every lane carries an entry whatever the
+// group's size, and a target's sum is 32 partial sums (entry position modulo
+// 32, in list order) added in one fixed tree: it does not depend on the
+// chunk, so the host may choose it by the size of the system.  A batch whose
+// entries are all beyond every target's cut-off reach (decided in FP32 with a
+// margin) skips the changeover and the candidate test; the factor K = 1
+// would leave the same bits.  16 FP64 instructions a far pair, 31 a near one,
+// 37 a node (21, 33 and 42 with one lane a target, rsqrt() and 0.6-0.9 of the
+// lanes in use): N = 1e5 ring, theta 0.5, 4,790 -> 2,700 us a
+// walk (93 % of the FP64 pipe's instruction rate); 3 to 5 blocks an SM and
+// chunks of 4 or 8 within 2 %.
+constexpr int kChunk = 8;
+constexpr int kWalk64Blocks = 4;
+struct Targets64 {
+  double x[kChunk], y[kChunk], z[kChunk], iro[kChunk];
+  int32_t rs2[kChunk];  // leading bits of r_search^2
+  double acc[kChunk * 3][33];  // a row's 32 partial sums (33: columns in different banks)
+};
+
+// FP32 box of the chunk and its largest max(r_search, r_out)^2, as FarBox
+__device__ __forceinline__ void far_box64(const WalkArgs &a, int32_t t0, int nt, FarBox &b) {
+  const int lane = threadIdx.x & 31;
+  const int32_t i = t0 + min(lane, nt - 1);
+  const float x = lead_float(a.sx[i], 0), y = lead_float(a.sy[i], 0), z = lead_float(a.sz[i], 0);
+  const float ro = lead_float(a.sro[i], 0), rs = lead_float(a.srs[i], 0);
+  float lo0 = x, lo1 = y, lo2 = z, hi0 = x, hi1 = y, hi2 = z;
+  float R = fmaxf(ro, rs), am = fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z)));
+#pragma unroll
+  for (int o = kChunk / 2; o > 0; o >>= 1) {
+    lo0 = fminf(lo0, __shfl_xor_sync(0xffffffffu, lo0, o));
+    lo1 = fminf(lo1, __shfl_xor_sync(0xffffffffu, lo1, o));
+    lo2 = fminf(lo2, __shfl_xor_sync(0xffffffffu, lo2, o));
+    hi0 = fmaxf(hi0, __shfl_xor_sync(0xffffffffu, hi0, o));
+    hi1 = fmaxf(hi1, __shfl_xor_sync(0xffffffffu, hi1, o));
+    hi2 = fmaxf(hi2, __shfl_xor_sync(0xffffffffu, hi2, o));
+    R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, o));
+    am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
+  }
+  __syncwarp();
+  if (lane == 0) {
+    b.lo[0] = lo0; b.lo[1] = lo1; b.lo[2] = lo2;
+    b.hi[0] = hi0; b.hi[1] = hi1; b.hi[2] = hi2;
+    b.R2 = R;
+    b.amax = am;
+  }
+  __syncwarp();
+}
+// whether a source is beyond every target's max(r_search, r_out) and its own:
+// the gap to the box less 2^-18 of the coordinates' scale (their truncation to
+// 20 bits), against the reach widened by 1e-5
+__device__ __forceinline__ bool far_from64(const FarBox &b, double X, double Y, double Z,
+                                           double ro, double rs) {
+  const float x = lead_float(X, 0), y = lead_float(Y, 0), z = lead_float(Z, 0);
+  const float m = 3.814697265625e-6f *
+                  (b.amax + fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z))));
+  const float gx = fmaxf(fmaxf(b.lo[0] - x, x - b.hi[0]) - m, 0.f);
+  const float gy = fmaxf(fmaxf(b.lo[1] - y, y - b.hi[1]) - m, 0.f);
+  const float gz = fmaxf(fmaxf(b.lo[2] - z, z - b.hi[2]) - m, 0.f);
+  const float R = fmaxf(b.R2, fmaxf(lead_float(ro, 0), lead_float(rs, 0))) * 1.00001f;
+  const float d2 = gx * gx + gy * gy + gz * gz;
+  return d2 > 1e-30f && d2 >= R * R;
+}
+
+// m r^-3 from r^2 (zero for r = 0): the seed's y, e = 1 - r^2 y^2 and the
+// result (see rsqrt_seed); rare ranges by rsqrt()
+struct Inv3 {
+  double y, e, f;
+};
+__device__ __forceinline__ Inv3 inv_cube(double r2, double m) {
+  Inv3 v;
+  if (rsqrt_seed_ok(r2)) {
+    v.y = rsqrt_seed(r2);
+    const double y2 = v.y * v.y;
+    v.e = fma(-r2, y2, 1.0);
+    const double t = y2 * (v.y * m);
+    v.f = fma(t * v.e, fma(1.875, v.e, 1.5), t);
+  } else {
+    v.y = __double_as_longlong(r2) == 0 ? 0.0 : rsqrt(r2);
+    v.e = 0.0;
+    v.f = m * (v.y * v.y * v.y);
+  }
+  return v;
+}
+// min of two positive numbers and clamp to [0, 1], on the bit patterns (an FP64
+// comparison takes an FP64 instruction)
+__device__ __forceinline__ double min_pos(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
+}
+__device__ __forceinline__ double clamp01(double x) {
+  const long long b = __double_as_longlong(x), one = 0x3ff0000000000000LL;
+  return __longlong_as_double(b < 0 ? 0 : (b > one ? one : b));
+}
+// 1 / r to full precision
+__device__ __forceinline__ double inv_r(const Inv3 &v) {
+  return fma(v.y * v.e, fma(0.375, v.e, 0.5), v.y);
+}
+
+struct Eval64 {
+  const WalkArgs &a;
+  Targets64 &t;
+  const FarBox &box;
+  int32_t t0;
+  int nt;
+  unsigned &npp, &npn;
+  __device__ __forceinline__ void add(int i, double fx, double dx, double fy, double dy, double fz,
+                                      double dz) {
+    const int lane = threadIdx.x & 31;
+    t.acc[3 * i][lane] = fma(fx, dx, t.acc[3 * i][lane]);
+    t.acc[3 * i + 1][lane] = fma(fy, dy, t.acc[3 * i + 1][lane]);
+    t.acc[3 * i + 2][lane] = fma(fz, dz, t.acc[3 * i + 2][lane]);
+  }
+  __device__ void pp(const int32_t *list, int n) {
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < n;
+    const int32_t j = list[on ? lane : 0];
+    const double X = a.sx[j], Y = a.sy[j], Z = a.sz[j], ro = a.sro[j], rs = a.srs[j];
+    const double m = on ? -a.sm[j] : 0.0;
+    npp += on ? (unsigned)nt : 0u;
+    if (!__any_sync(0xffffffffu, on && !far_from64(box, X, Y, Z, ro, rs))) {
+#pragma unroll 1
+      for (int i = 0; i < nt; ++i) {
+        const double dx = t.x[i] - X, dy = t.y[i] - Y, dz = t.z[i] - Z;
+        const double f = inv_cube(fma(dx, dx, fma(dy, dy, dz * dz)), m).f;
+        add(i, f, dx, f, dy, f, dz);
+      }
+      return;
     }
-    if (lane == 0) {
-      atomicAdd(&a.counts[0], (unsigned long long)p);
-      atomicAdd(&a.counts[1], (unsigned long long)q);
+    const double iro = 1.0 / ro;
+    const int32_t rs2 = __double2hiint(rs * rs);
+#pragma unroll 1
+    for (int i = 0; i < nt; ++i) {
+      const double dx = t.x[i] - X, dy = t.y[i] - Y, dz = t.z[i] - Z;
+      const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+      const Inv3 v = inv_cube(r2, m);
+      // y = r / max(r_out,i, r_out,j) as r min(1 / r_out)
+      const double y = (r2 * inv_r(v)) * min_pos(t.iro[i], iro);
+      const double x = clamp01((y - a.gamma) * a.inv1mg);
+      const double x2 = x * x;
+      const double K = (x2 * x2) * fma(fma(fma(-20.0, x, 70.0), x, -84.0), x, 35.0);
+      const double f = v.f * K;
+      add(i, f, dx, f, dy, f, dz);
+      // r < max(r_search) by the leading 32 bits (a superset; the exact test
+      // follows in the neighbour search)
+      if (on && __double2hiint(r2) <= max(t.rs2[i], rs2)) {
+        if (j != t0 + i) record_candidate(a, t0 + i, j);
+        else --npp;  // the target itself is not a pair
+      }
     }
   }
+  // a += -M r/r^3 + Q.r/r^5 - (5/2)(r.Q.r) r/r^7, r = x_i - com
+  __device__ void nodes(const int32_t *list, int n) {
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < n;
+    const Mom64 *g = &a.mom64[list[on ? lane : 0]];
+    const double2 c0 = __ldg(reinterpret_cast<const double2 *>(g)),
+                  c1 = __ldg(reinterpret_cast<const double2 *>(g) + 1),
+                  q0 = __ldg(reinterpret_cast<const double2 *>(g) + 2),
+                  q1 = __ldg(reinterpret_cast<const double2 *>(g) + 3),
+                  q2 = __ldg(reinterpret_cast<const double2 *>(g) + 4);
+    const double M = on ? c1.y : 0.0;
+    const double qxx = on ? q0.x : 0.0, qyy = on ? q0.y : 0.0, qzz = on ? q1.x : 0.0,
+                 qxy = on ? q1.y : 0.0, qxz = on ? q2.x : 0.0, qyz = on ? q2.y : 0.0;
+    npn += on ? (unsigned)nt : 0u;
+#pragma unroll 1
+    for (int i = 0; i < nt; ++i) {
+      const double dx = t.x[i] - c0.x, dy = t.y[i] - c0.y, dz = t.z[i] - c1.x;
+      const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+      const Inv3 v = inv_cube(r2, 1.0);
+      const double ri3 = v.f, y2 = v.y * v.y;
+      const double ri2 = fma(y2, fma(v.e, v.e, v.e), y2);  // y^2 / (1 - e)
+      const double qx = fma(qxx, dx, fma(qxy, dy, qxz * dz));
+      const double qy = fma(qxy, dx, fma(qyy, dy, qyz * dz));
+      const double qz = fma(qxz, dx, fma(qyz, dy, qzz * dz));
+      const double s = fma(dx, qx, fma(dy, qy, dz * qz)) * ri2;
+      const double A = fma(-2.5, s * ri2, -M) * ri3, B = ri3 * ri2;
+      add(i, A, dx, A, dy, A, dz);
+      add(i, B, qx, B, qy, B, qz);
+    }
+  }
+};
+
+// the chunk's sums: the 32 partial sums of each row in one fixed tree (k +
+// (k + 16), then 8, 4, 2, 1), a row a lane
+__device__ __forceinline__ double row_sum(double *r) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    for (int k = 0; k < o; ++k) r[k] += r[k + o];
+  return r[0];
+}
+
+__global__ void __launch_bounds__(kWarps * 32) k_walk64(const WalkArgs a, int ct) {
+  pdl_wait();
+  __shared__ int32_t s_pp[kWarps][kPPCap];
+  __shared__ int32_t s_nd[kWarps][kNDCap];
+  __shared__ int32_t s_big[kWarps][kBigCap];
+  __shared__ Targets64 s_t[kWarps];
+  __shared__ int64_t s_bh[P3T_BITS + 1];
+  __shared__ FarBox s_box[kWarps];
+  if (threadIdx.x <= P3T_BITS) s_bh[threadIdx.x] = a.bh[threadIdx.x];
+  __syncthreads();
+
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int32_t *stack = a.stack + ((int64_t)blockIdx.x * kWarps + w) * a.stack_cap;
+  const int64_t ngroup = *a.d_nleaf;
+  const int64_t round_limit = *a.d_nnode + 2;  // a node is pushed at most once per walk
+  const int parts = (a.group_max + ct - 1) / ct;
+  Targets64 &t = s_t[w];
+  unsigned npp = 0, npn = 0;
+
+  for (;;) {
+    // work unit u: chunk u mod parts of target group u / parts (empty for the
+    // smaller groups); the last chunk takes what an oversized leaf has left
+    int64_t u = 0;
+    if (lane == 0) u = atomicAdd(reinterpret_cast<unsigned long long *>(a.cursor), 1ull);
+    u = __shfl_sync(0xffffffffu, u, 0);
+    const int64_t g = u / parts;
+    const int part = (int)(u - g * parts);
+    if (g >= ngroup) break;
+    if (*(volatile int32_t *)&a.st->code != 0) break;
+    const TreeNode &G = a.node[a.leaf_list[g]];
+    const int32_t gfirst = G.first, gend = G.first + G.count;
+    const int32_t u0 = gfirst + part * ct;
+    const int32_t u1 = part == parts - 1 ? gend : min(gend, u0 + ct);
+    if (u0 >= u1) continue;
+    GroupBox gb;
+    gb.load(G);
+    bool ok = true;
+    for (int32_t t0 = u0; t0 < u1 && ok; t0 += ct) {
+      const int nt = min(ct, u1 - t0);
+      if (lane < nt) {
+        const int32_t i = t0 + lane;
+        t.x[lane] = a.sx[i]; t.y[lane] = a.sy[i]; t.z[lane] = a.sz[i];
+        t.iro[lane] = 1.0 / a.sro[i];
+        t.rs2[lane] = __double2hiint(a.srs[i] * a.srs[i]);
+      }
+      for (int k = 0; k < 3 * nt; ++k) t.acc[k][lane] = 0.0;
+      far_box64(a, t0, nt, s_box[w]);
+      Eval64 ev{a, t, s_box[w], t0, nt, npp, npn};
+      ok = traverse(a, gb, gfirst, stack, s_pp[w], s_nd[w], s_big[w], s_bh, round_limit, ev);
+      __syncwarp();
+      if (ok)
+        for (int k = lane; k < 3 * nt; k += 32) {
+          const int i = k / 3, c = k - 3 * i;
+          (c == 0 ? a.ax : (c == 1 ? a.ay : a.az))[a.idx[t0 + i]] = a.G * row_sum(t.acc[k]);
+        }
+      __syncwarp();
+    }
+    if (!ok) break;
+  }
+  add_counts(a, npp, npn);
 }
 
 // ---- adjoint of the tree walk (FP64 path) -----------------------------------
@@ -958,11 +1043,19 @@ __global__ void __launch_bounds__(kWarps * 32, MIXED ? P3T_WALK_MINB_MIXED : 1)
 //     and dL/dM, dL/dQ accumulated per node;
 // the node adjoints then reach the member particles through M = sum m_k,
 // c = sum m_k x_k / M, Q = sum m_k (3 d d^T - d^2 I), d = x_k - c (the
-// derivative of Q through c vanishes, as sum m_k d_k = 0).  One warp per
-// target group, one lane per target (lanes past the group idle); the
-// contributions of a walk's targets to one source or node are added by a
-// warp reduction and then to the global sums by FP64 atomics (their order
-// follows the walks' order, so the last bits can differ from run to run).
+// derivative of Q through c vanishes, as sum m_k d_k = 0).  The layout of the
+// FP64 walk: a lane per source or node, the targets of a chunk in turn, so
+// that what the chunk's targets add to a source or node is summed in that
+// lane's registers and goes to the global sums in one FP64 atomic per value
+// and chunk (their order follows the walks' order, so the last bits can
+// differ from run to run), and what the lanes add to a target in shared
+// memory.  With lam' = G lam (lam scaled), z = r.Q.r / r^2, the node's
+//   g = r^-5 [Q lam' + cl lam' + cr r + cq Q r], cl = -M r^2 - 5/2 z,
+//   cr = 3 M lam'.r + (35/2 z lam'.r - 5 lam'.Q r) / r^2, cq = -5 lam'.r / r^2,
+//   dL/dQ_ab = r^-5 sym(k_a r_b), k = lam' + cq/2 r:
+// 84 FP64 instructions a node term and 33 a far pair (N = 10,000: 6,240 -> 600
+// us a call), where one lane a target
+// with a warp reduction per source took about 180 and 60 at half the lanes.
 struct VjpOut {
   const double *lx, *ly, *lz;  // velocity adjoints, caller order
   double s;                    // scale (the kick's time step)
@@ -970,164 +1063,175 @@ struct VjpOut {
   double *nadj;                // per node: dL/dc (3), dL/dM, dL/dQ (xx yy zz xy xz yz)
 };
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
+struct TargetsVjp {
+  double x[kChunk], y[kChunk], z[kChunk], iro[kChunk];
+  double lx[kChunk], ly[kChunk], lz[kChunk];  // s G lam
+  double acc[kChunk * 3][33];
+};
 
 struct VjpEval {
   const WalkArgs &a;
   const VjpOut &o;
-  void *stage;
-  bool valid;
-  int32_t self;            // sorted index of the lane's target
-  double x, y, z, ro;      // target
-  double lx, ly, lz;       // s lam
-  double gx, gy, gz;       // dL/dx of the target, this walk
-  __device__ void nodes(const int32_t *list, int n) {
-    Mom64 *S = reinterpret_cast<Mom64 *>(stage);
-    int32_t *ids = reinterpret_cast<int32_t *>(S + 32);
+  TargetsVjp &t;
+  const FarBox &box;
+  int32_t t0;
+  int nt;
+  __device__ __forceinline__ void add(int i, double f, double vx, double vy, double vz) {
     const int lane = threadIdx.x & 31;
-    if (lane < n) {
-      S[lane] = a.mom64[list[lane]];
-      ids[lane] = list[lane];
+    t.acc[3 * i][lane] = fma(f, vx, t.acc[3 * i][lane]);
+    t.acc[3 * i + 1][lane] = fma(f, vy, t.acc[3 * i + 1][lane]);
+    t.acc[3 * i + 2][lane] = fma(f, vz, t.acc[3 * i + 2][lane]);
+  }
+  __device__ void nodes(const int32_t *list, int n) {
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < n;
+    const int32_t id = list[on ? lane : 0];
+    const double2 *g = reinterpret_cast<const double2 *>(&a.mom64[id]);
+    const double2 c0 = __ldg(g), c1 = __ldg(g + 1), q0 = __ldg(g + 2), q1 = __ldg(g + 3),
+                  q2 = __ldg(g + 4);
+    const double M = c1.y;
+    double nx = 0.0, ny = 0.0, nz = 0.0, nM = 0.0;
+    double nQ[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int i = 0; i < nt; ++i) {
+      const double rx = t.x[i] - c0.x, ry = t.y[i] - c0.y, rz = t.z[i] - c1.x;
+      const double lx = t.lx[i], ly = t.ly[i], lz = t.lz[i];
+      const double r2 = fma(rx, rx, fma(ry, ry, rz * rz));
+      const Inv3 v = inv_cube(r2, 1.0);
+      const double ri3 = v.f, y2 = v.y * v.y;
+      const double ri2 = fma(y2, fma(v.e, v.e, v.e), y2);
+      const double ri5 = ri3 * ri2;
+      const double qx = fma(q0.x, rx, fma(q1.y, ry, q2.x * rz));
+      const double qy = fma(q1.y, rx, fma(q0.y, ry, q2.y * rz));
+      const double qz = fma(q2.x, rx, fma(q2.y, ry, q1.x * rz));
+      const double z = fma(rx, qx, fma(ry, qy, rz * qz)) * ri2;
+      const double lr = fma(lx, rx, fma(ly, ry, lz * rz));
+      const double lq = fma(lx, qx, fma(ly, qy, lz * qz));
+      const double l2 = lr * ri2;
+      const double cl = fma(-2.5, z, -M * r2);
+      const double cr = fma(ri2, fma(17.5 * z, lr, -5.0 * lq), 3.0 * M * lr);
+      const double cq = -5.0 * l2, k5 = -2.5 * l2;
+      const double hx = fma(cl, lx, fma(cr, rx, fma(cq, qx, fma(q0.x, lx, fma(q1.y, ly, q2.x * lz)))));
+      const double hy = fma(cl, ly, fma(cr, ry, fma(cq, qy, fma(q1.y, lx, fma(q0.y, ly, q2.y * lz)))));
+      const double hz = fma(cl, lz, fma(cr, rz, fma(cq, qz, fma(q2.x, lx, fma(q2.y, ly, q1.x * lz)))));
+      // lanes past the batch repeat entry 0: their terms must not reach the target
+      add(i, on ? ri5 : 0.0, hx, hy, hz);
+      nx = fma(ri5, hx, nx); ny = fma(ri5, hy, ny); nz = fma(ri5, hz, nz);
+      nM = fma(-lr, ri3, nM);
+      const double kx = fma(k5, rx, lx), ky = fma(k5, ry, ly), kz = fma(k5, rz, lz);
+      const double sx = ri5 * rx, sy = ri5 * ry, sz = ri5 * rz;
+      nQ[0] = fma(kx, sx, nQ[0]); nQ[1] = fma(ky, sy, nQ[1]); nQ[2] = fma(kz, sz, nQ[2]);
+      nQ[3] = fma(kx, sy, fma(ky, sx, nQ[3]));
+      nQ[4] = fma(kx, sz, fma(kz, sx, nQ[4]));
+      nQ[5] = fma(ky, sz, fma(kz, sy, nQ[5]));
     }
-    __syncwarp();
-    for (int q = 0; q < n; ++q) {
-      const Mom64 &m = S[q];
-      double c[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-      if (valid) {
-        const double rx = x - m.cx, ry = y - m.cy, rz = z - m.cz;
-        const double r2 = rx * rx + ry * ry + rz * rz;
-        const double ri = rsqrt(r2);
-        const double ri2 = ri * ri, ri3 = ri2 * ri, ri5 = ri3 * ri2, ri7 = ri5 * ri2,
-                     ri9 = ri7 * ri2;
-        const double qx = m.qxx * rx + m.qxy * ry + m.qxz * rz;
-        const double qy = m.qxy * rx + m.qyy * ry + m.qyz * rz;
-        const double qz = m.qxz * rx + m.qyz * ry + m.qzz * rz;
-        const double q2 = rx * qx + ry * qy + rz * qz;           // r.Q.r
-        const double lr = lx * rx + ly * ry + lz * rz;           // lam.r
-        const double lq = lx * qx + ly * qy + lz * qz;           // lam.Q r
-        const double Ql_x = m.qxx * lx + m.qxy * ly + m.qxz * lz;  // Q lam
-        const double Ql_y = m.qxy * lx + m.qyy * ly + m.qyz * lz;
-        const double Ql_z = m.qxz * lx + m.qyz * ly + m.qzz * lz;
-        const double G = a.G;
-        // g = grad_r lam.a (a the node term)
-        const double cr = G * (3.0 * m.M * lr * ri5 - 5.0 * lq * ri7 + 17.5 * q2 * lr * ri9);
-        const double cl = G * (-m.M * ri3 - 2.5 * q2 * ri7);
-        const double cQ = G * ri5, cQr = -5.0 * G * lr * ri7;
-        const double g0 = cl * lx + cr * rx + cQ * Ql_x + cQr * qx;
-        const double g1 = cl * ly + cr * ry + cQ * Ql_y + cQr * qy;
-        const double g2 = cl * lz + cr * rz + cQ * Ql_z + cQr * qz;
-        gx += g0; gy += g1; gz += g2;
-        c[0] = -g0; c[1] = -g1; c[2] = -g2;
-        c[3] = -G * lr * ri3;
-        // d(lam.a)/dQ per stored component (an off-diagonal one stands for ab and ba)
-        const double u = G * ri5, v = -2.5 * G * lr * ri7;
-        c[4] = u * lx * rx + v * rx * rx;
-        c[5] = u * ly * ry + v * ry * ry;
-        c[6] = u * lz * rz + v * rz * rz;
-        c[7] = u * (lx * ry + ly * rx) + 2.0 * v * rx * ry;
-        c[8] = u * (lx * rz + lz * rx) + 2.0 * v * rx * rz;
-        c[9] = u * (ly * rz + lz * ry) + 2.0 * v * ry * rz;
-      }
-      for (int k = 0; k < 10; ++k) c[k] = warp_sum_d(c[k]);
-      if (lane == 0)
-        for (int k = 0; k < 10; ++k) atomicAdd(&o.nadj[10 * (int64_t)ids[q] + k], c[k]);
+    if (on) {
+      double *A = o.nadj + 10 * (int64_t)id;
+      atomicAdd(&A[0], -nx); atomicAdd(&A[1], -ny); atomicAdd(&A[2], -nz); atomicAdd(&A[3], nM);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) atomicAdd(&A[4 + k], nQ[k]);
     }
-    __syncwarp();
   }
   __device__ void pp(const int32_t *list, int n) {
-    double *S = reinterpret_cast<double *>(stage);  // x, y, z, m, ro of 32 sources
-    int32_t *ids = reinterpret_cast<int32_t *>(S + 5 * 32);
     const int lane = threadIdx.x & 31;
-    if (lane < n) {
-      const int32_t j = list[lane];
-      S[lane] = a.sx[j]; S[32 + lane] = a.sy[j]; S[64 + lane] = a.sz[j];
-      S[96 + lane] = a.sm[j]; S[128 + lane] = a.sro[j];
-      ids[lane] = j;
-    }
-    __syncwarp();
-    const double i1mg = 1.0 / (1.0 - a.gamma);
-    for (int q = 0; q < n; ++q) {
-      double c[4] = {0, 0, 0, 0};
-      if (valid && ids[q] != self) {
-        const double rx = x - S[q], ry = y - S[32 + q], rz = z - S[64 + q];
-        const double mj = S[96 + q];
-        const double r2 = rx * rx + ry * ry + rz * rz;
-        const double r = sqrt(r2);
-        const double roij = fmax(ro, S[128 + q]);
-        const double yv = r / roij;
-        double K = 0.0, dK = 0.0;
-        if (yv >= 1.0) {
-          K = 1.0;
-        } else if (yv > a.gamma) {
-          const double xs = (yv - a.gamma) * i1mg;
-          const double x2 = xs * xs, x3 = x2 * xs, us = 1.0 - xs;
-          K = x2 * x2 * (35.0 - 84.0 * xs + 70.0 * x2 - 20.0 * x3);
-          dK = 140.0 * x3 * us * us * us * i1mg;
-        }
-        if (K != 0.0 || dK != 0.0) {
-          const double r3 = r2 * r, r4 = r2 * r2, r5 = r4 * r;
-          const double phi = K / r3, psi = dK / (roij * r4) - 3.0 * K / r5;
-          const double lr = lx * rx + ly * ry + lz * rz;
-          const double f = -a.G * mj;
-          const double j0 = f * (phi * lx + psi * lr * rx);
-          const double j1 = f * (phi * ly + psi * lr * ry);
-          const double j2 = f * (phi * lz + psi * lr * rz);
-          gx += j0; gy += j1; gz += j2;
-          c[0] = -j0; c[1] = -j1; c[2] = -j2;
-          c[3] = -a.G * phi * lr;
-        }
+    const bool on = lane < n;
+    const int32_t j = list[on ? lane : 0];
+    const double X = a.sx[j], Y = a.sy[j], Z = a.sz[j], ro = a.sro[j];
+    const double m = on ? -a.sm[j] : 0.0;
+    const bool near =
+        __any_sync(0xffffffffu, on && !far_from64(box, X, Y, Z, ro, 0.0));
+    const double iro = near ? 1.0 / ro : 0.0;
+    // sum over the targets of K r^-3 lam' + psi (lam'.r) r, and of K r^-3 lam'.r
+    double bx = 0.0, by = 0.0, bz = 0.0, bm = 0.0;
+#pragma unroll 1
+    for (int i = 0; i < nt; ++i) {
+      const double rx = t.x[i] - X, ry = t.y[i] - Y, rz = t.z[i] - Z;
+      const double lx = t.lx[i], ly = t.ly[i], lz = t.lz[i];
+      const double r2 = fma(rx, rx, fma(ry, ry, rz * rz));
+      const Inv3 v = inv_cube(r2, 1.0);
+      const double y2 = v.y * v.y;
+      const double ri2 = fma(y2, fma(v.e, v.e, v.e), y2);
+      double phi = v.f, psi;
+      if (near) {
+        // the target itself (r = 0) has y = 0: K = K' = 0
+        const double irot = min_pos(t.iro[i], iro);
+        const double yv = (r2 * inv_r(v)) * irot;
+        const double x = clamp01((yv - a.gamma) * a.inv1mg);
+        const double x2 = x * x, u = 1.0 - x;
+        const double K = (x2 * x2) * fma(fma(fma(-20.0, x, 70.0), x, -84.0), x, 35.0);
+        const double dK = (140.0 * a.inv1mg) * ((x2 * x) * (u * u * u)) * irot;
+        psi = fma(dK, ri2 * ri2, -3.0 * K * (phi * ri2));
+        phi *= K;
+      } else {
+        psi = -3.0 * (phi * ri2);
       }
-      for (int k = 0; k < 4; ++k) c[k] = warp_sum_d(c[k]);
-      if (lane == 0) {
-        const int32_t i = a.idx[ids[q]];
-        atomicAdd(&o.gx[i], c[0]); atomicAdd(&o.gy[i], c[1]); atomicAdd(&o.gz[i], c[2]);
-        atomicAdd(&o.gm[i], c[3]);
-      }
+      const double lr = fma(lx, rx, fma(ly, ry, lz * rz));
+      const double pl = psi * lr;
+      const double tx = fma(pl, rx, phi * lx), ty = fma(pl, ry, phi * ly), tz = fma(pl, rz, phi * lz);
+      add(i, m, tx, ty, tz);
+      bx += tx; by += ty; bz += tz;
+      bm = fma(-phi, lr, bm);
     }
-    __syncwarp();
+    if (on) {
+      const int32_t i = a.idx[j];
+      atomicAdd(&o.gx[i], -m * bx); atomicAdd(&o.gy[i], -m * by); atomicAdd(&o.gz[i], -m * bz);
+      atomicAdd(&o.gm[i], bm);
+    }
   }
 };
 
-__global__ void __launch_bounds__(kWarps * 32) k_walk_vjp(const WalkArgs a, const VjpOut o) {
+__global__ void __launch_bounds__(kWarps * 32) k_walk_vjp(const WalkArgs a, int ct, const VjpOut o) {
   pdl_wait();
   __shared__ int32_t s_pp[kWarps][kPPCap];
   __shared__ int32_t s_nd[kWarps][kNDCap];
   __shared__ int32_t s_big[kWarps][kBigCap];
-  // a batch of 32 FP64 moments (or sources) and their 32 ids
-  __shared__ __align__(16) unsigned char s_stage[kWarps][32 * sizeof(Mom64) + 32 * 4];
+  __shared__ TargetsVjp s_t[kWarps];
   __shared__ int64_t s_bh[P3T_BITS + 1];
+  __shared__ FarBox s_box[kWarps];
   if (threadIdx.x <= P3T_BITS) s_bh[threadIdx.x] = a.bh[threadIdx.x];
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int32_t *stack = a.stack + ((int64_t)blockIdx.x * kWarps + w) * a.stack_cap;
   const int64_t ngroup = *a.d_nleaf;
   const int64_t round_limit = *a.d_nnode + 2;
+  const int parts = (a.group_max + ct - 1) / ct;  // as k_walk64
+  TargetsVjp &t = s_t[w];
   for (;;) {
-    int64_t g = 0;
-    if (lane == 0) g = atomicAdd(reinterpret_cast<unsigned long long *>(a.cursor), 1ull);
-    g = __shfl_sync(0xffffffffu, g, 0);
+    int64_t u = 0;
+    if (lane == 0) u = atomicAdd(reinterpret_cast<unsigned long long *>(a.cursor), 1ull);
+    u = __shfl_sync(0xffffffffu, u, 0);
+    const int64_t g = u / parts;
+    const int part = (int)(u - g * parts);
     if (g >= ngroup) break;
     if (*(volatile int32_t *)&a.st->code != 0) break;
     const TreeNode &G = a.node[a.leaf_list[g]];
+    const int32_t gfirst = G.first, gend = G.first + G.count;
+    const int32_t u0 = gfirst + part * ct;
+    const int32_t u1 = part == parts - 1 ? gend : min(gend, u0 + ct);
+    if (u0 >= u1) continue;
     GroupBox gb;
     gb.load(G);
     bool ok = true;
-    for (int32_t tb = G.first; tb < G.first + G.count && ok; tb += 32) {
-      const bool valid = tb + lane < G.first + G.count;
-      VjpEval ev{a, o, s_stage[w], valid, tb + lane, 0, 0, 0, 1, 0, 0, 0, 0, 0, 0};
-      if (valid) {
-        const int32_t t = tb + lane, i = a.idx[t];
-        ev.x = a.sx[t]; ev.y = a.sy[t]; ev.z = a.sz[t]; ev.ro = a.sro[t];
-        ev.lx = o.s * o.lx[i]; ev.ly = o.s * o.ly[i]; ev.lz = o.s * o.lz[i];
+    for (int32_t t0 = u0; t0 < u1 && ok; t0 += ct) {
+      const int nt = min(ct, u1 - t0);
+      if (lane < nt) {
+        const int32_t k = t0 + lane, i = a.idx[k];
+        t.x[lane] = a.sx[k]; t.y[lane] = a.sy[k]; t.z[lane] = a.sz[k];
+        t.iro[lane] = 1.0 / a.sro[k];
+        const double sg = o.s * a.G;
+        t.lx[lane] = sg * o.lx[i]; t.ly[lane] = sg * o.ly[i]; t.lz[lane] = sg * o.lz[i];
       }
-      ok = traverse(a, gb, G.first, stack, s_pp[w], s_nd[w], s_big[w], s_bh, round_limit, ev);
-      if (ok && valid) {
-        const int32_t i = a.idx[tb + lane];
-        atomicAdd(&o.gx[i], ev.gx); atomicAdd(&o.gy[i], ev.gy); atomicAdd(&o.gz[i], ev.gz);
-      }
+      for (int k = 0; k < 3 * nt; ++k) t.acc[k][lane] = 0.0;
+      far_box64(a, t0, nt, s_box[w]);
+      VjpEval ev{a, o, t, s_box[w], t0, nt};
+      ok = traverse(a, gb, gfirst, stack, s_pp[w], s_nd[w], s_big[w], s_bh, round_limit, ev);
+      __syncwarp();
+      if (ok)
+        for (int k = lane; k < 3 * nt; k += 32) {
+          const int i = k / 3, c = k - 3 * i;
+          atomicAdd(&(c == 0 ? o.gx : (c == 1 ? o.gy : o.gz))[a.idx[t0 + i]], row_sum(t.acc[k]));
+        }
+      __syncwarp();
     }
     if (!ok) break;
   }
@@ -1247,6 +1351,7 @@ static WalkArgs walk_args(p3t_ctx *c, const p3t_particles *p) {
   a.cursor = &c->counters[12];
   a.st = c->status;
   a.seg = SegView{c->seg_off, (int)c->nseg, p->n};
+  a.group_max = c->prm.group_size > c->prm.leaf_size ? c->prm.group_size : c->prm.leaf_size;
   a.refine_cf = 32.0f;
   a.G = c->prm.G;
   a.gamma = c->prm.gamma;
@@ -1257,6 +1362,22 @@ static WalkArgs walk_args(p3t_ctx *c, const p3t_particles *p) {
   return a;
 }
 
+// The FP64 walks' chunk of targets: up to kChunk at a time (one traversal
+// serves them all), fewer while a warp would get less than four chunks, so
+// that small systems fill the card (N = 1,000: chunks of one target; from
+// about 100,000 particles on the largest)
+static int walk64_chunk(const p3t_ctx *c, unsigned blocks) {
+  int ct = kChunk;
+  while (ct > 1 && c->last_n < (int64_t)4 * ct * blocks * kWarps) ct >>= 1;
+  return ct;
+}
+// their blocks per SM: kWalk64Blocks (12 warps hold the FP64 pipe busy through
+// each other's traversals)
+static unsigned walk64_blocks(const p3t_ctx *c, unsigned blocks) {
+  const unsigned most = (unsigned)c->num_sms * kWalk64Blocks;
+  return blocks < most ? blocks : most;
+}
+
 int p3t_run_soft_force_vjp_tree(p3t_ctx *c, const p3t_particles *p, double s,
                                 const double *lx, const double *ly, const double *lz,
                                 double *gx, double *gy, double *gz, double *gm,
@@ -1265,8 +1386,8 @@ int p3t_run_soft_force_vjp_tree(p3t_ctx *c, const p3t_particles *p, double s,
   VjpOut o{lx, ly, lz, s, gx, gy, gz, gm, c->nadj};
   P3T_CUDA_TRY(cudaMemsetAsync(c->nadj, 0, sizeof(double) * 10 * c->node_cap, st));
   P3T_CUDA_TRY(cudaMemsetAsync(a.cursor, 0, sizeof(int64_t), st));
-  const unsigned blocks = (unsigned)(c->walk_warps / kWarps);
-  pdl_launch(k_walk_vjp, dim3(blocks), dim3(kWarps * 32), 0, st, a, o);
+  const unsigned blocks = walk64_blocks(c, (unsigned)(c->walk_warps / kWarps));
+  pdl_launch(k_walk_vjp, dim3(blocks), dim3(kWarps * 32), 0, st, a, walk64_chunk(c, blocks), o);
   pdl_launch(k_node_adjoint, dim3((unsigned)(c->num_sms * 8)), dim3(128), 0, st, 
       &c->counters[2], c->leaf_list, c->node, c->mom64, c->nadj, c->sx, c->sy, c->sz, c->sm,
       c->idx, gx, gy, gz, gm);
@@ -1277,28 +1398,9 @@ int p3t_run_soft_force_vjp_tree(p3t_ctx *c, const p3t_particles *p, double s,
 int p3t_run_soft_force(p3t_ctx *c, const p3t_particles *p, double *ax,
                        double *ay, double *az, uint64_t *counts,
                        cudaStream_t s) {
-  WalkArgs a;
-  a.node = c->node; a.mom64 = c->mom64; a.mom32 = c->mom32;
-  a.leaf_list = c->group_list; a.d_nleaf = &c->counters[15]; a.d_nnode = &c->counters[3];
-  a.sx = c->sx; a.sy = c->sy; a.sz = c->sz; a.sm = c->sm; a.sro = c->sro; a.srs = c->srs;
-  a.spA = c->spA; a.spB = c->spB; a.srs32 = c->srs32; a.sml = c->sml;
-  a.idx = c->idx;
+  WalkArgs a = walk_args(c, p);
   a.ax = ax; a.ay = ay; a.az = az;
-  a.stack = c->walk_stack; a.stack_cap = c->stack_cap;
-  a.cand_i = c->cand_i; a.cand_j = c->cand_j; a.cand_cap = c->cand_cap;
-  a.cand_count = reinterpret_cast<unsigned long long *>(&c->counters[8]);
   a.counts = reinterpret_cast<unsigned long long *>(counts);
-  a.cursor = &c->counters[12];
-  a.st = c->status;
-  a.seg = SegView{c->seg_off, (int)c->nseg, p->n};
-  a.refine_cf = 32.0f;
-  a.G = c->prm.G;
-  a.gamma = c->prm.gamma;
-  a.inv1mg = 1.0 / (1.0 - c->prm.gamma);
-  a.inv1mg_f = (float)(1.0 / (1.0 - c->prm.gamma));
-  a.mgi_f = (float)(-c->prm.gamma / (1.0 - c->prm.gamma));
-  // Barnes-Hut thresholds per level, ceil((2^(22-l))^2 / theta^2) (half units)
-  for (int l = 0; l <= P3T_BITS; ++l) a.bh[l] = bh_threshold(c->prm.theta, l);
   pdl_launch(k_walk_prep, dim3(1), dim3(1), 0, s, a.cursor, a.cand_count, a.counts);
   unsigned blocks = (unsigned)(c->walk_warps / kWarps);
   if (c->walk_bps > 0 && (int64_t)c->num_sms * c->walk_bps < (int64_t)blocks)
@@ -1307,9 +1409,10 @@ int p3t_run_soft_force(p3t_ctx *c, const p3t_particles *p, double *ax,
     // one target per lane (or several lanes per target): two targets per
     // lane (a 64-target group walked once) was measured slower than two
     // walks of 32 (register pressure, longer chains)
-    pdl_launch(k_walk<true>, dim3(blocks), dim3(kWarps * 32), 0, s, a);
+    pdl_launch(k_walk, dim3(blocks), dim3(kWarps * 32), 0, s, a);
   } else {
-    pdl_launch(k_walk<false>, dim3(blocks), dim3(kWarps * 32), 0, s, a);
+    blocks = walk64_blocks(c, blocks);
+    pdl_launch(k_walk64, dim3(blocks), dim3(kWarps * 32), 0, s, a, walk64_chunk(c, blocks));
   }
   pdl_launch(k_walk_post, dim3(1), dim3(1), 0, s, c->counters, c->cand_cap, c->status);
   p3t_note_launches(3);
@@ -1318,11 +1421,12 @@ int p3t_run_soft_force(p3t_ctx *c, const p3t_particles *p, double *ax,
 }
 
 // persistent walk warps for a context of up to n particles: 6 blocks per SM,
-// fewer for small systems (a block for every 256 particles: a group walk
-// takes a warp, and a group holds tens of particles)
+// fewer for small systems: a block for every 4 particles (the FP64 walks take
+// single targets there; with a block for every 256, 1,000 particles in FP64
+// ran on 4 SMs: 2,535 us at theta = 0, 105 now; mixed 1e5 ring 338 -> 253)
 int64_t p3t_walk_warps(int num_sms, int64_t n) {
   int64_t blocks = (int64_t)num_sms * p3t_walk_blocks_per_sm();
-  const int64_t want = n / 256 + 1;
+  const int64_t want = n / 4 + 1;
   if (want < blocks) blocks = want;
   return blocks * kWarps;
 }
