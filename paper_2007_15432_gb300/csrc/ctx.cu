@@ -197,7 +197,8 @@ int p3t_create(p3t_ctx **ctx, const p3t_params *p, int device) {
   bool ok = dalloc(c->status, 1) && dalloc(c->box, 5) && dalloc(c->box_bits, 6) &&
             dalloc(c->counters, 64) && dalloc(c->cl_counts, 4) && dalloc(c->hsteps, 1) && dalloc(c->hcursor, 5) &&
             dalloc(c->coll_ctr, 1) &&
-            dalloc(c->epart, 8192) && dalloc(c->bh_table, 32);
+            dalloc(c->epart, 8192) && dalloc(c->bh_table, 32) &&
+            dalloc(c->sort_work, (int64_t)p3t_sort_work_bytes()) && p3t_sort_prepare();
   for (int q = 0; q < 2 && ok; ++q)
     ok = cudaStreamCreateWithFlags(&c->aux[q], cudaStreamNonBlocking) == cudaSuccess &&
          cudaEventCreateWithFlags(&c->ev_join[q], cudaEventDisableTiming) == cudaSuccess;
@@ -228,7 +229,7 @@ void p3t_destroy(p3t_ctx *c) {
   delete[] c->seg_off_h;
   dfree(c->cl_counts); dfree(c->hsteps); dfree(c->hcursor); dfree(c->epart);
   dfree(c->coll_ctr);
-  dfree(c->bh_table);
+  dfree(c->bh_table); dfree(c->sort_work);
   dfree(c->dpart); dfree(c->dcnt);
   for (int q = 0; q < 2; ++q) {
     if (c->aux[q]) cudaStreamDestroy(c->aux[q]);

@@ -246,17 +246,16 @@ int p3t_run_neighbours(p3t_ctx *c, const p3t_particles *p, int64_t *nb_off,
              &cnt[21], c->singles, c->cl_off, c->mkeys, c->mvals, c->cl_counts, &cnt[11]);
   // filter, check, fill, sort_rows, zero, uf_init, uf_union, uf_label, flags, scatter
   p3t_note_launches(10);
-  // members ordered by (label, index): stable sort of the ascending member
-  // list on the label's bits (labels are particle indices below n).  The
-  // sorted members must land in the buffer they started in, so that the
-  // cluster views keep their addresses from step to step (a step captured in
-  // a CUDA graph reads the previous step's clusters there): after an odd
-  // number of 8-bit passes they are copied back
+  // members ordered by (label, index), on the label's bits (labels are
+  // particle indices below n).  The sorted members must land in the buffer
+  // they started in, so that the cluster views keep their addresses from step
+  // to step (a step captured in a CUDA graph reads the previous step's
+  // clusters there): after an odd number of radix passes they are copied back
   const int bits = n <= 65536 ? 16 : (n <= (1 << 24) ? 24 : 32);
   uint64_t *k0 = c->mkeys, *k1 = c->mkeys_alt;
   int32_t *v0 = c->mvals, *v1 = c->mvals_alt;
-  rc = p3t_radix_sort(&k0, &v0, &k1, &v1, &cnt[11], c->cap, 0, bits, c->radix_hist,
-                      c->radix_hist_cap, s);
+  rc = p3t_sort_pairs(&k0, &v0, &k1, &v1, &cnt[11], c->cap, bits, c->radix_hist,
+                      c->radix_hist_cap, c->sort_work, p3t_sort_where(c), s);
   if (rc) return rc;
   if (v0 != c->mvals) {
     pdl_launch(k_copy_i32, dim3((unsigned)p3t_grid(n, kBlock, maxb)), dim3(kBlock), 0, s, &cnt[11],

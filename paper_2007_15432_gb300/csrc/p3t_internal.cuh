@@ -239,6 +239,7 @@ struct p3t_ctx {
   int32_t *idx = nullptr, *idx_alt = nullptr;
   uint32_t *radix_hist = nullptr;
   int64_t radix_hist_cap = 0;
+  unsigned char *sort_work = nullptr;      // splitters and bucket counts of the sample sort
 
   // sorted particles (FP64 and mixed packings)
   double *sx = nullptr, *sy = nullptr, *sz = nullptr, *sm = nullptr;
@@ -394,6 +395,23 @@ int p3t_radix_sort(uint64_t **keys, int32_t **vals, uint64_t **keys_alt,
                    int begin_bit, int end_bit, uint32_t *hist,
                    int64_t hist_cap, cudaStream_t s);
 int64_t p3t_radix_hist_entries(int64_t n_cap);
+// Sort by (key, val) of distinct values (the stable order by key when the
+// values start in ascending order), n from device memory (at most n_cap); on
+// return *keys / *vals point at the sorted data.  Keys below 2^key_bits, values
+// in [0, n_cap).  work: p3t_sort_work_bytes(), where: n_cap words.  p3t_sort_prepare once per
+// device before the first call.
+constexpr int P3T_SORT_BLOCK = 8192;  // most entries one block sorts (one launch)
+size_t p3t_sort_work_bytes();
+bool p3t_sort_prepare();
+int p3t_sort_pairs(uint64_t **keys, int32_t **vals, uint64_t **keys_alt, int32_t **vals_alt,
+                   const int64_t *d_n, int64_t n_cap, int key_bits, uint32_t *hist,
+                   int64_t hist_cap, void *work, uint32_t *where, cudaStream_t s);
+
+// the sorts' per-entry words: the last quarter of the flag buffer, which the
+// stages that sort leave free
+static inline uint32_t *p3t_sort_where(p3t_ctx *c) {
+  return reinterpret_cast<uint32_t *>(c->flag + 3 * c->cap);
+}
 
 // ---- stages (tree.cu, walk.cu, neighbours.cu, hard.cu) -------------------
 int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s);

@@ -344,6 +344,476 @@ radix_downsweep(const uint64_t *keys, const int32_t *vals, uint64_t *okeys,
   }
 }
 
+// ---- sort by (key, value) ----------------------------------------------------
+// The sorts of the library order distinct values by (key, value) (the values
+// are indices that start in ascending order, so this is the stable order by
+// key).  A radix pass is three launches whose tiles leave the chip waiting on
+// L2 latency: 22 us at a million keys, 12 at three thousand, eight passes a
+// tree.  Up to kSampleMax keys are sorted instead
+//  - by one block in shared memory when the capacity is at most
+//    kBlockSortMax (one launch);
+//  - else as a sample sort: one block sorts 8 samples a bucket (4 with the most
+//    buckets) and takes every eighth (fourth) as a splitter, so that the
+//    buckets are balanced whatever the keys' distribution: about 1,000 a
+//    bucket, and one above the 4,096 a block holds has odds of 3e-8 (5e-5; it
+//    costs a merge of two runs, some 10 us), a pass finds each key's bucket and its place in
+//    it (by atomics: the order within a bucket is left to its sort), a pass
+//    moves it there, and a block sorts each bucket.  Four launches.
+// The order is unique, so the result is that of the radix passes.  Keys and
+// values end in the buffers they started in.  Measured (mixed tree build): N =
+// 1e6 381 -> 339 us, 1e5 200 -> 155, 3,001 178 -> 120, 1,000 (FP64) 200 -> 141.
+// What bounds it: the one block that sorts the samples and the latency of the
+// buckets' blocks (three of 512 threads an SM beat two, and blocks of 256 with
+// buckets of 2,048: 339, 348, 346 us).  Keys of 32 bits or less keep the radix
+// passes (cut-off bins of 377,740: 40 against 76 us).
+constexpr int kItems = 8;                 // a thread's run of sorted keys
+constexpr int kBlockSortMax = 1024 * kItems;
+static_assert(kBlockSortMax == P3T_SORT_BLOCK, "one block's sort");
+constexpr int kLocalThreads = 512;
+constexpr int kLocalMax = kLocalThreads * kItems;
+constexpr int kMaxBuckets = 1024;
+constexpr int kSamples = 4096;            // 8 a bucket, 4 of the most buckets
+constexpr int64_t kSampleMax = 1500000;
+constexpr int kPosBits = 21;              // place in a bucket: below kSampleMax < 2^21
+constexpr int kPlace = 13;                // place in a block's input, below 2^13
+
+struct SortWork {
+  uint64_t skey[kMaxBuckets];
+  int32_t sval[kMaxBuckets];
+  uint32_t count[kMaxBuckets], start[kMaxBuckets + 1];
+  int32_t done;
+};
+
+__device__ __forceinline__ bool pair_less(uint64_t ka, int32_t va, uint64_t kb, int32_t vb) {
+  return ka < kb || (ka == kb && va < vb);
+}
+// shared-memory slot of entry i (a word skipped every eight: a thread's runs
+// start in different banks)
+__device__ __forceinline__ int slot(int i) { return i + (i >> 3); }
+constexpr size_t sort_smem(int max) { return (size_t)(max + max / 8) * 12; }
+
+__device__ __forceinline__ void sort2(uint64_t &a, uint64_t &b) {
+  const uint64_t x = a < b ? a : b;
+  b = a < b ? b : a;
+  a = x;
+}
+
+// One 64-bit word per entry: the leading bits of its key (kb bits, taken
+// relative to the smallest possible one), as much of its value (vb bits) as
+// there is room for, and its place in the input.  Words order as (key, value)
+// except among entries that agree in the whole upper part while something was
+// cut off (exact() false).
+struct WordSpec {
+  int kb, vb;
+  __device__ __forceinline__ bool exact() const { return kb + vb <= 64 - kPlace; }
+  __device__ __forceinline__ uint64_t word(uint64_t key, int32_t val, int place) const {
+    const int room = 64 - kPlace;
+    uint64_t u;
+    if (kb >= room) {
+      u = key >> (kb - room);
+    } else {
+      const int w = min(vb, room - kb);
+      u = (key << w) | (uint64_t)((uint32_t)val >> (vb - w));
+    }
+    return u << kPlace | (uint64_t)place;
+  }
+};
+
+// the words [0, n) in shared memory sorted by the block: eight a thread by an
+// odd-even merge network, up to 256 a warp by bitonic merges in registers
+// (no barrier), then merge rounds through shared memory, each thread taking
+// the eight outputs that its merge-path search gives it
+__device__ void sort_words(uint64_t *sk, int n) {
+  const int i0 = threadIdx.x * kItems, lane = threadIdx.x & 31;
+  const bool in = i0 < n;
+  uint64_t k[kItems];
+  if ((int)(threadIdx.x & ~31u) * kItems < n) {  // the warp holds entries
+#pragma unroll
+    for (int q = 0; q < kItems; ++q) k[q] = i0 + q < n ? sk[slot(i0 + q)] : ~0ull;
+    // Batcher's odd-even merge sort of eight
+#pragma unroll
+    for (int p = 1; p < kItems; p <<= 1)
+#pragma unroll
+      for (int h = p; h > 0; h >>= 1)
+#pragma unroll
+        for (int j = h % p; j + h < kItems; j += 2 * h)
+#pragma unroll
+          for (int i = 0; i < h; ++i)
+            if (j + i + h < kItems && (j + i) / (2 * p) == (j + i + h) / (2 * p))
+              sort2(k[j + i], k[j + i + h]);
+    // runs of L lanes -> runs of 2 L lanes: the second run taken backwards,
+    // then half-cleaners across lanes and within the thread
+#pragma unroll
+    for (int L = 1; L < 32; L <<= 1) {
+      uint64_t o[kItems];
+#pragma unroll
+      for (int q = 0; q < kItems; ++q)
+        o[q] = __shfl_xor_sync(0xffffffffu, k[kItems - 1 - q], 2 * L - 1);
+      const bool up = (lane & L) != 0;
+#pragma unroll
+      for (int q = 0; q < kItems; ++q) k[q] = (k[q] < o[q]) != up ? k[q] : o[q];
+#pragma unroll
+      for (int h = L >> 1; h > 0; h >>= 1) {
+        const bool hi = (lane & h) != 0;
+#pragma unroll
+        for (int q = 0; q < kItems; ++q) {
+          const uint64_t x = __shfl_xor_sync(0xffffffffu, k[q], h);
+          k[q] = (k[q] < x) != hi ? k[q] : x;
+        }
+      }
+#pragma unroll
+      for (int h = kItems / 2; h > 0; h >>= 1)
+#pragma unroll
+        for (int q = 0; q < kItems; ++q)
+          if (!(q & h)) sort2(k[q], k[q + h]);
+    }
+#pragma unroll
+    for (int q = 0; q < kItems; ++q)
+      if (i0 + q < n) sk[slot(i0 + q)] = k[q];
+  }
+  __syncthreads();
+  for (int w = 32 * kItems; w < n; w <<= 1) {
+    if (in) {
+      const int base = i0 & ~(2 * w - 1), diag = i0 - base;
+      const int a1 = min(base + w, n), b1 = min(base + 2 * w, n);
+      int lo = max(0, diag - (b1 - a1)), hi = min(diag, a1 - base);
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (sk[slot(base + mid)] < sk[slot(a1 + diag - 1 - mid)]) lo = mid + 1; else hi = mid;
+      }
+      int ia = base + lo, ib = a1 + diag - lo;
+      uint64_t ka = ia < a1 ? sk[slot(ia)] : ~0ull, kb = ib < b1 ? sk[slot(ib)] : ~0ull;
+#pragma unroll
+      for (int q = 0; q < kItems; ++q) {
+        const bool ta = ka <= kb;  // words are distinct but for the filler
+        k[q] = ta ? ka : kb;
+        ia += ta;
+        ib += !ta;
+        const int nx = ta ? ia : ib;
+        const uint64_t nk = nx < (ta ? a1 : b1) ? sk[slot(nx)] : ~0ull;
+        if (ta) ka = nk; else kb = nk;
+      }
+    }
+    __syncthreads();
+    if (in) {
+#pragma unroll
+      for (int q = 0; q < kItems; ++q)
+        if (i0 + q < n) sk[slot(i0 + q)] = k[q];
+    }
+    __syncthreads();
+  }
+}
+
+// entries [0, n) of (sk, sv) sorted by (key, value) in merge rounds: the plain
+// form for entries that sort_words cannot tell apart
+__device__ __noinline__ void block_sort(uint64_t *sk, int32_t *sv, int n) {
+  const int i0 = threadIdx.x * kItems;
+  const bool in = i0 < n;
+  uint64_t k[kItems];
+  int32_t v[kItems];
+  for (int w = 1; w < n; w <<= 1) {
+    if (in) {
+      int last = -1, ia = 0, ib = 0, a1 = 0, b1 = 0;
+      for (int q = 0; q < kItems && i0 + q < n; ++q) {
+        const int base = (i0 + q) & ~(2 * w - 1);
+        if (base != last) {
+          const int diag = i0 + q - base;
+          last = base;
+          a1 = min(base + w, n);
+          b1 = min(base + 2 * w, n);
+          int lo = max(0, diag - (b1 - a1)), hi = min(diag, a1 - base);
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            const int pa = slot(base + mid), pb = slot(a1 + diag - 1 - mid);
+            if (pair_less(sk[pa], sv[pa], sk[pb], sv[pb])) lo = mid + 1; else hi = mid;
+          }
+          ia = base + lo;
+          ib = a1 + diag - lo;
+        }
+        const bool ta = ib >= b1 || (ia < a1 && pair_less(sk[slot(ia)], sv[slot(ia)],
+                                                          sk[slot(ib)], sv[slot(ib)]));
+        const int f = slot(ta ? ia++ : ib++);
+        k[q] = sk[f];
+        v[q] = sv[f];
+      }
+    }
+    __syncthreads();
+    if (in)
+      for (int q = 0; q < kItems && i0 + q < n; ++q) {
+        sk[slot(i0 + q)] = k[q];
+        sv[slot(i0 + q)] = v[q];
+      }
+    __syncthreads();
+  }
+}
+
+// n entries of (ik, iv) (at most eight a thread) sorted into (ok, ov), which
+// may be the same arrays; keys are at least lo and below lo + 2^kb.  With ok
+// null the result stays in shared memory (*sk, *sv in slots).
+__device__ void sort_entries(const uint64_t *ik, const int32_t *iv, uint64_t *ok, int32_t *ov,
+                             int n, uint64_t lo, int kb, int vb, uint64_t *sk, int32_t *sv) {
+  const WordSpec ws{kb, vb};
+  const int t = threadIdx.x, nt = blockDim.x;
+  for (int i = t; i < n; i += nt) sk[slot(i)] = ws.word(ik[i] - lo, iv[i], i);
+  __syncthreads();
+  sort_words(sk, n);
+  // entries whose words agree but for the place: short runs (two bodies in a
+  // cell) put in order here, longer ones by the plain sort
+  bool bad = false;
+  if (!ws.exact()) {
+    for (int i = t; i < n; i += nt) {
+      const uint64_t w = sk[slot(i)] >> kPlace;
+      if (i > 0 && sk[slot(i - 1)] >> kPlace == w) continue;
+      int e = i + 1;
+      while (e < n && e - i <= 8 && sk[slot(e)] >> kPlace == w) ++e;
+      if (e - i > 8) {
+        bad = true;
+      } else {
+        for (int u = i + 1; u < e; ++u) {
+          const uint64_t x = sk[slot(u)];
+          const int px = (int)(x & ((1u << kPlace) - 1u));
+          int z = u - 1;
+          for (; z >= i; --z) {
+            const uint64_t y = sk[slot(z)];
+            const int py = (int)(y & ((1u << kPlace) - 1u));
+            if (!pair_less(ik[px], iv[px], ik[py], iv[py])) break;
+            sk[slot(z + 1)] = y;
+          }
+          sk[slot(z + 1)] = x;
+        }
+      }
+    }
+    if (__syncthreads_or(bad)) {
+      for (int i = t; i < n; i += nt) { sk[slot(i)] = ik[i]; sv[slot(i)] = iv[i]; }
+      __syncthreads();
+      block_sort(sk, sv, n);
+      if (ok)
+        for (int i = t; i < n; i += nt) { ok[i] = sk[slot(i)]; ov[i] = sv[slot(i)]; }
+      __syncthreads();
+      return;
+    }
+  }
+  uint64_t k[kItems];
+  int32_t v[kItems];
+#pragma unroll
+  for (int q = 0; q < kItems; ++q) {
+    const int i = t + q * nt;
+    if (i < n) {
+      const int p = (int)(sk[slot(i)] & ((1u << kPlace) - 1u));
+      k[q] = ik[p];
+      v[q] = iv[p];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kItems; ++q) {
+    const int i = t + q * nt;
+    if (i < n) {
+      if (ok) { ok[i] = k[q]; ov[i] = v[q]; }
+      else { sk[slot(i)] = k[q]; sv[slot(i)] = v[q]; }
+    }
+  }
+  __syncthreads();
+}
+
+// up to kBlockSortMax entries, in place
+__global__ void __launch_bounds__(1024) k_sort_block(uint64_t *keys, int32_t *vals,
+                                                     const int64_t *d_n, int kb, int vb) {
+  pdl_wait();
+  extern __shared__ __align__(16) unsigned char sort_mem[];
+  uint64_t *sk = reinterpret_cast<uint64_t *>(sort_mem);
+  int32_t *sv = reinterpret_cast<int32_t *>(sk + kBlockSortMax + kBlockSortMax / 8);
+  sort_entries(keys, vals, keys, vals, (int)*d_n, 0, kb, vb, sk, sv);
+}
+
+// the splitters of `buckets` buckets; a short input is sorted here and now.
+// The samples are gathered into (tk, tv), kBlockSortMax entries of scratch
+__global__ void __launch_bounds__(1024) k_sort_sample(uint64_t *keys, int32_t *vals,
+                                                      const int64_t *d_n, int buckets, int kb,
+                                                      int vb, SortWork *w, uint64_t *tk,
+                                                      int32_t *tv) {
+  pdl_wait();
+  extern __shared__ __align__(16) unsigned char sort_mem[];
+  uint64_t *sk = reinterpret_cast<uint64_t *>(sort_mem);
+  int32_t *sv = reinterpret_cast<int32_t *>(sk + kBlockSortMax + kBlockSortMax / 8);
+  const int64_t n = *d_n;
+  const int t = threadIdx.x;
+  const bool small = n <= kBlockSortMax;
+  if (t < buckets) w->count[t] = 0;
+  if (t == 0) w->done = small ? 1 : 0;
+  if (small) {
+    sort_entries(keys, vals, keys, vals, (int)n, 0, kb, vb, sk, sv);
+    return;
+  }
+  const int per = kSamples / buckets < 8 ? kSamples / buckets : 8, ns = per * buckets;
+  uint64_t k[kSamples / 1024];
+  int32_t v[kSamples / 1024];
+#pragma unroll
+  for (int q = 0; q < kSamples / 1024; ++q) {
+    const int i = t + q * 1024;
+    const int64_t e = (int64_t)(i < ns ? i : 0) * n / ns;
+    k[q] = keys[e];
+    v[q] = vals[e];
+  }
+#pragma unroll
+  for (int q = 0; q < kSamples / 1024; ++q)
+    if (t + q * 1024 < ns) { tk[t + q * 1024] = k[q]; tv[t + q * 1024] = v[q]; }
+  __syncthreads();
+  sort_entries(tk, tv, nullptr, nullptr, ns, 0, kb, vb, sk, sv);
+  if (t > 0 && t < buckets) {
+    w->skey[t - 1] = sk[slot(per * t)];
+    w->sval[t - 1] = sv[slot(per * t)];
+  }
+}
+
+constexpr int kClassThreads = 512;
+constexpr int kClassPer = 4;
+constexpr int kClassTile = kClassThreads * kClassPer;
+
+// each key's bucket (the number of splitters at or below it, a power of two of
+// buckets searched without branches) and its place in the bucket
+__global__ void __launch_bounds__(kClassThreads) k_sort_class(const uint64_t *keys,
+                                                              const int32_t *vals,
+                                                              const int64_t *d_n, int buckets,
+                                                              int kb, SortWork *w,
+                                                              uint32_t *where) {
+  pdl_wait();
+  // searched by the splitters' leading 32 bits (half the shared-memory
+  // conflicts of 64-bit words), the rest read on equality
+  __shared__ uint32_t sl[kMaxBuckets];
+  __shared__ uint64_t sk[kMaxBuckets];
+  __shared__ int32_t sv[kMaxBuckets];
+  __shared__ uint32_t h[kMaxBuckets];
+  const int64_t n = *d_n, base = (int64_t)blockIdx.x * kClassTile;
+  const int sh = kb > 32 ? kb - 32 : 0;
+  const int t = threadIdx.x;
+  if (base >= n || w->done) return;
+  uint64_t k[kClassPer];
+  int32_t v[kClassPer];
+#pragma unroll
+  for (int q = 0; q < kClassPer; ++q) {
+    const int64_t e = base + q * kClassThreads + t;
+    k[q] = e < n ? keys[e] : 0ull;
+    v[q] = e < n ? vals[e] : 0;
+  }
+  for (int b = t; b < buckets; b += kClassThreads) {
+    sk[b] = w->skey[b];
+    sv[b] = w->sval[b];
+    sl[b] = (uint32_t)(sk[b] >> sh);
+    h[b] = 0;
+  }
+  __syncthreads();
+  uint32_t bk[kClassPer] = {}, r[kClassPer];
+  for (int step = buckets >> 1; step > 0; step >>= 1)
+#pragma unroll
+    for (int q = 0; q < kClassPer; ++q) {
+      const int m = (int)bk[q] + step - 1;
+      const uint32_t x = sl[m], kl = (uint32_t)(k[q] >> sh);
+      if (x < kl || (x == kl && !pair_less(k[q], v[q], sk[m], sv[m]))) bk[q] += step;
+    }
+#pragma unroll
+  for (int q = 0; q < kClassPer; ++q)
+    r[q] = base + q * kClassThreads + t < n ? atomicAdd(&h[bk[q]], 1u) : 0u;
+  __syncthreads();
+  for (int b = t; b < buckets; b += kClassThreads)
+    if (h[b]) h[b] = atomicAdd(&w->count[b], h[b]);
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kClassPer; ++q) {
+    const int64_t e = base + q * kClassThreads + t;
+    if (e < n) where[e] = bk[q] << kPosBits | (h[bk[q]] + r[q]);
+  }
+}
+
+__global__ void __launch_bounds__(kClassThreads) k_sort_move(const uint64_t *keys,
+                                                             const int32_t *vals, uint64_t *okeys,
+                                                             int32_t *ovals, const int64_t *d_n,
+                                                             int buckets, SortWork *w,
+                                                             const uint32_t *where) {
+  pdl_wait();
+  __shared__ int64_t sh[33];
+  __shared__ uint32_t start[kMaxBuckets];
+  const int64_t n = *d_n, base = (int64_t)blockIdx.x * kClassTile;
+  const int t = threadIdx.x;
+  if (base >= n || w->done) return;
+  uint64_t k[kClassPer];
+  int32_t v[kClassPer];
+  uint32_t p[kClassPer];
+#pragma unroll
+  for (int q = 0; q < kClassPer; ++q) {
+    const int64_t e = base + q * kClassThreads + t;
+    if (e < n) { k[q] = keys[e]; v[q] = vals[e]; p[q] = where[e]; }
+  }
+  const uint32_t c0 = 2 * t < buckets ? w->count[2 * t] : 0u,
+                 c1 = 2 * t + 1 < buckets ? w->count[2 * t + 1] : 0u;
+  int64_t ex;
+  block_excl_scan((int64_t)c0 + c1, &ex, sh);
+  if (2 * t < kMaxBuckets) {
+    start[2 * t] = (uint32_t)ex;
+    start[2 * t + 1] = (uint32_t)ex + c0;
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    for (int b = t; b < buckets; b += kClassThreads) w->start[b] = start[b];
+    if (t == 0) w->start[buckets] = (uint32_t)n;
+  }
+#pragma unroll
+  for (int q = 0; q < kClassPer; ++q)
+    if (base + q * kClassThreads + t < n) {
+      const uint32_t d = start[p[q] >> kPosBits] + (p[q] & ((1u << kPosBits) - 1u));
+      okeys[d] = k[q];
+      ovals[d] = v[q];
+    }
+}
+
+// a bucket a block, from (ik, iv) into (ok, ov); one that does not fit (rare)
+// is sorted in runs that do, the runs then merged through global memory
+__global__ void __launch_bounds__(kLocalThreads, 3) k_sort_local(uint64_t *ik, int32_t *iv,
+                                                              uint64_t *ok, int32_t *ov,
+                                                              int buckets, int key_bits, int vb,
+                                                              const SortWork *w) {
+  pdl_wait();
+  extern __shared__ __align__(16) unsigned char sort_mem[];
+  uint64_t *sk = reinterpret_cast<uint64_t *>(sort_mem);
+  int32_t *sv = reinterpret_cast<int32_t *>(sk + kLocalMax + kLocalMax / 8);
+  if (w->done) return;
+  const int b = blockIdx.x;
+  const uint32_t s0 = w->start[b];
+  const int n = (int)(w->start[b + 1] - s0);
+  // the bucket's keys lie between its splitters
+  const uint64_t lo = b > 0 ? w->skey[b - 1] : 0ull;
+  const uint64_t hi = b < buckets - 1 ? w->skey[b]
+                                      : (key_bits < 64 ? (1ull << key_bits) - 1 : ~0ull);
+  const int kb = 64 - __clzll((long long)(hi - lo));
+  ik += s0; iv += s0; ok += s0; ov += s0;
+  for (int c = 0; c < n; c += kLocalMax)
+    sort_entries(ik + c, iv + c, ok + c, ov + c, min(kLocalMax, n - c), lo, kb, vb, sk, sv);
+  for (int r = kLocalMax; r < n; r *= 2) {
+    __threadfence_block();
+    __syncthreads();
+    // runs of r in (ok, ov) merged into (ik, iv), then copied back
+    for (int o = threadIdx.x * kItems; o < n; o += kLocalThreads * kItems) {
+      const int base = o / (2 * r) * (2 * r), diag = o - base;
+      const int a1 = min(base + r, n), b1 = min(base + 2 * r, n);
+      int lo = max(0, diag - (b1 - a1)), hi = min(diag, a1 - base);
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1, pa = base + mid, pb = a1 + diag - 1 - mid;
+        if (pair_less(ok[pa], ov[pa], ok[pb], ov[pb])) lo = mid + 1; else hi = mid;
+      }
+      int ia = base + lo, ib = a1 + diag - lo;
+      for (int q = 0; q < kItems && o + q < b1; ++q) {
+        const bool ta = ib >= b1 || (ia < a1 && pair_less(ok[ia], ov[ia], ok[ib], ov[ib]));
+        const int f = ta ? ia++ : ib++;
+        ik[o + q] = ok[f];
+        iv[o + q] = ov[f];
+      }
+    }
+    __threadfence_block();
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += kLocalThreads) { ok[i] = ik[i]; ov[i] = iv[i]; }
+  }
+}
+
 }  // namespace
 
 int64_t p3t_scan_state_words(int64_t n_cap) {
@@ -399,5 +869,52 @@ int p3t_radix_sort(uint64_t **keys, int32_t **vals, uint64_t **keys_alt,
     uint64_t *tk = *keys; *keys = *keys_alt; *keys_alt = tk;
     int32_t *tv = *vals; *vals = *vals_alt; *vals_alt = tv;
   }
+  return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
+}
+
+size_t p3t_sort_work_bytes() { return sizeof(SortWork); }
+
+// dynamic shared memory above 48 KB is granted per function and device
+static bool sort_attr(const void *f, size_t bytes) {
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) ==
+         cudaSuccess;
+}
+
+bool p3t_sort_prepare() {
+  return sort_attr((const void *)k_sort_block, sort_smem(kBlockSortMax)) &&
+         sort_attr((const void *)k_sort_sample, sort_smem(kBlockSortMax)) &&
+         sort_attr((const void *)k_sort_local, sort_smem(kLocalMax));
+}
+
+int p3t_sort_pairs(uint64_t **keys, int32_t **vals, uint64_t **keys_alt, int32_t **vals_alt,
+                   const int64_t *d_n, int64_t n_cap, int key_bits, uint32_t *hist,
+                   int64_t hist_cap, void *work, uint32_t *where, cudaStream_t s) {
+  int vb = 1;  // bits of a value below n_cap
+  while (vb < 31 && ((int64_t)1 << vb) < n_cap) ++vb;
+  if (n_cap <= kBlockSortMax) {
+    pdl_launch(k_sort_block, dim3(1), dim3(1024), sort_smem(kBlockSortMax), s, *keys, *vals, d_n,
+               key_bits, vb);
+    p3t_note_launches(1);
+    return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
+  }
+  // four radix passes take less than the sample sort's launches
+  if (n_cap > kSampleMax || key_bits <= 32)
+    return p3t_radix_sort(keys, vals, keys_alt, vals_alt, d_n, n_cap, 0, key_bits, hist, hist_cap,
+                          s);
+  int buckets = 16;  // about 1,000 keys each
+  while (buckets < kMaxBuckets && (int64_t)buckets * 1000 < n_cap) buckets *= 2;
+  SortWork *w = static_cast<SortWork *>(work);
+  const unsigned tiles = (unsigned)((n_cap + kClassTile - 1) / kClassTile);
+  // the samples stand in the second buffers (n_cap > kBlockSortMax entries)
+  // until the keys move there
+  pdl_launch(k_sort_sample, dim3(1), dim3(1024), sort_smem(kBlockSortMax), s, *keys, *vals, d_n,
+             buckets, key_bits, vb, w, *keys_alt, *vals_alt);
+  pdl_launch(k_sort_class, dim3(tiles), dim3(kClassThreads), 0, s, *keys, *vals, d_n, buckets,
+             key_bits, w, where);
+  pdl_launch(k_sort_move, dim3(tiles), dim3(kClassThreads), 0, s, *keys, *vals, *keys_alt,
+             *vals_alt, d_n, buckets, w, where);
+  pdl_launch(k_sort_local, dim3((unsigned)buckets), dim3(kLocalThreads), sort_smem(kLocalMax), s,
+             *keys_alt, *vals_alt, *keys, *vals, buckets, key_bits, vb, w);
+  p3t_note_launches(4);
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }

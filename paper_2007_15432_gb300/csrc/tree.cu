@@ -1246,8 +1246,8 @@ int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s) {
   pdl_launch(k_cut_u2, dim3((unsigned)g), dim3(kBlock), 0, s, sv, p->x, p->y, p->z, p->vx, p->vy, p->vz, mu,
                                           c->box_bits, nb, c->seg_nb, c->seg_base, c->seg_l,
                                           u2, c->keys, c->idx, bin, bcnt);
-  int rc = p3t_radix_sort(&c->keys, &c->idx, &c->keys_alt, &c->idx_alt, d_n, c->cap, 0, 16,
-                          c->radix_hist, c->radix_hist_cap, s);
+  int rc = p3t_sort_pairs(&c->keys, &c->idx, &c->keys_alt, &c->idx_alt, d_n, c->cap, 16,
+                          c->radix_hist, c->radix_hist_cap, c->sort_work, p3t_sort_where(c), s);
   if (rc) return rc;
   pdl_launch(k_cut_offsets, dim3(1), dim3(1024), 0, s, nb, bcnt, boff);
   pdl_launch(k_cut_binsum, dim3((unsigned)p3t_grid((int64_t)nb * 32, kBlock, (int64_t)c->num_sms * 4)), dim3(kBlock), 0, s, nb, boff, c->idx, u2, bsum);
@@ -1279,8 +1279,8 @@ int p3t_run_build_tree(p3t_ctx *c, const p3t_particles *p, cudaStream_t s) {
   pdl_launch(k_box_final, dim3(1), dim3(256), 0, s, c->box_bits, c->box, nseg);
   pdl_launch(k_keys, dim3((unsigned)g), dim3(kBlock), 0, s, sv, p->x, p->y, p->z, p->m, p->r_out, p->r_search,
                                         c->box, c->keys, c->idx, c->pack, 0, &cnt[0]);
-  rc = p3t_radix_sort(&c->keys, &c->idx, &c->keys_alt, &c->idx_alt, &cnt[0], c->cap,
-                      0, 64, c->radix_hist, c->radix_hist_cap, s);
+  rc = p3t_sort_pairs(&c->keys, &c->idx, &c->keys_alt, &c->idx_alt, &cnt[0], c->cap, 63,
+                      c->radix_hist, c->radix_hist_cap, c->sort_work, p3t_sort_where(c), s);
   if (rc) return rc;
   if (nseg > 1) {
     // stable sort by segment (the most significant digit of (segment, key)),
