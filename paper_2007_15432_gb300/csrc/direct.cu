@@ -8,11 +8,25 @@
 // the pair arithmetic's type; a block is 8 warps over 64 targets (two per
 // lane); each warp takes one eighth of the block's source range and stages
 // it 32 sources at a time in its own shared-memory slots (one broadcast load
-// per 4-vector, shared by the lane's two targets).  A grid column
-// (blockIdx.y) is one split of the sources; each block adds its 8 warps in
-// order and writes its per-target sums to part[(split * C + c) * n + k];
-// the last block of a target tile to finish adds the splits in order: the
-// result does not depend on scheduling.
+// per 4-vector, shared by the lane's two targets).  A grid column (blockIdx.y) is one split of the sources; each
+// block adds its 8 warps in order and writes its per-target sums to
+// part[(split * C + c) * n + k]; the last block of a target tile to finish
+// adds the splits in order: the result does not depend on scheduling.
+//
+// Far sources: with the particles in no spatial order a source is inside the
+// cut-off reach of some target of a warp about once in a thousand times (ring
+// of 10,000: 1e-5 a pair).  Each source carries a bound T on max(r_out)^2 over
+// the warp's targets and itself; a chunk of 32 sources is summed without the
+// changeover (K = 1, K' = 0: the same bits in FP32 for 18 packed instructions
+// instead of 32 a pair, 43 instead of 63 for the VJP), and when some r^2 of
+// the warp was within its bound it is summed again in full (and the next one
+// in full at once, as long as near pairs are met); in FP64, where a vote costs
+// little beside a pair, each source is voted on.  What bounds the kernels is
+// the FP32 (FP64) pipe: a packed instruction holds it two cycles (73 % active at
+// N = 50,000).  Measured per call, FP32: force N = 1e4 150 -> 125 us, 5e4 2,550
+// -> 1,670, VJP 242 -> 199, 4,663 -> 3,352; FP64: force N = 8,191 3,000 -> 2,130,
+// VJP N = 1e4 8,984 -> 7,370.  Four targets a lane: 1,590 us at 5e4, 128 at 1e4
+// and 50 instead of 45 at 1,000 (fewer, longer blocks): two kept.
 //
 // Precision: FP64 throughout, or (MIXED) float-float positions whose
 // difference (hi_k - hi_j) + (lo_k - lo_j) carries the relative coordinate
@@ -21,8 +35,6 @@
 // instruction runs inside the pair loop.
 #include <math.h>
 
-#include <type_traits>
-
 #include "p3t_internal.cuh"
 
 namespace {
@@ -30,6 +42,7 @@ namespace {
 constexpr int kDW = 8;          // warps per block
 constexpr int kDT = 2;          // targets per lane
 constexpr int kDTB = 32 * kDT;  // targets per block
+constexpr int kSplitBlocks = 3;  // blocks an SM that the sources' split counts with
 #ifndef P3T_DIRECT_MINB_MIXED
 #define P3T_DIRECT_MINB_MIXED 3  // resident blocks per SM asked of the FP32 kernels
 #endif
@@ -48,8 +61,6 @@ struct DT<true> {
   using T = float;
 };
 
-__device__ __forceinline__ double rsq(double a) { return rsqrt(a); }
-
 // hi + lo += p without losing the rounding error of the addition (TwoSum)
 __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float p) {
   const float s = hi + p;
@@ -58,44 +69,57 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float p) {
   hi = s;
 }
 
-// one pair term: k the target (its mass, 1/r_out and adjoint), j the source
-template <typename T, bool VJP>
-__device__ __forceinline__ void pair_term(T rx, T ry, T rz, const Q4<T> &A, T iroj,
-                                          const Q4<T> &L, T mk, T irok, T lxk, T lyk, T lzk,
-                                          T g, T i1mg, T *acc) {
-  // the FP64 path's term (the mixed path uses pair_term2)
-  static_assert(std::is_same<T, double>::value, "FP64 pair term");
-  const T r2 = rx * rx + ry * ry + rz * rz;
-  const T ir = rsq(r2);
-  const T irout = irok < iroj ? irok : iroj;  // 1 / max(r_out,k, r_out,j)
-  const T yv = r2 * ir * irout;
-  // y <= gamma: K = K' = 0.  The target itself (r2 = 0) gives 0 * inf = NaN
-  // and leaves here too.
-  if (!(yv > g)) return;
-  T K = 1, dKr = 0;     // K(y) and K'(y) / r_out
-  if (yv < (T)1) {
-    const T u = (yv - g) * i1mg, u2 = u * u, u3 = u2 * u;
-    K = u2 * u2 * ((T)35 - (T)84 * u + (T)70 * u2 - (T)20 * u3);
+// r^-3 from r^2 with the seed's y and e = 1 - r^2 y^2 (see rsqrt_seed); 0 for
+// r = 0
+__device__ __forceinline__ double inv_cube(double r2, double &y, double &e) {
+  y = rsqrt_seed(r2);
+  const double y2 = y * y, y3 = y2 * y;
+  e = fma(-r2, y2, 1.0);
+  return fma(y3 * e, fma(1.875, e, 1.5), y3);
+}
+
+// one FP64 pair term: k the target (its mass, 1/r_out and adjoint), j the
+// source; NEAR: with the changeover.  The target itself (r = 0) has y = 0, K =
+// K' = 0.
+template <bool VJP, bool NEAR>
+__device__ __forceinline__ void pair_term(double rx, double ry, double rz, double r2,
+                                          const Q4<double> &A, double iroj, const Q4<double> &L,
+                                          double mk, double irok, double lxk, double lyk,
+                                          double lzk, double g, double i1mg, double *acc) {
+  double y, e;
+  double phi = inv_cube(r2, y, e);  // K / r^3 below
+  double dKr = 0.0, K = 1.0;        // K'(y) / r_out
+  if constexpr (NEAR) {
+    const double irout = irok < iroj ? irok : iroj;  // 1 / max(r_out,k, r_out,j)
+    const double ir = fma(y * e, fma(0.375, e, 0.5), y);
+    const double yv = r2 * ir * irout;
+    const double t = (yv - g) * i1mg;
+    // NaN (r = 0 with r_out = 0) stays below
+    const double u = t > 0.0 ? (t < 1.0 ? t : 1.0) : 0.0, u2 = u * u;
+    K = (u2 * u2) * fma(fma(fma(-20.0, u, 70.0), u, -84.0), u, 35.0);
+    phi *= K;
     if constexpr (VJP) {
-      const T v = (T)1 - u;
-      dKr = (T)140 * u3 * (v * v * v) * i1mg * irout;
+      // zero at both ends also where 1 / r_out is infinite
+      const double v = 1.0 - u, ie = u > 0.0 && u < 1.0 ? irout : 0.0;
+      dKr = 140.0 * (u2 * u) * (v * v * v) * i1mg * ie;
     }
   }
-  const T ir2 = ir * ir;
-  const T phi = K * ir2 * ir;
   if constexpr (!VJP) {
-    const T w = A.w * phi;  // m_j K / r^3
-    acc[0] += w * rx;
-    acc[1] += w * ry;
-    acc[2] += w * rz;
+    const double w = A.w * phi;  // m_j K / r^3
+    acc[0] = fma(w, rx, acc[0]);
+    acc[1] = fma(w, ry, acc[1]);
+    acc[2] = fma(w, rz, acc[2]);
   } else {
-    const T psi = ir2 * ir2 * (dKr - (T)3 * K * ir);
-    const T wx = mk * L.x - A.w * lxk, wy = mk * L.y - A.w * lyk, wz = mk * L.z - A.w * lzk;
-    const T prw = psi * (rx * wx + ry * wy + rz * wz);
-    acc[0] += phi * wx + prw * rx;
-    acc[1] += phi * wy + prw * ry;
-    acc[2] += phi * wz + prw * rz;
-    acc[3] += phi * (L.x * rx + L.y * ry + L.z * rz);
+    const double y2 = y * y, ir2 = fma(y2, fma(e, e, e), y2);  // y^2 / (1 - e)
+    double psi = -3.0 * (phi * ir2);
+    if constexpr (NEAR) psi = fma(ir2 * ir2, dKr, psi);
+    const double wx = fma(mk, L.x, -A.w * lxk), wy = fma(mk, L.y, -A.w * lyk),
+                 wz = fma(mk, L.z, -A.w * lzk);
+    const double prw = psi * fma(rx, wx, fma(ry, wy, rz * wz));
+    acc[0] += fma(phi, wx, prw * rx);
+    acc[1] += fma(phi, wy, prw * ry);
+    acc[2] += fma(phi, wz, prw * rz);
+    acc[3] = fma(phi, fma(L.x, rx, fma(L.y, ry, L.z * rz)), acc[3]);
   }
 }
 
@@ -135,6 +159,35 @@ __device__ __forceinline__ void pair_term2(f2 rx, f2 ry, f2 rz, const Q4<float> 
     const f2 v = sub2(k.one, u);
     const f2 dKr = mul2(mul2(mul2(k.c140i, u3), mul2(mul2(v, v), v)), irout);
     const f2 psi = mul2(mul2(ir2, ir2), sub2(dKr, mul2(mul2(k.three, K), ir)));
+    const f2 mA = f2_dup(A.w);
+    const f2 wx = sub2(mul2(mk, f2_dup(L.x)), mul2(mA, lxk));
+    const f2 wy = sub2(mul2(mk, f2_dup(L.y)), mul2(mA, lyk));
+    const f2 wz = sub2(mul2(mk, f2_dup(L.z)), mul2(mA, lzk));
+    const f2 prw = mul2(psi, fma2(rx, wx, fma2(ry, wy, mul2(rz, wz))));
+    acc[0] = add2(acc[0], fma2(phi, wx, mul2(prw, rx)));
+    acc[1] = add2(acc[1], fma2(phi, wy, mul2(prw, ry)));
+    acc[2] = add2(acc[2], fma2(phi, wz, mul2(prw, rz)));
+    acc[3] = fma2(phi, fma2(f2_dup(L.x), rx, fma2(f2_dup(L.y), ry, mul2(f2_dup(L.z), rz))),
+                  acc[3]);
+  }
+}
+
+// the same with K = 1 and K' = 0 (every r beyond max(r_out)): pair_term2's
+// operations without those that return their operand, so the same bits
+template <bool VJP>
+__device__ __forceinline__ void pair_far2(f2 rx, f2 ry, f2 rz, f2 r2, const Q4<float> &A,
+                                          const Q4<float> &L, f2 mk, f2 lxk, f2 lyk, f2 lzk,
+                                          f2 m3, f2 *acc) {
+  const f2 ir = f2_pk(rsqrtf(f2_lo(r2)), rsqrtf(f2_hi(r2)));
+  const f2 ir2 = mul2(ir, ir);
+  const f2 phi = mul2(ir2, ir);
+  if constexpr (!VJP) {
+    const f2 w = mul2(f2_dup(A.w), phi);
+    acc[0] = fma2(w, rx, acc[0]);
+    acc[1] = fma2(w, ry, acc[1]);
+    acc[2] = fma2(w, rz, acc[2]);
+  } else {
+    const f2 psi = mul2(mul2(ir2, ir2), mul2(m3, ir));  // m3 = -3
     const f2 mA = f2_dup(A.w);
     const f2 wx = sub2(mul2(mk, f2_dup(L.x)), mul2(mA, lxk));
     const f2 wy = sub2(mul2(mk, f2_dup(L.y)), mul2(mA, lyk));
@@ -189,6 +242,11 @@ __global__ void k_direct_pack(int64_t n, const double *x, const double *y, const
   }
 }
 
+// the targets of one packed pair
+struct Pair2 {
+  f2 xh, yh, zh, xl, yl, zl, m, iro, lx, ly, lz;
+};
+
 template <bool MIXED, bool VJP>
 __global__ void __launch_bounds__(kDW * 32, MIXED ? P3T_DIRECT_MINB_MIXED : 1)
     k_direct(int64_t n, int64_t chunk, const Q4<typename DT<MIXED>::T> *__restrict__ PA,
@@ -198,53 +256,69 @@ __global__ void __launch_bounds__(kDW * 32, MIXED ? P3T_DIRECT_MINB_MIXED : 1)
   pdl_wait();
   using T = typename DT<MIXED>::T;
   constexpr int NC = VJP ? 4 : 3;
+  constexpr int DTL = kDT, DTB = kDTB;
+  constexpr int NP = MIXED ? DTL / 2 : 1;           // packed pairs a lane
   __shared__ Q4<T> sA[kDW][32];                     // x_hi, y_hi, z_hi, m
   __shared__ Q4<T> sB[kDW][32];                     // x_lo, y_lo, z_lo, 1 / r_out
   __shared__ Q4<T> sL[VJP ? kDW : 1][VJP ? 32 : 1];  // lam
+  __shared__ T sT[kDW][32];                          // bound on max(r_out)^2, widened
   // the 8 warps' sums: FP64, or (MIXED) float-float pairs added with FP32
-  // instructions only (an FP64 instruction costs 64 FP32 issue slots here)
-  __shared__ double red[MIXED ? 1 : kDW][NC][MIXED ? 1 : kDTB];
-  __shared__ float red_h[MIXED ? kDW : 1][NC][MIXED ? kDTB : 1];
-  __shared__ float red_l[MIXED ? kDW : 1][NC][MIXED ? kDTB : 1];
+  // instructions only (an FP64 instruction costs 64 FP32 issue slots here);
+  // the mixed running sums stand here too
+  __shared__ double red[MIXED ? 1 : kDW][NC][MIXED ? 1 : DTB];
+  __shared__ float red_h[MIXED ? kDW : 1][NC][MIXED ? DTB : 1];
+  __shared__ float red_l[MIXED ? kDW : 1][NC][MIXED ? DTB : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const T g = (T)gamma, i1mg = (T)(1.0 / (1.0 - gamma));
 
-  T txh[kDT], tyh[kDT], tzh[kDT], txl[kDT], tyl[kDT], tzl[kDT];
-  T tm[kDT], tiro[kDT], tlx[kDT], tly[kDT], tlz[kDT];
+  T txh[DTL], tyh[DTL], tzh[DTL], txl[DTL], tyl[DTL], tzl[DTL];
+  T tm[DTL], tiro[DTL], tlx[DTL], tly[DTL], tlz[DTL];
+  T tmax = 0;  // largest r_out^2 of the lane's targets
 #pragma unroll
-  for (int t = 0; t < kDT; ++t) {
-    const int64_t k = (int64_t)blockIdx.x * kDTB + t * 32 + lane;
-    txh[t] = tyh[t] = tzh[t] = txl[t] = tyl[t] = tzl[t] = 0;
+  for (int t = 0; t < DTL; ++t) {
+    const int64_t k = (int64_t)blockIdx.x * DTB + t * 32 + lane;
+    txh[t] = tyh[t] = tzh[t] = (T)1e18;  // far from every source
+    txl[t] = tyl[t] = tzl[t] = 0;
     tm[t] = tiro[t] = tlx[t] = tly[t] = tlz[t] = 0;  // 1/r_out = 0: no pair term
     if (k < n) {
       const Q4<T> a = PA[k], b = PB[k];
       txh[t] = a.x; tyh[t] = a.y; tzh[t] = a.z; tm[t] = a.w;
       txl[t] = b.x; tyl[t] = b.y; tzl[t] = b.z; tiro[t] = b.w;
+      const T ro = (T)1 / b.w;
+      tmax = fmax(tmax, ro * ro);
       if constexpr (VJP) {
         const Q4<T> l = PL[k];
         tlx[t] = l.x; tly[t] = l.y; tlz[t] = l.z;
       }
     }
   }
-  struct TP {
-    f2 xh, yh, zh, xl, yl, zl, m, iro, lx, ly, lz;
-  } P{};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tmax = fmax(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+  Pair2 P[NP];
   PairConst2 kc{};
   if constexpr (MIXED) {
-    P = TP{f2_pk(txh[0], txh[1]), f2_pk(tyh[0], tyh[1]), f2_pk(tzh[0], tzh[1]),
-           f2_pk(txl[0], txl[1]), f2_pk(tyl[0], tyl[1]), f2_pk(tzl[0], tzl[1]),
-           f2_pk(tm[0], tm[1]), f2_pk(tiro[0], tiro[1]), f2_pk(tlx[0], tlx[1]),
-           f2_pk(tly[0], tly[1]), f2_pk(tlz[0], tlz[1])};
+#pragma unroll
+    for (int p = 0; p < NP; ++p)
+      P[p] = Pair2{f2_pk(txh[2 * p], txh[2 * p + 1]), f2_pk(tyh[2 * p], tyh[2 * p + 1]),
+                   f2_pk(tzh[2 * p], tzh[2 * p + 1]), f2_pk(txl[2 * p], txl[2 * p + 1]),
+                   f2_pk(tyl[2 * p], tyl[2 * p + 1]), f2_pk(tzl[2 * p], tzl[2 * p + 1]),
+                   f2_pk(tm[2 * p], tm[2 * p + 1]), f2_pk(tiro[2 * p], tiro[2 * p + 1]),
+                   f2_pk(tlx[2 * p], tlx[2 * p + 1]), f2_pk(tly[2 * p], tly[2 * p + 1]),
+                   f2_pk(tlz[2 * p], tlz[2 * p + 1])};
     kc = PairConst2{f2_dup((float)g), f2_dup((float)i1mg), f2_dup(35.f), f2_dup(84.f),
                     f2_dup(70.f), f2_dup(20.f), f2_dup(1.f), f2_dup(3.f),
                     f2_dup((float)(140.0 * (1.0 / (1.0 - gamma))))};
+#pragma unroll
+    for (int t = 0; t < DTL; ++t)
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+        red_h[warp][c][t * 32 + lane] = red_l[warp][c][t * 32 + lane] = 0.0f;
   }
-  float fh[kDT][NC], fl[kDT][NC];  // MIXED running sums (float-float)
-  double dd[kDT][NC];              // FP64 running sums
+  double dd[MIXED ? 1 : DTL][NC];  // FP64 running sums
 #pragma unroll
-  for (int t = 0; t < kDT; ++t)
+  for (int t = 0; t < (MIXED ? 1 : DTL); ++t)
 #pragma unroll
-    for (int c = 0; c < NC; ++c) fh[t][c] = fl[t][c] = 0.0f, dd[t][c] = 0.0;
+    for (int c = 0; c < NC; ++c) dd[t][c] = 0.0;
 
   // the split's sources, cut into 8 contiguous, equal (to one source) warp
   // ranges, walked in chunks of 32
@@ -252,79 +326,128 @@ __global__ void __launch_bounds__(kDW * 32, MIXED ? P3T_DIRECT_MINB_MIXED : 1)
   const int64_t b_len = max((int64_t)0, min(n, b_lo + chunk) - b_lo);
   const int64_t s_lo = b_lo + b_len * warp / kDW;
   const int64_t s_hi = b_lo + b_len * (warp + 1) / kDW;
+  bool full = false;  // the last chunk had a near pair: take the next in full form
   for (int64_t cb = s_lo; cb < s_hi; cb += 32) {
     const int lim = (int)min((int64_t)32, s_hi - cb);
     __syncwarp();
     if (lane < lim) {
       const int64_t j = cb + lane;
+      const Q4<T> b = PB[j];
       sA[warp][lane] = PA[j];
-      sB[warp][lane] = PB[j];
+      sB[warp][lane] = b;
       if constexpr (VJP) sL[warp][lane] = PL[j];
+      // widened beyond the rounding of r^2 and 1 / r_out; pairs below 1e-17
+      // (the target itself) take the near form, which bounds r^2 from below
+      const T ro = (T)1 / b.w;
+      sT[warp][lane] = fmax(fmax(tmax, ro * ro) * (T)1.0001, (T)1e-17);
     }
     __syncwarp();
-    T acc[kDT][NC];
-#pragma unroll
-    for (int t = 0; t < kDT; ++t)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) acc[t][c] = 0;
     if constexpr (MIXED) {
-      // the lane's two targets as the halves of packed pairs
-      static_assert(kDT == 2, "two targets per lane");
-      f2 a2[NC];
+      // the lane's targets in packed pairs
+      f2 a2[NP][NC];
+      const f2 m3 = f2_dup(-3.f);
+      bool near = false;
+      if (!full) {
 #pragma unroll
-      for (int c = 0; c < NC; ++c) a2[c] = 0ull;
+        for (int p = 0; p < NP; ++p)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) a2[p][c] = 0ull;
+#pragma unroll 4
+        for (int q = 0; q < lim; ++q) {
+          const Q4<T> A = sA[warp][q], B = sB[warp][q];
+          const float Tq = sT[warp][q];
+          Q4<T> L{0, 0, 0, 0};
+          if constexpr (VJP) L = sL[warp][q];
+#pragma unroll
+          for (int p = 0; p < NP; ++p) {
+            const f2 rx = add2(sub2(P[p].xh, f2_dup(A.x)), sub2(P[p].xl, f2_dup(B.x)));
+            const f2 ry = add2(sub2(P[p].yh, f2_dup(A.y)), sub2(P[p].yl, f2_dup(B.y)));
+            const f2 rz = add2(sub2(P[p].zh, f2_dup(A.z)), sub2(P[p].zl, f2_dup(B.z)));
+            const f2 r2 = fma2(rx, rx, fma2(ry, ry, mul2(rz, rz)));
+            near = near || !(fminf(f2_lo(r2), f2_hi(r2)) > Tq);
+            pair_far2<VJP>(rx, ry, rz, r2, A, L, P[p].m, P[p].lx, P[p].ly, P[p].lz, m3, a2[p]);
+          }
+        }
+        full = __any_sync(0xffffffffu, near);
+      }
+      if (full) {
+#pragma unroll
+        for (int p = 0; p < NP; ++p)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) a2[p][c] = 0ull;
+        near = false;
+#pragma unroll 2
+        for (int q = 0; q < lim; ++q) {
+          const Q4<T> A = sA[warp][q], B = sB[warp][q];
+          const float Tq = sT[warp][q];
+          Q4<T> L{0, 0, 0, 0};
+          if constexpr (VJP) L = sL[warp][q];
+#pragma unroll
+          for (int p = 0; p < NP; ++p) {
+            const f2 rx = add2(sub2(P[p].xh, f2_dup(A.x)), sub2(P[p].xl, f2_dup(B.x)));
+            const f2 ry = add2(sub2(P[p].yh, f2_dup(A.y)), sub2(P[p].yl, f2_dup(B.y)));
+            const f2 rz = add2(sub2(P[p].zh, f2_dup(A.z)), sub2(P[p].zl, f2_dup(B.z)));
+            const f2 r2 = fma2(rx, rx, fma2(ry, ry, mul2(rz, rz)));
+            near = near || !(fminf(f2_lo(r2), f2_hi(r2)) > Tq);
+            pair_term2<VJP>(rx, ry, rz, A, B.w, L, P[p].m, P[p].iro, P[p].lx, P[p].ly, P[p].lz,
+                            kc, a2[p]);
+          }
+        }
+        full = __any_sync(0xffffffffu, near);
+      }
+#pragma unroll
+      for (int t = 0; t < DTL; ++t)
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+          two_sum_acc(red_h[warp][c][t * 32 + lane], red_l[warp][c][t * 32 + lane],
+                      t & 1 ? f2_hi(a2[t / 2][c]) : f2_lo(a2[t / 2][c]));
+    } else {
+      double acc[DTL][NC];
+#pragma unroll
+      for (int t = 0; t < DTL; ++t)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[t][c] = 0.0;
 #pragma unroll 2
       for (int q = 0; q < lim; ++q) {
         const Q4<T> A = sA[warp][q], B = sB[warp][q];
+        const int hT = __double2hiint(sT[warp][q]);
         Q4<T> L{0, 0, 0, 0};
         if constexpr (VJP) L = sL[warp][q];
-        const f2 rx = add2(sub2(P.xh, f2_dup(A.x)), sub2(P.xl, f2_dup(B.x)));
-        const f2 ry = add2(sub2(P.yh, f2_dup(A.y)), sub2(P.yl, f2_dup(B.y)));
-        const f2 rz = add2(sub2(P.zh, f2_dup(A.z)), sub2(P.zl, f2_dup(B.z)));
-        pair_term2<VJP>(rx, ry, rz, A, B.w, L, P.m, P.iro, P.lx, P.ly, P.lz, kc, a2);
-      }
+        double rx[DTL], ry[DTL], rz[DTL], r2[DTL];
+        int low = 0x7fffffff;  // by the leading 32 bits: an FP64 comparison takes the pipe
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        acc[0][c] = f2_lo(a2[c]);
-        acc[1][c] = f2_hi(a2[c]);
-      }
-    } else {
-#pragma unroll 4
-      for (int q = 0; q < lim; ++q) {
-        const Q4<T> A = sA[warp][q], B = sB[warp][q];
-        Q4<T> L{0, 0, 0, 0};
-        if constexpr (VJP) L = sL[warp][q];
+        for (int t = 0; t < DTL; ++t) {
+          rx[t] = txh[t] - A.x; ry[t] = tyh[t] - A.y; rz[t] = tzh[t] - A.z;
+          r2[t] = fma(rx[t], rx[t], fma(ry[t], ry[t], rz[t] * rz[t]));
+          low = min(low, __double2hiint(r2[t]));
+        }
+        if (__any_sync(0xffffffffu, low <= hT)) {
 #pragma unroll
-        for (int t = 0; t < kDT; ++t) {
-          T rx = txh[t] - A.x, ry = tyh[t] - A.y, rz = tzh[t] - A.z;
-          pair_term<T, VJP>(rx, ry, rz, A, B.w, L, tm[t], tiro[t], tlx[t], tly[t], tlz[t], g,
-                            i1mg, acc[t]);
+          for (int t = 0; t < DTL; ++t)
+            pair_term<VJP, true>(rx[t], ry[t], rz[t], r2[t], A, B.w, L, tm[t], tiro[t], tlx[t],
+                                 tly[t], tlz[t], g, i1mg, acc[t]);
+        } else {
+#pragma unroll
+          for (int t = 0; t < DTL; ++t)
+            pair_term<VJP, false>(rx[t], ry[t], rz[t], r2[t], A, B.w, L, tm[t], tiro[t], tlx[t],
+                                  tly[t], tlz[t], g, i1mg, acc[t]);
         }
       }
+#pragma unroll
+      for (int t = 0; t < DTL; ++t)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) dd[t][c] += acc[t][c];
     }
-#pragma unroll
-    for (int t = 0; t < kDT; ++t)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        if constexpr (MIXED) two_sum_acc(fh[t][c], fl[t][c], acc[t][c]);
-        else dd[t][c] += acc[t][c];
-      }
   }
+  if constexpr (!MIXED)
 #pragma unroll
-  for (int t = 0; t < kDT; ++t)
+    for (int t = 0; t < DTL; ++t)
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      if constexpr (MIXED) {
-        red_h[warp][c][t * 32 + lane] = fh[t][c];
-        red_l[warp][c][t * 32 + lane] = fl[t][c];
-      } else {
-        red[warp][c][t * 32 + lane] = dd[t][c];
-      }
-    }
+      for (int c = 0; c < NC; ++c) red[warp][c][t * 32 + lane] = dd[t][c];
   __syncthreads();
-  for (int e = threadIdx.x; e < NC * kDTB; e += kDW * 32) {
-    const int c = e / kDTB, tt = e - c * kDTB;
-    const int64_t k = (int64_t)blockIdx.x * kDTB + tt;
+  for (int e = threadIdx.x; e < NC * DTB; e += kDW * 32) {
+    const int c = e / DTB, tt = e - c * DTB;
+    const int64_t k = (int64_t)blockIdx.x * DTB + tt;
     if (k >= n) continue;
     double s = 0.0;
     if constexpr (MIXED) {
@@ -355,9 +478,9 @@ __global__ void __launch_bounds__(kDW * 32, MIXED ? P3T_DIRECT_MINB_MIXED : 1)
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int e = threadIdx.x; e < NC * kDTB; e += kDW * 32) {
-    const int c = e / kDTB, tt = e - c * kDTB;
-    const int64_t k = (int64_t)blockIdx.x * kDTB + tt;
+  for (int e = threadIdx.x; e < NC * DTB; e += kDW * 32) {
+    const int c = e / DTB, tt = e - c * DTB;
+    const int64_t k = (int64_t)blockIdx.x * DTB + tt;
     if (k >= n) continue;
     double s = 0.0;
 #pragma unroll 8
@@ -368,43 +491,24 @@ __global__ void __launch_bounds__(kDW * 32, MIXED ? P3T_DIRECT_MINB_MIXED : 1)
   if (threadIdx.x == 0) tile_cnt[blockIdx.x] = 0;
 }
 
-// Work split: blocks of 64 targets x one source split.  With fewer than 8
-// waves of target tiles alone, the sources are split so that the grid is at
-// least 8 waves of resident blocks (the last, partial wave then costs at most
-// an eighth); every split keeps at least 256 sources (a chunk per warp).
-// With ns >= 2 splits, (ns - 1) n < 8 slots 64, so the partial sums, C ns n
-// doubles, fit in 4 * 2 * 8 * slots * 64 (direct_part_doubles).
-template <bool MIXED, bool VJP>
-int blocks_per_sm() {
-  static int b = 0;
-  if (b == 0) {
-    int v = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_direct<MIXED, VJP>, kDW * 32, 0) !=
-            cudaSuccess || v < 1)
-      v = 1;
-    b = v;
-  }
-  return b;
-}
-
-int max_blocks_per_sm() {
-  int b = blocks_per_sm<true, true>();
-  b = b > blocks_per_sm<true, false>() ? b : blocks_per_sm<true, false>();
-  b = b > blocks_per_sm<false, true>() ? b : blocks_per_sm<false, true>();
-  b = b > blocks_per_sm<false, false>() ? b : blocks_per_sm<false, false>();
-  return b;
-}
-
+// Work split: tiles of 64 targets x one source split.  With fewer than 8 waves
+// of target tiles alone (three blocks an SM), the sources are split so that the
+// grid is at least 8 waves of resident blocks (the last, partial wave then
+// costs at most an eighth); every split keeps at least 256 sources (a chunk
+// per warp).  With ns >= 2 splits, (ns - 1) n < 8 slots 64, so the partial
+// sums, C ns n doubles, fit in 4 * 2 * 8 * slots * 64 (direct_part_doubles).
+// The split sets the order of the sums, so it does not follow the kernels'
+// occupancy.
 struct Split {
-  int64_t tiles, chunk;
+  int64_t chunk;
   int nsplit;
 };
-Split split_for(const p3t_ctx *c, int64_t n, int bps) {
+Split split_for(const p3t_ctx *c, int64_t n) {
   Split s;
-  s.tiles = (n + kDTB - 1) / kDTB;
-  const int64_t slots = (int64_t)c->num_sms * bps;
+  const int64_t tiles = (n + kDTB - 1) / kDTB;
+  const int64_t slots = (int64_t)c->num_sms * kSplitBlocks;
   int64_t ns = 1;
-  if (s.tiles < 8 * slots) ns = (8 * slots + s.tiles - 1) / s.tiles;
+  if (tiles < 8 * slots) ns = (8 * slots + tiles - 1) / tiles;
   const int64_t ns_max = (n + kDW * 32 - 1) / (kDW * 32);
   ns = ns > ns_max ? ns_max : ns;
   ns = ns < 1 ? 1 : ns;
@@ -419,15 +523,16 @@ int launch_direct(p3t_ctx *c, const p3t_particles *p, const double *lx, const do
                   const double *lz, DOut out, cudaStream_t s) {
   constexpr int NC = VJP ? 4 : 3;
   const int64_t n = p->n;
-  const Split sp = split_for(c, n, blocks_per_sm<MIXED, VJP>());
+  const Split sp = split_for(c, n);
+  const int64_t tiles = (n + kDTB - 1) / kDTB;
   if (sp.nsplit > 1 && (int64_t)NC * sp.nsplit * n > c->dpart_cap) return P3T_ERR_CAPACITY;
   using T = typename DT<MIXED>::T;
   Q4<T> *A = reinterpret_cast<Q4<T> *>(c->hw);  // 3 n packed 4-vectors <= 96 n bytes
   Q4<T> *B = A + n, *L = B + n;
   pdl_launch(k_direct_pack<MIXED, VJP>, dim3((unsigned)p3t_grid(n, 256, (int64_t)c->num_sms * 4)), dim3(256), 0, s, 
       n, p->x, p->y, p->z, p->m, p->r_out, lx, ly, lz, A, B, L);
-  if (sp.nsplit > 1 && sp.tiles > c->dcnt_cap) return P3T_ERR_CAPACITY;
-  const dim3 grid((unsigned)sp.tiles, (unsigned)sp.nsplit);
+  if (sp.nsplit > 1 && tiles > c->dcnt_cap) return P3T_ERR_CAPACITY;
+  const dim3 grid((unsigned)tiles, (unsigned)sp.nsplit);
   pdl_launch(k_direct<MIXED, VJP>, dim3(grid), dim3(kDW * 32), 0, s, n, sp.chunk, A, B, L, c->prm.gamma, c->dpart,
                                                 c->dcnt, out);
   p3t_note_launches(2);
@@ -437,12 +542,12 @@ int launch_direct(p3t_ctx *c, const p3t_particles *p, const double *lx, const do
 }  // namespace
 
 int64_t p3t_direct_part_doubles(const p3t_ctx *c) {
-  return (int64_t)4 * 2 * 8 * c->num_sms * max_blocks_per_sm() * kDTB;
+  return (int64_t)4 * 2 * 8 * c->num_sms * kSplitBlocks * kDTB;
 }
 
 // with several splits there are fewer than 8 slots target tiles
 int64_t p3t_direct_tile_counters(const p3t_ctx *c) {
-  return (int64_t)8 * c->num_sms * max_blocks_per_sm();
+  return (int64_t)8 * c->num_sms * kSplitBlocks;
 }
 
 int p3t_run_soft_force_direct(p3t_ctx *c, const p3t_particles *p, double *ax, double *ay,

@@ -66,15 +66,18 @@ __device__ __forceinline__ FF ff_rsqrt(FF r2) {
 // over all leading mantissas), x^(-3/2) = y^3 (1 - e)^(-3/2) = y^3 (1 + 3/2 e +
 // 15/8 e^2 + O(2.2 e^3)): the rest is below 2^-55, so the result carries only
 // its last rounding and y^3's, and takes 6 FP64 instructions where rsqrt()
-// cubed takes 7 to 8 and three more roundings.  Valid for x well inside the
-// normal range (rsqrt_seed_ok); x = 0 must be excluded by the caller.
+// cubed takes 7 to 8 and three more roundings.  Outside 2^-511 <= x < 2^513 the
+// seed is rsqrt() itself (0 for x = 0), out of line: inlined, the compiler
+// predicates its FP64 instructions into every use, and predicated-off ones
+// still take the pipe.
+static __device__ __noinline__ double rsqrt_rare(double x) {
+  return __double_as_longlong(x) == 0 ? 0.0 : rsqrt(x);
+}
 __device__ __forceinline__ double rsqrt_seed(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  if ((unsigned)((__double2hiint(x) >> 20) - 512) >= 1024u) y = rsqrt_rare(x);
   return y;
-}
-__device__ __forceinline__ bool rsqrt_seed_ok(double x) {  // 2^-511 <= x < 2^513
-  return (unsigned)((__double2hiint(x) >> 20) - 512) < 1024u;
 }
 // x 2^k in FP32 from the leading 20 bits of x (relative error below 2^-20,
 // towards zero); zero below and infinity above FP32's normal range

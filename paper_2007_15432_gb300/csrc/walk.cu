@@ -841,23 +841,17 @@ __device__ __forceinline__ bool far_from64(const FarBox &b, double X, double Y, 
 }
 
 // m r^-3 from r^2 (zero for r = 0): the seed's y, e = 1 - r^2 y^2 and the
-// result (see rsqrt_seed); rare ranges by rsqrt()
+// result (see rsqrt_seed)
 struct Inv3 {
   double y, e, f;
 };
 __device__ __forceinline__ Inv3 inv_cube(double r2, double m) {
   Inv3 v;
-  if (rsqrt_seed_ok(r2)) {
-    v.y = rsqrt_seed(r2);
-    const double y2 = v.y * v.y;
-    v.e = fma(-r2, y2, 1.0);
-    const double t = y2 * (v.y * m);
-    v.f = fma(t * v.e, fma(1.875, v.e, 1.5), t);
-  } else {
-    v.y = __double_as_longlong(r2) == 0 ? 0.0 : rsqrt(r2);
-    v.e = 0.0;
-    v.f = m * (v.y * v.y * v.y);
-  }
+  v.y = rsqrt_seed(r2);
+  const double y2 = v.y * v.y;
+  v.e = fma(-r2, y2, 1.0);
+  const double t = y2 * (v.y * m);
+  v.f = fma(t * v.e, fma(1.875, v.e, 1.5), t);
   return v;
 }
 // min of two positive numbers and clamp to [0, 1], on the bit patterns (an FP64
