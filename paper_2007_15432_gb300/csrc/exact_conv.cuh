@@ -64,7 +64,7 @@ __device__ __forceinline__ uint64_t quantise(double v, double lo, CellScale cs) 
 
 // A node's search reach in grid cells, R = ceil(rs / u) + 1 with the FP64
 // quotient (rounded to nearest) as the definition has it, capped at 2^23.
-__device__ __noinline__ int32_t reach_cells_fp64(double rs, double L) {
+static __device__ __noinline__ int32_t reach_cells_fp64(double rs, double L) {
   const double rq = ceil(rs / ldexp(L, -P3T_BITS)) + 1.0;
   return rq < 8388608.0 ? (int32_t)rq : 8388608;
 }
@@ -104,7 +104,7 @@ __device__ __forceinline__ int32_t reach_cells(double rs, double L, const CellSc
 // the FP64 conversions, out of line: inlined, the compiler predicates them
 // into every call, and predicated-off FP64 instructions still occupy the
 // FP64 pipe
-__device__ __noinline__ void split_f32_fp64(double x, float &hi, float &lo) {
+static __device__ __noinline__ void split_f32_fp64(double x, float &hi, float &lo) {
   hi = (float)x;
   lo = (float)(x - (double)hi);
 }
