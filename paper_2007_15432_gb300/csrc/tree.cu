@@ -818,7 +818,19 @@ __device__ __forceinline__ int64_t max_bits(int64_t a, double v) {
   return b > a ? b : a;
 }
 
-__device__ __forceinline__ int32_t leaf_moments32(
+// What bounds the mixed moments: for few leaves latency (a leaf's serial sums,
+// then a chain of a dozen parents, each an atomic, a fence, the children's
+// records from L2 and some 400 dependent instructions when one thread does
+// it, 4 us a level), for many the leaves' instructions.  A node is therefore
+// taken by eight lanes (group mask gm, lane `sub` of the group), a child a
+// lane, the children added in the fixed tree by shuffles.  A leaf is taken by
+// eight lanes where that fits the resident threads (its members are multiplied
+// out one a lane; the sums, serial in the member order, are dealt to the
+// lanes from shared memory) and by one thread above (eight lanes for all: 233
+// us at N = 1e6).  The same operations in the same order in every form.
+// Measured (whole mixed tree build): N = 3,001 96 -> 84 us, 1e5 146 -> 130, 1e6
+// 330 -> 326; one thread a leaf throughout 91, 138, 320.
+__device__ __forceinline__ int32_t leaf_moments32_thread(
     int64_t b, TreeNode *node, Mom32 *m32, double *nrs, const float4 *spA, const float4 *spB,
     const float *sml, const double *srs, const int32_t *sq, const double *box,
     const SegView &sv) {
@@ -869,144 +881,244 @@ __device__ __forceinline__ int32_t leaf_moments32(
   }
 }
 
-// One internal node of the mixed path from its children's Mom32 records, by
-// one thread, the eight child slots added in the fixed pairwise tree ((s0 +
-// s4) + (s2 + s6)) + ((s1 + s5) + (s3 + s7)) (zero past the last child).  The
-// children were written by other threads of the same launch: read through L2.
-template <int NQ, class T, class F, class A>
-__device__ __forceinline__ void tree8_acc(int nch, F slot, A add, T (&r)[NQ]) {
-  // the children fill slots 0 .. nch - 1; an empty slot is zero and adding
-  // zero to a (normalised) sum returns it, so empty slots and their additions
-  // are skipped: the same values as the full tree
-  T a[NQ], b[NQ], c[NQ], d[NQ];
-  slot(0, a);
-  if (nch > 4) {
-    slot(4, b);
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) a[q] = add(a[q], b[q]);
-  }
-  if (nch > 2) {
-    slot(2, b);
-    if (nch > 6) {
-      slot(6, c);
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) b[q] = add(b[q], c[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) a[q] = add(a[q], b[q]);
-  }
-  if (nch > 1) {
-    slot(1, b);
-    if (nch > 5) {
-      slot(5, c);
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) b[q] = add(b[q], c[q]);
-    }
-    if (nch > 3) {
-      slot(3, c);
-      if (nch > 7) {
-        slot(7, d);
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) c[q] = add(c[q], d[q]);
-      }
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) b[q] = add(b[q], c[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) r[q] = add(a[q], b[q]);
-  } else {
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) r[q] = a[q];
-  }
+constexpr int kLeavesByLanes = 4;  // leaves a warp up to which eight lanes take each
+struct LeafTerms {
+  float v[14][32];  // m (h, l), m d (h, l) x 3, m d rounded x 3, d x 3; a column a lane
+};
+template <class T>
+__device__ __forceinline__ T grp_shfl(unsigned gm, T v, int src) {
+  return __shfl_sync(gm, v, src, 8);
 }
-
-__device__ __forceinline__ Mom32 ldcg_mom32(const Mom32 *m) {
-  Mom32 o;
-  o.hi = __ldcg(&m->hi); o.lo = __ldcg(&m->lo); o.q0 = __ldcg(&m->q0); o.q1 = __ldcg(&m->q1);
-  return o;
+__device__ __forceinline__ FF grp_shfl(unsigned gm, FF v, int src) {
+  return {__shfl_sync(gm, v.h, src, 8), __shfl_sync(gm, v.l, src, 8)};
 }
-
-__device__ int32_t node_moments32(int64_t b, TreeNode *node, Mom32 *m32, double *nrs,
-                                  const double *box, const SegView &sv) {
-  TreeNode *pn = &node[b];
-  const int4 r2 = __ldcg(reinterpret_cast<const int4 *>(pn) + 2),
-             r3 = __ldcg(reinterpret_cast<const int4 *>(pn) + 3);
-  const int32_t c0 = r3.x, nch = r3.y;
-  if (nch < 1 || nch > 8) return r2.w;  // only a node with children is completed
-  int64_t rsb = 0;
-  int32_t plo[3] = {P3T_QMAX, P3T_QMAX, P3T_QMAX}, phi[3] = {-1, -1, -1};
-  for (int k = 0; k < nch; ++k) {
-    rsb = max_bits(rsb, __ldcg(&nrs[c0 + k]));
-    const TreeNode *cn = &node[c0 + k];
+__device__ __forceinline__ FF grp_xor(unsigned gm, FF v, int o) {
+  return {__shfl_xor_sync(gm, v.h, o), __shfl_xor_sync(gm, v.l, o)};
+}
+// box and largest r_search over the group's lanes
+__device__ __forceinline__ void grp_box(unsigned gm, int32_t (&lo)[3], int32_t (&hi)[3],
+                                        int64_t &rsb) {
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-      plo[a] = min(plo[a], __ldcg(&cn->qlo[a]));
-      phi[a] = max(phi[a], __ldcg(&cn->qhi[a]));
+      lo[a] = min(lo[a], __shfl_xor_sync(gm, lo[a], o));
+      hi[a] = max(hi[a], __shfl_xor_sync(gm, hi[a], o));
     }
+    const int64_t r = __shfl_xor_sync(gm, rsb, o);
+    rsb = r > rsb ? r : rsb;
   }
-  FF P[4];
-  tree8_acc<4>(nch, [&](int k, FF (&t)[4]) {
-    const float4 hi = __ldcg(&m32[c0 + k].hi), lo = __ldcg(&m32[c0 + k].lo);
-    const FF M = ff_fast(hi.w, lo.w);
-    t[0] = M;
-    t[1] = ff_mul(M, ff_fast(hi.x, lo.x));
-    t[2] = ff_mul(M, ff_fast(hi.y, lo.y));
-    t[3] = ff_mul(M, ff_fast(hi.z, lo.z));
-  }, [](FF x, FF y) { return ff_add(x, y); }, P);
-  const FF pc[3] = {ff_div(P[1], P[0]), ff_div(P[2], P[0]), ff_div(P[3], P[0])};
-  float Q[6];
-  tree8_acc<6>(nch, [&](int k, float (&t)[6]) {
-    {
-      const Mom32 cm = ldcg_mom32(&m32[c0 + k]);
-      const float M = cm.hi.w;
-      const float dx = ff_add(ff_fast(cm.hi.x, cm.lo.x), ff_neg(pc[0])).h;
-      const float dy = ff_add(ff_fast(cm.hi.y, cm.lo.y), ff_neg(pc[1])).h;
-      const float dz = ff_add(ff_fast(cm.hi.z, cm.lo.z), ff_neg(pc[2])).h;
-      const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-      const float tx = 3.f * dx, ty = 3.f * dy;
-      t[0] = fmaf(M, fmaf(tx, dx, -d2), cm.q0.x);
-      t[1] = fmaf(M, fmaf(ty, dy, -d2), cm.q0.y);
-      t[2] = fmaf(M, fmaf(3.f * dz, dz, -d2), cm.q0.z);
-      t[3] = fmaf(M, tx * dy, cm.q0.w);
-      t[4] = fmaf(M, tx * dz, cm.q1.x);
-      t[5] = fmaf(M, ty * dz, cm.q1.y);
-    }
-  }, [](float x, float y) { return x + y; }, Q);
-  Mom32 o;
-  o.hi = make_float4(pc[0].h, pc[1].h, pc[2].h, P[0].h);
-  o.lo = make_float4(pc[0].l, pc[1].l, pc[2].l, P[0].l);
-  o.q0 = make_float4(Q[0], Q[1], Q[2], Q[3]);
-  o.q1 = make_float4(Q[4], Q[5], 0.f, 0.f);
-  for (int a = 0; a < 3; ++a) { pn->qlo[a] = plo[a]; pn->qhi[a] = phi[a]; }
+}
+// the group writes a node: box, reach and largest r_search, moments
+__device__ __forceinline__ void grp_store(int64_t b, int sub, TreeNode *node, Mom32 *m32,
+                                          double *nrs, const int32_t (&lo)[3],
+                                          const int32_t (&hi)[3], int level, int64_t rsb, double L,
+                                          const Mom32 &o) {
+  int4 *n4 = reinterpret_cast<int4 *>(&node[b]);
   const double rs = __longlong_as_double(rsb);
-  nrs[b] = rs;
-  const double L = box[5 * seg_at(sv, r3.z) + 3];
-  pn->R = reach_cells(rs, L, cell_scale(L));
-  m32[b] = o;
+  if (sub == 0) m32[b].hi = o.hi;
+  if (sub == 1) m32[b].lo = o.lo;
+  if (sub == 2) m32[b].q0 = o.q0;
+  if (sub == 3) m32[b].q1 = o.q1;
+  if (sub == 4) n4[0] = make_int4(lo[0], lo[1], lo[2], reach_cells(rs, L, cell_scale(L)));
+  if (sub == 5) n4[1] = make_int4(hi[0], hi[1], hi[2], level);
+  if (sub == 6) nrs[b] = rs;
+}
+
+__device__ __forceinline__ int32_t leaf_moments32_lanes(
+    int64_t b, unsigned gm, int sub, LeafTerms &T, TreeNode *node, Mom32 *m32, double *nrs,
+    const float4 *spA, const float4 *spB, const float *sml, const double *srs, const int32_t *sq,
+    const double *box, const SegView &sv) {
+  const int col0 = (threadIdx.x & 31) - sub;
+  const int4 *n4 = reinterpret_cast<const int4 *>(&node[b]);
+  const int4 r1 = n4[1], r2 = n4[2], r3 = n4[3];
+  const int32_t f = r3.z, c = r3.w;
+  const double L = box[5 * seg_at(sv, f) + 3];
+  const float4 A0 = spA[f], B0 = spB[f];
+  // lanes 0-3: M, D; lanes 4-6: (Sxx, Sxy), (Syy, Sxz), (Szz, Syz)
+  FF acc{0.f, 0.f};
+  float s0 = 0.f, s1 = 0.f;
+  const int k0 = sub == 4 ? 8 : (sub == 5 ? 9 : 10), l0 = sub == 4 ? 11 : (sub == 5 ? 12 : 13);
+  const int k1 = sub == 6 ? 9 : 8, l1 = sub == 4 ? 12 : 13;
+  int64_t rsb = 0;
+  int32_t lo[3] = {P3T_QMAX, P3T_QMAX, P3T_QMAX}, hi[3] = {-1, -1, -1};
+  for (int32_t base = 0; base < c; base += 8) {
+    const int32_t i = f + base + sub;
+    if (base + sub < c) {
+      const float4 A = spA[i], B = spB[i];
+      const FF dx = ff_add({A.x, B.x}, {-A0.x, -B0.x});
+      const FF dy = ff_add({A.y, B.y}, {-A0.y, -B0.y});
+      const FF dz = ff_add({A.z, B.z}, {-A0.z, -B0.z});
+      const FF m = ff_fast(A.w, sml[i]);
+      const FF tx = ff_mul(m, dx), ty = ff_mul(m, dy), tz = ff_mul(m, dz);
+      const int l = col0 + sub;
+      T.v[0][l] = m.h; T.v[1][l] = m.l;
+      T.v[2][l] = tx.h; T.v[3][l] = tx.l;
+      T.v[4][l] = ty.h; T.v[5][l] = ty.l;
+      T.v[6][l] = tz.h; T.v[7][l] = tz.l;
+      T.v[8][l] = m.h * dx.h; T.v[9][l] = m.h * dy.h; T.v[10][l] = m.h * dz.h;
+      T.v[11][l] = dx.h; T.v[12][l] = dy.h; T.v[13][l] = dz.h;
+      rsb = max_bits(rsb, srs[i]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        lo[a] = min(lo[a], sq[3 * i + a]);
+        hi[a] = max(hi[a], sq[3 * i + a]);
+      }
+    }
+    __syncwarp(gm);
+    const int nb = min(8, c - base);
+    if (sub < 4) {
+      for (int j = 0; j < nb; ++j)
+        acc = ff_add(acc, {T.v[2 * sub][col0 + j], T.v[2 * sub + 1][col0 + j]});
+    } else if (sub < 7) {
+      for (int j = 0; j < nb; ++j) {
+        s0 = fmaf(T.v[k0][col0 + j], T.v[l0][col0 + j], s0);
+        s1 = fmaf(T.v[k1][col0 + j], T.v[l1][col0 + j], s1);
+      }
+    }
+    __syncwarp(gm);
+  }
+  grp_box(gm, lo, hi, rsb);
+  const FF M = grp_shfl(gm, acc, 0);
+  const FF D[3] = {grp_shfl(gm, acc, 1), grp_shfl(gm, acc, 2), grp_shfl(gm, acc, 3)};
+  const float S[6] = {grp_shfl(gm, s0, 4), grp_shfl(gm, s0, 5), grp_shfl(gm, s0, 6),
+                      grp_shfl(gm, s1, 4), grp_shfl(gm, s1, 5), grp_shfl(gm, s1, 6)};
+  const FF e[3] = {ff_div(D[0], M), ff_div(D[1], M), ff_div(D[2], M)};
+  const FF cx = ff_add({A0.x, B0.x}, e[0]), cy = ff_add({A0.y, B0.y}, e[1]),
+           cz = ff_add({A0.z, B0.z}, e[2]);
+  const float Mh = M.h, ex = e[0].h, ey = e[1].h, ez = e[2].h;
+  const float Cxx = S[0] - Mh * ex * ex, Cyy = S[1] - Mh * ey * ey, Czz = S[2] - Mh * ez * ez;
+  const float tr = Cxx + Cyy + Czz;
+  Mom32 o;
+  o.hi = make_float4(cx.h, cy.h, cz.h, M.h);
+  o.lo = make_float4(cx.l, cy.l, cz.l, M.l);
+  o.q0 = make_float4(3.f * Cxx - tr, 3.f * Cyy - tr, 3.f * Czz - tr, 3.f * (S[3] - Mh * ex * ey));
+  o.q1 = make_float4(3.f * (S[4] - Mh * ex * ez), 3.f * (S[5] - Mh * ey * ez), 0.f, 0.f);
+  grp_store(b, sub, node, m32, nrs, lo, hi, r1.w, rsb, L, o);
   return r2.w;
 }
 
-// All moments of the mixed path in one launch, bottom-up: a thread per leaf
-// computes the leaf, then counts itself off at its parent (node_done, preset
-// to the number of children by k_nodes_bfs); the child that brings the count
-// to zero computes the parent from all its children and climbs on (each
-// node's record gives its parent in the same load as its children).  Nothing waits, and a node's result does
-// not depend on which child arrives last.  (In FP32 and float-float a node
-// costs a few thousand cycles of latency, so the climb's serial tail at the
-// top levels is short; the FP64 path keeps its level launches.)
-__global__ void k_moments_up32(
+// One internal node of the mixed path from its children's Mom32 records, a
+// child a lane, the eight slots added in the fixed pairwise tree ((s0 + s4) +
+// (s2 + s6)) + ((s1 + s5) + (s3 + s7)), zero past the last child (adding zero
+// to a normalised sum returns it); lane 0 holds the sums.  The children were
+// written by other threads of the same launch: read through L2.
+__device__ int32_t node_moments32(int64_t b, unsigned gm, int sub, TreeNode *node, Mom32 *m32,
+                                  double *nrs, const double *box, const SegView &sv) {
+  const int4 *n4 = reinterpret_cast<const int4 *>(&node[b]);
+  const int4 r1 = __ldcg(n4 + 1), r2 = __ldcg(n4 + 2), r3 = __ldcg(n4 + 3);
+  const int32_t c0 = r3.x, nch = r3.y;
+  if (nch < 1 || nch > 8) return r2.w;  // only a node with children is completed
+  int64_t rsb = 0;
+  int32_t lo[3] = {P3T_QMAX, P3T_QMAX, P3T_QMAX}, hi[3] = {-1, -1, -1};
+  const bool on = sub < nch;
+  Mom32 cm;
+  cm.hi = cm.lo = cm.q0 = cm.q1 = make_float4(0.f, 0.f, 0.f, 0.f);
+  FF P[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  if (on) {
+    const Mom32 *m = &m32[c0 + sub];
+    cm.hi = __ldcg(&m->hi); cm.lo = __ldcg(&m->lo); cm.q0 = __ldcg(&m->q0); cm.q1 = __ldcg(&m->q1);
+    const int4 *cn = reinterpret_cast<const int4 *>(&node[c0 + sub]);
+    const int4 q0 = __ldcg(cn), q1 = __ldcg(cn + 1);
+    rsb = max_bits(0, __ldcg(&nrs[c0 + sub]));
+    lo[0] = q0.x; lo[1] = q0.y; lo[2] = q0.z;
+    hi[0] = q1.x; hi[1] = q1.y; hi[2] = q1.z;
+    P[0] = ff_fast(cm.hi.w, cm.lo.w);
+    P[1] = ff_mul(P[0], ff_fast(cm.hi.x, cm.lo.x));
+    P[2] = ff_mul(P[0], ff_fast(cm.hi.y, cm.lo.y));
+    P[3] = ff_mul(P[0], ff_fast(cm.hi.z, cm.lo.z));
+  }
+  grp_box(gm, lo, hi, rsb);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) P[q] = ff_add(P[q], grp_xor(gm, P[q], o));
+#pragma unroll
+  for (int q = 0; q < 4; ++q) P[q] = grp_shfl(gm, P[q], 0);
+  const FF pc[3] = {ff_div(P[1], P[0]), ff_div(P[2], P[0]), ff_div(P[3], P[0])};
+  float Q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (on) {
+    const float M = cm.hi.w;
+    const float dx = ff_add(ff_fast(cm.hi.x, cm.lo.x), ff_neg(pc[0])).h;
+    const float dy = ff_add(ff_fast(cm.hi.y, cm.lo.y), ff_neg(pc[1])).h;
+    const float dz = ff_add(ff_fast(cm.hi.z, cm.lo.z), ff_neg(pc[2])).h;
+    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    const float tx = 3.f * dx, ty = 3.f * dy;
+    Q[0] = fmaf(M, fmaf(tx, dx, -d2), cm.q0.x);
+    Q[1] = fmaf(M, fmaf(ty, dy, -d2), cm.q0.y);
+    Q[2] = fmaf(M, fmaf(3.f * dz, dz, -d2), cm.q0.z);
+    Q[3] = fmaf(M, tx * dy, cm.q0.w);
+    Q[4] = fmaf(M, tx * dz, cm.q1.x);
+    Q[5] = fmaf(M, ty * dz, cm.q1.y);
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) Q[q] = Q[q] + __shfl_xor_sync(gm, Q[q], o);
+  Mom32 o;
+  o.hi = make_float4(pc[0].h, pc[1].h, pc[2].h, P[0].h);
+  o.lo = make_float4(pc[0].l, pc[1].l, pc[2].l, P[0].l);
+#pragma unroll
+  for (int q = 0; q < 6; ++q) Q[q] = grp_shfl(gm, Q[q], 0);
+  o.q0 = make_float4(Q[0], Q[1], Q[2], Q[3]);
+  o.q1 = make_float4(Q[4], Q[5], 0.f, 0.f);
+  grp_store(b, sub, node, m32, nrs, lo, hi, r1.w, rsb, box[5 * seg_at(sv, r3.z) + 3], o);
+  return r2.w;
+}
+
+// All moments of the mixed path in one launch, bottom-up: a leaf, once
+// computed, is counted off at its parent (node_done, preset to the number of
+// children by k_nodes_bfs); the child that brings the count to zero makes the
+// parent ready, which its warp takes next, four nodes at a time (each node's
+// record gives its parent in the same load as its children).  Nothing waits,
+// and a node's result does not depend on which child arrives last.
+__global__ void __launch_bounds__(128) k_moments_up32(
     const int64_t *d_nleaf, const int32_t *leaf_list, TreeNode *node, Mom32 *m32, double *nrs,
     const float4 *spA, const float4 *spB, const float *sml, const double *srs,
     const int32_t *sq, const double *box, SegView sv, int32_t *node_done) {
   pdl_wait();
+  __shared__ LeafTerms s_t[4];
+  __shared__ int32_t s_ready[4][32];
   const int64_t nleaf = *d_nleaf;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nleaf;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    int32_t p = leaf_moments32(leaf_list[t], node, m32, nrs, spA, spB, sml, srs, sq, box, sv);
-    while (p >= 0) {
-      __threadfence();  // this node's record before the count
-      if (atomicSub(&node_done[p], 1) != 1) break;  // siblings still to come
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane & 7, grp = lane >> 3;
+  const unsigned gm = 0xffu << (lane & 24), lt = (1u << lane) - 1u;
+  int32_t *ready = s_ready[w];
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const bool lanes = nleaf <= nwarps * kLeavesByLanes;  // leaves a warp takes at once
+  const int per = lanes ? 4 : 32;
+  for (int64_t t0 = warp * per; t0 < nleaf; t0 += nwarps * per) {
+    const int64_t t = t0 + (lanes ? grp : lane);
+    int32_t p = -1;  // held by one lane a leaf
+    if (lanes) {
+      if (t < nleaf) {
+        p = leaf_moments32_lanes(leaf_list[t], gm, sub, s_t[w], node, m32, nrs, spA, spB, sml, srs,
+                                 sq, box, sv);
+        if (sub != 0) p = -1;
+      }
+    } else if (t < nleaf) {
+      p = leaf_moments32_thread(leaf_list[t], node, m32, nrs, spA, spB, sml, srs, sq, box, sv);
+    }
+    int n = 0;  // nodes ready, all of their children done
+    for (;;) {
+      __threadfence();  // the nodes' records before the counts
+      __syncwarp();
+      const bool last = p >= 0 && atomicSub(&node_done[p], 1) == 1;
+      const unsigned m = __ballot_sync(0xffffffffu, last);
+      if (last) ready[n + __popc(m & lt)] = p;
+      n += __popc(m);
+      __syncwarp();
+      if (n == 0) break;
       __threadfence();  // the siblings' records after their counts
-      p = node_moments32(p, node, m32, nrs, box, sv);
+      const int take = n < 4 ? n : 4;
+      const int32_t b = grp < take ? ready[n - 1 - grp] : -1;
+      n -= take;
+      __syncwarp();
+      p = -1;
+      if (b >= 0) {
+        p = node_moments32(b, gm, sub, node, m32, nrs, box, sv);
+        if (sub != 0) p = -1;
+      }
     }
   }
 }
@@ -1327,7 +1439,7 @@ int p3t_run_build_tree(p3t_ctx *c, const p3t_particles *p, cudaStream_t s) {
   pdl_launch(k_lists, dim3((unsigned)gn), dim3(kBlock), 0, s, &cnt[3], c->node_cap, c->node_flag,
              c->flag_pos, c->pre2bfs, &cnt[19], c->leaf_list, c->group_list, &cnt[2], &cnt[15]);
   if (c->prm.precision == P3T_MIXED) {
-    pdl_launch(k_moments_up32, dim3((unsigned)p3t_grid(c->node_cap, 128, maxb)), dim3(128), 0, s, 
+    pdl_launch(k_moments_up32, dim3((unsigned)p3t_grid(c->node_cap * 8, 128, maxb)), dim3(128), 0, s, 
         &cnt[2], c->leaf_list, c->node, c->mom32, c->nrs, c->spA, c->spB, c->sml, c->srs,
         c->sq, c->box, sv, c->node_done);
     p3t_note_launches(1);
