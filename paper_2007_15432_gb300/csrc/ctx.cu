@@ -82,7 +82,7 @@ void free_particle_buffers(p3t_ctx *c) {
   dfree(c->node_done); dfree(c->leaf_list); dfree(c->node_flag); dfree(c->flag_pos);
   dfree(c->group_list);
   dfree(c->walk_stack); dfree(c->cand_i); dfree(c->cand_j); dfree(c->cand_keep);
-  dfree(c->deg); dfree(c->fill); dfree(c->parent); dfree(c->label); dfree(c->csize);
+  dfree(c->deg); dfree(c->parent); dfree(c->label); dfree(c->csize);
   dfree(c->flag); dfree(c->pos); dfree(c->singles); dfree(c->cl_off); dfree(c->hlist);
   // cl_mem aliases one of the mvals buffers
   c->cl_mem = nullptr;
@@ -137,7 +137,7 @@ int reserve(p3t_ctx *c, int64_t n, int64_t cand_cap) {
   ok &= dalloc(c->group_list, NC);
   ok &= dalloc(c->walk_stack, c->walk_warps * c->stack_cap);
   ok &= dalloc(c->cand_i, cand_cap) && dalloc(c->cand_j, cand_cap) && dalloc(c->cand_keep, cand_cap);
-  ok &= dalloc(c->deg, N + 1) && dalloc(c->fill, N + 1);
+  ok &= dalloc(c->deg, N + 1);
   ok &= dalloc(c->parent, N) && dalloc(c->label, N) && dalloc(c->csize, N);
   ok &= dalloc(c->flag, 4 * N) && dalloc(c->pos, 4 * N);
   ok &= dalloc(c->singles, N) && dalloc(c->cl_off, N + 1);
@@ -195,6 +195,7 @@ int p3t_create(p3t_ctx **ctx, const p3t_params *p, int device) {
     return P3T_ERR_CUDA;
   }
   bool ok = dalloc(c->status, 1) && dalloc(c->box, 5) && dalloc(c->box_bits, 6) &&
+            dalloc(c->box_part, 6 * p3t_box_blocks(c->num_sms)) &&
             dalloc(c->counters, 64) && dalloc(c->cl_counts, 4) && dalloc(c->hsteps, 1) && dalloc(c->hcursor, 5) &&
             dalloc(c->coll_ctr, 1) &&
             dalloc(c->epart, 8192) && dalloc(c->bh_table, 32) &&
@@ -224,7 +225,7 @@ void p3t_destroy(p3t_ctx *c) {
   DeviceGuard g(c->device);
   cudaDeviceSynchronize();
   free_particle_buffers(c);
-  dfree(c->status); dfree(c->box); dfree(c->box_bits); dfree(c->counters);
+  dfree(c->status); dfree(c->box); dfree(c->box_bits); dfree(c->box_part); dfree(c->counters);
   dfree(c->seg_off); dfree(c->seg_nb); dfree(c->seg_base); dfree(c->seg_l);
   delete[] c->seg_off_h;
   dfree(c->cl_counts); dfree(c->hsteps); dfree(c->hcursor); dfree(c->epart);

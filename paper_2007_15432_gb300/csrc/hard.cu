@@ -1411,8 +1411,12 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 20 : 1) k_hermite_block(
   if (tid == 0 && steps_out && steps) atomicAdd(steps_out, steps);
 }
 
-__global__ void k_zero_i64_five(int64_t *p) {
-  pdl_wait(); p[0] = 0; p[1] = 0; p[2] = 0; p[3] = 0; p[4] = 0; }
+// the step count and the Hermite kernels' cursors and list lengths to zero
+__global__ void k_zero_hard(unsigned long long *steps, int64_t *p) {
+  pdl_wait();
+  if (threadIdx.x < 5) p[threadIdx.x] = 0;
+  if (threadIdx.x == 5) *steps = 0ull;
+}
 
 // the clusters of more than hw members: up to kHMax into list[0..), larger
 // ones into list[cap..); their numbers into n[0], n[1] (zeroed before).  The
@@ -1431,9 +1435,6 @@ __global__ void k_cluster_classes(const int64_t *d_ncl, const int64_t *cl_off, i
     if (slot < cap) list[big * cap + slot] = (int32_t)c;
   }
 }
-
-__global__ void k_zero_u64(unsigned long long *p) {
-  pdl_wait(); *p = 0ull; }
 
 // ---- energy ----------------------------------------------------------------
 __device__ __forceinline__ void two_sum_f(float &hi, float &lo, float b) {
@@ -1731,8 +1732,7 @@ int p3t_run_hard_step(p3t_ctx *c, p3t_particles *p, const p3t_clusters *cl,
   const CollOut co = coll_out(c);
   unsigned long long *steps = n_steps ? reinterpret_cast<unsigned long long *>(n_steps)
                                       : c->hsteps;
-  pdl_launch(k_zero_u64, dim3(1), dim3(1), 0, s, steps);
-  pdl_launch(k_zero_i64_five, dim3(1), dim3(1), 0, s, c->hcursor);
+  pdl_launch(k_zero_hard, dim3(1), dim3(32), 0, s, steps, c->hcursor);
   // the clusters of the four-warp and workspace kernels, listed once so that
   // those kernels do not step through every small cluster
   const int hw = c->hwarp_max;
@@ -1786,7 +1786,7 @@ int p3t_run_hard_step(p3t_ctx *c, p3t_particles *p, const p3t_clusters *cl,
   P3T_CUDA_TRY(cudaEventRecord(c->ev_join[1], c->aux[1]));
   P3T_CUDA_TRY(cudaStreamWaitEvent(s, c->ev_join[0], 0));
   P3T_CUDA_TRY(cudaStreamWaitEvent(s, c->ev_join[1], 0));
-  p3t_note_launches(7);
+  p3t_note_launches(6);
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }
 

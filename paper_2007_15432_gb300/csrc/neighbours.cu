@@ -53,34 +53,41 @@ __global__ void k_nb_filter(const int64_t *d_ncand, const int32_t *cand_i,
   }
 }
 
-__global__ void k_nb_check(const int64_t *nb_total, int64_t nb_cap, DevStatus *st) {
-  pdl_wait();
-  if (*nb_total > nb_cap) dev_fail(st, P3T_ERR_CAPACITY, 50, *nb_total);
-}
-
+// the kept candidates into their rows (in any order; deg counts down to zero).
+// A total above the capacity is recorded and nothing is written
 __global__ void k_nb_fill(const int64_t *d_ncand, const int32_t *cand_i,
                           const int32_t *cand_j, const int32_t *idx,
-                          const int32_t *keep, const int64_t *nb_off,
-                          int32_t *fill, int32_t *nb_idx, const DevStatus *st) {
+                          const int32_t *keep, const int64_t *nb_off, const int64_t *nb_total,
+                          int64_t nb_cap, int32_t *deg, int32_t *nb_idx, DevStatus *st) {
   pdl_wait();
+  if (*nb_total > nb_cap) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) dev_fail(st, P3T_ERR_CAPACITY, 50, *nb_total);
+    return;
+  }
   if (st->code != 0) return;
   const int64_t nc = *d_ncand;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nc;
        k += (int64_t)gridDim.x * blockDim.x) {
     if (!keep[k]) continue;
     const int32_t i = idx[cand_i[k]], j = idx[cand_j[k]];
-    const int32_t q = atomicAdd(&fill[i], 1);
+    const int32_t q = atomicSub(&deg[i], 1) - 1;
     nb_idx[nb_off[i] + q] = j;
   }
 }
 
-// rows are short (<n_b> << 1 in the paper's runs): insertion sort per row
+// rows are short (<n_b> << 1 in the paper's runs): insertion sort per row; and
+// the start of the union-find: every particle its own root, counts zero
 __global__ void k_nb_sort_rows(int64_t n, const int64_t *nb_off, int32_t *nb_idx,
+                               int32_t *parent, int32_t *csize, int64_t *cl_counts,
                                const DevStatus *st) {
   pdl_wait();
-  if (st->code != 0) return;
+  if (blockIdx.x == 0 && threadIdx.x < 4) cl_counts[threadIdx.x] = 0;
+  const bool failed = st->code != 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
+    parent[i] = (int32_t)i;
+    csize[i] = 0;
+    if (failed) continue;
     const int64_t b = nb_off[i], e = nb_off[i + 1];
     for (int64_t u = b + 1; u < e; ++u) {
       const int32_t v = nb_idx[u];
@@ -97,15 +104,6 @@ __device__ __forceinline__ int32_t uf_find(const int32_t *parent, int32_t x) {
   int64_t guard = 0;
   while (p != x && guard++ < kUFLimit) { x = p; p = __ldcg(&parent[x]); }
   return x;
-}
-
-__global__ void k_uf_init(int64_t n, int32_t *parent, int32_t *csize) {
-  pdl_wait();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    parent[i] = (int32_t)i;
-    csize[i] = 0;
-  }
 }
 
 __global__ void k_uf_union(int64_t n, const int64_t *nb_off, const int32_t *nb_idx,
@@ -203,11 +201,6 @@ __global__ void k_copy_i32(const int64_t *d_n, const int32_t *src, int32_t *dst)
     dst[i] = src[i];
 }
 
-__global__ void k_zero_i64(int64_t *p, int k) {
-  pdl_wait();
-  if (threadIdx.x < k) p[threadIdx.x] = 0;
-}
-
 }  // namespace
 
 int p3t_run_neighbours(p3t_ctx *c, const p3t_particles *p, int64_t *nb_off,
@@ -220,18 +213,15 @@ int p3t_run_neighbours(p3t_ctx *c, const p3t_particles *p, int64_t *nb_off,
   int rc;
   // ---- neighbour lists ----
   P3T_CUDA_TRY(cudaMemsetAsync(c->deg, 0, sizeof(int32_t) * (n + 1), s));
-  P3T_CUDA_TRY(cudaMemsetAsync(c->fill, 0, sizeof(int32_t) * (n + 1), s));
   pdl_launch(k_nb_filter, dim3((unsigned)gc), dim3(kBlock), 0, s, &cnt[9], c->cand_i, c->cand_j, c->idx, *p,
                                               c->prm, c->cand_keep, c->deg, c->status);
   rc = p3t_scan_i32_to_i64(c->deg, nb_off, &cnt[0], c->cap, nb_off + n, c->scan_state, c->scan_words, c->status, c->poll_limit, s);
   if (rc) return rc;
-  pdl_launch(k_nb_check, dim3(1), dim3(1), 0, s, nb_off + n, nb_cap, c->status);
-  pdl_launch(k_nb_fill, dim3((unsigned)gc), dim3(kBlock), 0, s, &cnt[9], c->cand_i, c->cand_j, c->idx,
-                                            c->cand_keep, nb_off, c->fill, nb_idx, c->status);
-  pdl_launch(k_nb_sort_rows, dim3((unsigned)g), dim3(kBlock), 0, s, n, nb_off, nb_idx, c->status);
+  pdl_launch(k_nb_fill, dim3((unsigned)gc), dim3(kBlock), 0, s, &cnt[9], c->cand_i, c->cand_j,
+             c->idx, c->cand_keep, nb_off, nb_off + n, nb_cap, c->deg, nb_idx, c->status);
+  pdl_launch(k_nb_sort_rows, dim3((unsigned)g), dim3(kBlock), 0, s, n, nb_off, nb_idx, c->parent,
+             c->csize, c->cl_counts, c->status);
   // ---- neighbour clusters ----
-  pdl_launch(k_zero_i64, dim3(1), dim3(32), 0, s, c->cl_counts, 4);
-  pdl_launch(k_uf_init, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->parent, c->csize);
   pdl_launch(k_uf_union, dim3((unsigned)g), dim3(kBlock), 0, s, n, nb_off, nb_idx, c->parent, c->status);
   pdl_launch(k_uf_label, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->parent, c->label, c->csize);
   pdl_launch(k_cl_flags, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->label, c->csize, c->flag, c->cl_counts);
@@ -244,8 +234,8 @@ int p3t_run_neighbours(p3t_ctx *c, const p3t_particles *p, int64_t *nb_off,
   }
   pdl_launch(k_cl_scatter, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->label, c->flag, c->pos,
              &cnt[21], c->singles, c->cl_off, c->mkeys, c->mvals, c->cl_counts, &cnt[11]);
-  // filter, check, fill, sort_rows, zero, uf_init, uf_union, uf_label, flags, scatter
-  p3t_note_launches(10);
+  // filter, fill, sort_rows, uf_union, uf_label, flags, scatter
+  p3t_note_launches(7);
   // members ordered by (label, index), on the label's bits (labels are
   // particle indices below n).  The sorted members must land in the buffer
   // they started in, so that the cluster views keep their addresses from step

@@ -234,8 +234,9 @@ struct p3t_ctx {
   DevStatus *status = nullptr;
   // root box {x0, y0, z0, L} and scalar counters
   double *box = nullptr;
-  unsigned long long *box_bits = nullptr;  // ordered-bits min/max workspace [6]
-  int64_t *counters = nullptr;             // misc device counters [64] (32..53: tree level offsets)
+  unsigned long long *box_bits = nullptr;  // the cut-off stage's ordered-bits min/max
+  unsigned long long *box_part = nullptr;  // the root cubes' partial min/max, six a block
+  int64_t *counters = nullptr;             // misc device counters [64]
 
   // sort
   uint64_t *keys = nullptr, *keys_alt = nullptr;
@@ -279,7 +280,7 @@ struct p3t_ctx {
 
   // neighbours and clusters
   int32_t *cand_keep = nullptr;
-  int32_t *deg = nullptr, *fill = nullptr;
+  int32_t *deg = nullptr;
   int32_t *parent = nullptr, *label = nullptr, *csize = nullptr;
   int32_t *flag = nullptr;
   int64_t *pos = nullptr;
@@ -392,11 +393,12 @@ int p3t_scan_flag_pairs(const int32_t *in, int64_t *out, const int64_t *d_n, int
                         DevStatus *st, int64_t poll_limit, cudaStream_t s);
 // Stable LSD radix sort of (key, val) on bits [begin_bit, end_bit), n from
 // device memory (at most n_cap).  Ping-pongs between the two buffers; on
-// return *keys / *vals point at the sorted data.
+// return *keys / *vals point at the sorted data.  inv: null, or receives each
+// value's place in the sorted order (values are indices).
 int p3t_radix_sort(uint64_t **keys, int32_t **vals, uint64_t **keys_alt,
                    int32_t **vals_alt, const int64_t *d_n, int64_t n_cap,
                    int begin_bit, int end_bit, uint32_t *hist,
-                   int64_t hist_cap, cudaStream_t s);
+                   int64_t hist_cap, cudaStream_t s, int32_t *inv = nullptr);
 int64_t p3t_radix_hist_entries(int64_t n_cap);
 // Sort by (key, val) of distinct values (the stable order by key when the
 // values start in ascending order), n from device memory (at most n_cap); on
@@ -410,6 +412,10 @@ int p3t_sort_pairs(uint64_t **keys, int32_t **vals, uint64_t **keys_alt, int32_t
                    const int64_t *d_n, int64_t n_cap, int key_bits, uint32_t *hist,
                    int64_t hist_cap, void *work, uint32_t *where, cudaStream_t s);
 
+// most blocks of the root cube reduction: four an SM, or one a segment
+static inline int64_t p3t_box_blocks(int num_sms) {
+  return 4 * num_sms > P3T_MAX_SEGMENTS ? 4 * num_sms : P3T_MAX_SEGMENTS;
+}
 // the sorts' per-entry words: the last quarter of the flag buffer, which the
 // stages that sort leave free
 static inline uint32_t *p3t_sort_where(p3t_ctx *c) {

@@ -78,7 +78,8 @@ scan_onepass(const int32_t *in, int64_t *out, const int64_t *d_n, int64_t *d_tot
   const int64_t used = (n + kScanTile - 1) / kScanTile;
   const int64_t takers = used < 1 ? 1 : (used < (int64_t)gridDim.x ? used : (int64_t)gridDim.x);
   if ((int64_t)blockIdx.x >= takers) return;
-  if (t == 0) s_tile = atomicAdd(&state[0], 1ull);
+  const bool alone = used <= 1;  // one tile: no look-back, no state
+  if (t == 0) s_tile = alone ? 0ull : atomicAdd(&state[0], 1ull);
   __syncthreads();
   const int64_t tile = (int64_t)s_tile;
   const int64_t base = tile * kScanTile;
@@ -104,7 +105,7 @@ scan_onepass(const int32_t *in, int64_t *out, const int64_t *d_n, int64_t *d_tot
     if (warp == 0) {
       int64_t prefix = 0;
       if (tile == 0) {
-        if (lane == 0) {
+        if (lane == 0 && !alone) {
           __threadfence();
           __stcg(&ts[0], kFlagInc | (unsigned long long)agg);
         }
@@ -158,6 +159,7 @@ scan_onepass(const int32_t *in, int64_t *out, const int64_t *d_n, int64_t *d_tot
   } else if (t == 0 && tile == 0 && d_total) {
     *d_total = 0;  // n = 0
   }
+  if (alone) return;
   // the last block out resets the tile words and the counters
   __shared__ bool s_last;
   __syncthreads();
@@ -256,7 +258,7 @@ __device__ __forceinline__ uint32_t match_digit(uint32_t d, bool valid) {
 __global__ void __launch_bounds__(kSortThreads)
 radix_downsweep(const uint64_t *keys, const int32_t *vals, uint64_t *okeys,
                 int32_t *ovals, const int64_t *d_n, int shift,
-                const uint32_t *hist, int ntiles, const uint32_t *digit_total) {
+                const uint32_t *hist, int ntiles, const uint32_t *digit_total, int32_t *inv) {
   pdl_wait();
   __shared__ uint32_t s_warp[kSortThreads / 32][kRadix];
   __shared__ uint32_t s_run[kRadix];
@@ -340,6 +342,7 @@ radix_downsweep(const uint64_t *keys, const int32_t *vals, uint64_t *okeys,
       const uint32_t dst = s_gbase[d] + ((uint32_t)i - s_lbase[d]);
       okeys[dst] = k;
       ovals[dst] = s_val[i];
+      if (inv) inv[s_val[i]] = (int32_t)dst;
     }
   }
 }
@@ -854,7 +857,7 @@ int64_t p3t_radix_hist_entries(int64_t n_cap) {
 int p3t_radix_sort(uint64_t **keys, int32_t **vals, uint64_t **keys_alt,
                    int32_t **vals_alt, const int64_t *d_n, int64_t n_cap,
                    int begin_bit, int end_bit, uint32_t *hist,
-                   int64_t hist_cap, cudaStream_t s) {
+                   int64_t hist_cap, cudaStream_t s, int32_t *inv) {
   int64_t ntiles = (n_cap + kSortTile - 1) / kSortTile;
   if (ntiles < 1) ntiles = 1;
   if (ntiles * kRadix + kRadix > hist_cap) return P3T_ERR_CAPACITY;
@@ -864,7 +867,8 @@ int p3t_radix_sort(uint64_t **keys, int32_t **vals, uint64_t **keys_alt,
                                                             hist, (int)ntiles);
     pdl_launch(radix_row_scan, dim3(kRadix), dim3(kRadix), 0, s, hist, (int)ntiles, digit_total, d_n);
     pdl_launch(radix_downsweep, dim3((unsigned)ntiles), dim3(kSortThreads), 0, s, 
-        *keys, *vals, *keys_alt, *vals_alt, d_n, shift, hist, (int)ntiles, digit_total);
+        *keys, *vals, *keys_alt, *vals_alt, d_n, shift, hist, (int)ntiles, digit_total,
+        shift + kRadixBits >= end_bit ? inv : (int32_t *)nullptr);
     p3t_note_launches(3);
     uint64_t *tk = *keys; *keys = *keys_alt; *keys_alt = tk;
     int32_t *tv = *vals; *vals = *vals_alt; *vals_alt = tv;

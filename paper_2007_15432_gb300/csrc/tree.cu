@@ -3,6 +3,8 @@
 // and the integer grid geometry must be bit-identical on every IEEE machine.
 #include <math.h>
 
+#include <algorithm>
+
 #include "p3t_internal.cuh"
 #include "exact_conv.cuh"
 
@@ -28,9 +30,10 @@ __device__ __forceinline__ double ord_double(unsigned long long b) {
 // per segment d: bits[4d] min R, bits[4d + 1] max R, bits[4d + 2], [4d + 3]
 // the largest r_out and r_search (shared scheme)
 __global__ void k_cut_init(unsigned long long *bits, int nseg, double *bsum,
-                           unsigned long long *bcnt, int nb) {
+                           unsigned long long *bcnt, int nb, int64_t *d_n, int64_t n) {
   pdl_wait();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t == 0) *d_n = n;  // for the sort
   for (int d = t; d < nseg; d += gridDim.x * blockDim.x) {
     bits[4 * d] = ~0ull; bits[4 * d + 1] = 0ull; bits[4 * d + 2] = 0ull; bits[4 * d + 3] = 0ull;
   }
@@ -310,25 +313,19 @@ __global__ void k_cut_shared(SegView sv, const unsigned long long *bits, double 
 // =========================================================================
 // Keys, sort, octree, moments.
 // =========================================================================
-__global__ void k_set_i64(int64_t *dst, int64_t v) {
-  pdl_wait(); *dst = v; }
-
-__global__ void k_box_init(unsigned long long *bits, int nseg) {
-  pdl_wait();
-  for (int d = threadIdx.x; d < nseg; d += blockDim.x)
-    for (int a = 0; a < 3; ++a) { bits[6 * d + a] = ~0ull; bits[6 * d + 3 + a] = 0ull; }
-}
-
 // min / max of the positions of each segment: warp and block reductions over
-// a block's slice of its segment, then six atomics per block
+// a block's slice of its segment into part; the last block to finish (arrival
+// counter, left at zero) reduces the slices of each segment, a warp a segment,
+// to its root cube: corner at the per-axis minimum, side = largest extent;
+// box[5 d ..]: corner, side L, quantisation scale S
 __global__ void k_box(SegView sv, int slices, const double *x, const double *y,
-                      const double *z, unsigned long long *bits6) {
+                      const double *z, unsigned long long *part, int64_t *arrived, double *box5) {
   pdl_wait();
   __shared__ unsigned long long red[6][kBlock / 32];
+  __shared__ bool s_last;
   int d;
   int64_t sa, sb;
   seg_slice(sv, slices, d, sa, sb);
-  unsigned long long *bits = bits6 + 6 * d;
   unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
   // four elements a trip, their loads issued before the first is used
   for (int64_t i0 = sa + threadIdx.x; i0 < sb; i0 += 4 * (int64_t)blockDim.x) {
@@ -365,23 +362,47 @@ __global__ void k_box(SegView sv, int slices, const double *x, const double *y,
     unsigned long long r = red[a][0];
     for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
       r = a < 3 ? (red[a][w] < r ? red[a][w] : r) : (red[a][w] > r ? red[a][w] : r);
-    if (a < 3) atomicMin(&bits[a], r); else atomicMax(&bits[a], r);
+    part[6 * (int64_t)blockIdx.x + a] = r;
+    __threadfence();
   }
-}
-
-// root cube of each segment: corner at the per-axis minimum, side = largest
-// extent; box[5 d ..]: corner, side L, quantisation scale S
-__global__ void k_box_final(const unsigned long long *bits6, double *box5, int nseg) {
-  pdl_wait();
-  for (int d = threadIdx.x; d < nseg; d += blockDim.x) {
-    const unsigned long long *bits = bits6 + 6 * d;
-    double *box = box5 + 5 * d;
-    double lo[3], hi[3];
-    for (int a = 0; a < 3; ++a) { lo[a] = ord_double(bits[a]); hi[a] = ord_double(bits[3 + a]); }
-    double L = fmax(hi[0] - lo[0], fmax(hi[1] - lo[1], hi[2] - lo[2]));
-    if (!(L > 0.0)) L = 1.0;
-    box[0] = lo[0]; box[1] = lo[1]; box[2] = lo[2]; box[3] = L;
-    box[4] = (double)P3T_QMAX / L;  // quantisation scale S
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_last = atomicAdd(reinterpret_cast<unsigned long long *>(arrived), 1ull) ==
+             (unsigned long long)gridDim.x - 1;
+    if (s_last) *arrived = 0;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const int lane = threadIdx.x & 31;
+  for (int seg = threadIdx.x >> 5; seg < sv.nseg; seg += blockDim.x >> 5) {
+    unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0ull, 0ull, 0ull};
+    for (int q = lane; q < slices; q += 32) {
+      const unsigned long long *v = part + 6 * ((int64_t)seg * slices + q);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const unsigned long long l = __ldcg(&v[a]), h = __ldcg(&v[3 + a]);
+        mn[a] = l < mn[a] ? l : mn[a];
+        mx[a] = h > mx[a] ? h : mx[a];
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long l = __shfl_xor_sync(0xffffffffu, mn[a], o);
+        const unsigned long long h = __shfl_xor_sync(0xffffffffu, mx[a], o);
+        mn[a] = l < mn[a] ? l : mn[a];
+        mx[a] = h > mx[a] ? h : mx[a];
+      }
+    if (lane == 0) {
+      double *box = box5 + 5 * seg;
+      double lo0[3], hi0[3];
+      for (int a = 0; a < 3; ++a) { lo0[a] = ord_double(mn[a]); hi0[a] = ord_double(mx[a]); }
+      double L = fmax(hi0[0] - lo0[0], fmax(hi0[1] - lo0[1], hi0[2] - lo0[2]));
+      if (!(L > 0.0)) L = 1.0;
+      box[0] = lo0[0]; box[1] = lo0[1]; box[2] = lo0[2]; box[3] = L;
+      box[4] = (double)P3T_QMAX / L;  // quantisation scale S
+    }
   }
 }
 
@@ -444,43 +465,6 @@ __global__ void k_segkey(SegView sv, const int32_t *idx, uint64_t *keys) {
     keys[s] = (uint64_t)seg_of(sv, idx[s]);
 }
 
-// gather sorted copies: the FP64 arrays the FP64 path reads, or the
-// float-float packing the mixed path reads (each path writes only its own)
-template <bool MIXED>
-__global__ void k_gather(int64_t n, const int32_t *idx, const uint64_t *keys,
-                         const double *pack, double *sx, double *sy, double *sz, double *sm,
-                         double *sro, double *srs, int32_t *sq, float4 *spA,
-                         float4 *spB, float *srs32, float *sml) {
-  pdl_wait();
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
-       s += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t i = idx[s];
-    const double2 *rec = reinterpret_cast<const double2 *>(pack + 6 * (int64_t)i);
-    const double2 r0 = rec[0], r1 = rec[1], r2 = rec[2];
-    const double X = r0.x, Y = r0.y, Z = r1.x, M = r1.y, RO = r2.x, RS = r2.y;
-    srs[s] = RS;
-    const uint64_t k = keys[s];
-    sq[3 * s + 0] = (int32_t)compact3(k >> 2);
-    sq[3 * s + 1] = (int32_t)compact3(k >> 1);
-    sq[3 * s + 2] = (int32_t)compact3(k);
-    if constexpr (!MIXED) {
-      sx[s] = X; sy[s] = Y; sz[s] = Z; sm[s] = M; sro[s] = RO;
-      continue;
-    }
-    float xh, xl, yh, yl, zh, zl, mh, ml, roh, rol, r2h, r2l;
-    split_f32(X, xh, xl);
-    split_f32(Y, yh, yl);
-    split_f32(Z, zh, zl);
-    split_f32(M, mh, ml);
-    split_f32(RO, roh, rol);
-    split_f32(RS * RS, r2h, r2l);
-    spA[s] = make_float4(xh, yh, zh, mh);
-    sml[s] = ml;
-    spB[s] = make_float4(xl, yl, zl, 1.0f / roh);  // FP32 path only
-    srs32[s] = r2h * 1.00001f;  // walk's candidate test: r^2 vs r_search^2, widened
-  }
-}
-
 // common prefix of two keys in levels (0..21)
 __device__ __forceinline__ int lcp_levels(uint64_t a, uint64_t b) {
   uint64_t d = a ^ b;
@@ -488,43 +472,76 @@ __device__ __forceinline__ int lcp_levels(uint64_t a, uint64_t b) {
   return (__clzll((long long)d) - 1) / 3;
 }
 
-// Each particle's common prefix with its predecessor (lp, levels; -1 at a
-// segment's first particle), its leaf level and the number of nodes it starts.
-// The cell of i at level l holds more than `leaf` particles iff some window
-// of leaf + 1 consecutive sorted particles containing i (within its segment)
-// shares the level-l prefix; the window prefixes w(a) = lcp(a, a + leaf) of a
-// block's tile and the `leaf` positions before it are formed once in shared
-// memory.  (Each segment's particles are a contiguous sorted run with a tree
-// of its own.)
+// Per sorted particle, a tile of a block's threads at a time:
+//  - the sorted copies: the FP64 arrays the FP64 path reads, or the float-float
+//    packing the mixed path reads (each path writes only its own);
+//  - its common prefix with its predecessor (lp, levels; -1 at a segment's
+//    first particle), its leaf level and the number of nodes it starts.  The
+//    cell of i at level l holds more than `leaf` particles iff some window of
+//    leaf + 1 consecutive sorted particles containing i (within its segment)
+//    shares the level-l prefix; the window prefixes w(a) = lcp(a, a + leaf) of
+//    the tile and the `leaf` positions before it are formed once in shared
+//    memory.  (Each segment's particles are a contiguous sorted run with a
+//    tree of its own.)
 constexpr int kLevelTile = 256;  // = kBlock
+template <bool MIXED>
 __global__ void __launch_bounds__(kLevelTile)
-k_lcp_levels(SegView sv, const uint64_t *keys, int leaf, int8_t *lp, int8_t *lv,
-             int32_t *ncount) {
+k_gather(SegView sv, const int32_t *idx, const uint64_t *keys, const double *pack, double *sx,
+         double *sy, double *sz, double *sm, double *sro, double *srs, int32_t *sq, float4 *spA,
+         float4 *spB, float *srs32, float *sml, int leaf, int8_t *lp, int8_t *lv,
+         int32_t *ncount) {
   pdl_wait();
   __shared__ int8_t w[kLevelTile + 32];  // leaf <= 32
   const int64_t n = sv.n;
   for (int64_t t0 = (int64_t)blockIdx.x * kLevelTile; t0 < n;
        t0 += (int64_t)gridDim.x * kLevelTile) {
+    const int64_t s = t0 + threadIdx.x;
+    double2 r0, r1, r2;
+    uint64_t k = 0;
+    if (s < n) {  // the record's loads are in flight during the window prefixes
+      const double2 *rec = reinterpret_cast<const double2 *>(pack + 6 * (int64_t)idx[s]);
+      r0 = rec[0]; r1 = rec[1]; r2 = rec[2];
+      k = keys[s];
+    }
     __syncthreads();
     for (int j = threadIdx.x; j < kLevelTile + leaf; j += kLevelTile) {
       const int64_t a = t0 - leaf + j;
       w[j] = (a >= 0 && a + leaf < n) ? (int8_t)lcp_levels(keys[a], keys[a + leaf]) : (int8_t)-1;
     }
     __syncthreads();
-    const int64_t i = t0 + threadIdx.x;
-    if (i < n) {
-      const int d = seg_at(sv, i);
+    if (s >= n) continue;
+    {
+      const int d = seg_at(sv, s);
       const int64_t s0 = seg_lo(sv, d), s1 = seg_hi(sv, d);
-      const uint64_t k = keys[i];
-      const int p = i == s0 ? -1 : lcp_levels(keys[i - 1], k);
-      lp[i] = (int8_t)p;
+      const int p = s == s0 ? -1 : lcp_levels(keys[s - 1], k);
+      lp[s] = (int8_t)p;
       int D = -1;
-      const int64_t a0 = i - leaf > s0 ? i - leaf : s0;
-      const int64_t a1 = i < s1 - 1 - leaf ? i : s1 - 1 - leaf;
+      const int64_t a0 = s - leaf > s0 ? s - leaf : s0;
+      const int64_t a1 = s < s1 - 1 - leaf ? s : s1 - 1 - leaf;
       for (int64_t a = a0; a <= a1; ++a) D = max(D, (int)w[a - (t0 - leaf)]);
       const int L = min(D + 1, P3T_BITS);
-      lv[i] = (int8_t)L;
-      ncount[i] = max(0, L - p);
+      lv[s] = (int8_t)L;
+      ncount[s] = max(0, L - p);
+    }
+    const double X = r0.x, Y = r0.y, Z = r1.x, M = r1.y, RO = r2.x, RS = r2.y;
+    srs[s] = RS;
+    sq[3 * s + 0] = (int32_t)compact3(k >> 2);
+    sq[3 * s + 1] = (int32_t)compact3(k >> 1);
+    sq[3 * s + 2] = (int32_t)compact3(k);
+    if constexpr (!MIXED) {
+      sx[s] = X; sy[s] = Y; sz[s] = Z; sm[s] = M; sro[s] = RO;
+    } else {
+      float xh, xl, yh, yl, zh, zl, mh, ml, roh, rol, r2h, r2l;
+      split_f32(X, xh, xl);
+      split_f32(Y, yh, yl);
+      split_f32(Z, zh, zl);
+      split_f32(M, mh, ml);
+      split_f32(RO, roh, rol);
+      split_f32(RS * RS, r2h, r2l);
+      spA[s] = make_float4(xh, yh, zh, mh);
+      sml[s] = ml;
+      spB[s] = make_float4(xl, yl, zl, 1.0f / roh);  // FP32 path only
+      srs32[s] = r2h * 1.00001f;  // walk's candidate test: r^2 vs r_search^2, widened
     }
   }
 }
@@ -623,13 +640,59 @@ __global__ void k_node_counts(SegView sv, const uint64_t *keys, const int64_t *d
   }
 }
 
-__global__ void k_pre2bfs(const int64_t *d_nnode, int64_t node_cap,
-                          const int32_t *bfs2pre, int32_t *pre2bfs) {
+// Breadth-first order of the nodes of a small system by one block: the stable
+// order by level of the preorder nodes.  A warp takes 32 consecutive nodes at a
+// time and counts each level among them by the match of the lanes; a warp a
+// level then scans the counts, and the nodes go to their places.  (Larger
+// systems take a radix pass: three launches.)
+constexpr int kOrderMax = 16384;
+__global__ void __launch_bounds__(1024) k_level_order(const int64_t *d_nnode,
+                                                      const int32_t *pre_level, int32_t *bfs2pre,
+                                                      int32_t *pre2bfs) {
   pdl_wait();
-  const int64_t nn = min(*d_nnode, node_cap);
-  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nn;
-       b += (int64_t)gridDim.x * blockDim.x)
-    pre2bfs[bfs2pre[b]] = (int32_t)b;
+  constexpr int kLevels = P3T_BITS + 1, kGroups = kOrderMax / 32;
+  __shared__ uint16_t s_cnt[kLevels][kGroups];  // per level and 32 nodes
+  __shared__ int s_tot[kLevels];
+  const int nn = (int)*d_nnode, t = threadIdx.x, lane = t & 31, wp = t >> 5;
+  const int ng = (nn + 31) >> 5;
+  for (int g = wp; g < ng; g += 32) {
+    const int id = 32 * g + lane;
+    const int l = id < nn ? pre_level[id] : -1;
+    const unsigned m = __match_any_sync(0xffffffffu, l);
+    if (lane < kLevels) s_cnt[lane][g] = 0;
+    __syncwarp();
+    if (l >= 0 && lane == __ffs(m) - 1) s_cnt[l][g] = (uint16_t)__popc(m);
+  }
+  __syncthreads();
+  if (wp < kLevels) {
+    int run = 0;
+    for (int g0 = 0; g0 < ng; g0 += 32) {
+      const int c = g0 + lane < ng ? s_cnt[wp][g0 + lane] : 0;
+      int v = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+      }
+      if (g0 + lane < ng) s_cnt[wp][g0 + lane] = (uint16_t)(run + v - c);
+      run += __shfl_sync(0xffffffffu, v, 31);
+    }
+    if (lane == 0) s_tot[wp] = run;
+  }
+  __syncthreads();
+  int first = 0;  // lane l: the nodes of the levels above l
+  for (int l = 0; l < kLevels; ++l)
+    if (l < lane) first += s_tot[l];
+  for (int g = wp; g < ng; g += 32) {
+    const int id = 32 * g + lane;
+    const int l = id < nn ? pre_level[id] : -1;
+    const unsigned m = __match_any_sync(0xffffffffu, l);
+    const int base = __shfl_sync(0xffffffffu, first, l < 0 ? 0 : l);
+    if (l < 0) continue;  // the last group's tail: no shuffle follows for it
+    const int pos = base + s_cnt[l][g] + __popc(m & ((1u << lane) - 1u));
+    bfs2pre[pos] = id;
+    pre2bfs[id] = pos;
+  }
 }
 
 __global__ void k_nodes_bfs(const int64_t *d_nnode, int64_t node_cap,
@@ -654,12 +717,21 @@ __global__ void k_nodes_bfs(const int64_t *d_nnode, int64_t node_cap,
     const bool internal = l < (int)lv[first];
     if (internal && pre + 1 < nn) {
       nd.child0 = pre2bfs[pre + 1];
+      // the children in preorder; each gets its parent link and its flags
+      // (bit 0: a leaf; bit 1: a target group, a node holding <= gs particles,
+      // or a leaf, whose parent holds more) from here
       const int64_t e = (int64_t)first + count;
+      const bool big = count > gs;
       int k = 0;
       int64_t c = pre + 1;
       for (;;) {
+        const int32_t cfirst = pre_first[c], ccount = pre_count[c];
+        const bool cleaf = l + 1 >= (int)lv[cfirst];
+        flags[c] = (cleaf ? 1 : 0) | (big && (ccount <= gs || cleaf) ? 2 : 0);
+        if ((int64_t)nd.child0 + k < nn && nd.child0 > b)
+          node[nd.child0 + k].parent = (int32_t)b;
         ++k;
-        const int64_t cend = (int64_t)pre_first[c] + pre_count[c];
+        const int64_t cend = (int64_t)cfirst + ccount;
         if (cend >= e) break;
         c = nstart[cend] + (l + 1) - ((int)lp[cend] + 1);
         if (k >= 8 || c <= pre || c >= nn) {  // cannot happen in a consistent tree
@@ -674,37 +746,18 @@ __global__ void k_nodes_bfs(const int64_t *d_nnode, int64_t node_cap,
       nd.nchild = 0;
       node_done[b] = 0;
     }
-    // bit 0: a leaf; bit 1: a target group without a parent (a root; the
-    // parents flag the others)
-    const bool small = count <= gs || nd.nchild == 0;
-    flags[pre] = (internal ? 0 : 1) | (l == 0 && small ? 2 : 0);
-    // geometry (qlo, qhi, R) is filled bottom-up by k_moments and the parent
-    // links by k_parents
+    // a root's own flags (a target group when it is small)
+    if (l == 0) {
+      const bool small = count <= gs || nd.nchild == 0;
+      flags[pre] = (internal ? 0 : 1) | (small ? 2 : 0);
+    }
+    // geometry (qlo, qhi, R) is filled bottom-up by the moments, the parent
+    // link by the parent
     TreeNode *o = &node[b];
     o->level = nd.level; o->first = nd.first; o->count = nd.count;
     o->c2[0] = nd.c2[0]; o->c2[1] = nd.c2[1]; o->c2[2] = nd.c2[2];
     o->child0 = nd.child0; o->nchild = nd.nchild;
-    o->parent = -1;  // set for children by k_parents
-  }
-}
-
-// parent links, and the target-group flag (bit 1 of the preorder flags) of
-// every child: a node holding <= gs particles (or a leaf) whose parent holds
-// more
-__global__ void k_parents(const int64_t *d_nnode, int64_t node_cap, TreeNode *node,
-                          const int32_t *bfs2pre, int gs, int32_t *flags) {
-  pdl_wait();
-  const int64_t nn = min(*d_nnode, node_cap);
-  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nn;
-       b += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t c0 = node[b].child0, nc = node[b].nchild;
-    if (nc > 0 && (c0 <= b || (int64_t)c0 + nc > nn)) continue;  // inconsistent: skip
-    const bool big = node[b].count > gs;
-    for (int k = 0; k < nc; ++k) {
-      TreeNode &cn = node[c0 + k];
-      cn.parent = (int32_t)b;
-      if (big && (cn.count <= gs || cn.nchild == 0)) flags[bfs2pre[c0 + k]] |= 2;
-    }
+    if (l == 0) o->parent = -1;
   }
 }
 
@@ -1341,7 +1394,8 @@ int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s) {
   double *bsum = c->epart;  // reuse: >= 4096 doubles
   unsigned long long *bcnt = reinterpret_cast<unsigned long long *>(c->epart + 4096);
   const int64_t g = p3t_grid(n, kBlock, (int64_t)c->num_sms * P3T_NSM_BLOCKS);
-  pdl_launch(k_cut_init, dim3(4), dim3(kBlock), 0, s, c->box_bits, (int)c->nseg, bsum, bcnt, nb);
+  pdl_launch(k_cut_init, dim3(4), dim3(kBlock), 0, s, c->box_bits, (int)c->nseg, bsum, bcnt, nb,
+             &c->counters[18], n);
   const int rsl = c->nseg == 1 ? (int)g : (int)((g + c->nseg - 1) / c->nseg);
   pdl_launch(k_cut_range, dim3((unsigned)(rsl * c->nseg)), dim3(kBlock), 0, s, sv, rsl, p->x, p->y, c->box_bits);
   if (c->nseg > 1)
@@ -1353,7 +1407,6 @@ int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s) {
   double *u2 = c->hw;
   int64_t *boff = c->pos;
   int64_t *d_n = &c->counters[18];
-  pdl_launch(k_set_i64, dim3(1), dim3(1), 0, s, d_n, n);
   int32_t *bin = c->flag;  // the bins of k_cut_u2, read by k_cut_final (N int32)
   pdl_launch(k_cut_u2, dim3((unsigned)g), dim3(kBlock), 0, s, sv, p->x, p->y, p->z, p->vx, p->vy, p->vz, mu,
                                           c->box_bits, nb, c->seg_nb, c->seg_base, c->seg_l,
@@ -1368,9 +1421,9 @@ int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s) {
                                              p->r_out, p->r_search);
   if (c->prm.cutoff_mode == P3T_CUT_SHARED)
     pdl_launch(k_cut_shared, dim3((unsigned)g), dim3(kBlock), 0, s, sv, c->box_bits, p->r_out, p->r_search);
-  // init, range, n, u2, offsets, bin sums, final (+ shared, + segment bins);
+  // init, range, u2, offsets, bin sums, final (+ shared, + segment bins);
   // the sort counts itself
-  p3t_note_launches(7 + (c->prm.cutoff_mode == P3T_CUT_SHARED) + (c->nseg > 1));
+  p3t_note_launches(6 + (c->prm.cutoff_mode == P3T_CUT_SHARED) + (c->nseg > 1));
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }
 
@@ -1384,11 +1437,11 @@ int p3t_run_build_tree(p3t_ctx *c, const p3t_particles *p, cudaStream_t s) {
   const int nseg = (int)c->nseg;
   const SegView sv{c->seg_off, nseg, n};
   // one root cube per segment: a few blocks per SM in all, in slices of the
-  // segments
-  const int bsl = nseg >= 4 * c->num_sms ? 1 : 4 * c->num_sms / nseg;
-  pdl_launch(k_box_init, dim3(1), dim3(256), 0, s, c->box_bits, nseg);
-  pdl_launch(k_box, dim3((unsigned)(bsl * nseg)), dim3(kBlock), 0, s, sv, bsl, p->x, p->y, p->z, c->box_bits);
-  pdl_launch(k_box_final, dim3(1), dim3(256), 0, s, c->box_bits, c->box, nseg);
+  // segments of no less than a trip of a block (four elements a thread)
+  const int64_t bmax = nseg >= 4 * c->num_sms ? 1 : 4 * c->num_sms / nseg;
+  const int bsl = (int)std::min(bmax, (n / nseg + 4 * kBlock - 1) / (4 * kBlock) + 1);
+  pdl_launch(k_box, dim3((unsigned)(bsl * nseg)), dim3(kBlock), 0, s, sv, bsl, p->x, p->y, p->z,
+             c->box_part, &cnt[24], c->box);
   pdl_launch(k_keys, dim3((unsigned)g), dim3(kBlock), 0, s, sv, p->x, p->y, p->z, p->m, p->r_out, p->r_search,
                                         c->box, c->keys, c->idx, c->pack, 0, &cnt[0]);
   rc = p3t_sort_pairs(&c->keys, &c->idx, &c->keys_alt, &c->idx_alt, &cnt[0], c->cap, 63,
@@ -1408,11 +1461,9 @@ int p3t_run_build_tree(p3t_ctx *c, const p3t_particles *p, cudaStream_t s) {
     p3t_note_launches(2);
   }
   auto gather = c->prm.precision == P3T_MIXED ? k_gather<true> : k_gather<false>;
-  pdl_launch(gather, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->idx, c->keys, c->pack, c->sx, c->sy, c->sz,
-                                          c->sm, c->sro, c->srs, c->sq, c->spA, c->spB,
-                                          c->srs32, c->sml);
-  pdl_launch(k_lcp_levels, dim3((unsigned)p3t_grid(n, kLevelTile, maxb)), dim3(kLevelTile), 0, s, 
-      sv, c->keys, leaf, c->lp, c->lv, c->ncount);
+  pdl_launch(gather, dim3((unsigned)p3t_grid(n, kLevelTile, maxb)), dim3(kLevelTile), 0, s, sv,
+             c->idx, c->keys, c->pack, c->sx, c->sy, c->sz, c->sm, c->sro, c->srs, c->sq, c->spA,
+             c->spB, c->srs32, c->sml, leaf, c->lp, c->lv, c->ncount);
   rc = p3t_scan_i32_to_i64(c->ncount, c->nstart, &cnt[0], c->cap, &cnt[1], c->scan_state, c->scan_words, c->status, c->poll_limit, s);
   if (rc) return rc;
   pdl_launch(k_nodes_pre, dim3((unsigned)g), dim3(kBlock), 0, s, sv, c->lp, c->lv, c->nstart, cnt, c->node_cap,
@@ -1420,18 +1471,25 @@ int p3t_run_build_tree(p3t_ctx *c, const p3t_particles *p, cudaStream_t s) {
                                              c->bfs2pre, c->status);
   pdl_launch(k_node_counts, dim3((unsigned)p3t_grid(c->node_cap, kBlock, maxb)), dim3(kBlock), 0, s, 
       sv, c->keys, &cnt[1], c->node_cap, c->pre_first, c->pre_level, c->pre_count, c->status);
-  rc = p3t_radix_sort(&c->lvl_keys, &c->bfs2pre, &c->lvl_keys_alt, &c->bfs2pre_alt, &cnt[3],
-                      c->node_cap, 0, 8, c->radix_hist, c->radix_hist_cap, s);
-  if (rc) return rc;
+  // breadth-first order: one block's counts, or a radix pass on the level that
+  // also writes the inverse.  One block's time grows with the nodes, three
+  // launches cost about the same at any size (whole tree build, block / pass: N
+  // = 1,000 58 / 63 us, 3,001 71 / 75, 4,800, near the limit, 79 / 82)
+  if (c->node_cap <= kOrderMax) {
+    pdl_launch(k_level_order, dim3(1), dim3(1024), 0, s, &cnt[3], c->pre_level, c->bfs2pre,
+               c->pre2bfs);
+    p3t_note_launches(1);
+  } else {
+    rc = p3t_radix_sort(&c->lvl_keys, &c->bfs2pre, &c->lvl_keys_alt, &c->bfs2pre_alt, &cnt[3],
+                        c->node_cap, 0, 8, c->radix_hist, c->radix_hist_cap, s, c->pre2bfs);
+    if (rc) return rc;
+  }
   const int64_t gn = p3t_grid(c->node_cap, kBlock, maxb);
-  pdl_launch(k_pre2bfs, dim3((unsigned)gn), dim3(kBlock), 0, s, &cnt[3], c->node_cap, c->bfs2pre, c->pre2bfs);
   pdl_launch(k_nodes_bfs, dim3((unsigned)gn), dim3(kBlock), 0, s, &cnt[3], c->node_cap, c->bfs2pre, c->pre2bfs,
                                               c->pre_first, c->pre_count, c->pre_level,
                                               c->lp, c->lv, c->nstart, c->sq, c->node,
                                               c->prm.group_size, c->node_flag, c->node_done,
                                               c->status);
-  pdl_launch(k_parents, dim3((unsigned)gn), dim3(kBlock), 0, s, &cnt[3], c->node_cap, c->node,
-             c->bfs2pre, c->prm.group_size, c->node_flag);
   // leaves (bit 0) and target groups (bit 1) counted by one scan
   rc = p3t_scan_flag_pairs(c->node_flag, c->flag_pos, &cnt[3], c->node_cap, &cnt[19],
                            c->scan_state, c->scan_words, c->status, c->poll_limit, s);
@@ -1460,10 +1518,9 @@ int p3t_run_build_tree(p3t_ctx *c, const p3t_particles *p, cudaStream_t s) {
                                                            c->mom32, c->nrs, c->box, sv, wt);
     p3t_note_launches(3 + kDeepLevel);  // leaves, level offsets, deep levels, one a level
   }
-  // own kernels here (the scans, sorts and moments count themselves): box 3,
-  // keys, gather, lcp_levels, nodes_pre, node_counts, pre2bfs, nodes_bfs,
-  // parents, lists
-  p3t_note_launches(12);
+  // own kernels here (the scans, sorts and moments count themselves): box,
+  // keys, gather, nodes_pre, node_counts, nodes_bfs, lists
+  p3t_note_launches(7);
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }
 

@@ -1266,21 +1266,22 @@ __global__ void k_node_adjoint(const int64_t *d_nleaf, const int32_t *leaf_list,
   }
 }
 
-__global__ void k_walk_prep(int64_t *cursor, unsigned long long *cand_count,
-                            unsigned long long *counts) {
-  pdl_wait();
-  *cursor = 0;
-  *cand_count = 0ull;
-  if (counts) { counts[0] = 0ull; counts[1] = 0ull; }
-}
-
-// candidates found -> device status (for growth on the host) and clamped count
-__global__ void k_walk_post(int64_t *cnt, int64_t cand_cap, DevStatus *st) {
+// after a walk: the candidates found to the device status (for growth on the
+// host) and clamped for the neighbour search, the interaction counts to the
+// caller's, and the walk's counters back to zero for the next one
+// (cnt: [8] candidates, [9] clamped, [12] cursor, [25] p-p, [26] p-node)
+__global__ void k_walk_post(int64_t *cnt, int64_t cand_cap, unsigned long long *counts,
+                            DevStatus *st) {
   pdl_wait();
   const int64_t nc = cnt[8];
   st->cand_need = nc;
   if (nc > cand_cap) dev_fail(st, P3T_ERR_CAPACITY, 42, nc);
   cnt[9] = nc < cand_cap ? nc : cand_cap;
+  if (counts) {
+    counts[0] = (unsigned long long)cnt[25];
+    counts[1] = (unsigned long long)cnt[26];
+  }
+  cnt[8] = cnt[12] = cnt[25] = cnt[26] = 0;
 }
 
 // T M^2 >= 2^K for T < 2^49, M < 2^53, K >= 0: the product formed exactly in
@@ -1378,6 +1379,7 @@ int p3t_run_soft_force_vjp_tree(p3t_ctx *c, const p3t_particles *p, double s,
                                 cudaStream_t st) {
   WalkArgs a = walk_args(c, p);
   VjpOut o{lx, ly, lz, s, gx, gy, gz, gm, c->nadj};
+  a.cursor = &c->counters[27];  // the forward walk leaves its own at zero
   P3T_CUDA_TRY(cudaMemsetAsync(c->nadj, 0, sizeof(double) * 10 * c->node_cap, st));
   P3T_CUDA_TRY(cudaMemsetAsync(a.cursor, 0, sizeof(int64_t), st));
   const unsigned blocks = walk64_blocks(c, (unsigned)(c->walk_warps / kWarps));
@@ -1394,8 +1396,7 @@ int p3t_run_soft_force(p3t_ctx *c, const p3t_particles *p, double *ax,
                        cudaStream_t s) {
   WalkArgs a = walk_args(c, p);
   a.ax = ax; a.ay = ay; a.az = az;
-  a.counts = reinterpret_cast<unsigned long long *>(counts);
-  pdl_launch(k_walk_prep, dim3(1), dim3(1), 0, s, a.cursor, a.cand_count, a.counts);
+  a.counts = reinterpret_cast<unsigned long long *>(&c->counters[25]);
   unsigned blocks = (unsigned)(c->walk_warps / kWarps);
   if (c->walk_bps > 0 && (int64_t)c->num_sms * c->walk_bps < (int64_t)blocks)
     blocks = (unsigned)(c->num_sms * c->walk_bps);
@@ -1408,8 +1409,9 @@ int p3t_run_soft_force(p3t_ctx *c, const p3t_particles *p, double *ax,
     blocks = walk64_blocks(c, blocks);
     pdl_launch(k_walk64, dim3(blocks), dim3(kWarps * 32), 0, s, a, walk64_chunk(c, blocks));
   }
-  pdl_launch(k_walk_post, dim3(1), dim3(1), 0, s, c->counters, c->cand_cap, c->status);
-  p3t_note_launches(3);
+  pdl_launch(k_walk_post, dim3(1), dim3(1), 0, s, c->counters, c->cand_cap,
+             reinterpret_cast<unsigned long long *>(counts), c->status);
+  p3t_note_launches(2);
   (void)p;
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }
