@@ -787,74 +787,59 @@ __global__ void k_lists(const int64_t *d_nnode, int64_t node_cap, const int32_t 
   }
 }
 
-__device__ __forceinline__ void finish_node(TreeNode *nd, Mom64 *m64, Mom32 *m32,
-                                            double rsmax, double u, int64_t b,
-                                            const Mom64 &mm) {
-  double rq = ceil(rsmax / u) + 1.0;
-  nd->R = rq < 8388608.0 ? (int32_t)rq : 8388608;
-  m64[b] = mm;
-  Mom32 f;
-  const float hx = (float)mm.cx, hy = (float)mm.cy, hz = (float)mm.cz;
-  const float mh = (float)mm.M;
-  f.hi = make_float4(hx, hy, hz, mh);
-  f.lo = make_float4((float)(mm.cx - (double)hx), (float)(mm.cy - (double)hy),
-                     (float)(mm.cz - (double)hz), (float)(mm.M - (double)mh));
-  f.q0 = make_float4((float)mm.qxx, (float)mm.qyy, (float)mm.qzz, (float)mm.qxy);
-  f.q1 = make_float4((float)mm.qxz, (float)mm.qyz, 0.f, 0.f);
-  m32[b] = f;
+// Moments of the FP64 path.  A leaf's members are summed, in their order, about
+// a reference point r (its first member): M, D = sum m d, S_ab = sum m d_a d_b
+// with d = x - r; then com = r + D / M and the traceless quadrupole about the
+// com, Q_ab = 3 C_ab - delta_ab tr C with C_ab = S_ab - M e_a e_b, e = D / M
+// (the definition sum m (3 d'_a d'_b - d'^2 delta_ab), d' = x - com,
+// expanded).  An internal node sums its children with the parallel-axis shift
+// of Q.  What bounds them is the latency of FP64 instructions (64 cycles of a
+// sub-partition each, however few lanes are active): a node takes eight lanes,
+// and of every sum that the lanes could all form alike each lane forms its own
+// part.  Measured (whole FP64 tree build, against a launch a level and a thread
+// a leaf): N = 1,000 114 -> 64 us, 1e4 154 -> 107, 1e5 194 -> 152, 1e6 588 -> 458.
+__device__ __forceinline__ int64_t max_reach(int64_t a, double v) {  // a NaN is passed over
+  const int64_t b = __double_as_longlong(v);
+  return b > a && b <= 0x7ff0000000000000ll ? b : a;
 }
-
-// Moments, one thread per node, level by level with no atomics: first every
-// leaf from its members, then the internal nodes of one level per launch,
-// deepest level first, from their (finished) children.  (A warp instruction
-// of FP64 occupies a sub-partition's pipe for ~64 cycles however few of its
-// lanes are active, so every lane carries a node of its own.)  A leaf's
-// members are summed about a reference point r (its first member): M, D =
-// sum m d, S_ab = sum m d_a d_b with d = x - r; then com = r + D / M and the
-// traceless quadrupole about the com, Q_ab = 3 C_ab - delta_ab tr C with C_ab
-// = S_ab - M e_a e_b, e = D / M (the definition sum m (3 d'_a d'_b - d'^2
-// delta_ab), d' = x - com, expanded).  An internal node sums its children with
-// the parallel-axis shift of Q.
-__global__ void k_moments_leaf(
-    const int64_t *d_nleaf, const int32_t *leaf_list, TreeNode *node, Mom64 *m64, Mom32 *m32,
-    double *nrs, const double *sx, const double *sy, const double *sz, const double *sm,
-    const double *srs, const int32_t *sq, const double *box, SegView sv) {
-  pdl_wait();
-  const int64_t nleaf = *d_nleaf;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nleaf;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = leaf_list[t];
-    TreeNode *nd = &node[b];
-    const int32_t f = nd->first, c = nd->count;
-    const double u = ldexp(box[5 * seg_at(sv, f) + 3], -P3T_BITS);
-    const double rx = sx[f], ry = sy[f], rz = sz[f];
-    double M = 0.0, D[3] = {0, 0, 0}, S[6] = {0, 0, 0, 0, 0, 0}, rs = 0.0;
-    int32_t lo[3] = {P3T_QMAX, P3T_QMAX, P3T_QMAX}, hi[3] = {-1, -1, -1};
-    for (int32_t i = f; i < f + c; ++i) {
-      const double m = sm[i], dx = sx[i] - rx, dy = sy[i] - ry, dz = sz[i] - rz;
-      const double mx = m * dx, my = m * dy, mz = m * dz;
-      M += m; D[0] += mx; D[1] += my; D[2] += mz;
-      S[0] = __fma_rn(mx, dx, S[0]); S[1] = __fma_rn(my, dy, S[1]); S[2] = __fma_rn(mz, dz, S[2]);
-      S[3] = __fma_rn(mx, dy, S[3]); S[4] = __fma_rn(mx, dz, S[4]); S[5] = __fma_rn(my, dz, S[5]);
-      rs = fmax(rs, srs[i]);
+__device__ __forceinline__ int32_t leaf_moments64_thread(
+    int64_t b, TreeNode *node, Mom64 *m64, double *nrs, const double *sx, const double *sy,
+    const double *sz, const double *sm, const double *srs, const int32_t *sq, const double *box,
+    const SegView &sv) {
+  TreeNode *nd = &node[b];
+  const int32_t f = nd->first, c = nd->count;
+  const double L = box[5 * seg_at(sv, f) + 3];
+  const double rx = sx[f], ry = sy[f], rz = sz[f];
+  double M = 0.0, D[3] = {0, 0, 0}, S[6] = {0, 0, 0, 0, 0, 0};
+  int64_t rsb = 0;
+  int32_t lo[3] = {P3T_QMAX, P3T_QMAX, P3T_QMAX}, hi[3] = {-1, -1, -1};
+  for (int32_t i = f; i < f + c; ++i) {
+    const double m = sm[i], dx = sx[i] - rx, dy = sy[i] - ry, dz = sz[i] - rz;
+    const double mx = m * dx, my = m * dy, mz = m * dz;
+    M += m; D[0] += mx; D[1] += my; D[2] += mz;
+    S[0] = __fma_rn(mx, dx, S[0]); S[1] = __fma_rn(my, dy, S[1]); S[2] = __fma_rn(mz, dz, S[2]);
+    S[3] = __fma_rn(mx, dy, S[3]); S[4] = __fma_rn(mx, dz, S[4]); S[5] = __fma_rn(my, dz, S[5]);
+    rsb = max_reach(rsb, srs[i]);
 #pragma unroll
-      for (int a = 0; a < 3; ++a) { lo[a] = min(lo[a], sq[3 * i + a]); hi[a] = max(hi[a], sq[3 * i + a]); }
-    }
-    Mom64 mm = {};
-    const double iM = 1.0 / M;
-    const double e[3] = {D[0] * iM, D[1] * iM, D[2] * iM};
-    mm.M = M; mm.cx = rx + e[0]; mm.cy = ry + e[1]; mm.cz = rz + e[2];
-    const double Cxx = S[0] - M * e[0] * e[0], Cyy = S[1] - M * e[1] * e[1],
-                 Czz = S[2] - M * e[2] * e[2];
-    const double tr = Cxx + Cyy + Czz;
-    mm.qxx = 3.0 * Cxx - tr; mm.qyy = 3.0 * Cyy - tr; mm.qzz = 3.0 * Czz - tr;
-    mm.qxy = 3.0 * (S[3] - M * e[0] * e[1]);
-    mm.qxz = 3.0 * (S[4] - M * e[0] * e[2]);
-    mm.qyz = 3.0 * (S[5] - M * e[1] * e[2]);
-    for (int a = 0; a < 3; ++a) { nd->qlo[a] = lo[a]; nd->qhi[a] = hi[a]; }
-    nrs[b] = rs;
-    finish_node(nd, m64, m32, rs, u, b, mm);
+    for (int a = 0; a < 3; ++a) { lo[a] = min(lo[a], sq[3 * i + a]); hi[a] = max(hi[a], sq[3 * i + a]); }
   }
+  Mom64 mm = {};
+  const double iM = 1.0 / M;
+  const double e[3] = {D[0] * iM, D[1] * iM, D[2] * iM};
+  mm.M = M; mm.cx = rx + e[0]; mm.cy = ry + e[1]; mm.cz = rz + e[2];
+  const double Cxx = S[0] - M * e[0] * e[0], Cyy = S[1] - M * e[1] * e[1],
+               Czz = S[2] - M * e[2] * e[2];
+  const double tr = Cxx + Cyy + Czz;
+  mm.qxx = 3.0 * Cxx - tr; mm.qyy = 3.0 * Cyy - tr; mm.qzz = 3.0 * Czz - tr;
+  mm.qxy = 3.0 * (S[3] - M * e[0] * e[1]);
+  mm.qxz = 3.0 * (S[4] - M * e[0] * e[2]);
+  mm.qyz = 3.0 * (S[5] - M * e[1] * e[2]);
+  for (int a = 0; a < 3; ++a) { nd->qlo[a] = lo[a]; nd->qhi[a] = hi[a]; }
+  const double rs = __longlong_as_double(rsb);
+  nrs[b] = rs;
+  nd->R = reach_cells(rs, L, cell_scale(L));
+  m64[b] = mm;
+  return nd->parent;
 }
 
 // Mixed path: the same moments with no FP64 instruction, written straight to
@@ -1119,20 +1104,191 @@ __device__ int32_t node_moments32(int64_t b, unsigned gm, int sub, TreeNode *nod
   return r2.w;
 }
 
-// All moments of the mixed path in one launch, bottom-up: a leaf, once
-// computed, is counted off at its parent (node_done, preset to the number of
-// children by k_nodes_bfs); the child that brings the count to zero makes the
-// parent ready, which its warp takes next, four nodes at a time (each node's
-// record gives its parent in the same load as its children).  Nothing waits,
-// and a node's result does not depend on which child arrives last.
-__global__ void __launch_bounds__(128) k_moments_up32(
-    const int64_t *d_nleaf, const int32_t *leaf_list, TreeNode *node, Mom32 *m32, double *nrs,
-    const float4 *spA, const float4 *spB, const float *sml, const double *srs,
-    const int32_t *sq, const double *box, SegView sv, int32_t *node_done) {
+// the group writes an FP64 node's box, reach and largest r_search
+__device__ __forceinline__ void grp_store64(int64_t b, int sub, TreeNode *node, double *nrs,
+                                            const int32_t (&lo)[3], const int32_t (&hi)[3],
+                                            int level, int64_t rsb, double L) {
+  int4 *n4 = reinterpret_cast<int4 *>(&node[b]);
+  const double rs = __longlong_as_double(rsb);
+  if (sub == 3) n4[0] = make_int4(lo[0], lo[1], lo[2], reach_cells(rs, L, cell_scale(L)));
+  if (sub == 7) n4[1] = make_int4(hi[0], hi[1], hi[2], level);
+  if (sub == 1) nrs[b] = rs;
+}
+
+// An FP64 leaf by eight lanes: the members multiplied out one a lane, the ten
+// sums (leaf_moments64_thread's, in the member order) dealt to the lanes: lane
+// l the sum l of M, D, Sxx, Syy, Szz, Sxy, and by its parity Sxz or Syz
+struct LeafTerms64 {
+  double v[7][32];  // m, m d, d; a column a lane
+};
+__device__ __forceinline__ int32_t leaf_moments64_lanes(
+    int64_t b, unsigned gm, int sub, LeafTerms64 &T, TreeNode *node, Mom64 *m64, double *nrs,
+    const double *sx, const double *sy, const double *sz, const double *sm, const double *srs,
+    const int32_t *sq, const double *box, const SegView &sv) {
+  const int col0 = (threadIdx.x & 31) - sub;
+  const int4 *n4 = reinterpret_cast<const int4 *>(&node[b]);
+  const int4 r1 = n4[1], r2 = n4[2], r3 = n4[3];
+  const int32_t f = r3.z, c = r3.w;
+  const double L = box[5 * seg_at(sv, f) + 3];
+  const double rx = sx[f], ry = sy[f], rz = sz[f];
+  // the factors' rows of the lane's two sums (row k1 < 4: the factor is one)
+  const int k0 = sub < 4 ? sub : (sub == 7 ? 1 : sub - 3), k1 = sub < 4 ? 0 : (sub == 7 ? 5 : sub);
+  const int h0 = 1 + (sub & 1);
+  double s0 = 0.0, s1 = 0.0;
+  int64_t rsb = 0;
+  int32_t lo[3] = {P3T_QMAX, P3T_QMAX, P3T_QMAX}, hi[3] = {-1, -1, -1};
+  for (int32_t base = 0; base < c; base += 8) {
+    const int32_t i = f + base + sub;
+    if (base + sub < c) {
+      const double m = sm[i], dx = sx[i] - rx, dy = sy[i] - ry, dz = sz[i] - rz;
+      const int l = col0 + sub;
+      T.v[0][l] = m;
+      T.v[1][l] = m * dx; T.v[2][l] = m * dy; T.v[3][l] = m * dz;
+      T.v[4][l] = dx; T.v[5][l] = dy; T.v[6][l] = dz;
+      rsb = max_reach(rsb, srs[i]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        lo[a] = min(lo[a], sq[3 * i + a]);
+        hi[a] = max(hi[a], sq[3 * i + a]);
+      }
+    }
+    __syncwarp(gm);
+    const int nb = min(8, c - base);
+    for (int j = 0; j < nb; ++j) {
+      const double w = T.v[k1][col0 + j];
+      s0 = __fma_rn(T.v[k0][col0 + j], k1 < 4 ? 1.0 : w, s0);
+      s1 = __fma_rn(T.v[h0][col0 + j], T.v[6][col0 + j], s1);
+    }
+    __syncwarp(gm);
+  }
+  grp_box(gm, lo, hi, rsb);
+  const double M = grp_shfl(gm, s0, 0);
+  const double iM = 1.0 / M;
+  const double el = s0 * iM;  // lanes 1-3: e
+  const double e[3] = {grp_shfl(gm, el, 1), grp_shfl(gm, el, 2), grp_shfl(gm, el, 3)};
+  // lane 4 + q: C of xx, yy, zz, xy; lanes 0, 1: xz, yz
+  const double ea = sub == 4 || sub == 7 || sub == 0 ? e[0] : (sub == 6 ? e[2] : e[1]);
+  const double eb = sub == 4 ? e[0] : (sub == 5 || sub == 7 ? e[1] : e[2]);
+  const double C = (sub >= 4 ? s0 : s1) - M * ea * eb;
+  const double tr = grp_shfl(gm, C, 4) + grp_shfl(gm, C, 5) + grp_shfl(gm, C, 6);
+  const double C3 = 3.0 * C, Q = C3 - tr;
+  double *o = reinterpret_cast<double *>(&m64[b]);
+  if (sub == 0) o[3] = M;
+  if (sub >= 1 && sub < 4) o[sub - 1] = (sub == 1 ? rx : (sub == 2 ? ry : rz)) + el;
+  if (sub >= 4) o[sub] = sub < 7 ? Q : C3;
+  if (sub < 2) o[8 + sub] = C3;
+  grp_store64(b, sub, node, nrs, lo, hi, r1.w, rsb, L);
+  return r2.w;
+}
+
+// One step of the sum over the group's eight lanes: the lanes with the bit set
+// keep the upper half of the values, the others the lower half, each added to
+// the partner's (so that every value is added once a step, not in every lane)
+template <int N>
+__device__ __forceinline__ void halve(unsigned gm, bool up, int bit, double (&v)[N]) {
+  constexpr int H = (N + 1) / 2;
+#pragma unroll
+  for (int q = 0; q < H; ++q) {
+    const int u = q + N / 2;  // an odd middle value is kept by both
+    const double keep = up ? v[u] : v[q], give = up ? v[q] : v[u];
+    v[q] = keep + __shfl_xor_sync(gm, give, bit);
+  }
+}
+
+// One internal node of the FP64 path, a child a lane, the eight slots (zero
+// past the last child) added in the same fixed pairwise tree as the mixed
+// path's
+__device__ int32_t node_moments64(int64_t b, unsigned gm, int sub, TreeNode *node, Mom64 *m64,
+                                  double *nrs, const double *box, const SegView &sv) {
+  const int4 *n4 = reinterpret_cast<const int4 *>(&node[b]);
+  const int4 r1 = __ldcg(n4 + 1), r2 = __ldcg(n4 + 2), r3 = __ldcg(n4 + 3);
+  const int32_t c0 = r3.x, nch = r3.y;
+  if (nch < 1 || nch > 8) return r2.w;  // only a node with children is completed
+  int64_t rsb = 0;
+  int32_t lo[3] = {P3T_QMAX, P3T_QMAX, P3T_QMAX}, hi[3] = {-1, -1, -1};
+  const bool on = sub < nch;
+  double2 g[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) g[k] = make_double2(0.0, 0.0);
+  if (on) {
+    const double2 *m = reinterpret_cast<const double2 *>(&m64[c0 + sub]);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) g[k] = __ldcg(m + k);
+    const int4 *cn = reinterpret_cast<const int4 *>(&node[c0 + sub]);
+    const int4 q0 = __ldcg(cn), q1 = __ldcg(cn + 1);
+    rsb = max_bits(0, __ldcg(&nrs[c0 + sub]));
+    lo[0] = q0.x; lo[1] = q0.y; lo[2] = q0.z;
+    hi[0] = q1.x; hi[1] = q1.y; hi[2] = q1.z;
+  }
+  grp_box(gm, lo, hi, rsb);
+  const double m = g[1].y;
+  double t4[4] = {m, m * g[0].x, m * g[0].y, m * g[1].x};
+  const bool b4 = sub & 4, b2 = sub & 2, b1 = sub & 1;
+  halve(gm, b4, 4, t4);
+  double t2[2] = {t4[0], t4[1]};
+  halve(gm, b2, 2, t2);
+  const double t = t2[0] + __shfl_xor_sync(gm, t2[0], 1);  // lane 2c: sum c of M, M com
+  const double M = grp_shfl(gm, t, 0);
+  const double iM = 1.0 / M;
+  const double cl = t * iM;
+  const double cx = grp_shfl(gm, cl, 2), cy = grp_shfl(gm, cl, 4), cz = grp_shfl(gm, cl, 6);
+  double Q[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if (on) {
+    const double dx = g[0].x - cx, dy = g[0].y - cy, dz = g[1].x - cz;
+    const double d2 = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
+    const double tx = 3.0 * dx, ty = 3.0 * dy;
+    Q[0] = __fma_rn(m, __fma_rn(tx, dx, -d2), g[2].x);
+    Q[1] = __fma_rn(m, __fma_rn(ty, dy, -d2), g[2].y);
+    Q[2] = __fma_rn(m, __fma_rn(3.0 * dz, dz, -d2), g[3].x);
+    Q[3] = __fma_rn(m, tx * dy, g[3].y);
+    Q[4] = __fma_rn(m, tx * dz, g[4].x);
+    Q[5] = __fma_rn(m, ty * dz, g[4].y);
+  }
+  halve(gm, b4, 4, Q);
+  double Q3[3] = {Q[0], Q[1], Q[2]};
+  // three values: the lower lanes keep 0 and 1, the upper ones 2 (in [1])
+  halve(gm, b2, 2, Q3);
+  const double keep = b2 ? Q3[1] : (b1 ? Q3[1] : Q3[0]), give = b2 ? Q3[1] : (b1 ? Q3[0] : Q3[1]);
+  const double q = keep + __shfl_xor_sync(gm, give, 1);
+  double *o = reinterpret_cast<double *>(&m64[b]);
+  if (sub == 0) o[3] = M;
+  if (sub == 2) o[0] = cl;
+  if (sub == 4) o[1] = cl;
+  if (sub == 6) o[2] = cl;
+  if ((sub & 3) != 3) o[4 + (b4 ? 3 : 0) + (sub & 3)] = q;
+  grp_store64(b, sub, node, nrs, lo, hi, r1.w, rsb, box[5 * seg_at(sv, r3.z) + 3]);
+  return r2.w;
+}
+
+// All moments in one launch, bottom-up: a leaf, once computed, is counted off
+// at its parent (node_done, preset to the number of children by k_nodes_bfs);
+// the child that brings the count to zero makes the parent ready, which its
+// warp takes next, four nodes at a time (each node's record gives its parent
+// in the same load as its children).  Nothing waits, and a node's result does
+// not depend on which child arrives last.
+struct MomArgs {
+  const int64_t *nleaf;
+  const int32_t *leaf_list;
+  TreeNode *node;
+  Mom32 *m32;
+  Mom64 *m64;
+  double *nrs;
+  const float4 *spA, *spB;
+  const float *sml;
+  const double *sx, *sy, *sz, *sm, *srs;
+  const int32_t *sq;
+  const double *box;
+  SegView sv;
+  int32_t *node_done;
+};
+template <bool MIXED> struct MomTerms { using type = LeafTerms; };
+template <> struct MomTerms<false> { using type = LeafTerms64; };
+template <bool MIXED>
+__global__ void __launch_bounds__(128) k_moments_up(MomArgs g) {
   pdl_wait();
-  __shared__ LeafTerms s_t[4];
+  __shared__ typename MomTerms<MIXED>::type s_t[4];
   __shared__ int32_t s_ready[4][32];
-  const int64_t nleaf = *d_nleaf;
+  const int64_t nleaf = *g.nleaf;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane & 7, grp = lane >> 3;
   const unsigned gm = 0xffu << (lane & 24), lt = (1u << lane) - 1u;
   int32_t *ready = s_ready[w];
@@ -1145,18 +1301,29 @@ __global__ void __launch_bounds__(128) k_moments_up32(
     int32_t p = -1;  // held by one lane a leaf
     if (lanes) {
       if (t < nleaf) {
-        p = leaf_moments32_lanes(leaf_list[t], gm, sub, s_t[w], node, m32, nrs, spA, spB, sml, srs,
-                                 sq, box, sv);
+        const int32_t b = g.leaf_list[t];
+        if constexpr (MIXED)
+          p = leaf_moments32_lanes(b, gm, sub, s_t[w], g.node, g.m32, g.nrs, g.spA, g.spB, g.sml,
+                                   g.srs, g.sq, g.box, g.sv);
+        else
+          p = leaf_moments64_lanes(b, gm, sub, s_t[w], g.node, g.m64, g.nrs, g.sx, g.sy, g.sz,
+                                   g.sm, g.srs, g.sq, g.box, g.sv);
         if (sub != 0) p = -1;
       }
     } else if (t < nleaf) {
-      p = leaf_moments32_thread(leaf_list[t], node, m32, nrs, spA, spB, sml, srs, sq, box, sv);
+      const int32_t b = g.leaf_list[t];
+      if constexpr (MIXED)
+        p = leaf_moments32_thread(b, g.node, g.m32, g.nrs, g.spA, g.spB, g.sml, g.srs, g.sq, g.box,
+                                  g.sv);
+      else
+        p = leaf_moments64_thread(b, g.node, g.m64, g.nrs, g.sx, g.sy, g.sz, g.sm, g.srs, g.sq,
+                                  g.box, g.sv);
     }
     int n = 0;  // nodes ready, all of their children done
     for (;;) {
       __threadfence();  // the nodes' records before the counts
       __syncwarp();
-      const bool last = p >= 0 && atomicSub(&node_done[p], 1) == 1;
+      const bool last = p >= 0 && atomicSub(&g.node_done[p], 1) == 1;
       const unsigned m = __ballot_sync(0xffffffffu, last);
       if (last) ready[n + __popc(m & lt)] = p;
       n += __popc(m);
@@ -1169,177 +1336,12 @@ __global__ void __launch_bounds__(128) k_moments_up32(
       __syncwarp();
       p = -1;
       if (b >= 0) {
-        p = node_moments32(b, gm, sub, node, m32, nrs, box, sv);
+        if constexpr (MIXED)
+          p = node_moments32(b, gm, sub, g.node, g.m32, g.nrs, g.box, g.sv);
+        else
+          p = node_moments64(b, gm, sub, g.node, g.m64, g.nrs, g.box, g.sv);
         if (sub != 0) p = -1;
       }
-    }
-  }
-}
-
-// first breadth-first id at level >= l (levels ascend in breadth-first order)
-__device__ __forceinline__ int64_t level_begin(const TreeNode *node, int64_t nn, int l) {
-  int64_t lo = 0, hi = nn;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (node[mid].level < l) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-// first breadth-first id of every level 0..21 and the node count (levels
-// ascend in breadth-first order): one thread per level
-__global__ void k_level_offsets(const int64_t *d_nnode, int64_t node_cap, const TreeNode *node,
-                                int64_t *lvl_start) {
-  pdl_wait();
-  const int64_t nn = min(*d_nnode, node_cap);
-  const int l = threadIdx.x;
-  if (l <= P3T_BITS + 1) lvl_start[l] = l == P3T_BITS + 1 ? nn : level_begin(node, nn, l);
-}
-
-// The internal nodes of one level (levels 0..20), one thread per node, from
-// their finished children; launched level by level, deepest first.  (A grid
-// barrier between levels in one cooperative launch was measured slower than
-// the launches: its waits dominated.)
-// Internal nodes of one level from their finished children.  Every level is
-// small enough that its time is the latency of one warp's FP64 instruction
-// stream (one FP64 warp instruction per 64 cycles of a sub-partition), so a
-// node's children are spread over L lanes (L = 8, 4, 2 or 1, the largest that
-// keeps the level within about one warp per sub-partition), lane sub holding
-// the child slots sub, sub + L, ... of the node's eight.  Each child's terms
-// are rounded on their own and the eight slots (zero where there is no child)
-// are added in one fixed pairwise tree, slots s and s + 4, then s + 2, then
-// s + 1: in registers while the stride is a multiple of L, by shuffles below
-// it.  The sums are therefore the same bits for every L, so a node's moments
-// do not depend on how many nodes share its level (a tree built alone or
-// beside other systems' trees).  The loop runs in warp-uniform chunks so that
-// every lane reaches every shuffle; groups past the level's end or at leaves
-// contribute nothing.
-__device__ __forceinline__ double shfl_down_group(double v, int o) {
-  return __shfl_xor_sync(0xffffffffu, v, o);
-}
-
-// the fixed pairwise tree over slots: J = 8 / L slots in this lane's
-// registers, then the shuffles between the L lanes of the group
-template <int L, int NQ>
-__device__ __forceinline__ void slot_tree(double (&v)[8 / L][NQ]) {
-#pragma unroll
-  for (int S = 4; S >= L; S >>= 1)
-#pragma unroll
-    for (int j = 0; j < S / L; ++j)
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) v[j][q] += v[j + S / L][q];
-#pragma unroll
-  for (int o = L >> 1; o > 0; o >>= 1)
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) v[0][q] += shfl_down_group(v[0][q], o);
-}
-
-template <int L>
-__device__ void moments_level_L(int64_t b0, int64_t nn, TreeNode *node, Mom64 *m64, Mom32 *m32,
-                                double *nrs, const double *box, const SegView &sv) {
-  constexpr int J = 8 / L;
-  const int lane = threadIdx.x & 31, sub = lane & (L - 1);
-  const int per_warp = 32 / L;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t wb = warp * per_warp; wb < nn; wb += nwarps * per_warp) {
-    const int64_t gi = wb + lane / L;
-    const bool valid = gi < nn;
-    const int64_t b = b0 + (valid ? gi : 0);
-    TreeNode *pn = &node[b];
-    const int32_t c0 = valid ? pn->child0 : 0, nch = valid ? pn->nchild : 0;
-    double prs = 0.0;
-    int32_t plo[3] = {P3T_QMAX, P3T_QMAX, P3T_QMAX}, phi[3] = {-1, -1, -1};
-    double t[J][4];  // M, M cx, M cy, M cz
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const int k = sub + j * L;
-      t[j][0] = t[j][1] = t[j][2] = t[j][3] = 0.0;
-      if (k < nch) {
-        const Mom64 &cm = m64[c0 + k];
-        t[j][0] = cm.M;
-        t[j][1] = cm.M * cm.cx;
-        t[j][2] = cm.M * cm.cy;
-        t[j][3] = cm.M * cm.cz;
-        prs = fmax(prs, nrs[c0 + k]);
-        const TreeNode &cn = node[c0 + k];
-        for (int a = 0; a < 3; ++a) { plo[a] = min(plo[a], cn.qlo[a]); phi[a] = max(phi[a], cn.qhi[a]); }
-      }
-    }
-    slot_tree<L, 4>(t);
-    for (int o = L >> 1; o > 0; o >>= 1) {
-      for (int a = 0; a < 3; ++a) {
-        plo[a] = min(plo[a], __shfl_xor_sync(0xffffffffu, plo[a], o));
-        phi[a] = max(phi[a], __shfl_xor_sync(0xffffffffu, phi[a], o));
-      }
-      prs = fmax(prs, shfl_down_group(prs, o));
-    }
-    Mom64 pm = {};
-    if (nch > 0) {
-      const double iM = 1.0 / t[0][0];
-      pm.M = t[0][0]; pm.cx = t[0][1] * iM; pm.cy = t[0][2] * iM; pm.cz = t[0][3] * iM;
-    }
-    double Q[J][6];  // xx, yy, zz, xy, xz, yz
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const int k = sub + j * L;
-      for (int q = 0; q < 6; ++q) Q[j][q] = 0.0;
-      if (k < nch) {
-        const Mom64 &cm = m64[c0 + k];
-        const double dx = cm.cx - pm.cx, dy = cm.cy - pm.cy, dz = cm.cz - pm.cz;
-        const double d2 = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
-        const double tx = 3.0 * dx, ty = 3.0 * dy;
-        Q[j][0] = __fma_rn(cm.M, __fma_rn(tx, dx, -d2), cm.qxx);
-        Q[j][1] = __fma_rn(cm.M, __fma_rn(ty, dy, -d2), cm.qyy);
-        Q[j][2] = __fma_rn(cm.M, __fma_rn(3.0 * dz, dz, -d2), cm.qzz);
-        Q[j][3] = __fma_rn(cm.M, tx * dy, cm.qxy);
-        Q[j][4] = __fma_rn(cm.M, tx * dz, cm.qxz);
-        Q[j][5] = __fma_rn(cm.M, ty * dz, cm.qyz);
-      }
-    }
-    slot_tree<L, 6>(Q);
-    if (valid && nch > 0 && sub == 0) {
-      pm.qxx = Q[0][0]; pm.qyy = Q[0][1]; pm.qzz = Q[0][2];
-      pm.qxy = Q[0][3]; pm.qxz = Q[0][4]; pm.qyz = Q[0][5];
-      for (int a = 0; a < 3; ++a) { pn->qlo[a] = plo[a]; pn->qhi[a] = phi[a]; }
-      nrs[b] = prs;
-      finish_node(pn, m64, m32, prs, ldexp(box[5 * seg_at(sv, pn->first) + 3], -P3T_BITS), b,
-                  pm);
-    }
-  }
-}
-
-__device__ void moments_level(int level, const int64_t *lvl_start, TreeNode *node, Mom64 *m64,
-                              Mom32 *m32, double *nrs, const double *box, const SegView &sv,
-                              int64_t warp_target) {
-  const int64_t b0 = lvl_start[level], b1 = lvl_start[level + 1];
-  const int64_t nn = b1 - b0;
-  if (nn <= 0) return;
-  int L = 8;
-  while (L > 1 && nn * L > 32 * warp_target) L >>= 1;
-  switch (L) {
-    case 8: moments_level_L<8>(b0, nn, node, m64, m32, nrs, box, sv); break;
-    case 4: moments_level_L<4>(b0, nn, node, m64, m32, nrs, box, sv); break;
-    case 2: moments_level_L<2>(b0, nn, node, m64, m32, nrs, box, sv); break;
-    default: moments_level_L<1>(b0, nn, node, m64, m32, nrs, box, sv); break;
-  }
-}
-
-// levels kDeepLevel and deeper share one single-block launch
-constexpr int kDeepLevel = 12;
-
-
-// levels level_hi down to level_lo; several levels only with a single block
-// (a block barrier between levels)
-__global__ void k_moments_level(int level_hi, int level_lo, const int64_t *lvl_start,
-                                TreeNode *node, Mom64 *m64, Mom32 *m32, double *nrs,
-                                const double *box, SegView sv, int64_t warp_target) {
-  pdl_wait();
-  for (int l = level_hi; l >= level_lo; --l) {
-    moments_level(l, lvl_start, node, m64, m32, nrs, box, sv, warp_target);
-    if (l > level_lo) {
-      __threadfence_block();
-      __syncthreads();
     }
   }
 }
@@ -1496,31 +1498,13 @@ int p3t_run_build_tree(p3t_ctx *c, const p3t_particles *p, cudaStream_t s) {
   if (rc) return rc;
   pdl_launch(k_lists, dim3((unsigned)gn), dim3(kBlock), 0, s, &cnt[3], c->node_cap, c->node_flag,
              c->flag_pos, c->pre2bfs, &cnt[19], c->leaf_list, c->group_list, &cnt[2], &cnt[15]);
-  if (c->prm.precision == P3T_MIXED) {
-    pdl_launch(k_moments_up32, dim3((unsigned)p3t_grid(c->node_cap * 8, 128, maxb)), dim3(128), 0, s, 
-        &cnt[2], c->leaf_list, c->node, c->mom32, c->nrs, c->spA, c->spB, c->sml, c->srs,
-        c->sq, c->box, sv, c->node_done);
-    p3t_note_launches(1);
-  } else {
-    pdl_launch(k_moments_leaf, dim3((unsigned)p3t_grid(c->node_cap, 128, maxb)), dim3(128), 0, s, 
-        &cnt[2], c->leaf_list, c->node, c->mom64, c->mom32, c->nrs, c->sx, c->sy, c->sz, c->sm,
-        c->srs, c->sq, c->box, sv);
-    // internal nodes, level by level, deepest first
-    int64_t *lvl_start = c->counters + 32;  // [P3T_BITS + 2]
-    pdl_launch(k_level_offsets, dim3(1), dim3(32), 0, s, &cnt[3], c->node_cap, c->node, lvl_start);
-    // the deep levels (empty or nearly so in a disk) in one single-block
-    // launch, then one launch a level at about one warp per sub-partition
-    pdl_launch(k_moments_level, dim3(1), dim3(128), 0, s, P3T_BITS - 1, kDeepLevel, lvl_start, c->node, c->mom64,
-                                      c->mom32, c->nrs, c->box, sv, 4);
-    const int64_t wt = (int64_t)c->num_sms * 4;
-    for (int l = kDeepLevel - 1; l >= 0; --l)
-      pdl_launch(k_moments_level, dim3((unsigned)c->num_sms), dim3(128), 0, s, l, l, lvl_start, c->node, c->mom64,
-                                                           c->mom32, c->nrs, c->box, sv, wt);
-    p3t_note_launches(3 + kDeepLevel);  // leaves, level offsets, deep levels, one a level
-  }
-  // own kernels here (the scans, sorts and moments count themselves): box,
-  // keys, gather, nodes_pre, node_counts, nodes_bfs, lists
-  p3t_note_launches(7);
+  const MomArgs ma{&cnt[2], c->leaf_list, c->node, c->mom32, c->mom64, c->nrs, c->spA, c->spB,
+                   c->sml, c->sx, c->sy, c->sz, c->sm, c->srs, c->sq, c->box, sv, c->node_done};
+  auto moments = c->prm.precision == P3T_MIXED ? k_moments_up<true> : k_moments_up<false>;
+  pdl_launch(moments, dim3((unsigned)p3t_grid(c->node_cap * 8, 128, maxb)), dim3(128), 0, s, ma);
+  // own kernels here (the scans and sorts count themselves): box, keys, gather,
+  // nodes_pre, node_counts, nodes_bfs, lists, moments
+  p3t_note_launches(8);
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }
 
