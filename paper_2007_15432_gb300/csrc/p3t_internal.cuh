@@ -50,6 +50,13 @@ __device__ __forceinline__ FF ff_div(FF a, FF b) {
 
 // 1 / sqrt(r2): the FP32 estimate and one Newton step y (3 - r2 y^2) / 2 with
 // the residual 1 - r2 y^2 formed in float-float
+// rsqrtf of a normal number (the same bits): without flushing, rsqrtf adds a
+// comparison and two multiplications that only a subnormal needs
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ FF ff_rsqrt(FF r2) {
   const float y = rsqrtf(r2.h);
   const float p = y * y;

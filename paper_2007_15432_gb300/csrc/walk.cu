@@ -25,6 +25,8 @@
 // replicas split a batch by pairs, and each pair slot keeps its own partial
 // sum (even and odd entries) until the batch is folded.  The FP64 path
 // (k_walk64) shares the traversal and has a layout of its own.
+#include <algorithm>
+
 #include "p3t_internal.cuh"
 
 namespace {
@@ -95,12 +97,6 @@ __device__ __forceinline__ void two_sum(float &hi, float &lo, float b) {
   hi = s;
   lo += err;
 }
-
-#ifndef P3T_PAIR_UNROLL
-#define P3T_PAIR_UNROLL 1  // pair slots in flight per loop iteration
-#endif
-constexpr int kPairUnroll = P3T_PAIR_UNROLL;
-
 
 // ---- per-target state (one lane per target) ---------------------------------
 struct Target {
@@ -206,7 +202,7 @@ __device__ __forceinline__ void pp_pair(const WalkArgs &a, Target &t,
   const f2 dz = add2(sub2(t.Z, azw.x), sub2(t.ZL, bzw.x));
   const f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
   const float r2a = f2_lo(r2), r2b = f2_hi(r2);
-  const f2 rinv = f2_pk(rsqrtf(fmaxf(r2a, 1e-30f)), rsqrtf(fmaxf(r2b, 1e-30f)));
+  const f2 rinv = f2_pk(rsqrt_normal(fmaxf(r2a, 1e-30f)), rsqrt_normal(fmaxf(r2b, 1e-30f)));
   const f2 r = mul2(r2, rinv);
   const float ya = f2_lo(r) * fminf(t.inv_ro, f2_lo(bzw.y));
   const float yb = f2_hi(r) * fminf(t.inv_ro, f2_hi(bzw.y));
@@ -267,7 +263,7 @@ __device__ __forceinline__ void pp_pair_far(Target &t, const StagePP32 &S, int p
   const f2 dy = add2(sub2(t.Y, axy.y), sub2(t.YL, bxy.y));
   const f2 dz = add2(sub2(t.Z, azw.x), sub2(t.ZL, bzw.x));
   const f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-  const f2 rinv = f2_pk(rsqrtf(f2_lo(r2)), rsqrtf(f2_hi(r2)));
+  const f2 rinv = f2_pk(rsqrt_normal(f2_lo(r2)), rsqrt_normal(f2_hi(r2)));
   const f2 r = mul2(r2, rinv);
   const f2 f = mul2(mul2(azw.y, rinv), mul2(rinv, rinv));
   BX = fma2(f, dx, BX);
@@ -283,6 +279,7 @@ __device__ __forceinline__ void fold_pairs(Target &t, f2 BX, f2 BY, f2 BZ, f2 TB
   t.tabs += f2_lo(TB) + f2_hi(TB);
 }
 
+template <int U>
 __device__ __forceinline__ void eval_pp(const WalkArgs &a, Target &t, const int32_t *list,
                                         int nsrc, void *stage, const FarBox &box,
                                         unsigned &npp) {
@@ -312,10 +309,10 @@ __device__ __forceinline__ void eval_pp(const WalkArgs &a, Target &t, const int3
   npp += (t.valid && t.rep == 0) ? (unsigned)nsrc : 0u;
   const int np = (nsrc + 1) >> 1;
   if (any_near) {
-#pragma unroll kPairUnroll
+#pragma unroll U
     for (int p = t.rep; p < np; p += t.nrep) pp_pair(a, t, S, p, BX, BY, BZ, TB, npp);
   } else {
-#pragma unroll kPairUnroll
+#pragma unroll U
     for (int p = t.rep; p < np; p += t.nrep) pp_pair_far(t, S, p, BX, BY, BZ, TB);
   }
   __syncwarp();
@@ -333,7 +330,8 @@ __device__ __forceinline__ void node_pair(Target &t, const StageND32 &S, int p, 
   const f2 dy = add2(sub2(t.Y, hxy.y), sub2(t.YL, lxy.y));
   const f2 dz = add2(sub2(t.Z, hzw.x), sub2(t.ZL, lzw.x));
   const f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-  const f2 rinv = f2_pk(rsqrtf(fmaxf(f2_lo(r2), 1e-30f)), rsqrtf(fmaxf(f2_hi(r2), 1e-30f)));
+  const f2 rinv = f2_pk(rsqrt_normal(fmaxf(f2_lo(r2), 1e-30f)),
+                        rsqrt_normal(fmaxf(f2_hi(r2), 1e-30f)));
   const f2 rinv2 = mul2(rinv, rinv);
   const f2 rinv3 = mul2(rinv2, rinv);
   const f2 rinv5 = mul2(rinv3, rinv2);
@@ -349,6 +347,7 @@ __device__ __forceinline__ void node_pair(Target &t, const StageND32 &S, int p, 
   TB = fma2(hzw.y, rinv2, TB);  // -M / r^2
 }
 
+template <int U>
 __device__ __forceinline__ void eval_nodes(const WalkArgs &a, Target &t,
                                            const int32_t *list, int nnd, void *stage,
                                            unsigned &npn) {
@@ -373,7 +372,7 @@ __device__ __forceinline__ void eval_nodes(const WalkArgs &a, Target &t,
   f2 BX = 0ull, BY = 0ull, BZ = 0ull, TB = 0ull;
   npn += (t.valid && t.rep == 0) ? (unsigned)nnd : 0u;
   const int np = (nnd + 1) >> 1;
-#pragma unroll kPairUnroll
+#pragma unroll U
   for (int p = t.rep; p < np; p += t.nrep) node_pair(t, S, p, BX, BY, BZ, TB);
   __syncwarp();
   // force sums as they are; the magnitude sum was of -M / r^2
@@ -548,15 +547,18 @@ __device__ bool traverse(const WalkArgs &a, const GroupBox &gb, int32_t first, i
 }
 
 // up to 32 targets of a group (each on nrep lanes), batches staged in shared
-// memory
+// memory, U pair slots in flight
+template <int U>
 struct GroupEval {
   const WalkArgs &a;
   Target &t;
   void *stage;
   const FarBox &box;
   unsigned &npp, &npn;
-  __device__ void nodes(const int32_t *list, int n) { eval_nodes(a, t, list, n, stage, npn); }
-  __device__ void pp(const int32_t *list, int n) { eval_pp(a, t, list, n, stage, box, npp); }
+  __device__ void nodes(const int32_t *list, int n) { eval_nodes<U>(a, t, list, n, stage, npn); }
+  __device__ void pp(const int32_t *list, int n) {
+    eval_pp<U>(a, t, list, n, stage, box, npp);
+  }
 };
 
 // the walk's FarBox from its (valid) targets, written by lane 0
@@ -698,10 +700,6 @@ __device__ bool refine_group(const WalkArgs &a, const GroupBox &gb, bool redo, i
   return true;
 }
 
-#ifndef P3T_WALK_MINB_MIXED
-#define P3T_WALK_MINB_MIXED 6  // resident blocks per SM asked of the mixed walk
-#endif
-
 // the warp's interaction counts to the caller's: a lane that met its target's
 // own entry holds npp below zero, the warp sum is taken modulo 2^32, where a
 // warp's true count fits
@@ -715,7 +713,15 @@ __device__ __forceinline__ void add_counts(const WalkArgs &a, unsigned p, unsign
   }
 }
 
-__global__ void __launch_bounds__(kWarps * 32, P3T_WALK_MINB_MIXED)
+// Two forms of the mixed walk, the same arithmetic in the same order.  Many
+// units of work (U = 1): 80 registers, six blocks an SM, one pair slot at a
+// time; a second slot in flight costs registers and is slower (N = 1e6: 1,219
+// us, 1,514 with four blocks of two slots).  Fewer units than warps (U = 4): a
+// unit has a sub-partition nearly to itself and its time is the latency of its
+// own chain, which four slots in flight shorten.
+constexpr int kFewU = 4, kManyBlocks = 6, kFewBlocks = 3;
+template <int U>
+__global__ void __launch_bounds__(kWarps * 32, U == 1 ? kManyBlocks : kFewBlocks)
     k_walk(const WalkArgs a) {
   pdl_wait();
   __shared__ int32_t s_pp[kWarps][kPPCap];
@@ -734,19 +740,23 @@ __global__ void __launch_bounds__(kWarps * 32, P3T_WALK_MINB_MIXED)
   unsigned npp = 0, npn = 0;
 
   for (;;) {
-    // work unit u: target group u / 2, its first 32 targets (u even) or the
-    // rest (u odd; empty for a group of at most 32): half-group units keep
-    // the warps' finishing times within one such unit of each other
+    // work unit u: the first 32 targets of target group u, then, once all of
+    // those are taken, the rest of group u - nleaf (empty for a group of at
+    // most 32): units of at most 32 targets keep the warps' finishing times
+    // close, and the rests, mostly small, are left for the end (against a
+    // group's rest right after its first 32: N = 3e5 463 -> 441 us, 1e5 254 ->
+    // 250, 1e6 the same)
     int64_t u = 0;
     if (lane == 0) u = atomicAdd(reinterpret_cast<unsigned long long *>(a.cursor), 1ull);
     u = __shfl_sync(0xffffffffu, u, 0);
-    const int64_t g = u >> 1;
+    const bool rest = u >= nleaf;
+    const int64_t g = rest ? u - nleaf : u;
     if (g >= nleaf) break;
     if (*(volatile int32_t *)&a.st->code != 0) break;
     const TreeNode &G = a.node[a.leaf_list[g]];
     const int32_t gfirst = G.first, gcount = G.count;
-    const int32_t t0 = (u & 1) ? gfirst + 32 : gfirst;
-    const int32_t t1 = (u & 1) ? gfirst + gcount : min(gfirst + gcount, gfirst + 32);
+    const int32_t t0 = rest ? gfirst + 32 : gfirst;
+    const int32_t t1 = rest ? gfirst + gcount : min(gfirst + gcount, gfirst + 32);
     if (t0 >= t1) continue;
     GroupBox gb;
     gb.load(G);
@@ -757,7 +767,7 @@ __global__ void __launch_bounds__(kWarps * 32, P3T_WALK_MINB_MIXED)
       Target t;
       t.load(a, tb + (lane - rep * k), rep < nrep, rep < nrep ? rep : 0, nrep);
       far_box(t, s_box[w]);
-      GroupEval ev{a, t, s_stage[w], s_box[w], npp, npn};
+      GroupEval<U> ev{a, t, s_stage[w], s_box[w], npp, npn};
       ok = traverse(a, gb, gfirst, stack, s_pp[w], s_nd[w], s_big[w], s_bh, round_limit, ev);
       if (ok) {
         t.reduce(k);
@@ -1328,7 +1338,7 @@ int64_t bh_threshold(double theta, int level) {
 
 // blocks of 4 warps resident per SM: the mixed walk is compiled for 6 (80
 // registers; 30.5 KB of shared memory a block)
-int p3t_walk_blocks_per_sm() { return P3T_WALK_MINB_MIXED; }
+int p3t_walk_blocks_per_sm() { return kManyBlocks; }
 
 // the walk's arguments for the tree of context c built from particles p
 static WalkArgs walk_args(p3t_ctx *c, const p3t_particles *p) {
@@ -1356,6 +1366,12 @@ static WalkArgs walk_args(p3t_ctx *c, const p3t_particles *p) {
   for (int l = 0; l <= P3T_BITS; ++l) a.bh[l] = bh_threshold(c->prm.theta, l);
   return a;
 }
+
+// particles an SM up to which the mixed walk takes its few-units form (about
+// one unit a warp at three blocks an SM).  Force, few / many, wide disk: N =
+// 3,001 96 / 107 us, 1e4 99 / 122, 3e4 116 / 133, 4.5e4 132 / 147, 6e4 194 / 184;
+// ring: 3e4 117 / 138, 6e4 216 / 174, 1e5 439 / 247
+constexpr int kFewTargets = 200;
 
 // The FP64 walks' chunk of targets: up to kChunk at a time (one traversal
 // serves them all), fewer while a warp would get less than four chunks, so
@@ -1404,7 +1420,12 @@ int p3t_run_soft_force(p3t_ctx *c, const p3t_particles *p, double *ax,
     // one target per lane (or several lanes per target): two targets per
     // lane (a 64-target group walked once) was measured slower than two
     // walks of 32 (register pressure, longer chains)
-    pdl_launch(k_walk, dim3(blocks), dim3(kWarps * 32), 0, s, a);
+    if (c->last_n <= (int64_t)kFewTargets * c->num_sms) {
+      blocks = std::min(blocks, (unsigned)(c->num_sms * kFewBlocks));
+      pdl_launch(k_walk<kFewU>, dim3(blocks), dim3(kWarps * 32), 0, s, a);
+    } else {
+      pdl_launch(k_walk<1>, dim3(blocks), dim3(kWarps * 32), 0, s, a);
+    }
   } else {
     blocks = walk64_blocks(c, blocks);
     pdl_launch(k_walk64, dim3(blocks), dim3(kWarps * 32), 0, s, a, walk64_chunk(c, blocks));
