@@ -2,63 +2,17 @@
 // (the drift of a particle with no neighbours, Sec. 2.1.2) for the adjoint
 // of the soft kick-drift-kick (the soft force's VJP is in direct.cu).
 //
-// The state-transition matrix comes from the forward map evaluated in dual
-// numbers with six directions (one per input coordinate), the universal
-// anomaly's derivative from one Newton step taken in dual arithmetic at the
-// converged value (implicit-function theorem).
+// The product lam^T Phi is formed in reverse through the drift's formulas, the
+// universal anomaly's part from the implicit function theorem (F(chi) = 0
+// gives d chi = -dF / F').  What bounds it is the latency of one warp's FP64
+// instructions (64 cycles each): some 300 of them, against 1,200 for the
+// forward map in dual numbers with six directions.  Measured, N = 1e4:
+// 40.8 -> 14.8 us.
 #include <math.h>
 
 #include "p3t_internal.cuh"
 
 namespace {
-
-// ---- dual numbers with six directions ----------------------------------------
-struct D6 {
-  double v, d[6];
-};
-__device__ __forceinline__ D6 dc(double v) {
-  D6 r;
-  r.v = v;
-  for (int i = 0; i < 6; ++i) r.d[i] = 0.0;
-  return r;
-}
-__device__ __forceinline__ D6 operator+(const D6 &a, const D6 &b) {
-  D6 r; r.v = a.v + b.v;
-  for (int i = 0; i < 6; ++i) r.d[i] = a.d[i] + b.d[i];
-  return r;
-}
-__device__ __forceinline__ D6 operator-(const D6 &a, const D6 &b) {
-  D6 r; r.v = a.v - b.v;
-  for (int i = 0; i < 6; ++i) r.d[i] = a.d[i] - b.d[i];
-  return r;
-}
-__device__ __forceinline__ D6 operator*(const D6 &a, const D6 &b) {
-  D6 r; r.v = a.v * b.v;
-  for (int i = 0; i < 6; ++i) r.d[i] = a.d[i] * b.v + a.v * b.d[i];
-  return r;
-}
-__device__ __forceinline__ D6 operator*(double s, const D6 &a) {
-  D6 r; r.v = s * a.v;
-  for (int i = 0; i < 6; ++i) r.d[i] = s * a.d[i];
-  return r;
-}
-__device__ __forceinline__ D6 operator/(const D6 &a, const D6 &b) {
-  D6 r; r.v = a.v / b.v;
-  const double ib = 1.0 / b.v;
-  for (int i = 0; i < 6; ++i) r.d[i] = (a.d[i] - r.v * b.d[i]) * ib;
-  return r;
-}
-__device__ __forceinline__ D6 dsqrt(const D6 &a) {
-  D6 r; r.v = sqrt(a.v);
-  const double h = 0.5 / r.v;
-  for (int i = 0; i < 6; ++i) r.d[i] = a.d[i] * h;
-  return r;
-}
-__device__ __forceinline__ D6 dfun(const D6 &a, double f, double df) {
-  D6 r; r.v = f;
-  for (int i = 0; i < 6; ++i) r.d[i] = df * a.d[i];
-  return r;
-}
 
 // 1 / n! as a double (exact product of the integers up to 18!, then one
 // rounding per factor)
@@ -115,14 +69,6 @@ __device__ void stumpff4(double z, double &C, double &S, double &dC, double &dS)
   }
 }
 
-// C and S of a dual argument: values at z.v, derivatives by the chain rule
-__device__ __forceinline__ void stumpff_d(const D6 &z, D6 &C, D6 &S) {
-  double c, s_, dc_, ds_;
-  stumpff4(z.v, c, s_, dc_, ds_);
-  C = dfun(z, c, dc_);
-  S = dfun(z, s_, ds_);
-}
-
 // the universal anomaly (values only), Newton from the series inversion
 __device__ double chi_solve(double r0, double sig, double bet, double alpha, double tau,
                             double dt, double mu) {
@@ -146,58 +92,69 @@ __device__ double chi_solve(double r0, double sig, double bet, double alpha, dou
   return chi;
 }
 
-// lam_in = Phi^T lam_out for the drift of one particle by dt
+__device__ __forceinline__ double dot3(const double (&a)[3], const double (&b)[3]) {
+  return fma(a[0], b[0], fma(a[1], b[1], a[2] * b[2]));
+}
+
+// lam_in = Phi^T lam_out for the drift of one particle by dt (sq = sqrt mu, isq
+// = 1 / sq, imu = 1 / mu).  With C, S the Stumpff functions at z = alpha chi^2:
+// c2 = chi^2 C, c3 = chi^3 S, c1 = (z S - 1) chi; x' = f x + g v and v' = fd x
+// + gd v with f = 1 - c2 / r0, g = dt - c3 / sq, fd = sq c1 / (r r0), gd = 1 -
+// c2 / r.  A name ending in b is the adjoint of the name before it.
 __global__ void k_kepler_vjp(int64_t n, const double *x, const double *y, const double *z,
                              const double *vx, const double *vy, const double *vz, double dt,
-                             double mu, double *lx, double *ly, double *lz, double *lvx,
-                             double *lvy, double *lvz) {
+                             double mu, double sq, double isq, double imu, double *lx, double *ly,
+                             double *lz, double *lvx, double *lvy, double *lvz) {
   pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    D6 X[3] = {dc(x[i]), dc(y[i]), dc(z[i])}, V[3] = {dc(vx[i]), dc(vy[i]), dc(vz[i])};
-    for (int a = 0; a < 3; ++a) { X[a].d[a] = 1.0; V[a].d[3 + a] = 1.0; }
-    const double sq = sqrt(mu), isq = 1.0 / sq, imu = 1.0 / mu;
-    const D6 r0 = dsqrt(X[0] * X[0] + X[1] * X[1] + X[2] * X[2]);
-    const D6 v2 = V[0] * V[0] + V[1] * V[1] + V[2] * V[2];
-    const D6 rv = X[0] * V[0] + X[1] * V[1] + X[2] * V[2];
-    const D6 alpha = 2.0 * (dc(1.0) / r0) - imu * v2;
-    const D6 sig = isq * rv;
-    const D6 bet = dc(1.0) - alpha * r0;
-    const double tau = sq * dt;
-    const double chiv = chi_solve(r0.v, sig.v, bet.v, alpha.v, tau, dt, mu);
-    // one Newton step in dual arithmetic at the converged value
-    D6 chi = dc(chiv);
-    {
-      const D6 zz = alpha * chi * chi;
-      D6 C, S;
-      stumpff_d(zz, C, S);
-      const D6 chi2 = chi * chi;
-      const D6 F = sig * chi2 * C + bet * chi2 * chi * S + r0 * chi - dc(tau);
-      const D6 Fp = sig * chi * (dc(1.0) - zz * S) + bet * chi2 * C + r0;
-      chi = chi - F / Fp;
-    }
-    const D6 zz = alpha * chi * chi;
-    D6 C, S;
-    stumpff_d(zz, C, S);
-    const D6 chi2 = chi * chi;
-    const D6 f = dc(1.0) - chi2 * C / r0;
-    const D6 g = dc(dt) - isq * (chi2 * chi * S);
-    D6 nx[3];
+    const double X[3] = {x[i], y[i], z[i]}, V[3] = {vx[i], vy[i], vz[i]};
+    const double L[3] = {lx[i], ly[i], lz[i]}, Lv[3] = {lvx[i], lvy[i], lvz[i]};
+    const double r0 = sqrt(dot3(X, X)), ir0 = 1.0 / r0;
+    const double alpha = 2.0 * ir0 - imu * dot3(V, V);
+    const double sig = isq * dot3(X, V), bet = 1.0 - alpha * r0;
+    const double chi = chi_solve(r0, sig, bet, alpha, sq * dt, dt, mu);
+    const double chi2 = chi * chi, chi3 = chi2 * chi, zz = alpha * chi2;
+    double C, S, dC, dS;
+    stumpff4(zz, C, S, dC, dS);
+    const double w = zz * S - 1.0;
+    const double c1 = w * chi, c2 = chi2 * C, c3 = chi3 * S;
+    const double f = 1.0 - c2 * ir0, g = dt - isq * c3;
+    double nx[3];
     for (int a = 0; a < 3; ++a) nx[a] = f * X[a] + g * V[a];
-    const D6 r = dsqrt(nx[0] * nx[0] + nx[1] * nx[1] + nx[2] * nx[2]);
-    const D6 fd = sq * ((zz * S - dc(1.0)) * chi / (r * r0));
-    const D6 gd = dc(1.0) - chi2 * C / r;
-    D6 nv[3];
-    for (int a = 0; a < 3; ++a) nv[a] = fd * X[a] + gd * V[a];
-    const double lo[6] = {lx[i], ly[i], lz[i], lvx[i], lvy[i], lvz[i]};
-    double li[6];
-    for (int b = 0; b < 6; ++b) {
-      double s = 0.0;
-      for (int a = 0; a < 3; ++a) s += lo[a] * nx[a].d[b] + lo[3 + a] * nv[a].d[b];
-      li[b] = s;
+    const double ir = 1.0 / sqrt(dot3(nx, nx)), irr = sq * ir * ir0;
+    const double fd = irr * c1, gd = 1.0 - c2 * ir;
+    // v'
+    const double fdb = dot3(Lv, X), gdb = dot3(Lv, V);
+    const double c1b = fdb * irr;
+    const double rb = (gdb * c2 * ir - fdb * fd) * ir;
+    double r0b = -fdb * fd * ir0;
+    // x', with r = |x'|
+    const double rbr = rb * ir;
+    double nb[3];
+    for (int a = 0; a < 3; ++a) nb[a] = L[a] + rbr * nx[a];
+    const double fb = dot3(nb, X), gb = dot3(nb, V);
+    const double c2b = -gdb * ir - fb * ir0, c3b = -isq * gb;
+    r0b += fb * c2 * ir0 * ir0;
+    // c1, c2, c3 -> chi, z
+    const double zb = c1b * (S * chi + zz * chi * dS) + c3b * chi3 * dS + c2b * chi2 * dC;
+    const double chib = c1b * w + 2.0 * c2b * chi * C + 3.0 * c3b * chi2 * S +
+                        2.0 * zb * alpha * chi;
+    double ab = zb * chi2;
+    // chi: F = sig c2 + bet c3 + r0 chi - tau = 0
+    const double Fb = -chib / (bet * c2 - sig * c1 + r0);
+    ab += Fb * (sig * chi2 * dC + bet * chi3 * dS) * chi2;
+    const double rvb = isq * Fb * c2, betb = Fb * c3;
+    ab -= betb * r0;
+    r0b += Fb * chi - betb * alpha - 2.0 * ab * ir0 * ir0;
+    const double vb = -2.0 * imu * ab, xb = r0b * ir0;
+    double o[3], ov[3];
+    for (int a = 0; a < 3; ++a) {
+      o[a] = fd * Lv[a] + f * nb[a] + rvb * V[a] + xb * X[a];
+      ov[a] = gd * Lv[a] + g * nb[a] + rvb * X[a] + vb * V[a];
     }
-    lx[i] = li[0]; ly[i] = li[1]; lz[i] = li[2];
-    lvx[i] = li[3]; lvy[i] = li[4]; lvz[i] = li[5];
+    lx[i] = o[0]; ly[i] = o[1]; lz[i] = o[2];
+    lvx[i] = ov[0]; lvy[i] = ov[1]; lvz[i] = ov[2];
   }
 }
 
@@ -207,9 +164,10 @@ int p3t_run_kepler_vjp(p3t_ctx *c, const p3t_particles *p, double dt, double *lx
                        double *lz, double *lvx, double *lvy, double *lvz, cudaStream_t s) {
   const int64_t n = p->n;
   if (n == 0) return P3T_OK;
-  pdl_launch(k_kepler_vjp, dim3((unsigned)p3t_grid(n, 128, (int64_t)c->num_sms * P3T_NSM_BLOCKS)), dim3(128), 0, s, 
-      n, p->x, p->y, p->z, p->vx, p->vy, p->vz, dt, c->prm.G * c->prm.m_star, lx, ly, lz, lvx,
-      lvy, lvz);
+  const double mu = c->prm.G * c->prm.m_star, sq = sqrt(mu);
+  pdl_launch(k_kepler_vjp, dim3((unsigned)p3t_grid(n, 128, (int64_t)c->num_sms * P3T_NSM_BLOCKS)),
+             dim3(128), 0, s, n, p->x, p->y, p->z, p->vx, p->vy, p->vz, dt, mu, sq, 1.0 / sq,
+             1.0 / mu, lx, ly, lz, lvx, lvy, lvz);
   p3t_note_launches(1);
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }
