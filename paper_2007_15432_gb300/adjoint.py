@@ -23,7 +23,9 @@ kernels:
     Hermite, isolated particles by Kepler), the hard step's adjoint with the
     clusters and block schedule of the forward sweep (``p3t_hard_step_vjp``);
   * states are checkpointed every ``checkpoint`` steps; the backward pass
-    recomputes each segment forward from its checkpoint.
+    recomputes each segment forward from its checkpoint, up to its last drift.
+    The last segment, which the backward pass takes first, is kept by the
+    forward pass (the memory that one recomputed segment takes).
 
 Positions and velocities are (3, n) float64 CUDA tensors (rows x, y, z).
 """
@@ -113,19 +115,23 @@ class SoftKDK:
         else:
             P.p3t_soft_force_vjp(self.ctx, st, h, lv, lx, gm)
 
-    def _run(self, X, V, m, r_out, k0: int, k1: int, keep=None, have_force=False):
+    def _run(self, X, V, m, r_out, k0: int, k1: int, keep=None, have_force=False,
+             whole=True):
         """Steps k0..k1-1 in place on (X, V); with ``keep`` a list, appends
         (x_k, v'_k) (positions and velocities after the first kick) per step.
-        ``have_force``: self.acc already holds the force at X."""
+        ``have_force``: self.acc already holds the force at X.  Not ``whole``:
+        stops before the last step's drift, when all of ``keep`` is known."""
         h = 0.5 * self.params.dt_soft
         st = self._state(X, V, m, r_out)
         if not have_force:
             self._force(st)
-        for _ in range(k0, k1):
+        for k in range(k0, k1):
             P.p3t_kick(self.ctx, st, self.acc, h)
             if keep is not None:
                 keep.append((X.clone(), V.clone(),
                              self._copy_clusters() if self.hard == "p3t" else None))
+            if k == k1 - 1 and not whole:
+                break
             self._drift(st)
             self._force(st)
             P.p3t_kick(self.ctx, st, self.acc, h)
@@ -134,6 +140,9 @@ class SoftKDK:
     def forward(self, x0, v0, m, r_out, r_search=None):
         """Returns (x_N, v_N, tape); the tape holds the checkpoints.  The tree
         force needs the frozen search radii as well (``r_search``)."""
+        return self._forward(x0, v0, m, r_out, r_search, True)
+
+    def _forward(self, x0, v0, m, r_out, r_search, keep_last: bool):
         if self.force == "tree":
             if r_search is None:
                 raise ValueError("the tree force needs r_search")
@@ -144,7 +153,7 @@ class SoftKDK:
                 raise TypeError(f"expected a float64 tensor of shape {shape} on {self.dev}")
         X, V = x0.detach().clone().contiguous(), v0.detach().clone().contiguous()
         m, r_out = m.detach().contiguous(), r_out.detach().contiguous()
-        cps = []
+        cps, last = [], None
         for k0 in range(0, self.steps, self.checkpoint):
             if k0 == 0 and self.hard == "p3t":
                 self._force(self._state(X, V, m, r_out))
@@ -152,9 +161,12 @@ class SoftKDK:
             # it (the neighbour search saw the velocities before that kick)
             cl = self._copy_clusters() if self.hard == "p3t" else None
             cps.append((k0, X.clone(), V.clone(), cl))
-            self._run(X, V, m, r_out, k0, min(self.steps, k0 + self.checkpoint),
-                      have_force=k0 > 0 or self.hard == "p3t")
-        return X, V, dict(checkpoints=cps, m=m, r_out=r_out, xN=X.clone(), vN=V.clone())
+            k1 = min(self.steps, k0 + self.checkpoint)
+            if keep_last and k1 == self.steps:
+                last = []
+            self._run(X, V, m, r_out, k0, k1, last, have_force=k0 > 0 or self.hard == "p3t")
+        return X, V, dict(checkpoints=cps, last=last, m=m, r_out=r_out, xN=X.clone(),
+                          vN=V.clone())
 
     def backward(self, tape, lam_x, lam_v):
         """Adjoints (dL/dx_0, dL/dv_0, dL/dm) from those of (x_N, v_N)."""
@@ -168,15 +180,17 @@ class SoftKDK:
         for k0, Xc, Vc, clc in reversed(tape["checkpoints"]):
             k1 = min(self.steps, k0 + self.checkpoint)
             keep = []
-            if clc is not None:
+            if k1 == self.steps and tape["last"] is not None:
+                keep = tape["last"]
+            elif clc is not None:
                 # the checkpoint's force and clusters, as in the forward sweep
                 X, V = Xc.clone(), Vc.clone()
                 P.p3t_build_tree(self.ctx, self._state(X, V, m, r_out), False)
                 P.p3t_soft_force(self.ctx, self._state(X, V, m, r_out), self.acc)
                 self.cl = clc[1]
-                self._run(X, V, m, r_out, k0, k1, keep, have_force=True)
+                self._run(X, V, m, r_out, k0, k1, keep, have_force=True, whole=False)
             else:
-                self._run(Xc.clone(), Vc.clone(), m, r_out, k0, k1, keep)
+                self._run(Xc.clone(), Vc.clone(), m, r_out, k0, k1, keep, whole=False)
             for k in range(k1 - 1, k0 - 1, -1):
                 Xk, Vk, clk = keep[k - k0]
                 st = self._state(Xk, Vk, m, r_out)
@@ -196,7 +210,7 @@ class SoftKDK:
 class _KDK(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x0, v0, m, r_out, runner, r_search):
-        xN, vN, tape = runner.forward(x0, v0, m, r_out, r_search)
+        xN, vN, tape = runner._forward(x0, v0, m, r_out, r_search, any(ctx.needs_input_grad))
         ctx.runner, ctx.tape = runner, tape
         return xN, vN
 
