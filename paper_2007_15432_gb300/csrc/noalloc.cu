@@ -114,7 +114,9 @@ __device__ __forceinline__ int nz_bin(double R, double Rmin, double Rmax,
   if (Rmax > Rmin && R > Rmin) {
     const double t = (log(R) - lmin) / (lmax - lmin);
     const double f = floor(t * (double)nb);
-    k = f < 0.0 ? 0 : (f > (double)(nb - 1) ? nb - 1 : (int)f);
+    // a NaN (a particle on the axis: lmin is -infinity) takes bin 0; its
+    // conversion to int would be the smallest one
+    k = !(f >= 0.0) ? 0 : (f > (double)(nb - 1) ? nb - 1 : (int)f);
   }
   return k;
 }
