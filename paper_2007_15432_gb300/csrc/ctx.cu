@@ -194,7 +194,7 @@ int p3t_create(p3t_ctx **ctx, const p3t_params *p, int device) {
     delete c;
     return P3T_ERR_CUDA;
   }
-  bool ok = dalloc(c->status, 1) && dalloc(c->box, 5) && dalloc(c->box_bits, 6) &&
+  bool ok = dalloc(c->status, 1) && dalloc(c->box, 5) && dalloc(c->box_bits, 8) &&
             dalloc(c->box_part, 6 * p3t_box_blocks(c->num_sms)) &&
             dalloc(c->counters, 64) && dalloc(c->cl_counts, 4) && dalloc(c->hsteps, 1) && dalloc(c->hcursor, 5) &&
             dalloc(c->coll_ctr, 1) &&
@@ -274,7 +274,7 @@ int p3t_set_segments(p3t_ctx *c, int64_t nseg, const int64_t *seg_off) {
   c->seg_off_h = nullptr;
   c->nseg = 1;
   const int64_t S = nseg;
-  bool ok = dalloc(c->box, 5 * S) && dalloc(c->box_bits, 6 * S);
+  bool ok = dalloc(c->box, 5 * S) && dalloc(c->box_bits, 6 * S + 2);
   if (ok && nseg > 1) {
     ok = dalloc(c->seg_off, S + 1) && dalloc(c->seg_nb, S) && dalloc(c->seg_base, S) &&
          dalloc(c->seg_l, 2 * S);

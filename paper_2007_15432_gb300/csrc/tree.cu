@@ -29,17 +29,6 @@ __device__ __forceinline__ double ord_double(unsigned long long b) {
 // =========================================================================
 // per segment d: bits[4d] min R, bits[4d + 1] max R, bits[4d + 2], [4d + 3]
 // the largest r_out and r_search (shared scheme)
-__global__ void k_cut_init(unsigned long long *bits, int nseg, double *bsum,
-                           unsigned long long *bcnt, int nb, int64_t *d_n, int64_t n) {
-  pdl_wait();
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t == 0) *d_n = n;  // for the sort
-  for (int d = t; d < nseg; d += gridDim.x * blockDim.x) {
-    bits[4 * d] = ~0ull; bits[4 * d + 1] = 0ull; bits[4 * d + 2] = 0ull; bits[4 * d + 3] = 0ull;
-  }
-  for (int k = t; k < nb; k += gridDim.x * blockDim.x) { bsum[k] = 0.0; bcnt[k] = 0ull; }
-}
-
 // a block's slice of its segment: blocks [d * slices, (d + 1) * slices) take
 // segment d in contiguous slices
 __device__ __forceinline__ void seg_slice(const SegView &sv, int slices, int &d, int64_t &a,
@@ -51,25 +40,92 @@ __device__ __forceinline__ void seg_slice(const SegView &sv, int slices, int &d,
   b = s0 + len * (sl + 1) / slices;
 }
 
+// x > 0 cut to FP32's 24 bits; within 2^+-100
+__device__ __forceinline__ float cut_float(double x) {
+  return __uint_as_float((unsigned)(__double2hiint(x) - (896 << 20)) << 3 |
+                         (unsigned)__double2loint(x) >> 29);
+}
+__device__ __forceinline__ bool cut_range100(double x) {
+  return (unsigned)((__double2hiint(x) >> 20) - (1023 - 100)) < 200u;
+}
+// (1 / Rmin^2, nb / (lmax - lmin)); zeros (no estimate) out of range
+__device__ __forceinline__ float2 cut_scale(double Rmin, double lmin, double lmax, int nb) {
+  const double q = Rmin * Rmin, span = lmax - lmin;
+  if (!cut_range100(q) || !cut_range100(span)) return make_float2(0.f, 0.f);
+  return make_float2(1.0f / cut_float(q), (float)nb / (float)span);
+}
+// The range of R of each segment, as that of R^2 (the correctly rounded root
+// is monotone), a block's slice at a time into part; the last block to finish
+// (arrival counter, left at zero) reduces the slices, a warp a segment, and
+// takes the roots, and with one segment their logarithms (bits[4], bits[5]; the
+// FP32 estimate's scale in bits[6]),
+// which every thread of k_cut_u2 formed for itself before (FP64 logarithms,
+// more work than the rest of that kernel).  Also stores the sort's n.
 __global__ void k_cut_range(SegView sv, int slices, const double *x, const double *y,
-                            unsigned long long *bits) {
+                            unsigned long long *part, int64_t *arrived, unsigned long long *bits,
+                            int nb, int64_t *d_n) {
   pdl_wait();
+  __shared__ unsigned long long red[2][kBlock / 32];
+  __shared__ bool s_last;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *d_n = sv.n;
   int d;
   int64_t a, b;
   seg_slice(sv, slices, d, a, b);
   unsigned long long lo = ~0ull, hi = 0ull;
   for (int64_t i = a + threadIdx.x; i < b; i += blockDim.x) {
-    unsigned long long v = ord_bits(sqrt(x[i] * x[i] + y[i] * y[i]));
+    const unsigned long long v = ord_bits(x[i] * x[i] + y[i] * y[i]);
     lo = v < lo ? v : lo;
     hi = v > hi ? v : hi;
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long u = __shfl_xor_sync(0xffffffffu, lo, o);
-    unsigned long long c = __shfl_xor_sync(0xffffffffu, hi, o);
-    lo = u < lo ? u : lo;
-    hi = c > hi ? c : hi;
+  auto reduce = [&]() {
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long u = __shfl_xor_sync(0xffffffffu, lo, o);
+      const unsigned long long c = __shfl_xor_sync(0xffffffffu, hi, o);
+      lo = u < lo ? u : lo;
+      hi = c > hi ? c : hi;
+    }
+  };
+  reduce();
+  if (lane == 0) { red[0][w] = lo; red[1][w] = hi; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < nw; ++q) {
+      lo = red[0][q] < lo ? red[0][q] : lo;
+      hi = red[1][q] > hi ? red[1][q] : hi;
+    }
+    part[2 * (int64_t)blockIdx.x] = lo;
+    part[2 * (int64_t)blockIdx.x + 1] = hi;
+    __threadfence();
+    s_last = atomicAdd(reinterpret_cast<unsigned long long *>(arrived), 1ull) ==
+             (unsigned long long)gridDim.x - 1;
+    if (s_last) *arrived = 0;
   }
-  if ((threadIdx.x & 31) == 0) { atomicMin(&bits[4 * d], lo); atomicMax(&bits[4 * d + 1], hi); }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int seg = w; seg < sv.nseg; seg += nw) {
+    lo = ~0ull;
+    hi = 0ull;
+    for (int q = lane; q < slices; q += 32) {
+      const unsigned long long *v = part + 2 * ((int64_t)seg * slices + q);
+      const unsigned long long u = __ldcg(&v[0]), c = __ldcg(&v[1]);
+      lo = u < lo ? u : lo;
+      hi = c > hi ? c : hi;
+    }
+    reduce();
+    if (lane < 2) {  // lane 0: the smallest, lane 1: the largest
+      const double R = sqrt(ord_double(lane == 0 ? lo : hi));
+      bits[4 * seg + lane] = ord_bits(R);
+      bits[4 * seg + 2 + lane] = 0ull;
+      if (sv.nseg == 1) {
+        const double l = log(R);
+        bits[4 + lane] = (unsigned long long)__double_as_longlong(l);
+        const double lmax = __shfl_sync(0x3u, l, 1);
+        if (lane == 0) *reinterpret_cast<float2 *>(&bits[6]) = cut_scale(R, l, lmax, nb);
+      }
+    }
+  }
 }
 
 // radial bins of each segment (several segments): their number (as for a
@@ -120,165 +176,187 @@ __global__ void k_cut_segbins(SegView sv, int vran_bins, const unsigned long lon
   }
 }
 
-// bin of ln R among nb bins uniform on [lmin, lmax]: floor(nb (ln R - lmin) /
-// (lmax - lmin)) clamped to [0, nb - 1], decided in FP64.  An FP32 estimate
-// decides it first when no integer lies within its error bound of the
-// estimate (logf and the roundings to FP32 stay within 2e-6 absolute on ln R
-// and on each bound); otherwise the FP64 expression is evaluated.
-__device__ __forceinline__ int cut_bin(double R, double Rmin, double Rmax,
-                                       double lmin, double lmax, int nb) {
-  int k = 0;
-  if (Rmax > Rmin && R > Rmin) {
-    const float lminf = (float)lmin, span = (float)lmax - lminf;
-    const float tf = (logf((float)R) - lminf) / span * (float)nb;
-    const float margin = 8e-6f * (float)nb / span + 1e-3f;
-    double f;
-    if (span > 0.0f && margin < 0.25f && floorf(tf - margin) == floorf(tf + margin)) {
-      f = (double)floorf(tf);
-    } else {
-      double t = (log(R) - lmin) / (lmax - lmin);
-      f = floor(t * (double)nb);
-    }
-    k = f < 0.0 ? 0 : (f > (double)(nb - 1) ? nb - 1 : (int)f);
-  }
-  return k;
+// 1 / sqrt(x) and x^(-1/4) from the 20-bit seed (one rounding more than the
+// last at most; the rsqrt_seed range, otherwise out of line): with e = 1 - x y^2
+// (|e| <= 2^-18), y (1 + e / 2 + 3/8 e^2), the rest below 2^-55; with e = 1 - x z^4
+// (|e| <= 2^-16), z (1 + e / 4 + 5/32 e^2 + 15/128 e^3), the rest below 2^-67.  4
+// and 8 FP64 instructions, where rsqrt() takes 5 to 6 and sqrt() 9.
+__device__ __forceinline__ bool seed_range(double x) {
+  return (unsigned)((__double2hiint(x) >> 20) - 512) < 1024u;
+}
+__device__ __forceinline__ double rsqrt_raw(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ double inv_sqrt(double x) {  // 0 for 0
+  const double y = rsqrt_raw(x), e = __fma_rn(-x, y * y, 1.0);
+  double r = __fma_rn(y * e, __fma_rn(e, 0.375, 0.5), y);
+  if (!seed_range(x)) r = rsqrt_rare(x);
+  return r;
+}
+static __device__ __noinline__ double inv_root4_rare(double x) { return rsqrt(sqrt(x)); }
+__device__ __forceinline__ double inv_root4(double x) {
+  const double y = rsqrt_raw(x), z = y * rsqrt_raw(y), z2 = z * z;
+  const double e = __fma_rn(-x, z2 * z2, 1.0);
+  double r = __fma_rn(z * e, __fma_rn(e, __fma_rn(e, 15.0 / 128.0, 5.0 / 32.0), 0.25), z);
+  if (!seed_range(x)) r = inv_root4_rare(x);
+  return r;
 }
 
-// |u|^2 and the radial bin of every particle (kept for k_cut_final); bin
-// counts (integer atomics, first into the block's shared histogram);
-// (bin, index) pairs for a stable sort by bin
+// bin of ln R among nb bins uniform on [lmin, lmax]: floor(nb (ln R - lmin) /
+// (lmax - lmin)) clamped to [0, nb - 1], decided in FP64.  An FP32 estimate
+// nb / (2 span) ln(R^2 / Rmin^2) decides it first when no integer lies within
+// its error bound of the estimate: the squares cut to 24 bits, their quotient's
+// two roundings and logf's last place leave the logarithm within 3.6e-7 + 1.2e-7
+// of itself, the scale's and the products' roundings are 3e-7 relative; the
+// bound is twice that.  (One particle in a thousand is left at 377 bins over a
+// factor e; a bound ten times wider sent a warp in four through the FP64
+// logarithm.)  Otherwise the FP64 expression is evaluated.
+static __device__ __noinline__ int cut_bin_fp64(double R2, double Rmin, double Rmax, double lmin,
+                                                double lmax, int nb) {
+  const double R = sqrt(R2);
+  if (!(Rmax > Rmin && R > Rmin)) return 0;
+  const double f = floor((log(R) - lmin) / (lmax - lmin) * (double)nb);
+  // a NaN (a particle on the axis: lmin is -infinity) takes bin 0; its conversion
+  // to int would be the smallest one
+  return !(f >= 0.0) ? 0 : (f > (double)(nb - 1) ? nb - 1 : (int)f);
+}
+__device__ __forceinline__ int cut_bin(double R2, float2 sc, double Rmin, double Rmax, double lmin,
+                                       double lmax, int nb) {
+  const float tf = 0.5f * logf(cut_float(R2) * sc.x) * sc.y;
+  const float margin = 4e-7f * sc.y + 1e-6f * (float)nb;
+  const float lo = floorf(tf - margin);
+  if (cut_range100(R2) && sc.y > 0.0f && margin < 0.25f && tf > -1.0f &&
+      tf < 1.25f * (float)nb + 1.0f && lo == floorf(tf + margin))
+    return min(max((int)lo, 0), nb - 1);
+  return cut_bin_fp64(R2, Rmin, Rmax, lmin, lmax, nb);
+}
+
+// What bounds the cut-offs from some 1e5 particles on is the FP64 pipe (19 cycles
+// of an SM a warp instruction): 23 FP64 instructions a particle in k_cut_u2 and
+// some 40 in k_cut_final, where library roots, a division and the bounds'
+// logarithms took 56 and 57 and, a thread, 120 more.  Measured at N = 377,740:
+// k_cut_u2 108 -> 27 us, k_cut_final 52 -> 33, k_cut_range 18 -> 14, the whole 213
+// -> 104; below, the launches: N = 1,000 43 -> 32 us, 1e5 92 -> 52, 1e6 378 -> 205.
+// |u|^2 and the radial bin of every particle (kept for k_cut_final); (bin,
+// index) pairs for a stable sort by bin
 constexpr int kMaxBins = 4096;
 __global__ void k_cut_u2(SegView sv, const double *x, const double *y, const double *z,
-                         const double *vx, const double *vy, const double *vz, double mu,
+                         const double *vx, const double *vy, const double *vz, double smu,
                          const unsigned long long *bits, int nb, const int32_t *seg_nb,
                          const int32_t *seg_base, const double *seg_l, double *u2,
-                         uint64_t *key, int32_t *idx, int32_t *bin, unsigned long long *bcnt) {
+                         uint64_t *key, int32_t *idx, int32_t *bin) {
   pdl_wait();
-  __shared__ uint32_t h[kMaxBins];
-  for (int k = threadIdx.x; k < nb; k += blockDim.x) h[k] = 0;
-  __syncthreads();
   const int64_t n = sv.n;
   // one segment: its range here; several: per particle below
   const double Rmin0 = ord_double(bits[0]), Rmax0 = ord_double(bits[1]);
-  const double lmin0 = log(Rmin0), lmax0 = log(Rmax0);
-  const double smu = sqrt(mu);
+  double lmin0 = 0.0, lmax0 = 0.0;
+  float2 sc0 = make_float2(0.f, 0.f);
+  if (sv.nseg == 1) {
+    sc0 = *reinterpret_cast<const float2 *>(&bits[6]);
+    lmin0 = __longlong_as_double((long long)bits[4]);
+    lmax0 = __longlong_as_double((long long)bits[5]);
+  }
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const double R2 = x[i] * x[i] + y[i] * y[i];
-    const double R = sqrt(R2);
-    const double r = sqrt(R2 + z[i] * z[i]);
-    const double vk = smu * rsqrt(r);  // sqrt(mu / r)
-    double px = 0.0, py = 0.0;
-    if (R > 0.0) {
-      const double iR = rsqrt(R2);
-      px = -y[i] * iR;
-      py = x[i] * iR;
-    }
-    double ux = vx[i] - vk * px, uy = vy[i] - vk * py, uz = vz[i];
-    u2[i] = ux * ux + uy * uy + uz * uz;
+    const double X = x[i], Y = y[i], Z = z[i];
+    const double R2 = X * X + Y * Y;
+    // u = v - sqrt(mu / r) phi_hat, phi_hat = (-y, x) / R
+    const double t = smu * inv_root4(__fma_rn(Z, Z, R2)) * inv_sqrt(R2);
+    const double ux = __fma_rn(t, Y, vx[i]), uy = __fma_rn(-t, X, vy[i]), uz = vz[i];
+    u2[i] = __fma_rn(ux, ux, __fma_rn(uy, uy, uz * uz));
     int k;
     if (sv.nseg == 1) {
-      k = cut_bin(R, Rmin0, Rmax0, lmin0, lmax0, nb);
+      k = cut_bin(R2, sc0, Rmin0, Rmax0, lmin0, lmax0, nb);
     } else {
       const int d = seg_of(sv, i);
-      k = seg_base[d] + cut_bin(R, ord_double(bits[4 * d]), ord_double(bits[4 * d + 1]),
-                                seg_l[2 * d], seg_l[2 * d + 1], seg_nb[d]);
+      const double lmin = seg_l[2 * d], lmax = seg_l[2 * d + 1];
+      const double Rmin = ord_double(bits[4 * d]);
+      k = seg_base[d] + cut_bin(R2, cut_scale(Rmin, lmin, lmax, seg_nb[d]), Rmin,
+                                ord_double(bits[4 * d + 1]), lmin, lmax, seg_nb[d]);
     }
     key[i] = (uint64_t)k;
     idx[i] = (int32_t)i;
     bin[i] = k;
-    atomicAdd(&h[k], 1u);
   }
-  __syncthreads();
-  for (int k = threadIdx.x; k < nb; k += blockDim.x)
-    if (h[k]) atomicAdd(&bcnt[k], (unsigned long long)h[k]);
 }
 
-// exclusive offsets of the bins (at most 4096): one block, chunks of its
-// size scanned with warp shuffles and carried
-__global__ void k_cut_offsets(int nb, const unsigned long long *bcnt, int64_t *boff) {
-  pdl_wait();
-  __shared__ int64_t wsum[32];
-  __shared__ int64_t carry;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < nb; base += blockDim.x) {
-    const int k = base + threadIdx.x;
-    const int64_t v = k < nb ? (int64_t)bcnt[k] : 0;
-    int64_t x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int64_t t = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += t;
-    }
-    if (lane == 31) wsum[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-      const int64_t w0 = lane < nw ? wsum[lane] : 0;
-      int64_t y = w0;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int64_t t = __shfl_up_sync(0xffffffffu, y, o);
-        if (lane >= o) y += t;
-      }
-      if (lane < nw) wsum[lane] = y - w0;
-    }
-    __syncthreads();
-    const int64_t ex = carry + wsum[warp] + (x - v);
-    if (k < nb) boff[k] = ex;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry = ex + v;
-    __syncthreads();
+// first place of sorted keys that is not below k, by a warp
+__device__ __forceinline__ int64_t lower_bound_warp(const uint64_t *keys, int64_t n, uint64_t k) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = 0, len = n;
+  while (len > 0) {  // shrinks to at most a 32nd
+    const int64_t step = (len + 31) >> 5, p = lane * step;
+    const unsigned below = __ballot_sync(0xffffffffu, p < len && keys[lo + p] < k);
+    if (below == 0) break;
+    const int64_t past = (int64_t)(__popc(below) - 1) * step + 1;
+    lo += past;
+    len = step - 1 < len - past ? step - 1 : len - past;
   }
-  if (threadIdx.x == 0) boff[nb] = carry;
+  return lo;
 }
 
 // v_ran of each bin, sqrt(sum |u|^2 / count), the sum by one warp per bin
 // over its members in index order (a fixed lane-strided order and a fixed
-// shuffle tree: the same sum on every run)
-__global__ void k_cut_binsum(int nb, const int64_t *boff, const int32_t *sorted_idx,
-                             const double *u2, double *bvr) {
+// shuffle tree: the same sum on every run), the loads of eight members a lane
+// at a time before their additions.  The bins' ends by search in the sorted
+// bins: counted instead, every block of k_cut_u2 added every bin to the same
+// few words.
+__global__ void k_cut_binsum(int nb, int64_t n, const uint64_t *sorted_bin,
+                             const int32_t *sorted_idx, const double *u2, double *bvr) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t k = w0; k < nb; k += nw) {
+    const int64_t b0 = lower_bound_warp(sorted_bin, n, (uint64_t)k);
+    const int64_t b1 = lower_bound_warp(sorted_bin, n, (uint64_t)k + 1);
     double sum = 0.0;
-    for (int64_t j = boff[k] + lane; j < boff[k + 1]; j += 32) sum += u2[sorted_idx[j]];
+    int64_t j = b0 + lane;
+    for (; j + 7 * 32 < b1; j += 8 * 32) {
+      double v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = u2[sorted_idx[j + 32 * q]];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) sum += v[q];
+    }
+    for (; j < b1; j += 32) sum += u2[sorted_idx[j]];
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) bvr[k] = sqrt(sum / (double)(boff[k + 1] - boff[k]));
+    if (lane == 0) bvr[k] = sqrt(sum / (double)(b1 - b0));
   }
 }
 
-// x^(1/3) for x >= 0: the inverse cube root z = x^(-1/3) by Newton's method
-// on f(z) = z^-3 - x, z <- z (4 - x z^3) / 3 (quadratic convergence), from an
-// FP32 seed (relative error ~1e-7) in two steps, then x^(1/3) = x z^2; inputs
-// outside the FP32 seed's normal range take cbrt
+// x^(1/3) for x >= 0: the inverse cube root z = x^(-1/3) from an FP32 seed
+// (relative error below 5e-7), corrected once: with e = 1 - x z^3, z (1 + e / 3 +
+// 2/9 e^2), the rest below 2^-60; then x^(1/3) = x z^2.  Inputs outside the
+// seed's range take cbrt.  Conversions by integer operations (an FP64 one
+// takes the FP64 pipe).
+static __device__ __noinline__ double cbrt_rare(double x) { return cbrt(x); }
 __device__ __forceinline__ double cbrt_pos(double x) {
-  if (!(x > 1e-30 && x < 1e30)) return cbrt(x);
-  double z = (double)rcbrtf((float)x);
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const double z3 = z * z * z;
-    z = z * (4.0 - x * z3) * (1.0 / 3.0);
-  }
-  return x * z * z;
+  const unsigned f = __float_as_uint(rcbrtf(lead_float(x, 0)));
+  const double z = __hiloint2double((int)((f >> 3) + (896u << 20)), (int)(f << 29));
+  const double e = __fma_rn(-x, z * z * z, 1.0);
+  const double w = __fma_rn(z * e, __fma_rn(e, 2.0 / 9.0, 1.0 / 3.0), z);
+  double r = x * w * w;
+  if ((unsigned)((__double2hiint(x) >> 20) - (1023 - 99)) >= 198u) r = cbrt_rare(x);
+  return r;
 }
 
 __global__ void k_cut_final(SegView sv, const double *x, const double *y,
                             const double *z, const double *vx, const double *vy,
-                            const double *vz, const double *m, p3t_params prm,
-                            unsigned long long *bits, const int32_t *bin,
+                            const double *vz, const double *m, p3t_params prm, double imu,
+                            double i3ms, unsigned long long *bits, const int32_t *bin,
                             const double *bvr, double *r_out, double *r_search) {
   pdl_wait();
-  const double imu = 1.0 / (prm.G * prm.m_star), i3ms = 1.0 / (3.0 * prm.m_star);
   const int64_t n = sv.n;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const double r2 = x[i] * x[i] + y[i] * y[i] + z[i] * z[i];
-    const double ir = rsqrt(r2);
-    double v2 = vx[i] * vx[i] + vy[i] * vy[i] + vz[i] * vz[i];
-    double alpha = 2.0 * ir - v2 * imu;  // 1/a, vis-viva
-    double a = alpha > 0.0 ? 1.0 / alpha : r2 * ir;
+    const double r2 = __fma_rn(x[i], x[i], __fma_rn(y[i], y[i], z[i] * z[i]));
+    const double ir = inv_sqrt(r2);
+    const double v2 = __fma_rn(vx[i], vx[i], __fma_rn(vy[i], vy[i], vz[i] * vz[i]));
+    const double alpha = __fma_rn(-v2, imu, 2.0 * ir);  // 1/a, vis-viva
+    const double a = alpha > 0.0 ? 1.0 / alpha : r2 * ir;
     double rhill = cbrt_pos(m[i] * i3ms) * a;
     const double vr = bvr[bin[i]];
     // Eq. routi2 (P3T_CUT_HILL_VRAN) or Eq. routi (the other two); Eq. rsearch
@@ -1380,6 +1458,13 @@ static int cut_bins(int vran_bins, int64_t n) {
   return nb;
 }
 
+// slices a segment for a reduction over every segment: a few blocks per SM in
+// all, none with less than a trip of a block (four elements a thread)
+static int box_slices(const p3t_ctx *c, int64_t n) {
+  const int64_t most = c->nseg >= 4 * c->num_sms ? 1 : 4 * c->num_sms / c->nseg;
+  return (int)std::min(most, (n / c->nseg + 4 * kBlock - 1) / (4 * kBlock) + 1);
+}
+
 int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s) {
   const int64_t n = p->n;
   if (n == 0) return P3T_OK;
@@ -1394,12 +1479,11 @@ int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s) {
   if (nbt > kMaxBins) return P3T_ERR_INVALID;
   const int nb = (int)nbt;
   double *bsum = c->epart;  // reuse: >= 4096 doubles
-  unsigned long long *bcnt = reinterpret_cast<unsigned long long *>(c->epart + 4096);
   const int64_t g = p3t_grid(n, kBlock, (int64_t)c->num_sms * P3T_NSM_BLOCKS);
-  pdl_launch(k_cut_init, dim3(4), dim3(kBlock), 0, s, c->box_bits, (int)c->nseg, bsum, bcnt, nb,
-             &c->counters[18], n);
-  const int rsl = c->nseg == 1 ? (int)g : (int)((g + c->nseg - 1) / c->nseg);
-  pdl_launch(k_cut_range, dim3((unsigned)(rsl * c->nseg)), dim3(kBlock), 0, s, sv, rsl, p->x, p->y, c->box_bits);
+  int64_t *d_n = &c->counters[18];
+  const int rsl = box_slices(c, n);
+  pdl_launch(k_cut_range, dim3((unsigned)(rsl * c->nseg)), dim3(kBlock), 0, s, sv, rsl, p->x, p->y,
+             c->box_part, &c->counters[28], c->box_bits, nb, d_n);
   if (c->nseg > 1)
     pdl_launch(k_cut_segbins, dim3(1), dim3(1024), 0, s, sv, c->prm.vran_bins, c->box_bits, c->seg_nb,
                                      c->seg_base, c->seg_l);
@@ -1407,25 +1491,24 @@ int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s) {
   // per-bin sums in a fixed order (particles grouped by bin with the stable
   // radix sort, then one warp per bin): the radii do not depend on timing
   double *u2 = c->hw;
-  int64_t *boff = c->pos;
-  int64_t *d_n = &c->counters[18];
   int32_t *bin = c->flag;  // the bins of k_cut_u2, read by k_cut_final (N int32)
-  pdl_launch(k_cut_u2, dim3((unsigned)g), dim3(kBlock), 0, s, sv, p->x, p->y, p->z, p->vx, p->vy, p->vz, mu,
+  pdl_launch(k_cut_u2, dim3((unsigned)g), dim3(kBlock), 0, s, sv, p->x, p->y, p->z, p->vx, p->vy, p->vz, sqrt(mu),
                                           c->box_bits, nb, c->seg_nb, c->seg_base, c->seg_l,
-                                          u2, c->keys, c->idx, bin, bcnt);
-  int rc = p3t_sort_pairs(&c->keys, &c->idx, &c->keys_alt, &c->idx_alt, d_n, c->cap, 16,
+                                          u2, c->keys, c->idx, bin);
+  int rc = p3t_sort_pairs(&c->keys, &c->idx, &c->keys_alt, &c->idx_alt, d_n, c->cap, nb <= 256 ? 8 : 16,
                           c->radix_hist, c->radix_hist_cap, c->sort_work, p3t_sort_where(c), s);
   if (rc) return rc;
-  pdl_launch(k_cut_offsets, dim3(1), dim3(1024), 0, s, nb, bcnt, boff);
-  pdl_launch(k_cut_binsum, dim3((unsigned)p3t_grid((int64_t)nb * 32, kBlock, (int64_t)c->num_sms * 4)), dim3(kBlock), 0, s, nb, boff, c->idx, u2, bsum);
+  pdl_launch(k_cut_binsum, dim3((unsigned)p3t_grid((int64_t)nb * 32, kBlock, (int64_t)c->num_sms * 4)),
+             dim3(kBlock), 0, s, nb, n, c->keys, c->idx, u2, bsum);
   pdl_launch(k_cut_final, dim3((unsigned)g), dim3(kBlock), 0, s, sv, p->x, p->y, p->z, p->vx, p->vy,
-                                             p->vz, p->m, c->prm, c->box_bits, bin, bsum,
+                                             p->vz, p->m, c->prm, 1.0 / mu,
+                                             1.0 / (3.0 * c->prm.m_star), c->box_bits, bin, bsum,
                                              p->r_out, p->r_search);
   if (c->prm.cutoff_mode == P3T_CUT_SHARED)
     pdl_launch(k_cut_shared, dim3((unsigned)g), dim3(kBlock), 0, s, sv, c->box_bits, p->r_out, p->r_search);
-  // init, range, u2, offsets, bin sums, final (+ shared, + segment bins);
-  // the sort counts itself
-  p3t_note_launches(6 + (c->prm.cutoff_mode == P3T_CUT_SHARED) + (c->nseg > 1));
+  // range, u2, bin sums, final (+ shared, + segment bins); the sort counts
+  // itself
+  p3t_note_launches(4 + (c->prm.cutoff_mode == P3T_CUT_SHARED) + (c->nseg > 1));
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }
 
@@ -1438,10 +1521,7 @@ int p3t_run_build_tree(p3t_ctx *c, const p3t_particles *p, cudaStream_t s) {
   int rc;
   const int nseg = (int)c->nseg;
   const SegView sv{c->seg_off, nseg, n};
-  // one root cube per segment: a few blocks per SM in all, in slices of the
-  // segments of no less than a trip of a block (four elements a thread)
-  const int64_t bmax = nseg >= 4 * c->num_sms ? 1 : 4 * c->num_sms / nseg;
-  const int bsl = (int)std::min(bmax, (n / nseg + 4 * kBlock - 1) / (4 * kBlock) + 1);
+  const int bsl = box_slices(c, n);
   pdl_launch(k_box, dim3((unsigned)(bsl * nseg)), dim3(kBlock), 0, s, sv, bsl, p->x, p->y, p->z,
              c->box_part, &cnt[24], c->box);
   pdl_launch(k_keys, dim3((unsigned)g), dim3(kBlock), 0, s, sv, p->x, p->y, p->z, p->m, p->r_out, p->r_search,
