@@ -1460,7 +1460,8 @@ constexpr int64_t kEBlocks = 152 * 4 * 8;  // blocks asked for: eight waves of f
 // with 1 / r from the 20-bit seed.  Sources are staged by tile, a tile's sum
 // in FP32 (FP64) per target, the tiles' sums in float-float (FP64).  Measured
 // (one scalar target a thread over all sources before): mixed N = 1e5 11,640 ->
-// 3,490 us, 1e4 703 -> 72; FP64 N = 1e4 10,950 -> 1,330.
+// 2,790 us, 1e4 703 -> 69; FP64 N = 1e4 10,950 -> 1,330.  (rsqrtf's subnormal
+// scaling on every pair: 3,490 and 72.)
 template <bool MIXED>
 __global__ void __launch_bounds__(kEThreads) k_energy(p3t_particles p, p3t_params prm, int tiles,
                                                       int chunk, double *part) {
@@ -1539,7 +1540,9 @@ __global__ void __launch_bounds__(kEThreads) k_energy(p3t_particles p, p3t_param
           const f2 dz = add2(sub2(TZ, f2_dup(H.z)), sub2(TZL, f2_dup(L.z)));
           const f2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
           const float ra = f2_lo(r2), rb = f2_hi(r2);
-          const f2 ri = f2_pk(ra > 0.f ? rsqrtf(ra) : 0.f, rb > 0.f ? rsqrtf(rb) : 0.f);
+          f2 ri = f2_pk(rsqrt_normal(ra), rsqrt_normal(rb));
+          if (!(ra >= 1.17549435e-38f && rb >= 1.17549435e-38f))  // zero or subnormal
+            ri = f2_pk(ra > 0.f ? rsqrtf(ra) : 0.f, rb > 0.f ? rsqrtf(rb) : 0.f);
           // one Newton step
           const f2 c = fma2(mul2(f2_dup(-0.5f), r2), mul2(ri, ri), f2_dup(1.5f));
           b = fma2(f2_dup(H.w), mul2(ri, c), b);
