@@ -1405,12 +1405,14 @@ static WalkArgs walk_args(p3t_ctx *c, const p3t_particles *p) {
 constexpr int kFewTargets = 200;
 
 // The FP64 walks' chunk of targets: up to kChunk at a time (one traversal
-// serves them all), fewer while a warp would get less than four chunks, so
-// that small systems fill the card (N = 1,000: chunks of one target; from
-// about 100,000 particles on the largest)
+// serves them all, and in the VJP one set of atomics a node), fewer while a
+// warp would get less than two chunks, so that small systems fill the card (N =
+// 1,000: chunks of one target; from about 50,000 particles on the largest).
+// Force / VJP with at least two, four and one chunk a warp: N = 1e4 216 / 461,
+// 229 / 522, 223 / 435 us; 3e4 724 / 1,573, 716 / 1,593, 794 / 1,611
 static int walk64_chunk(const p3t_ctx *c, unsigned blocks) {
   int ct = kChunk;
-  while (ct > 1 && c->last_n < (int64_t)4 * ct * blocks * kWarps) ct >>= 1;
+  while (ct > 1 && c->last_n < (int64_t)2 * ct * blocks * kWarps) ct >>= 1;
   return ct;
 }
 // their blocks per SM: kWalk64Blocks (12 warps hold the FP64 pipe busy through
