@@ -196,6 +196,8 @@ int p3t_create(p3t_ctx **ctx, const p3t_params *p, int device) {
   }
   bool ok = dalloc(c->status, 1) && dalloc(c->box, 5) && dalloc(c->box_bits, 8) &&
             dalloc(c->box_part, 6 * p3t_box_blocks(c->num_sms)) &&
+            dalloc(c->seg_done, P3T_MAX_SEGMENTS) &&
+            cudaMemset(c->seg_done, 0, P3T_MAX_SEGMENTS * sizeof(uint32_t)) == cudaSuccess &&
             dalloc(c->counters, 64) && dalloc(c->cl_counts, 4) && dalloc(c->hsteps, 1) && dalloc(c->hcursor, 5) &&
             dalloc(c->coll_ctr, 1) &&
             dalloc(c->epart, 8192) && dalloc(c->bh_table, 32) &&
@@ -225,7 +227,8 @@ void p3t_destroy(p3t_ctx *c) {
   DeviceGuard g(c->device);
   cudaDeviceSynchronize();
   free_particle_buffers(c);
-  dfree(c->status); dfree(c->box); dfree(c->box_bits); dfree(c->box_part); dfree(c->counters);
+  dfree(c->status); dfree(c->box); dfree(c->box_bits); dfree(c->box_part); dfree(c->seg_done);
+  dfree(c->counters);
   dfree(c->seg_off); dfree(c->seg_nb); dfree(c->seg_base); dfree(c->seg_l);
   delete[] c->seg_off_h;
   dfree(c->cl_counts); dfree(c->hsteps); dfree(c->hcursor); dfree(c->epart);
@@ -285,6 +288,9 @@ int p3t_set_segments(p3t_ctx *c, int64_t nseg, const int64_t *seg_off) {
       c->seg_off_h = new (std::nothrow) int64_t[S + 1];
       ok = c->seg_off_h != nullptr;
       if (ok) for (int64_t d = 0; d <= S; ++d) c->seg_off_h[d] = seg_off[d];
+      c->seg_max = 0;
+      for (int64_t d = 0; d < S; ++d)
+        if (seg_off[d + 1] - seg_off[d] > c->seg_max) c->seg_max = seg_off[d + 1] - seg_off[d];
     }
   }
   if (!ok) {

@@ -215,6 +215,7 @@ struct p3t_ctx {
   int64_t nseg = 1;
   int64_t *seg_off = nullptr;      // device, nseg + 1 offsets
   int64_t *seg_off_h = nullptr;    // host copy
+  int64_t seg_max = 0;             // longest segment (several segments)
   int32_t *seg_nb = nullptr;       // device, radial bins of each segment (cut-offs)
   int32_t *seg_base = nullptr;     //   and the first global bin of each
   double *seg_l = nullptr;         //   log R_min, log R_max of each (2 nseg)
@@ -242,6 +243,7 @@ struct p3t_ctx {
   // root box {x0, y0, z0, L} and scalar counters
   double *box = nullptr;
   unsigned long long *box_bits = nullptr;  // the cut-off stage's ordered-bits min/max
+  uint32_t *seg_done = nullptr;            // blocks done, a segment (left at zero)
   unsigned long long *box_part = nullptr;  // the root cubes' partial min/max, six a block
   int64_t *counters = nullptr;             // misc device counters [64]
 
@@ -418,6 +420,13 @@ bool p3t_sort_prepare();
 int p3t_sort_pairs(uint64_t **keys, int32_t **vals, uint64_t **keys_alt, int32_t **vals_alt,
                    const int64_t *d_n, int64_t n_cap, int key_bits, uint32_t *hist,
                    int64_t hist_cap, void *work, uint32_t *where, cudaStream_t s);
+
+// Sort by (key, val) within each segment, the longest of seg_max entries (at
+// most P3T_SORT_SEGMENT); keys and vals stay in their buffers.
+constexpr int P3T_SORT_SEGMENT = 2 * P3T_SORT_BLOCK;
+int p3t_sort_segments(const SegView &sv, uint64_t *keys, int32_t *vals, uint64_t *keys_alt,
+                      int32_t *vals_alt, int64_t seg_max, int64_t n_cap, int key_bits,
+                      cudaStream_t s);
 
 // most blocks of the root cube reduction: four an SM, or one a segment
 static inline int64_t p3t_box_blocks(int num_sms) {

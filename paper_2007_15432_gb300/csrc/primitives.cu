@@ -769,6 +769,36 @@ __global__ void __launch_bounds__(kClassThreads) k_sort_move(const uint64_t *key
     }
 }
 
+// merges runs of r of the n entries of (ik, iv) into runs of 2 r of (ok, ov);
+// thread t of nt takes the outputs from kItems t on
+__device__ void merge_round(const uint64_t *ik, const int32_t *iv, uint64_t *ok, int32_t *ov, int n,
+                            int r, int t, int nt) {
+  for (int o = t * kItems; o < n; o += nt * kItems) {
+    // a thread's outputs may cross into the next pair of runs
+    int base = -1, ia = 0, ib = 0, a1 = 0, b1 = 0;
+    for (int q = 0; q < kItems && o + q < n; ++q) {
+      const int nb = (o + q) / (2 * r) * (2 * r);
+      if (nb != base) {
+        base = nb;
+        const int diag = o + q - base;
+        a1 = min(base + r, n);
+        b1 = min(base + 2 * r, n);
+        int lo = max(0, diag - (b1 - a1)), hi = min(diag, a1 - base);
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1, pa = base + mid, pb = a1 + diag - 1 - mid;
+          if (pair_less(ik[pa], iv[pa], ik[pb], iv[pb])) lo = mid + 1; else hi = mid;
+        }
+        ia = base + lo;
+        ib = a1 + diag - lo;
+      }
+      const bool ta = ib >= b1 || (ia < a1 && pair_less(ik[ia], iv[ia], ik[ib], iv[ib]));
+      const int f = ta ? ia++ : ib++;
+      ok[o + q] = ik[f];
+      ov[o + q] = iv[f];
+    }
+  }
+}
+
 // a bucket a block, from (ik, iv) into (ok, ov); one that does not fit (rare)
 // is sorted in runs that do, the runs then merged through global memory
 __global__ void __launch_bounds__(kLocalThreads, 3) k_sort_local(uint64_t *ik, int32_t *iv,
@@ -795,26 +825,52 @@ __global__ void __launch_bounds__(kLocalThreads, 3) k_sort_local(uint64_t *ik, i
     __threadfence_block();
     __syncthreads();
     // runs of r in (ok, ov) merged into (ik, iv), then copied back
-    for (int o = threadIdx.x * kItems; o < n; o += kLocalThreads * kItems) {
-      const int base = o / (2 * r) * (2 * r), diag = o - base;
-      const int a1 = min(base + r, n), b1 = min(base + 2 * r, n);
-      int lo = max(0, diag - (b1 - a1)), hi = min(diag, a1 - base);
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1, pa = base + mid, pb = a1 + diag - 1 - mid;
-        if (pair_less(ok[pa], ov[pa], ok[pb], ov[pb])) lo = mid + 1; else hi = mid;
-      }
-      int ia = base + lo, ib = a1 + diag - lo;
-      for (int q = 0; q < kItems && o + q < b1; ++q) {
-        const bool ta = ib >= b1 || (ia < a1 && pair_less(ok[ia], ov[ia], ok[ib], ov[ib]));
-        const int f = ta ? ia++ : ib++;
-        ik[o + q] = ok[f];
-        iv[o + q] = ov[f];
-      }
-    }
+    merge_round(ok, ov, ik, iv, n, r, threadIdx.x, kLocalThreads);
     __threadfence_block();
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += kLocalThreads) { ok[i] = ik[i]; ov[i] = iv[i]; }
   }
+}
+
+// Entries of several systems, each segment's (at most P3T_SORT_SEGMENT) sorted
+// by (key, value): one, two or four runs of equal length, a run a block, then
+// merged pairwise.  The runs start in the buffer from which the merges end in
+// (keys, vals).
+__device__ __forceinline__ int segment_runs(int n) {
+  return n <= kLocalMax ? 1 : (n <= 2 * kLocalMax ? 2 : 4);
+}
+__global__ void __launch_bounds__(kLocalThreads, 3) k_sort_runs(SegView seg, uint64_t *keys,
+                                                             int32_t *vals, uint64_t *tk,
+                                                             int32_t *tv, int kb, int vb) {
+  pdl_wait();
+  extern __shared__ __align__(16) unsigned char sort_mem[];
+  uint64_t *sk = reinterpret_cast<uint64_t *>(sort_mem);
+  int32_t *sv = reinterpret_cast<int32_t *>(sk + kLocalMax + kLocalMax / 8);
+  const int d = blockIdx.x >> 2, q = blockIdx.x & 3;
+  const int64_t s0 = seg_lo(seg, d);
+  const int n = (int)(seg_hi(seg, d) - s0), runs = segment_runs(n);
+  if (q >= runs) return;
+  const int r = (n + runs - 1) / runs, n0 = q * r, len = min(r, n - n0);
+  const int64_t o = s0 + n0;
+  sort_entries(keys + o, vals + o, (runs == 2 ? tk : keys) + o, (runs == 2 ? tv : vals) + o, len, 0,
+               kb, vb, sk, sv);
+}
+// the first merges of four runs (keys -> tk), or the last ones (tk -> keys)
+constexpr int kMergeThreads = 256, kMergeBlocks = P3T_SORT_SEGMENT / (kMergeThreads * kItems);
+__global__ void __launch_bounds__(kMergeThreads) k_merge_runs(SegView seg, uint64_t *keys,
+                                                              int32_t *vals, uint64_t *tk,
+                                                              int32_t *tv, bool last) {
+  pdl_wait();
+  const int d = blockIdx.x / kMergeBlocks, q = blockIdx.x % kMergeBlocks;
+  const int64_t s0 = seg_lo(seg, d);
+  const int n = (int)(seg_hi(seg, d) - s0), runs = segment_runs(n);
+  if (runs < (last ? 2 : 4)) return;
+  const int r = (n + runs - 1) / runs, t = q * kMergeThreads + threadIdx.x;
+  constexpr int nt = kMergeBlocks * kMergeThreads;
+  if (last)
+    merge_round(tk + s0, tv + s0, keys + s0, vals + s0, n, runs == 4 ? 2 * r : r, t, nt);
+  else
+    merge_round(keys + s0, vals + s0, tk + s0, tv + s0, n, r, t, nt);
 }
 
 }  // namespace
@@ -887,6 +943,7 @@ static bool sort_attr(const void *f, size_t bytes) {
 bool p3t_sort_prepare() {
   return sort_attr((const void *)k_sort_block, sort_smem(kBlockSortMax)) &&
          sort_attr((const void *)k_sort_sample, sort_smem(kBlockSortMax)) &&
+         sort_attr((const void *)k_sort_runs, sort_smem(kLocalMax)) &&
          sort_attr((const void *)k_sort_local, sort_smem(kLocalMax));
 }
 
@@ -920,5 +977,20 @@ int p3t_sort_pairs(uint64_t **keys, int32_t **vals, uint64_t **keys_alt, int32_t
   pdl_launch(k_sort_local, dim3((unsigned)buckets), dim3(kLocalThreads), sort_smem(kLocalMax), s,
              *keys_alt, *vals_alt, *keys, *vals, buckets, key_bits, vb, w);
   p3t_note_launches(4);
+  return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
+}
+
+int p3t_sort_segments(const SegView &sv, uint64_t *keys, int32_t *vals, uint64_t *keys_alt,
+                      int32_t *vals_alt, int64_t seg_max, int64_t n_cap, int key_bits, cudaStream_t s) {
+  int vb = 1;  // bits of a value below n_cap
+  while (vb < 31 && ((int64_t)1 << vb) < n_cap) ++vb;
+  pdl_launch(k_sort_runs, dim3((unsigned)sv.nseg * 4), dim3(kLocalThreads), sort_smem(kLocalMax), s,
+             sv, keys, vals, keys_alt, vals_alt, key_bits, vb);
+  for (int last = seg_max > 2 * kLocalMax ? 0 : 1; last < 2 && seg_max > kLocalMax; ++last) {
+    pdl_launch(k_merge_runs, dim3((unsigned)sv.nseg * kMergeBlocks), dim3(kMergeThreads), 0, s, sv,
+               keys, vals, keys_alt, vals_alt, last == 1);
+    p3t_note_launches(1);
+  }
+  p3t_note_launches(1);
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }

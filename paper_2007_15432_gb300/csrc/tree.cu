@@ -55,14 +55,14 @@ __device__ __forceinline__ float2 cut_scale(double Rmin, double lmin, double lma
   return make_float2(1.0f / cut_float(q), (float)nb / (float)span);
 }
 // The range of R of each segment, as that of R^2 (the correctly rounded root
-// is monotone), a block's slice at a time into part; the last block to finish
-// (arrival counter, left at zero) reduces the slices, a warp a segment, and
-// takes the roots, and with one segment their logarithms (bits[4], bits[5]; the
-// FP32 estimate's scale in bits[6]),
-// which every thread of k_cut_u2 formed for itself before (FP64 logarithms,
-// more work than the rest of that kernel).  Also stores the sort's n.
+// is monotone), a block's slice at a time into part; the last block of a
+// segment to finish (done, left at zero) reduces the slices and takes the
+// roots, and with one segment their logarithms (bits[4], bits[5]; the FP32
+// estimate's scale in bits[6]), which every thread of k_cut_u2 formed for itself
+// before (FP64 logarithms, more work than the rest of that kernel).  Also
+// stores the sort's n.
 __global__ void k_cut_range(SegView sv, int slices, const double *x, const double *y,
-                            unsigned long long *part, int64_t *arrived, unsigned long long *bits,
+                            unsigned long long *part, uint32_t *done, unsigned long long *bits,
                             int nb, int64_t *d_n) {
   pdl_wait();
   __shared__ unsigned long long red[2][kBlock / 32];
@@ -97,18 +97,17 @@ __global__ void k_cut_range(SegView sv, int slices, const double *x, const doubl
     part[2 * (int64_t)blockIdx.x] = lo;
     part[2 * (int64_t)blockIdx.x + 1] = hi;
     __threadfence();
-    s_last = atomicAdd(reinterpret_cast<unsigned long long *>(arrived), 1ull) ==
-             (unsigned long long)gridDim.x - 1;
-    if (s_last) *arrived = 0;
+    s_last = atomicAdd(&done[d], 1u) == (unsigned)slices - 1;
+    if (s_last) done[d] = 0;
   }
   __syncthreads();
-  if (!s_last) return;
+  if (!s_last || threadIdx.x >= 32) return;
   __threadfence();
-  for (int seg = w; seg < sv.nseg; seg += nw) {
+  {
     lo = ~0ull;
     hi = 0ull;
     for (int q = lane; q < slices; q += 32) {
-      const unsigned long long *v = part + 2 * ((int64_t)seg * slices + q);
+      const unsigned long long *v = part + 2 * ((int64_t)d * slices + q);
       const unsigned long long u = __ldcg(&v[0]), c = __ldcg(&v[1]);
       lo = u < lo ? u : lo;
       hi = c > hi ? c : hi;
@@ -116,8 +115,8 @@ __global__ void k_cut_range(SegView sv, int slices, const double *x, const doubl
     reduce();
     if (lane < 2) {  // lane 0: the smallest, lane 1: the largest
       const double R = sqrt(ord_double(lane == 0 ? lo : hi));
-      bits[4 * seg + lane] = ord_bits(R);
-      bits[4 * seg + 2 + lane] = 0ull;
+      bits[4 * d + lane] = ord_bits(R);
+      bits[4 * d + 2 + lane] = 0ull;
       if (sv.nseg == 1) {
         const double l = log(R);
         bits[4 + lane] = (unsigned long long)__double_as_longlong(l);
@@ -392,12 +391,12 @@ __global__ void k_cut_shared(SegView sv, const unsigned long long *bits, double 
 // Keys, sort, octree, moments.
 // =========================================================================
 // min / max of the positions of each segment: warp and block reductions over
-// a block's slice of its segment into part; the last block to finish (arrival
-// counter, left at zero) reduces the slices of each segment, a warp a segment,
-// to its root cube: corner at the per-axis minimum, side = largest extent;
-// box[5 d ..]: corner, side L, quantisation scale S
+// a block's slice of its segment into part; the last block of a segment to
+// finish (done, left at zero) reduces the slices to its root cube: corner at
+// the per-axis minimum, side = largest extent; box[5 d ..]: corner, side L,
+// quantisation scale S
 __global__ void k_box(SegView sv, int slices, const double *x, const double *y,
-                      const double *z, unsigned long long *part, int64_t *arrived, double *box5) {
+                      const double *z, unsigned long long *part, uint32_t *done, double *box5) {
   pdl_wait();
   __shared__ unsigned long long red[6][kBlock / 32];
   __shared__ bool s_last;
@@ -445,18 +444,17 @@ __global__ void k_box(SegView sv, int slices, const double *x, const double *y,
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    s_last = atomicAdd(reinterpret_cast<unsigned long long *>(arrived), 1ull) ==
-             (unsigned long long)gridDim.x - 1;
-    if (s_last) *arrived = 0;
+    s_last = atomicAdd(&done[d], 1u) == (unsigned)slices - 1;
+    if (s_last) done[d] = 0;
   }
   __syncthreads();
-  if (!s_last) return;
+  if (!s_last || threadIdx.x >= 32) return;
   __threadfence();
-  const int lane = threadIdx.x & 31;
-  for (int seg = threadIdx.x >> 5; seg < sv.nseg; seg += blockDim.x >> 5) {
+  const int lane = threadIdx.x;
+  {
     unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0ull, 0ull, 0ull};
     for (int q = lane; q < slices; q += 32) {
-      const unsigned long long *v = part + 6 * ((int64_t)seg * slices + q);
+      const unsigned long long *v = part + 6 * ((int64_t)d * slices + q);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const unsigned long long l = __ldcg(&v[a]), h = __ldcg(&v[3 + a]);
@@ -473,7 +471,7 @@ __global__ void k_box(SegView sv, int slices, const double *x, const double *y,
         mx[a] = h > mx[a] ? h : mx[a];
       }
     if (lane == 0) {
-      double *box = box5 + 5 * seg;
+      double *box = box5 + 5 * d;
       double lo0[3], hi0[3];
       for (int a = 0; a < 3; ++a) { lo0[a] = ord_double(mn[a]); hi0[a] = ord_double(mx[a]); }
       double L = fmax(hi0[0] - lo0[0], fmax(hi0[1] - lo0[1], hi0[2] - lo0[2]));
@@ -1458,11 +1456,14 @@ static int cut_bins(int vran_bins, int64_t n) {
   return nb;
 }
 
-// slices a segment for a reduction over every segment: a few blocks per SM in
-// all, none with less than a trip of a block (four elements a thread)
+// slices a segment for a reduction over every segment, none with less than a
+// trip of a block (four elements a thread): of one system a few blocks per SM
+// in all, of several as many as the longest one asks for (two slices a segment
+// of 518 to 16,296 particles: 60 us for the root cubes, 27 now)
 static int box_slices(const p3t_ctx *c, int64_t n) {
-  const int64_t most = c->nseg >= 4 * c->num_sms ? 1 : 4 * c->num_sms / c->nseg;
-  return (int)std::min(most, (n / c->nseg + 4 * kBlock - 1) / (4 * kBlock) + 1);
+  const int64_t most = c->nseg == 1 ? 4 * c->num_sms : p3t_box_blocks(c->num_sms) / c->nseg;
+  const int64_t len = c->nseg == 1 ? n : c->seg_max;
+  return (int)std::min(most, (len + 4 * kBlock - 1) / (4 * kBlock) + 1);
 }
 
 int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s) {
@@ -1483,7 +1484,7 @@ int p3t_run_cutoffs(p3t_ctx *c, p3t_particles *p, cudaStream_t s) {
   int64_t *d_n = &c->counters[18];
   const int rsl = box_slices(c, n);
   pdl_launch(k_cut_range, dim3((unsigned)(rsl * c->nseg)), dim3(kBlock), 0, s, sv, rsl, p->x, p->y,
-             c->box_part, &c->counters[28], c->box_bits, nb, d_n);
+             c->box_part, c->seg_done, c->box_bits, nb, d_n);
   if (c->nseg > 1)
     pdl_launch(k_cut_segbins, dim3(1), dim3(1024), 0, s, sv, c->prm.vran_bins, c->box_bits, c->seg_nb,
                                      c->seg_base, c->seg_l);
@@ -1523,13 +1524,22 @@ int p3t_run_build_tree(p3t_ctx *c, const p3t_particles *p, cudaStream_t s) {
   const SegView sv{c->seg_off, nseg, n};
   const int bsl = box_slices(c, n);
   pdl_launch(k_box, dim3((unsigned)(bsl * nseg)), dim3(kBlock), 0, s, sv, bsl, p->x, p->y, p->z,
-             c->box_part, &cnt[24], c->box);
+             c->box_part, c->seg_done, c->box);
   pdl_launch(k_keys, dim3((unsigned)g), dim3(kBlock), 0, s, sv, p->x, p->y, p->z, p->m, p->r_out, p->r_search,
                                         c->box, c->keys, c->idx, c->pack, 0, &cnt[0]);
-  rc = p3t_sort_pairs(&c->keys, &c->idx, &c->keys_alt, &c->idx_alt, &cnt[0], c->cap, 63,
-                      c->radix_hist, c->radix_hist_cap, c->sort_work, p3t_sort_where(c), s);
+  // several systems of which none is above P3T_SORT_SEGMENT are sorted apart: 256
+  // disks of 518 to 16,296 particles 99 us of kernels, one sort of all with a
+  // pass by segment and the keys anew 204.  Above, a segment's merges would be
+  // more rounds over memory than the one sort's passes
+  const bool apart = nseg > 1 && c->seg_max <= P3T_SORT_SEGMENT;
+  if (apart)
+    rc = p3t_sort_segments(sv, c->keys, c->idx, c->keys_alt, c->idx_alt, c->seg_max, c->cap, 63,
+                           s);
+  else
+    rc = p3t_sort_pairs(&c->keys, &c->idx, &c->keys_alt, &c->idx_alt, &cnt[0], c->cap, 63,
+                        c->radix_hist, c->radix_hist_cap, c->sort_work, p3t_sort_where(c), s);
   if (rc) return rc;
-  if (nseg > 1) {
+  if (nseg > 1 && !apart) {
     // stable sort by segment (the most significant digit of (segment, key)),
     // then the keys of the new order
     int sbits = 0;
