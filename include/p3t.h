@@ -188,7 +188,7 @@ int p3t_cutoffs(p3t_ctx *ctx, p3t_particles *p, void *stream);
  *  - Runs on the CURRENT CUDA device; all particle pointers must be on it.
  *    p and *p are host memory; the arrays they point to are device memory
  *    owned by the caller (inputs x..m are read, r_out and r_search written).
- *  - Scratch: a fixed 98,320-byte array in device memory that every GPU
+ *  - Scratch: a fixed 98,368-byte array in device memory that every GPU
  *    loading the library holds until the process exits; at most 4096 radial
  *    bins (prm->vran_bins > 4096 returns P3T_ERR_INVALID; the automatic choice
  *    is at most 1024).  Each call clears what it uses before use.

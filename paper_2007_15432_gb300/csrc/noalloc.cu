@@ -21,24 +21,32 @@
 // to a multiple of 2^-88 (|u|^2 < 2^40 assumed; a larger term saturates) and
 // added as a 128-bit integer, so the order in which threads add them does not
 // matter and every run gives the same bits.
+//
+// Bound by the FP64 pipe like the context's kernels, whose arithmetic it shares
+// (cutoff_math.cuh); the range's logarithms and each bin's v_ran are formed once,
+// by the last block of the kernel before, where every thread formed them:
+// N = 1,000 61 -> 47 us, 1e5 106 -> 45, 1e6 623 -> 208.
 #include <math.h>
 
 #include <mutex>
 
+#include "cutoff_math.cuh"
 #include "p3t_internal.cuh"
 
 namespace {
 
 constexpr int kMaxBins = 4096;           // largest vran_bins this entry point accepts
-// range bits, 128-bit bin sums (low and high words), bin counts
-constexpr int kScratchWords = 2 + 3 * kMaxBins;
+// range bits, 128-bit bin sums (low and high words), bin counts, and the six
+// words from kExtra on
+constexpr int kExtra = 2 + 3 * kMaxBins;
+constexpr int kScratchWords = kExtra + 6;
 constexpr int kSharedBins = 2048;        // bins summed per block in shared memory first
 constexpr int kMaxDevices = 64;
 constexpr int kBlock = 256;
 
 }  // namespace
 
-// 16 + 3 * 4096 * 8 = 98,320 bytes per device
+// 16 + 3 * 4096 * 8 + 48 = 98,368 bytes per device
 static __device__ __align__(256) unsigned long long p3t_noalloc_scratch[kScratchWords];
 
 namespace {
@@ -79,10 +87,13 @@ __device__ __forceinline__ double nz_ord_double(unsigned long long b) {
 
 // scratch layout: [0] min and [1] max of R_cyl (ordered bits), then per bin
 // the low words [2, 2 + nb) and high words [2 + kMaxBins, ...) of the
-// fixed-point sums of |u|^2, and the counts [2 + 2 kMaxBins, ...)
+// fixed-point sums of |u|^2 (the low ones hold v_ran once all are in), and the
+// counts [2 + 2 kMaxBins, ...); from kExtra on: the blocks done in nz_range and
+// nz_bins, R's bounds, their logarithms' bits [2], [3], the FP32 estimate's
+// scale [4]
 __global__ void nz_clear(unsigned long long *sc, int nb) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t == 0) { sc[0] = ~0ull; sc[1] = 0ull; }
+  if (t == 0) { sc[0] = ~0ull; sc[1] = 0ull; sc[kExtra] = sc[kExtra + 1] = 0ull; }
   for (int k = t; k < nb; k += gridDim.x * blockDim.x) {
     sc[2 + k] = 0ull;
     sc[2 + kMaxBins + k] = 0ull;
@@ -90,12 +101,25 @@ __global__ void nz_clear(unsigned long long *sc, int nb) {
   }
 }
 
-__global__ void nz_range(int64_t n, const double *x, const double *y,
+// whether this is the last of the grid's blocks to call this (one word, cleared
+// before; no shared memory: the bins may take all of a block's default share)
+__device__ __forceinline__ bool nz_last(unsigned long long *done) {
+  __threadfence();
+  __syncthreads();
+  const bool last = __syncthreads_or(
+      threadIdx.x == 0 && atomicAdd(done, 1ull) == (unsigned long long)gridDim.x - 1);
+  __threadfence();
+  return last;
+}
+
+// R's range as that of R^2 (the correctly rounded root is monotone); the last
+// block takes the roots and their logarithms, once
+__global__ void nz_range(int64_t n, const double *x, const double *y, int nb,
                          unsigned long long *sc) {
   unsigned long long lo = ~0ull, hi = 0ull;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long b = nz_ord_bits(sqrt(x[i] * x[i] + y[i] * y[i]));
+    const unsigned long long b = nz_ord_bits(x[i] * x[i] + y[i] * y[i]);
     lo = b < lo ? b : lo;
     hi = b > hi ? b : hi;
   }
@@ -106,31 +130,33 @@ __global__ void nz_range(int64_t n, const double *x, const double *y,
     hi = c > hi ? c : hi;
   }
   if ((threadIdx.x & 31) == 0) { atomicMin(&sc[0], lo); atomicMax(&sc[1], hi); }
+  if (!nz_last(&sc[kExtra]) || threadIdx.x >= 2) return;
+  const int t = threadIdx.x;
+  const double R = sqrt(nz_ord_double(__ldcg(&sc[t]))), l = log(R);
+  __syncwarp(3u);
+  sc[t] = nz_ord_bits(R);
+  sc[kExtra + 2 + t] = (unsigned long long)__double_as_longlong(l);
+  const double lmax = __shfl_sync(3u, l, 1);
+  if (t == 0) *reinterpret_cast<float2 *>(&sc[kExtra + 4]) = cut_scale(R, l, lmax, nb);
 }
 
-__device__ __forceinline__ int nz_bin(double R, double Rmin, double Rmax,
-                                      double lmin, double lmax, int nb) {
-  int k = 0;
-  if (Rmax > Rmin && R > Rmin) {
-    const double t = (log(R) - lmin) / (lmax - lmin);
-    const double f = floor(t * (double)nb);
-    // a NaN (a particle on the axis: lmin is -infinity) takes bin 0; its
-    // conversion to int would be the smallest one
-    k = !(f >= 0.0) ? 0 : (f > (double)(nb - 1) ? nb - 1 : (int)f);
-  }
-  return k;
+__device__ __forceinline__ int nz_bin(double R2, const unsigned long long *sc, int nb) {
+  return cut_bin(R2, *reinterpret_cast<const float2 *>(&sc[kExtra + 4]), nz_ord_double(sc[0]),
+                 nz_ord_double(sc[1]), __longlong_as_double((long long)sc[kExtra + 2]),
+                 __longlong_as_double((long long)sc[kExtra + 3]), nb);
 }
 
-// t >= 0 as a 128-bit count of 2^-88 (truncated; saturated at 2^128 - 1):
-// the high word is floor(t 2^24), the low word the next 64 bits (both
-// products by powers of two and the fraction t 2^24 - hi are exact)
+// t >= 0 as a 128-bit count of 2^-88 (truncated; saturated at 2^128 - 1, from
+// 2^40 on), by shifts of its bits
 __device__ __forceinline__ void nz_fixed(double t, unsigned long long &lo,
                                          unsigned long long &hi) {
-  const double a = t * 16777216.0;  // t 2^(88 - 64)
-  if (!(a < 18446744073709551616.0)) { lo = hi = ~0ull; return; }
-  const double h = floor(a);
-  hi = (unsigned long long)h;
-  lo = (unsigned long long)((a - h) * 18446744073709551616.0);
+  const unsigned long long b = (unsigned long long)__double_as_longlong(t);
+  const int e = (int)(b >> 52);
+  if (e >= 1023 + 40) { lo = hi = ~0ull; return; }
+  const unsigned long long m = (b & 0xfffffffffffffull) | (e > 0 ? 1ull << 52 : 0ull);
+  const int s = (e > 0 ? e : 1) - 1075 + 88;  // t = m 2^(s - 88), s < 76
+  hi = s >= 64 ? m << (s - 64) : (s > 0 ? m >> (64 - s) : 0ull);
+  lo = s >= 64 ? 0ull : (s >= 0 ? m << s : (s > -64 ? m >> -s : 0ull));
 }
 
 // (lo, hi) += (a_lo, a_hi) with atomics: the carry out of the low word is
@@ -146,7 +172,7 @@ __device__ __forceinline__ void nz_add128(unsigned long long *lo, unsigned long 
 // (per block in shared memory first when the bins fit)
 __global__ void nz_bins(int64_t n, const double *x, const double *y,
                         const double *z, const double *vx, const double *vy,
-                        const double *vz, double mu, int nb,
+                        const double *vz, double smu, int nb,
                         unsigned long long *sc) {
   extern __shared__ unsigned long long s_w[];
   const bool shared = nb <= kSharedBins;
@@ -156,19 +182,14 @@ __global__ void nz_bins(int64_t n, const double *x, const double *y,
     __syncthreads();
   }
   unsigned long long *g_lo = sc + 2, *g_hi = sc + 2 + kMaxBins, *g_cnt = sc + 2 + 2 * kMaxBins;
-  const double Rmin = nz_ord_double(sc[0]), Rmax = nz_ord_double(sc[1]);
-  const double lmin = log(Rmin), lmax = log(Rmax);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const double R = sqrt(x[i] * x[i] + y[i] * y[i]);
-    const double r = sqrt(x[i] * x[i] + y[i] * y[i] + z[i] * z[i]);
-    const double vk = sqrt(mu / r);
-    double px = 0.0, py = 0.0;
-    if (R > 0.0) { px = -y[i] / R; py = x[i] / R; }
-    const double ux = vx[i] - vk * px, uy = vy[i] - vk * py, uz = vz[i];
-    const int k = nz_bin(R, Rmin, Rmax, lmin, lmax, nb);
+    const double X = x[i], Y = y[i], Z = z[i], R2 = X * X + Y * Y;
+    const double t = smu * inv_root4(__fma_rn(Z, Z, R2)) * inv_sqrt(R2);
+    const double ux = __fma_rn(t, Y, vx[i]), uy = __fma_rn(-t, X, vy[i]), uz = vz[i];
+    const int k = nz_bin(R2, sc, nb);
     unsigned long long lo, hi;
-    nz_fixed(ux * ux + uy * uy + uz * uz, lo, hi);
+    nz_fixed(__fma_rn(ux, ux, __fma_rn(uy, uy, uz * uz)), lo, hi);
     if (shared) {
       nz_add128(&s_lo[k], &s_hi[k], lo, hi);
       atomicAdd(&s_cnt[k], 1ull);
@@ -177,38 +198,40 @@ __global__ void nz_bins(int64_t n, const double *x, const double *y,
       atomicAdd(&g_cnt[k], 1ull);
     }
   }
-  if (!shared) return;
-  __syncthreads();
-  for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-    if (s_cnt[k]) {
-      nz_add128(&g_lo[k], &g_hi[k], s_lo[k], s_hi[k]);
-      atomicAdd(&g_cnt[k], s_cnt[k]);
+  if (shared) {
+    __syncthreads();
+    for (int k = threadIdx.x; k < nb; k += blockDim.x) {
+      if (s_cnt[k]) {
+        nz_add128(&g_lo[k], &g_hi[k], s_lo[k], s_hi[k]);
+        atomicAdd(&g_cnt[k], s_cnt[k]);
+      }
     }
+  }
+  if (!nz_last(&sc[kExtra + 1])) return;
+  // v_ran of every bin, the 128-bit sum to FP64: hi 2^-24 + lo 2^-88
+  for (int k = threadIdx.x; k < nb; k += blockDim.x) {
+    const double sum = (double)__ldcg(&g_hi[k]) * 5.9604644775390625e-08 +
+                       (double)__ldcg(&g_lo[k]) * 3.2311742677852644e-27;
+    const double vr = sqrt(sum / (double)__ldcg(&g_cnt[k]));
+    g_lo[k] = (unsigned long long)__double_as_longlong(vr);
   }
 }
 
 // r_out = max(R~cut,0 r_Hill, R~cut,1 v_ran dt), r_search = R~s,0 r_out + R~s,1 v_ran dt
 __global__ void nz_final(int64_t n, const double *x, const double *y,
                          const double *z, const double *vx, const double *vy,
-                         const double *vz, const double *m, p3t_params prm,
-                         int nb, const unsigned long long *sc, double *r_out,
+                         const double *vz, const double *m, p3t_params prm, double imu,
+                         double i3ms, int nb, const unsigned long long *sc, double *r_out,
                          double *r_search) {
-  const double mu = prm.G * prm.m_star;
-  const double Rmin = nz_ord_double(sc[0]), Rmax = nz_ord_double(sc[1]);
-  const double lmin = log(Rmin), lmax = log(Rmax);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const double R = sqrt(x[i] * x[i] + y[i] * y[i]);
-    const double r = sqrt(x[i] * x[i] + y[i] * y[i] + z[i] * z[i]);
-    const double v2 = vx[i] * vx[i] + vy[i] * vy[i] + vz[i] * vz[i];
-    const double alpha = 2.0 / r - v2 / mu;
-    const double a = alpha > 0.0 ? 1.0 / alpha : r;
-    const double rhill = cbrt(m[i] / (3.0 * prm.m_star)) * a;
-    const int k = nz_bin(R, Rmin, Rmax, lmin, lmax, nb);
-    // the bin's 128-bit sum to FP64: hi 2^-24 + lo 2^-88
-    const double sum = (double)sc[2 + kMaxBins + k] * 5.9604644775390625e-08 +
-                       (double)sc[2 + k] * 3.2311742677852644e-27;
-    const double vr = sqrt(sum / (double)sc[2 + 2 * kMaxBins + k]);
+    const double R2 = x[i] * x[i] + y[i] * y[i], r2 = __fma_rn(z[i], z[i], R2);
+    const double ir = inv_sqrt(r2);
+    const double v2 = __fma_rn(vx[i], vx[i], __fma_rn(vy[i], vy[i], vz[i] * vz[i]));
+    const double alpha = __fma_rn(-v2, imu, 2.0 * ir);  // 1/a, vis-viva
+    const double a = alpha > 0.0 ? 1.0 / alpha : r2 * ir;
+    const double rhill = cbrt_pos(m[i] * i3ms) * a;
+    const double vr = __longlong_as_double((long long)sc[2 + nz_bin(R2, sc, nb)]);
     const double ro = prm.cutoff_mode == P3T_CUT_HILL_VRAN
                           ? fmax(prm.rcut0 * rhill, prm.rcut1 * vr * prm.dt_soft)
                           : prm.rcut0 * rhill;
@@ -252,11 +275,12 @@ extern "C" int p3t_cutoffs_noalloc(const p3t_params *prm, p3t_particles *p,
   if (g < 1) g = 1;
   const double mu = prm->G * prm->m_star;
   nz_clear<<<4, kBlock, 0, s>>>(sc, nb);
-  nz_range<<<(unsigned)g, kBlock, 0, s>>>(n, p->x, p->y, sc);
+  nz_range<<<(unsigned)g, kBlock, 0, s>>>(n, p->x, p->y, nb, sc);
   const size_t smem = nb <= kSharedBins ? 3 * sizeof(unsigned long long) * nb : 0;
-  nz_bins<<<(unsigned)g, kBlock, smem, s>>>(n, p->x, p->y, p->z, p->vx, p->vy, p->vz, mu,
-                                            nb, sc);
+  nz_bins<<<(unsigned)g, kBlock, smem, s>>>(n, p->x, p->y, p->z, p->vx, p->vy, p->vz,
+                                            sqrt(mu), nb, sc);
   nz_final<<<(unsigned)g, kBlock, 0, s>>>(n, p->x, p->y, p->z, p->vx, p->vy, p->vz,
-                                          p->m, *prm, nb, sc, p->r_out, p->r_search);
+                                          p->m, *prm, 1.0 / mu, 1.0 / (3.0 * prm->m_star), nb, sc,
+                                          p->r_out, p->r_search);
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }

@@ -30,8 +30,8 @@ def _disk(kind, n):
 
 
 @pytest.mark.parametrize("kind", ["annulus", "far", "near", "axis", "circle", "spread"])
-@pytest.mark.parametrize("n,bins", [(1, 1), (2, 4096), (257, 256), (6000, 257), (50000, 4096),
-                                    (50000, 0)])
+@pytest.mark.parametrize("n,bins", [(1, 1), (2, 4096), (257, 256), (6000, 257), (6000, 2048),
+                                    (50000, 4096), (50000, 0)])
 def test_cutoffs_match_oracle(kind, n, bins):
     need_gpu()
     from paper_2007_15432_gb300 import build
