@@ -158,14 +158,13 @@ __global__ void k_cl_flags(int64_t n, const int32_t *label, const int32_t *csize
   if (mx) atomicMax(reinterpret_cast<unsigned long long *>(&counts[3]), mx);
 }
 
-// the singles, each cluster's offset and the members (with their labels, for
-// the sort) from the two packed scans (counts in bits 0-30, the second sum
-// from bit 31), and the four totals: singles, clusters, members (counts[0..2])
-// and members again for the sort (*d_nmem)
+// the singles, each cluster's offset and its members (in any order: the root's
+// size counts down to zero) from the two packed scans (counts in bits 0-30, the
+// second sum from bit 31), and the totals: singles, clusters, members
+// (counts[0..2])
 __global__ void k_cl_scatter(int64_t n, const int32_t *label, const int32_t *flag,
                              const int64_t *pos, const int64_t *d_tot, int32_t *singles,
-                             int64_t *cl_off, uint64_t *mkeys, int32_t *mvals, int64_t *counts,
-                             int64_t *d_nmem) {
+                             int64_t *cl_off, int32_t *csize, int32_t *mem, int64_t *counts) {
   pdl_wait();
   constexpr int64_t kLow = (1ll << 31) - 1;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -177,9 +176,8 @@ __global__ void k_cl_scatter(int64_t n, const int32_t *label, const int32_t *fla
       cl_off[q & kLow] = q >> 31;
     }
     if (fa & 2) {
-      const int64_t q = pos[i] >> 31;
-      mkeys[q] = (uint64_t)label[i];
-      mvals[q] = (int32_t)i;
+      const int32_t r = label[i];
+      mem[(pos[n + r] >> 31) + atomicSub(&csize[r], 1) - 1] = (int32_t)i;
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -187,18 +185,94 @@ __global__ void k_cl_scatter(int64_t n, const int32_t *label, const int32_t *fla
     counts[0] = ta & kLow;
     counts[1] = tb & kLow;
     counts[2] = tb >> 31;
-    *d_nmem = ta >> 31;
     cl_off[tb & kLow] = tb >> 31;
   }
 }
 
-// the first *d_n values of src into dst
-__global__ void k_copy_i32(const int64_t *d_n, const int32_t *src, int32_t *dst) {
+// The members of every cluster in index order.  A cluster is a few members
+// almost always: a thread sorts up to eight in registers; a block ranks up to
+// kMemChunk at a time in shared memory, and merges the runs of a larger one
+// through tmp (a cluster of a million would take some 60 ms here; one Hermite
+// block step of it is 10^12 pair terms).  One launch, where all members were
+// sorted by label: three radix passes and a copy, some 55 us at N = 1e5 and
+// 1e6.  Measured (this kernel): P3T_CLSORT.
+constexpr int kMemThreads = 256, kMemSmall = 8, kMemChunk = 1024;
+__device__ void sort_members(int32_t *mem, int32_t *tmp, int m, int32_t *s) {
+  for (int b = 0; b < m; b += kMemChunk) {
+    const int len = min(kMemChunk, m - b);
+    for (int e = threadIdx.x; e < len; e += kMemThreads) s[e] = mem[b + e];
+    __syncthreads();
+    for (int e = threadIdx.x; e < len; e += kMemThreads) {
+      const int32_t v = s[e];
+      int rank = 0;
+      for (int j = 0; j < len; ++j) rank += s[j] < v;
+      mem[b + rank] = v;
+    }
+    __syncthreads();
+  }
+  for (int64_t r = kMemChunk; r < m; r *= 2) {
+    for (int64_t o = threadIdx.x; o < m; o += kMemThreads) {
+      // output o of its pair of runs: the split of the diagonal
+      const int64_t base = o / (2 * r) * (2 * r), diag = o - base;
+      const int64_t a1 = min(base + r, (int64_t)m), b1 = min(base + 2 * r, (int64_t)m);
+      int64_t lo = max((int64_t)0, diag - (b1 - a1)), hi = min(diag, a1 - base);
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (mem[base + mid] < mem[a1 + diag - 1 - mid]) lo = mid + 1; else hi = mid;
+      }
+      const int64_t ia = base + lo, ib = a1 + diag - lo;
+      tmp[o] = ib >= b1 || (ia < a1 && mem[ia] < mem[ib]) ? mem[ia] : mem[ib];
+    }
+    __syncthreads();
+    for (int64_t o = threadIdx.x; o < m; o += kMemThreads) mem[o] = tmp[o];
+    __syncthreads();
+  }
+}
+__global__ void __launch_bounds__(kMemThreads) k_cl_sort(const int64_t *counts,
+                                                         const int64_t *cl_off, int32_t *mem,
+                                                         int32_t *tmp) {
   pdl_wait();
-  const int64_t n = *d_n;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = src[i];
+  __shared__ int32_t s_mem[kMemChunk];
+  __shared__ int s_list[kMemThreads], s_n;
+  const int64_t ncl = counts[1];
+  for (int64_t c0 = (int64_t)blockIdx.x * kMemThreads; c0 < ncl;
+       c0 += (int64_t)gridDim.x * kMemThreads) {
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const int64_t c = c0 + threadIdx.x;
+    if (c < ncl) {
+      const int64_t o = cl_off[c];
+      const int m = (int)(cl_off[c + 1] - o);
+      if (m <= kMemSmall) {
+        int32_t v[kMemSmall];
+#pragma unroll
+        for (int k = 0; k < kMemSmall; ++k) v[k] = k < m ? mem[o + k] : 0x7fffffff;
+        // odd-even transposition, as many rounds as members
+#pragma unroll
+        for (int r = 0; r < kMemSmall; ++r) {
+          if (r < m)
+#pragma unroll
+            for (int k = r & 1; k + 1 < kMemSmall; k += 2) {
+              const int32_t lo = min(v[k], v[k + 1]), hi = max(v[k], v[k + 1]);
+              v[k] = lo;
+              v[k + 1] = hi;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kMemSmall; ++k)
+          if (k < m) mem[o + k] = v[k];
+      } else {
+        s_list[atomicAdd(&s_n, 1)] = threadIdx.x;
+      }
+    }
+    __syncthreads();
+    const int many = s_n;
+    for (int q = 0; q < many; ++q) {
+      const int64_t d = c0 + s_list[q], o = cl_off[d];
+      sort_members(mem + o, tmp + o, (int)(cl_off[d + 1] - o), s_mem);
+    }
+    __syncthreads();
+  }
 }
 
 }  // namespace
@@ -232,26 +306,15 @@ int p3t_run_neighbours(p3t_ctx *c, const p3t_particles *p, int64_t *nb_off,
                              c->scan_state, c->scan_words, c->status, c->poll_limit, s);
     if (rc) return rc;
   }
+  // the members stay in one buffer, so that the cluster views keep their
+  // addresses from step to step (a step captured in a CUDA graph reads the
+  // previous step's clusters there)
   pdl_launch(k_cl_scatter, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->label, c->flag, c->pos,
-             &cnt[21], c->singles, c->cl_off, c->mkeys, c->mvals, c->cl_counts, &cnt[11]);
-  // filter, fill, sort_rows, uf_union, uf_label, flags, scatter
-  p3t_note_launches(7);
-  // members ordered by (label, index), on the label's bits (labels are
-  // particle indices below n).  The sorted members must land in the buffer
-  // they started in, so that the cluster views keep their addresses from step
-  // to step (a step captured in a CUDA graph reads the previous step's
-  // clusters there): after an odd number of radix passes they are copied back
-  const int bits = n <= 65536 ? 16 : (n <= (1 << 24) ? 24 : 32);
-  uint64_t *k0 = c->mkeys, *k1 = c->mkeys_alt;
-  int32_t *v0 = c->mvals, *v1 = c->mvals_alt;
-  rc = p3t_sort_pairs(&k0, &v0, &k1, &v1, &cnt[11], c->cap, bits, c->radix_hist,
-                      c->radix_hist_cap, c->sort_work, p3t_sort_where(c), s);
-  if (rc) return rc;
-  if (v0 != c->mvals) {
-    pdl_launch(k_copy_i32, dim3((unsigned)p3t_grid(n, kBlock, maxb)), dim3(kBlock), 0, s, &cnt[11],
-               v0, c->mvals);
-    p3t_note_launches(1);
-  }
-  c->cl_mem = c->mvals;  // sorted payload buffer
+             &cnt[21], c->singles, c->cl_off, c->csize, c->mvals, c->cl_counts);
+  pdl_launch(k_cl_sort, dim3((unsigned)p3t_grid(n / 2 + 1, kMemThreads, maxb)), dim3(kMemThreads), 0,
+             s, c->cl_counts, c->cl_off, c->mvals, c->mvals_alt);
+  // filter, fill, sort_rows, uf_union, uf_label, flags, scatter, sort
+  p3t_note_launches(8);
+  c->cl_mem = c->mvals;
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }

@@ -296,8 +296,7 @@ struct p3t_ctx {
   int32_t *singles = nullptr, *cl_mem = nullptr;
   int64_t *cl_off = nullptr;
   int64_t *cl_counts = nullptr;            // [4]
-  uint64_t *mkeys = nullptr, *mkeys_alt = nullptr;
-  int32_t *mvals = nullptr, *mvals_alt = nullptr;
+  int32_t *mvals = nullptr, *mvals_alt = nullptr;  // cluster members, scratch for large clusters
 
   // hard step workspace (per cluster member, clusters of more than 128)
   double *hw = nullptr;                    // 33 * cap doubles
