@@ -193,9 +193,9 @@ __global__ void k_cl_scatter(int64_t n, const int32_t *label, const int32_t *fla
 // almost always: a thread sorts up to eight in registers; a block ranks up to
 // kMemChunk at a time in shared memory, and merges the runs of a larger one
 // through tmp (a cluster of a million would take some 60 ms here; one Hermite
-// block step of it is 10^12 pair terms).  One launch, where all members were
-// sorted by label: three radix passes and a copy, some 55 us at N = 1e5 and
-// 1e6.  Measured (this kernel): P3T_CLSORT.
+// block step of it is 10^12 pair terms).  Bound by its launch and the members'
+// latency: equal-mass ring, N = 1e5, 3.7 us, wide disk, N = 1e6, 7.0; sorting all
+// members by label took three radix passes and a copy, some 55 us in both.
 constexpr int kMemThreads = 256, kMemSmall = 8, kMemChunk = 1024;
 __device__ void sort_members(int32_t *mem, int32_t *tmp, int m, int32_t *s) {
   for (int b = 0; b < m; b += kMemChunk) {
