@@ -86,7 +86,7 @@ void free_particle_buffers(p3t_ctx *c) {
   dfree(c->flag); dfree(c->pos); dfree(c->singles); dfree(c->cl_off); dfree(c->hlist);
   // cl_mem aliases mvals
   c->cl_mem = nullptr;
-  dfree(c->mvals); dfree(c->mvals_alt);
+  dfree(c->mvals);
   dfree(c->hw); dfree(c->ht); dfree(c->hl);
   dfree(c->coll_ent); dfree(c->coll_rec); dfree(c->coll_rec_e); dfree(c->coll_esoft);
   dfree(c->coll_slot); dfree(c->scan_state);
@@ -143,7 +143,7 @@ int reserve(p3t_ctx *c, int64_t n, int64_t cand_cap) {
   ok &= dalloc(c->singles, N) && dalloc(c->cl_off, N + 1);
   c->hlist_cap = N / 2 + 1;  // clusters have at least two members
   ok &= dalloc(c->hlist, 2 * c->hlist_cap);
-  ok &= dalloc(c->mvals, N) && dalloc(c->mvals_alt, N);
+  ok &= dalloc(c->mvals, N);
   ok &= dalloc(c->hw, 33 * N) && dalloc(c->ht, N) && dalloc(c->hl, 6 * N);
   ok &= dalloc(c->coll_ent, N) && dalloc(c->coll_rec, N / 2 + 1) && dalloc(c->coll_rec_e, N / 2 + 1);
   ok &= dalloc(c->coll_esoft, N) && dalloc(c->coll_slot, N);

@@ -158,6 +158,8 @@ __global__ void k_cl_flags(int64_t n, const int32_t *label, const int32_t *csize
   if (mx) atomicMax(reinterpret_cast<unsigned long long *>(&counts[3]), mx);
 }
 
+constexpr int kMemMax = 1024;  // members that a block ranks in shared memory
+
 // the singles, each cluster's offset and its members (in any order: the root's
 // size counts down to zero) from the two packed scans (counts in bits 0-30, the
 // second sum from bit 31), and the totals: singles, clusters, members
@@ -176,8 +178,13 @@ __global__ void k_cl_scatter(int64_t n, const int32_t *label, const int32_t *fla
       cl_off[q & kLow] = q >> 31;
     }
     if (fa & 2) {
+      // (of a cluster that will be listed from the labels, the root only)
       const int32_t r = label[i];
-      mem[(pos[n + r] >> 31) + atomicSub(&csize[r], 1) - 1] = (int32_t)i;
+      const int64_t o = pos[n + r] >> 31;
+      if ((flag[n + r] >> 1) <= kMemMax)
+        mem[o + atomicSub(&csize[r], 1) - 1] = (int32_t)i;
+      else if (i == r)
+        mem[o] = r;
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -190,54 +197,72 @@ __global__ void k_cl_scatter(int64_t n, const int32_t *label, const int32_t *fla
 }
 
 // The members of every cluster in index order.  A cluster is a few members
-// almost always: a thread sorts up to eight in registers; a block ranks up to
-// kMemChunk at a time in shared memory, and merges the runs of a larger one
-// through tmp (a cluster of a million would take some 60 ms here; one Hermite
-// block step of it is 10^12 pair terms).  Bound by its launch and the members'
-// latency: equal-mass ring, N = 1e5, 3.7 us, wide disk, N = 1e6, 7.0; sorting all
-// members by label took three radix passes and a copy, some 55 us in both.
-constexpr int kMemThreads = 256, kMemSmall = 8, kMemChunk = 1024;
-__device__ void sort_members(int32_t *mem, int32_t *tmp, int m, int32_t *s) {
-  for (int b = 0; b < m; b += kMemChunk) {
-    const int len = min(kMemChunk, m - b);
-    for (int e = threadIdx.x; e < len; e += kMemThreads) s[e] = mem[b + e];
-    __syncthreads();
-    for (int e = threadIdx.x; e < len; e += kMemThreads) {
-      const int32_t v = s[e];
-      int rank = 0;
-      for (int j = 0; j < len; ++j) rank += s[j] < v;
-      mem[b + rank] = v;
-    }
-    __syncthreads();
+// almost always: a thread sorts up to eight in registers, a warp ranks up to 32, a
+// block up to kMemMax in shared memory, and lists a larger one anew from the
+// labels (one pass over the particles).  Bound by its launch and the members'
+// latency: equal-mass ring, N = 1e5, 4 us, wide disk, N = 1e6, 5; sorting all
+// members by label took three radix passes and a copy, some 55 us in both.  One
+// cluster of 5,000 of 1e6 particles takes some 200 us, less than one block step of
+// its Hermite pairs.
+constexpr int kMemThreads = 1024, kMemSmall = 8;
+__device__ void rank_members(int32_t *mem, int m, int32_t *s) {
+  for (int e = threadIdx.x; e < m; e += kMemThreads) s[e] = mem[e];
+  __syncthreads();
+  for (int e = threadIdx.x; e < m; e += kMemThreads) {
+    const int32_t v = s[e];
+    int rank = 0;
+    for (int j = 0; j < m; ++j) rank += s[j] < v;
+    mem[rank] = v;
   }
-  for (int64_t r = kMemChunk; r < m; r *= 2) {
-    for (int64_t o = threadIdx.x; o < m; o += kMemThreads) {
-      // output o of its pair of runs: the split of the diagonal
-      const int64_t base = o / (2 * r) * (2 * r), diag = o - base;
-      const int64_t a1 = min(base + r, (int64_t)m), b1 = min(base + 2 * r, (int64_t)m);
-      int64_t lo = max((int64_t)0, diag - (b1 - a1)), hi = min(diag, a1 - base);
-      while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (mem[base + mid] < mem[a1 + diag - 1 - mid]) lo = mid + 1; else hi = mid;
-      }
-      const int64_t ia = base + lo, ib = a1 + diag - lo;
-      tmp[o] = ib >= b1 || (ia < a1 && mem[ia] < mem[ib]) ? mem[ia] : mem[ib];
+  __syncthreads();
+}
+// the particles labelled r (the smallest of them) into mem[0, m): a warp takes
+// 32 rows of 32 particles a pass, their loads in flight together, a lane
+// keeping each row's mask; s: the warps' counts
+__device__ void list_members(int64_t n, const int32_t *label, int32_t r, int32_t *mem, int m,
+                             int32_t *s) {
+  constexpr int kRows = 32;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int done = 0;
+  for (int64_t b = r; b < n && done < m; b += kMemThreads * kRows) {
+    const int64_t b0 = b + (int64_t)w * 32 * kRows;
+    unsigned rows = 0;  // lane k: the mask of row k
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+      const int64_t i = b0 + 32 * k + lane;
+      const unsigned in = __ballot_sync(0xffffffffu, i < n && label[i] == r);
+      if (lane == k) rows = in;
     }
+    const int own = __reduce_add_sync(0xffffffffu, __popc(rows));
+    if (lane == 0) s[w] = own;
     __syncthreads();
-    for (int64_t o = threadIdx.x; o < m; o += kMemThreads) mem[o] = tmp[o];
+    int at = done;
+    for (int q = 0; q < kMemThreads / 32; ++q) {
+      if (q < w) at += s[q];
+      done += s[q];
+    }
+    if (own)
+#pragma unroll 4
+      for (int k = 0; k < kRows; ++k) {
+        const unsigned in = __shfl_sync(0xffffffffu, rows, k);
+        const int o = at + __popc(in & ((1u << lane) - 1u));
+        if (((in >> lane) & 1u) && o < m) mem[o] = (int32_t)(b0 + 32 * k + lane);
+        at += __popc(in);
+      }
     __syncthreads();
   }
 }
 __global__ void __launch_bounds__(kMemThreads) k_cl_sort(const int64_t *counts,
-                                                         const int64_t *cl_off, int32_t *mem,
-                                                         int32_t *tmp) {
+                                                         const int64_t *cl_off, int64_t n,
+                                                         const int32_t *label, int32_t *mem) {
   pdl_wait();
-  __shared__ int32_t s_mem[kMemChunk];
-  __shared__ int s_list[kMemThreads], s_n;
+  __shared__ int32_t s_mem[kMemMax];
+  __shared__ int s_list[2][kMemThreads], s_n[2];  // clusters for a warp, for the block
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t ncl = counts[1];
   for (int64_t c0 = (int64_t)blockIdx.x * kMemThreads; c0 < ncl;
        c0 += (int64_t)gridDim.x * kMemThreads) {
-    if (threadIdx.x == 0) s_n = 0;
+    if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
     __syncthreads();
     const int64_t c = c0 + threadIdx.x;
     if (c < ncl) {
@@ -262,14 +287,29 @@ __global__ void __launch_bounds__(kMemThreads) k_cl_sort(const int64_t *counts,
         for (int k = 0; k < kMemSmall; ++k)
           if (k < m) mem[o + k] = v[k];
       } else {
-        s_list[atomicAdd(&s_n, 1)] = threadIdx.x;
+        const int q = m > 32;
+        s_list[q][atomicAdd(&s_n[q], 1)] = threadIdx.x;
       }
     }
     __syncthreads();
-    const int many = s_n;
-    for (int q = 0; q < many; ++q) {
-      const int64_t d = c0 + s_list[q], o = cl_off[d];
-      sort_members(mem + o, tmp + o, (int)(cl_off[d + 1] - o), s_mem);
+    for (int q = w; q < s_n[0]; q += kMemThreads / 32) {
+      const int64_t d = c0 + s_list[0][q], o = cl_off[d];
+      const int m = (int)(cl_off[d + 1] - o);
+      const int32_t v = lane < m ? mem[o + lane] : 0x7fffffff;
+      int rank = 0;
+      for (int j = 0; j < m; ++j) rank += __shfl_sync(0xffffffffu, v, j) < v;
+      if (lane < m) mem[o + rank] = v;
+    }
+    for (int q = 0; q < s_n[1]; ++q) {
+      const int64_t d = c0 + s_list[1][q], o = cl_off[d];
+      const int m = (int)(cl_off[d + 1] - o);
+      if (m <= kMemMax) {
+        rank_members(mem + o, m, s_mem);
+      } else {
+        const int32_t r = mem[o];
+        __syncthreads();  // mem[o] is read before it is written
+        list_members(n, label, r, mem + o, m, s_mem);
+      }
     }
     __syncthreads();
   }
@@ -311,8 +351,8 @@ int p3t_run_neighbours(p3t_ctx *c, const p3t_particles *p, int64_t *nb_off,
   // previous step's clusters there)
   pdl_launch(k_cl_scatter, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->label, c->flag, c->pos,
              &cnt[21], c->singles, c->cl_off, c->csize, c->mvals, c->cl_counts);
-  pdl_launch(k_cl_sort, dim3((unsigned)p3t_grid(n / 2 + 1, kMemThreads, maxb)), dim3(kMemThreads), 0,
-             s, c->cl_counts, c->cl_off, c->mvals, c->mvals_alt);
+  pdl_launch(k_cl_sort, dim3((unsigned)p3t_grid(n / 2 + 1, kMemThreads, c->num_sms)), dim3(kMemThreads), 0,
+             s, c->cl_counts, c->cl_off, n, c->label, c->mvals);
   // filter, fill, sort_rows, uf_union, uf_label, flags, scatter, sort
   p3t_note_launches(8);
   c->cl_mem = c->mvals;

@@ -296,7 +296,7 @@ struct p3t_ctx {
   int32_t *singles = nullptr, *cl_mem = nullptr;
   int64_t *cl_off = nullptr;
   int64_t *cl_counts = nullptr;            // [4]
-  int32_t *mvals = nullptr, *mvals_alt = nullptr;  // cluster members, scratch for large clusters
+  int32_t *mvals = nullptr;                // cluster members
 
   // hard step workspace (per cluster member, clusters of more than 128)
   double *hw = nullptr;                    // 33 * cap doubles

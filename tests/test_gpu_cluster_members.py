@@ -1,5 +1,5 @@
 """Members of neighbour clusters in index order at the sizes where their sort
-changes form: a thread's eight, a block's 1,024 and the merges above."""
+changes form: a thread's eight, a block's 1,024 and the listing above."""
 import numpy as np
 import pytest
 import torch
