@@ -49,8 +49,8 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # DRAM bytes (read + write) of one k_walk launch on the N = 10^6 wide disk,
 # group size 64, from a single-pass ncu capture of this kernel
-# (dram__bytes_read.sum 78.90 MB + dram__bytes_write.sum 16.13 MB)
-WALK_TRAFFIC_1E6 = 95.03e6
+# (dram__bytes_read.sum 110.27 MB + dram__bytes_write.sum 23.07 MB)
+WALK_TRAFFIC_1E6 = 133.34e6
 
 
 def parse():
@@ -825,8 +825,8 @@ def run_adjoint(args):
     torch.cuda.synchronize(dev)
     run.status()
     t_vjp = e[3].elapsed_time(e4) / 1e3 / 10
-    segs = (steps + ck - 1) // ck
-    forces = (steps + 1) + (steps + segs)  # forward sweep + recomputation
+    last = steps - ck * ((steps - 1) // ck)  # steps of the last segment, which is kept
+    forces = (steps + 1) + (steps - last)  # forward sweep + recomputation
     vjps = steps + 1
     pairs = float(n) * (n - 1)
     # FP32 work of one VJP pair term (float-float difference 9, r2 5, rsqrt,
