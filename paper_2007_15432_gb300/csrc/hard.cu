@@ -1244,11 +1244,9 @@ __device__ bool integrate_five(const V &S, HFive &F, int64_t off, int nc, const 
     } else {
       e = e_unit + P3T_KMAX;
     }
-    // the new step, first from norms good to 1e-5 (components by their leading
-    // 20 bits, approximate roots): |a| and |a2| in the position lanes, |j| and
-    // |a3| in the velocity lanes.  Its level is the exact one's unless it lies
-    // within 2^-14 of a power of two times dt (or out of range): then the
-    // criterion is evaluated as written
+    // the new step, first from squared norms of the components' leading 20 bits:
+    // |a| and |a2| in the position lanes, |j| and |a3| in the velocity lanes;
+    // where those do not decide its level, by the criterion as written
     double dtd;
     {
       const float x1 = lead_float(vel ? j1 : a1, vel ? e : 0);
@@ -1258,22 +1256,8 @@ __device__ bool integrate_five(const V &S, HFive &F, int64_t off, int nc, const 
                   o2 = __shfl_sync(0xffffffffu, n2, other);
       const float an = vel ? o1 : n1, jn = vel ? n1 : o1;  // squared
       const float a2n = vel ? o2 : n2, a3n = vel ? n2 : o2;
-      float r;
-      if (iter > 0) {
-        r = sqrt_approx(__fdividef(hc.etaf * (sqrt_approx(an * a2n) + jn),
-                                   sqrt_approx(jn * a3n) + a2n));
-      } else {  // first step eta0 |a| / |j|
-        r = hc.eta0f * sqrt_approx(__fdividef(an, jn));
-      }
-      const unsigned u = __float_as_uint(r);
-      const int er = (int)(u >> 23) - 127 + 1023 + e;
-      const bool fine = an > 1e-30f && an < 1e30f && jn > 1e-30f && jn < 1e30f &&
-                        (iter == 0 || (a2n > 1e-30f && a2n < 1e30f && a3n > 1e-30f && a3n < 1e30f)) &&
-                        r > 1e-30f && r < 1e30f && er > 0 && er < 2047;
-      const long long bs = (long long)er << 52 | (long long)(u & 0x7fffffu) << 29;
-      const long long frac = (bs - bd) & 0xfffffffffffffLL, lim = 1LL << 38;
-      dtd = __longlong_as_double(bs);
-      if (__any_sync(0xffffffffu, on && (!fine || frac < lim || frac > (1LL << 52) - lim)))
+      const bool decided = step_estimate(an, jn, a2n, a3n, e, iter > 0, hc, bd, dtd);
+      if (__any_sync(0xffffffffu, on && !decided))
         dtd = exact_step(vel ? j1 : a1, vel ? A3 : a2e, vel, other, gq, e, iter > 0, hc, dt);
     }
     if (on) {

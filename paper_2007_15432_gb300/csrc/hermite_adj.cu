@@ -413,27 +413,15 @@ __global__ void __launch_bounds__(128) k_tangent_lanes(
           dv = __fma_rn(B3, c4, __fma_rn(B2, c3, dpv));
         }
       }
-      // the new level: from norms good to 1e-5, the criterion as written when
-      // the step lies within 2^-14 of a power of two times dt (or out of range)
+      // the new level: from squared norms of the components' leading 20 bits, by
+      // the criterion as written where those do not decide it
       double dtd;
       {
         const float an = norm_lanes(lead_float(f.a, 0), b0), jn = norm_lanes(lead_float(f.j, e), b0);
         const float a2n = norm_lanes(lead_float(a2e, 2 * e), b0),
                     a3n = norm_lanes(lead_float(A3, 3 * e), b0);
-        const float r = blocks > 0
-                            ? sqrt_approx(__fdividef(hc.etaf * (sqrt_approx(an * a2n) + jn),
-                                                     sqrt_approx(jn * a3n) + a2n))
-                            : hc.eta0f * sqrt_approx(__fdividef(an, jn));
-        const unsigned b = __float_as_uint(r);
-        const int er = (int)(b >> 23) - 127 + 1023 + e;
-        const bool fine = an > 1e-30f && an < 1e30f && jn > 1e-30f && jn < 1e30f &&
-                          (blocks == 0 || (a2n > 1e-30f && a2n < 1e30f && a3n > 1e-30f && a3n < 1e30f)) &&
-                          r > 1e-30f && r < 1e30f && er > 0 && er < 2047;
-        const long long bs = (long long)er << 52 | (long long)(b & 0x7fffffu) << 29;
-        const long long frac = (bs - bd) & 0xfffffffffffffLL, lim = 1LL << 38;
-        dtd = __longlong_as_double(bs);
-        if (__any_sync(0xffffffffu,
-                       on && act && (!fine || frac < lim || frac > (1LL << 52) - lim)))
+        const bool decided = step_estimate(an, jn, a2n, a3n, e, blocks > 0, hc, bd, dtd);
+        if (__any_sync(0xffffffffu, on && act && !decided))
           dtd = exact_step64(f.a, f.j, a2e, A3, b0, blocks > 0, prm.eta, prm.eta0, dt);
       }
       if (act) {

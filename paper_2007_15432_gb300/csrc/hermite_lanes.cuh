@@ -100,3 +100,37 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
+
+// The step criterion (the first step eta0 |a| / |j|, or, `later`, sqrt(eta (|a|
+// |a2| + |j|^2) / (|j| |a3| + |a2|^2))) from squared norms good to 2e-6, by
+// approximate roots and quotient: dtd = its value times 2^e, good to 1e-5.
+// Returns whether dtd decides the level: it lies 2^-14 or more from every power
+// of two times dt (bd: dt's bits), and every squared norm, product, sum and
+// quotient formed is a normal number.  (The products of two squared norms are
+// the first to leave FP32's range: accelerations of 1e-9 with steps of a
+// twentieth of |a| / |j| have |j|^2 |a3|^2 of 4e-47.)
+__device__ __forceinline__ bool step_estimate(float an, float jn, float a2n, float a3n, int e,
+                                              bool later, const HConst &hc, long long bd,
+                                              double &dtd) {
+  float r;
+  bool fine = an > 1e-30f && an < 1e30f && jn > 1e-30f && jn < 1e30f;
+  if (later) {
+    const float p = an * a2n, q = jn * a3n;
+    const float num = hc.etaf * (sqrt_approx(p) + jn), den = sqrt_approx(q) + a2n;
+    const float s = __fdividef(num, den);
+    r = sqrt_approx(s);
+    fine = fine && a2n > 1e-30f && a2n < 1e30f && a3n > 1e-30f && a3n < 1e30f && p > 1e-37f &&
+           q > 1e-37f && num > 1e-37f && s > 1e-37f;
+  } else {
+    const float s = __fdividef(an, jn);
+    r = hc.eta0f * sqrt_approx(s);
+    fine = fine && s > 1e-37f;
+  }
+  const unsigned u = __float_as_uint(r);
+  const int er = (int)(u >> 23) - 127 + 1023 + e;
+  fine = fine && r > 1e-30f && r < 1e30f && er > 0 && er < 2047;
+  const long long bs = (long long)er << 52 | (long long)(u & 0x7fffffu) << 29;
+  const long long frac = (bs - bd) & 0xfffffffffffffLL, lim = 1LL << 38;
+  dtd = __longlong_as_double(bs);
+  return fine && frac >= lim && frac <= (1LL << 52) - lim;
+}
