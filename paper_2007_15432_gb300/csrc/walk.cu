@@ -836,7 +836,8 @@ __device__ __forceinline__ void far_box64(const WalkArgs &a, int32_t t0, int nt,
 }
 // whether a source is beyond every target's max(r_search, r_out) and its own:
 // the gap to the box less 2^-18 of the coordinates' scale (their truncation to
-// 20 bits), against the reach widened by 1e-5
+// 20 bits), against the reach widened by 1e-5.  A gap whose square leaves FP32's
+// range is not decided here: it would pass against a reach whose square does
 __device__ __forceinline__ bool far_from64(const FarBox &b, double X, double Y, double Z,
                                            double ro, double rs) {
   const float x = lead_float(X, 0), y = lead_float(Y, 0), z = lead_float(Z, 0);
@@ -847,7 +848,7 @@ __device__ __forceinline__ bool far_from64(const FarBox &b, double X, double Y, 
   const float gz = fmaxf(fmaxf(b.lo[2] - z, z - b.hi[2]) - m, 0.f);
   const float R = fmaxf(b.R2, fmaxf(lead_float(ro, 0), lead_float(rs, 0))) * 1.00001f;
   const float d2 = gx * gx + gy * gy + gz * gz;
-  return d2 > 1e-30f && d2 >= R * R;
+  return d2 > 1e-30f && d2 < 3e38f && d2 >= R * R;
 }
 
 // m r^-3 from r^2 (zero for r = 0): the seed's y, e = 1 - r^2 y^2 and the
