@@ -874,6 +874,10 @@ __device__ __forceinline__ double clamp01(double x) {
   const long long b = __double_as_longlong(x), one = 0x3ff0000000000000LL;
   return __longlong_as_double(b < 0 ? 0 : (b > one ? one : b));
 }
+// whether a clamped x lies strictly between 0 and 1
+__device__ __forceinline__ bool inside01(double x) {
+  return (unsigned long long)(__double_as_longlong(x) - 1) < 0x3fefffffffffffffULL;
+}
 // 1 / r to full precision
 __device__ __forceinline__ double inv_r(const Inv3 &v) {
   return fma(v.y * v.e, fma(0.375, v.e, 0.5), v.y);
@@ -1158,13 +1162,14 @@ struct VjpEval {
       const double ri2 = fma(y2, fma(v.e, v.e, v.e), y2);
       double phi = v.f, psi;
       if (near) {
-        // the target itself (r = 0) has y = 0: K = K' = 0
+        // the target itself (r = 0) has phi = 0, and K' = 0 at both ends also
+        // where 1 / r_out is infinite
         const double irot = min_pos(t.iro[i], iro);
         const double yv = (r2 * inv_r(v)) * irot;
         const double x = clamp01((yv - a.gamma) * a.inv1mg);
         const double x2 = x * x, u = 1.0 - x;
         const double K = (x2 * x2) * fma(fma(fma(-20.0, x, 70.0), x, -84.0), x, 35.0);
-        const double dK = (140.0 * a.inv1mg) * ((x2 * x) * (u * u * u)) * irot;
+        const double dK = (140.0 * a.inv1mg) * ((x2 * x) * (u * u * u)) * (inside01(x) ? irot : 0.0);
         psi = fma(dK, ri2 * ri2, -3.0 * K * (phi * ri2));
         phi *= K;
       } else {
