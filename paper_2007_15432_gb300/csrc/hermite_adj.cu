@@ -322,7 +322,8 @@ __device__ __forceinline__ TanOut hard_tangent(int nc, int k, int b0, int row0, 
       const double W = mid ? 1.0 - K : 1.0;
       const double dK = mid ? q2 * (xs * us) : 0.0;                    // K'(y)
       const double ddK = mid ? (3.0 * hc.i1mg) * (q2 * (us - xs)) : 0.0;  // K''(y)
-      const double rio = ri * irot, dy = s * rio;
+      // zero outside: irot is infinite between two members of zero radius
+      const double rio = mid ? ri * irot : 0.0, dy = s * rio;
       const double dW = -(dK * dy);
       const double ro = rv * rio;
       const double E = dK * ro;  // -dW/dt
