@@ -69,38 +69,37 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float p) {
   hi = s;
 }
 
-// r^-3 from r^2 with the seed's y and e = 1 - r^2 y^2 (see rsqrt_seed); 0 for
-// r = 0
-__device__ __forceinline__ double inv_cube(double r2, double &y, double &e) {
-  y = rsqrt_seed(r2);
-  const double y2 = y * y, y3 = y2 * y;
-  e = fma(-r2, y2, 1.0);
-  return fma(y3 * e, fma(1.875, e, 1.5), y3);
+// r^-3 from r^2's seed (see rsqrt_seed); 0 for r = 0
+__device__ __forceinline__ double inv_cube(const RsqrtSeed &s) {
+  const double y3 = s.y2 * s.y;
+  return fma(y3 * s.e, fma(1.875, s.e, 1.5), y3);
 }
 
 // one FP64 pair term: k the target (its mass, 1/r_out and adjoint), j the
-// source; NEAR: with the changeover.  The target itself (r = 0) has y = 0, K =
-// K' = 0.
+// source; NEAR: with the changeover.  A pair within gamma r_out adds nothing:
+// the target itself, bodies so near that r^-3 is infinite, and pairs whose r^2
+// is not finite.
 template <bool VJP, bool NEAR>
 __device__ __forceinline__ void pair_term(double rx, double ry, double rz, double r2,
                                           const Q4<double> &A, double iroj, const Q4<double> &L,
                                           double mk, double irok, double lxk, double lyk,
                                           double lzk, double g, double i1mg, double *acc) {
-  double y, e;
-  double phi = inv_cube(r2, y, e);  // K / r^3 below
+  const RsqrtSeed s = rsqrt_seed(r2);
+  double phi = inv_cube(s);         // K / r^3 below
   double dKr = 0.0, K = 1.0;        // K'(y) / r_out
   if constexpr (NEAR) {
     const double irout = irok < iroj ? irok : iroj;  // 1 / max(r_out,k, r_out,j)
-    const double ir = fma(y * e, fma(0.375, e, 0.5), y);
+    const double ir = fma(s.y * s.e, fma(0.375, s.e, 0.5), s.y);
     const double yv = r2 * ir * irout;
     const double t = (yv - g) * i1mg;
-    // NaN (r = 0 with r_out = 0) stays below
-    const double u = t > 0.0 ? (t < 1.0 ? t : 1.0) : 0.0, u2 = u * u;
+    // NaN too (r = 0 with r_out = 0; an infinite r^2)
+    if (!(t > 0.0)) return;
+    const double u = t < 1.0 ? t : 1.0, u2 = u * u;
     K = (u2 * u2) * fma(fma(fma(-20.0, u, 70.0), u, -84.0), u, 35.0);
     phi *= K;
     if constexpr (VJP) {
-      // zero at both ends also where 1 / r_out is infinite
-      const double v = 1.0 - u, ie = u > 0.0 && u < 1.0 ? irout : 0.0;
+      // zero at the end also where 1 / r_out is infinite
+      const double v = 1.0 - u, ie = u < 1.0 ? irout : 0.0;
       dKr = 140.0 * (u2 * u) * (v * v * v) * i1mg * ie;
     }
   }
@@ -110,7 +109,7 @@ __device__ __forceinline__ void pair_term(double rx, double ry, double rz, doubl
     acc[1] = fma(w, ry, acc[1]);
     acc[2] = fma(w, rz, acc[2]);
   } else {
-    const double y2 = y * y, ir2 = fma(y2, fma(e, e, e), y2);  // y^2 / (1 - e)
+    const double ir2 = fma(s.y2, fma(s.e, s.e, s.e), s.y2);  // y^2 / (1 - e)
     double psi = -3.0 * (phi * ir2);
     if constexpr (NEAR) psi = fma(ir2 * ir2, dKr, psi);
     const double wx = fma(mk, L.x, -A.w * lxk), wy = fma(mk, L.y, -A.w * lyk),
@@ -414,14 +413,16 @@ __global__ void __launch_bounds__(kDW * 32, MIXED ? P3T_DIRECT_MINB_MIXED : 1)
         Q4<T> L{0, 0, 0, 0};
         if constexpr (VJP) L = sL[warp][q];
         double rx[DTL], ry[DTL], rz[DTL], r2[DTL];
-        int low = 0x7fffffff;  // by the leading 32 bits: an FP64 comparison takes the pipe
+        // by the leading 32 bits: an FP64 comparison takes the pipe
+        int low = 0x7fffffff, high = 0;
 #pragma unroll
         for (int t = 0; t < DTL; ++t) {
           rx[t] = txh[t] - A.x; ry[t] = tyh[t] - A.y; rz[t] = tzh[t] - A.z;
           r2[t] = fma(rx[t], rx[t], fma(ry[t], ry[t], rz[t] * rz[t]));
           low = min(low, __double2hiint(r2[t]));
+          high = max(high, __double2hiint(r2[t]));
         }
-        if (__any_sync(0xffffffffu, low <= hT)) {
+        if (__any_sync(0xffffffffu, low <= hT || high >= 0x7ff00000)) {  // or not finite
 #pragma unroll
           for (int t = 0; t < DTL; ++t)
             pair_term<VJP, true>(rx[t], ry[t], rz[t], r2[t], A, B.w, L, tm[t], tiro[t], tlx[t],

@@ -1545,8 +1545,8 @@ __global__ void __launch_bounds__(kEThreads) k_energy(p3t_particles p, p3t_param
           for (int t = 0; t < 2; ++t) {
             const double dx = X[t] - hx, dy = Y[t] - hy, dz = Z[t] - hz;
             const double r2 = __fma_rn(dx, dx, __fma_rn(dy, dy, dz * dz));
-            const double y = rsqrt_seed(r2), e = __fma_rn(-r2, y * y, 1.0);
-            double ir = __fma_rn(y * e, __fma_rn(0.375, e, 0.5), y);
+            const RsqrtSeed u = rsqrt_seed(r2);
+            double ir = __fma_rn(u.y * u.e, __fma_rn(0.375, u.e, 0.5), u.y);
             // two bodies at one place: infinite, as 1 / r; the target itself: none
             if (__double_as_longlong(r2) == 0)
               ir = J == row && q == t * kEThreads + tid

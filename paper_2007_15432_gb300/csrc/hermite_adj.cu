@@ -270,7 +270,8 @@ __device__ __forceinline__ TanOut hard_tangent(int nc, int k, int b0, int row0, 
     row3(dv, b0, du);
     const double r2 = dot3(r, r), s = dot3(r, dr), rv = dot3(r, u);
     const double drv = dot3(dr, u) + dot3(r, du);
-    const double y = rsqrt_seed(r2), y2 = y * y, e = __fma_rn(-r2, y2, 1.0), y3 = y2 * y;
+    const RsqrtSeed i = rsqrt_seed(r2);
+    const double y = i.y, y2 = i.y2, e = i.e, y3 = y2 * y;
     const double ri3 = __fma_rn(y3 * e, __fma_rn(1.875, e, 1.5), y3);
     const double ri2 = __fma_rn(y2, __fma_rn(e, e, e), y2);
     const double g = -hc.gms * ri3, h = ri2 * s, r3i2 = 3.0 * ri2;
@@ -298,7 +299,8 @@ __device__ __forceinline__ TanOut hard_tangent(int nc, int k, int b0, int row0, 
     row3(duc, b0, du);
     const double r2 = dot3(r, r), s = dot3(r, dr), rv = dot3(r, u);
     const double drv = dot3(dr, u) + dot3(r, du);
-    const double y = rsqrt_seed(r2), y2 = y * y, e = __fma_rn(-r2, y2, 1.0), y3 = y2 * y;
+    const RsqrtSeed i = rsqrt_seed(r2);
+    const double y = i.y, y2 = i.y2, e = i.e, y3 = y2 * y;
     const double ri3 = __fma_rn(y3 * e, __fma_rn(1.875, e, 1.5), y3);
     const double ri2 = __fma_rn(y2, __fma_rn(e, e, e), y2);
     const double ri = __fma_rn(y * e, __fma_rn(0.375, e, 0.5), y);

@@ -80,11 +80,26 @@ __device__ __forceinline__ FF ff_rsqrt(FF r2) {
 static __device__ __noinline__ double rsqrt_rare(double x) {
   return __double_as_longlong(x) == 0 ? 0.0 : rsqrt(x);
 }
-__device__ __forceinline__ double rsqrt_seed(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  if ((unsigned)((__double2hiint(x) >> 20) - 512) >= 1024u) y = rsqrt_rare(x);
-  return y;
+static __device__ __noinline__ double2 rsqrt_rare2(double x) {
+  if (__double_as_longlong(x) == 0) return make_double2(0.0, 0.0);
+  const double y = rsqrt(x);
+  return make_double2(y, y * y);
+}
+struct RsqrtSeed {
+  double y, y2, e;  // y^2; out of range e = 0 (1 - x y^2 would be NaN for x = infinity)
+};
+__device__ __forceinline__ RsqrtSeed rsqrt_seed(double x) {
+  RsqrtSeed s;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(s.y) : "d"(x));
+  s.y2 = s.y * s.y;
+  s.e = __fma_rn(-x, s.y2, 1.0);
+  if ((unsigned)((__double2hiint(x) >> 20) - 512) >= 1024u) {
+    const double2 r = rsqrt_rare2(x);
+    s.y = r.x;
+    s.y2 = r.y;
+    s.e = 0.0;
+  }
+  return s;
 }
 // x 2^k in FP32 from the leading 20 bits of x (relative error below 2^-20,
 // towards zero); zero below and infinity above FP32's normal range

@@ -851,17 +851,18 @@ __device__ __forceinline__ bool far_from64(const FarBox &b, double X, double Y, 
   return d2 > 1e-30f && d2 < 3e38f && d2 >= R * R;
 }
 
-// m r^-3 from r^2 (zero for r = 0): the seed's y, e = 1 - r^2 y^2 and the
-// result (see rsqrt_seed)
+// m r^-3 from r^2 (zero for r = 0 and where r^2 is infinite): the seed's y, y^2
+// and e = 1 - r^2 y^2 and the result (see rsqrt_seed)
 struct Inv3 {
-  double y, e, f;
+  double y, y2, e, f;
 };
 __device__ __forceinline__ Inv3 inv_cube(double r2, double m) {
   Inv3 v;
-  v.y = rsqrt_seed(r2);
-  const double y2 = v.y * v.y;
-  v.e = fma(-r2, y2, 1.0);
-  const double t = y2 * (v.y * m);
+  const RsqrtSeed s = rsqrt_seed(r2);
+  v.y = s.y;
+  v.y2 = s.y2;
+  v.e = s.e;
+  const double t = v.y2 * (v.y * m);
   v.f = fma(t * v.e, fma(1.875, v.e, 1.5), t);
   return v;
 }
@@ -954,7 +955,7 @@ struct Eval64 {
       const double dx = t.x[i] - c0.x, dy = t.y[i] - c0.y, dz = t.z[i] - c1.x;
       const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
       const Inv3 v = inv_cube(r2, 1.0);
-      const double ri3 = v.f, y2 = v.y * v.y;
+      const double ri3 = v.f, y2 = v.y2;
       const double ri2 = fma(y2, fma(v.e, v.e, v.e), y2);  // y^2 / (1 - e)
       const double qx = fma(qxx, dx, fma(qxy, dy, qxz * dz));
       const double qy = fma(qxy, dx, fma(qyy, dy, qyz * dz));
@@ -1107,7 +1108,7 @@ struct VjpEval {
       const double lx = t.lx[i], ly = t.ly[i], lz = t.lz[i];
       const double r2 = fma(rx, rx, fma(ry, ry, rz * rz));
       const Inv3 v = inv_cube(r2, 1.0);
-      const double ri3 = v.f, y2 = v.y * v.y;
+      const double ri3 = v.f, y2 = v.y2;
       const double ri2 = fma(y2, fma(v.e, v.e, v.e), y2);
       const double ri5 = ri3 * ri2;
       const double qx = fma(q0.x, rx, fma(q1.y, ry, q2.x * rz));
@@ -1158,7 +1159,7 @@ struct VjpEval {
       const double lx = t.lx[i], ly = t.ly[i], lz = t.lz[i];
       const double r2 = fma(rx, rx, fma(ry, ry, rz * rz));
       const Inv3 v = inv_cube(r2, 1.0);
-      const double y2 = v.y * v.y;
+      const double y2 = v.y2;
       const double ri2 = fma(y2, fma(v.e, v.e, v.e), y2);
       double phi = v.f, psi;
       if (near) {
@@ -1172,6 +1173,7 @@ struct VjpEval {
         const double dK = (140.0 * a.inv1mg) * ((x2 * x) * (u * u * u)) * (inside01(x) ? irot : 0.0);
         psi = fma(dK, ri2 * ri2, -3.0 * K * (phi * ri2));
         phi *= K;
+        if (__double_as_longlong(x) == 0) phi = psi = 0.0;  // also where r^-3 is infinite
       } else {
         psi = -3.0 * (phi * ri2);
       }
