@@ -1,6 +1,7 @@
 // Soft step: neighbour lists and neighbour clusters
 // (Sec. 2.3).  Compiled with -fmad=false: the neighbour predicate is decided
 // in FP64 with a fixed evaluation order so that membership is bit-exact.
+#include "block_sort.cuh"
 #include "p3t_internal.cuh"
 
 namespace {
@@ -76,17 +77,18 @@ __global__ void k_nb_fill(const int64_t *d_ncand, const int32_t *cand_i,
 }
 
 // rows are short (<n_b> << 1 in the paper's runs): insertion sort per row; and
-// the start of the union-find: every particle its own root, counts zero
+// the start of the union-find: every particle its own root, of one member
 __global__ void k_nb_sort_rows(int64_t n, const int64_t *nb_off, int32_t *nb_idx,
                                int32_t *parent, int32_t *csize, int64_t *cl_counts,
-                               const DevStatus *st) {
+                               unsigned long long *huge, const DevStatus *st) {
   pdl_wait();
   if (blockIdx.x == 0 && threadIdx.x < 4) cl_counts[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 2) huge[threadIdx.x] = 0ull;
   const bool failed = st->code != 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     parent[i] = (int32_t)i;
-    csize[i] = 0;
+    csize[i] = 1;
     if (failed) continue;
     const int64_t b = nb_off[i], e = nb_off[i + 1];
     for (int64_t u = b + 1; u < e; ++u) {
@@ -128,21 +130,61 @@ __global__ void k_uf_union(int64_t n, const int64_t *nb_off, const int32_t *nb_i
   }
 }
 
+// each particle's root, the clusters' sizes (a root counts itself from the start)
+// and, from their counting, the others' places among their cluster's members (in
+// any order).  A warp's members of one cluster are counted by one addition
 __global__ void k_uf_label(int64_t n, const int32_t *parent, int32_t *label,
-                           int32_t *csize) {
+                           int32_t *csize, int32_t *place) {
   pdl_wait();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t r = uf_find(parent, (int32_t)i);
-    label[i] = r;
-    atomicAdd(&csize[r], 1);
+  const int lane = threadIdx.x & 31;
+  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x - lane); i0 < n;
+       i0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = i0 + lane;
+    int32_t r = -1;
+    if (i < n) {
+      r = uf_find(parent, (int32_t)i);
+      label[i] = r;
+      if (r == i) r = -1;
+    }
+    if (!__any_sync(0xffffffffu, r >= 0)) continue;
+    const unsigned same = __match_any_sync(0xffffffffu, r);
+    const int first = __ffs(same) - 1;
+    int32_t at = 0;
+    if (r >= 0 && lane == first) at = atomicAdd(&csize[r], __popc(same));
+    at = __shfl_sync(0xffffffffu, at, first);
+    if (r >= 0) place[i] = at + __popc(same & ((1u << lane) - 1u));
   }
 }
 
-// flags: [0, n) isolated, [n, 2n) cluster roots, [2n, 3n) root sizes,
-// [3n, 4n) members of clusters of >= 2
+// The members of every cluster in index order.  A cluster is a few members almost
+// always, but close to percolation there are many of any size, so each size has
+// a form of its own and consecutive clusters go to different blocks: a thread
+// sorts up to eight members in registers, a warp ranks up to 32 and sorts up to
+// 256, a block sorts up to kMemMax in shared memory.  Larger ones (at most n /
+// kMemMax) are numbered and placed in order: the particles are cut into kSlices
+// equal slices, k_cl_scatter counts each such cluster's members in each slice
+// and sums the counts before, and a warp a slice then writes its members.
+// Bound by its launch and the members' latency: equal-mass ring, N = 1e5, 4 us,
+// wide disk, N = 1e6, 5; sorting all members by label took three radix passes and
+// a copy, some 55 us in both.  The whole neighbour stage near percolation, with
+// that sort, with one block for all clusters above 32 members, and now: 1,000
+// clusters of 40 in 1e5 particles 100, 1,090, 71 us; 1,000 of 600 in 1e6 326,
+// 8,600, 320; 900 of 1,030 457, 229,000, 434; one of 200,000 340, 740, 328.
+constexpr int kMemThreads = 1024, kMemSmall = 8, kMemMax = kMemThreads * kItems;
+constexpr int kSlices = 1024;
+// the clusters above kMemMax: how many, the number of a root's cluster and, in the
+// union-find's words (free by then, n of them), a row of kSlices counts each
+struct Huge {
+  unsigned long long *count;  // [1]: the blocks of k_cl_scatter done
+  int32_t *number, *words;
+  __device__ __forceinline__ int32_t *row(int64_t h) const { return words + h * kSlices; }
+};
+__device__ __forceinline__ int slice_len(int64_t n) { return (int)((n + kSlices - 1) / kSlices); }
+
+// two flag words a particle: [0, n) isolated, member of a cluster; [n, 2n) root of
+// a cluster and its size
 __global__ void k_cl_flags(int64_t n, const int32_t *label, const int32_t *csize,
-                           int32_t *flag, int64_t *counts) {
+                           int32_t *flag, int64_t *counts, Huge huge) {
   pdl_wait();
   unsigned long long mx = 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -156,17 +198,24 @@ __global__ void k_cl_flags(int64_t n, const int32_t *label, const int32_t *csize
     if (root) mx = max(mx, (unsigned long long)csize[i]);
   }
   if (mx) atomicMax(reinterpret_cast<unsigned long long *>(&counts[3]), mx);
+  if (mx <= kMemMax) return;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (label[i] != i || csize[i] <= kMemMax) continue;
+    const int64_t h = (int64_t)atomicAdd(huge.count, 1ull);
+    huge.number[i] = (int32_t)h;
+    int4 *row = reinterpret_cast<int4 *>(huge.row(h));
+    for (int q = 0; q < kSlices / 4; ++q) row[q] = make_int4(0, 0, 0, 0);
+  }
 }
 
-constexpr int kMemMax = 1024;  // members that a block ranks in shared memory
-
-// the singles, each cluster's offset and its members (in any order: the root's
-// size counts down to zero) from the two packed scans (counts in bits 0-30, the
-// second sum from bit 31), and the totals: singles, clusters, members
-// (counts[0..2])
+// the singles, each cluster's offset and its members (in any order, by their
+// places) from the two packed scans (counts in bits 0-30, the second sum from
+// bit 31), and the totals: singles, clusters, members (counts[0..2])
 __global__ void k_cl_scatter(int64_t n, const int32_t *label, const int32_t *flag,
                              const int64_t *pos, const int64_t *d_tot, int32_t *singles,
-                             int64_t *cl_off, int32_t *csize, int32_t *mem, int64_t *counts) {
+                             int64_t *cl_off, const int32_t *place, int32_t *mem, int64_t *counts,
+                             Huge huge) {
   pdl_wait();
   constexpr int64_t kLow = (1ll << 31) - 1;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -178,13 +227,12 @@ __global__ void k_cl_scatter(int64_t n, const int32_t *label, const int32_t *fla
       cl_off[q & kLow] = q >> 31;
     }
     if (fa & 2) {
-      // (of a cluster that will be listed from the labels, the root only)
+      // (those of a cluster above kMemMax are counted by slice)
       const int32_t r = label[i];
-      const int64_t o = pos[n + r] >> 31;
       if ((flag[n + r] >> 1) <= kMemMax)
-        mem[o + atomicSub(&csize[r], 1) - 1] = (int32_t)i;
-      else if (i == r)
-        mem[o] = r;
+        mem[(pos[n + r] >> 31) + (r == i ? 0 : place[i])] = (int32_t)i;
+      else
+        atomicAdd(&huge.row(huge.number[r])[(int)i / slice_len(n)], 1);
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -194,77 +242,91 @@ __global__ void k_cl_scatter(int64_t n, const int32_t *label, const int32_t *fla
     counts[2] = tb >> 31;
     cl_off[tb & kLow] = tb >> 31;
   }
+  const int64_t nh = (int64_t)*huge.count;
+  if (nh == 0) return;
+  // the last block to finish: each row of counts to the sums of those before
+  __threadfence();
+  __syncthreads();
+  if (!__syncthreads_or(threadIdx.x == 0 && atomicAdd(&huge.count[1], 1ull) == gridDim.x - 1))
+    return;
+  __threadfence();
+  const int lane = threadIdx.x & 31;
+  for (int64_t h = threadIdx.x >> 5; h < nh; h += blockDim.x >> 5) {
+    int32_t *row = huge.row(h);
+    int run = 0;
+    for (int q = lane; q < kSlices; q += 128) {
+      int c[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) c[k] = __ldcg(&row[q + 32 * k]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        int v = c[k];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int u = __shfl_up_sync(0xffffffffu, v, o);
+          if (lane >= o) v += u;
+        }
+        row[q + 32 * k] = run + v - c[k];
+        run += __shfl_sync(0xffffffffu, v, 31);
+      }
+    }
+  }
 }
 
-// The members of every cluster in index order.  A cluster is a few members
-// almost always: a thread sorts up to eight in registers, a warp ranks up to 32, a
-// block up to kMemMax in shared memory, and lists a larger one anew from the
-// labels (one pass over the particles).  Bound by its launch and the members'
-// latency: equal-mass ring, N = 1e5, 4 us, wide disk, N = 1e6, 5; sorting all
-// members by label took three radix passes and a copy, some 55 us in both.  One
-// cluster of 5,000 of 1e6 particles takes some 200 us, less than one block step of
-// its Hermite pairs.
-constexpr int kMemThreads = 1024, kMemSmall = 8;
-__device__ void rank_members(int32_t *mem, int m, int32_t *s) {
-  for (int e = threadIdx.x; e < m; e += kMemThreads) s[e] = mem[e];
-  __syncthreads();
-  for (int e = threadIdx.x; e < m; e += kMemThreads) {
-    const int32_t v = s[e];
-    int rank = 0;
-    for (int j = 0; j < m; ++j) rank += s[j] < v;
-    mem[rank] = v;
-  }
-  __syncthreads();
-}
-// the particles labelled r (the smallest of them) into mem[0, m): a warp takes
-// 32 rows of 32 particles a pass, their loads in flight together, a lane
-// keeping each row's mask; s: the warps' counts
-__device__ void list_members(int64_t n, const int32_t *label, int32_t r, int32_t *mem, int m,
-                             int32_t *s) {
-  constexpr int kRows = 32;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int done = 0;
-  for (int64_t b = r; b < n && done < m; b += kMemThreads * kRows) {
-    const int64_t b0 = b + (int64_t)w * 32 * kRows;
-    unsigned rows = 0;  // lane k: the mask of row k
+// the members of the clusters above kMemMax, a warp a slice of the particles (its
+// cluster's word of the row is the warp's own)
+__device__ void place_huge(int64_t n, const Huge &huge, const int32_t *label, const int32_t *flag,
+                           const int64_t *pos, int32_t *mem) {
+  const int lane = threadIdx.x & 31, len = slice_len(n);
+  const int64_t warps = (int64_t)gridDim.x * (kMemThreads / 32);
+  // neighbouring slices to different blocks
+  for (int64_t sl = blockIdx.x + (int64_t)gridDim.x * (threadIdx.x >> 5); sl < kSlices;
+       sl += warps) {
+    const int64_t i0 = sl * len, i1 = min(n, i0 + len);
+    constexpr int kRows = 4;  // rows of 32 whose loads are in flight together
+    for (int64_t b = i0; b < i1; b += 32 * kRows) {
+      int32_t r[kRows], h[kRows];
+      int64_t o[kRows];
 #pragma unroll
-    for (int k = 0; k < kRows; ++k) {
-      const int64_t i = b0 + 32 * k + lane;
-      const unsigned in = __ballot_sync(0xffffffffu, i < n && label[i] == r);
-      if (lane == k) rows = in;
-    }
-    const int own = __reduce_add_sync(0xffffffffu, __popc(rows));
-    if (lane == 0) s[w] = own;
-    __syncthreads();
-    int at = done;
-    for (int q = 0; q < kMemThreads / 32; ++q) {
-      if (q < w) at += s[q];
-      done += s[q];
-    }
-    if (own)
-#pragma unroll 4
       for (int k = 0; k < kRows; ++k) {
-        const unsigned in = __shfl_sync(0xffffffffu, rows, k);
-        const int o = at + __popc(in & ((1u << lane) - 1u));
-        if (((in >> lane) & 1u) && o < m) mem[o] = (int32_t)(b0 + 32 * k + lane);
-        at += __popc(in);
+        const int64_t i = b + 32 * k + lane;
+        r[k] = i < i1 ? label[i] : -1;
       }
-    __syncthreads();
+#pragma unroll
+      for (int k = 0; k < kRows; ++k) {
+        const bool on = r[k] >= 0 && (flag[n + r[k]] >> 1) > kMemMax;
+        h[k] = on ? huge.number[r[k]] : -1;
+        o[k] = on ? pos[n + r[k]] >> 31 : 0;
+      }
+#pragma unroll
+      for (int k = 0; k < kRows; ++k) {
+        const unsigned same = __match_any_sync(0xffffffffu, h[k]);
+        const int first = __ffs(same) - 1;
+        int32_t at = 0;
+        if (h[k] >= 0 && lane == first) at = atomicAdd(&huge.row(h[k])[sl], __popc(same));
+        at = __shfl_sync(0xffffffffu, at, first);
+        if (h[k] >= 0)
+          mem[o[k] + at + __popc(same & ((1u << lane) - 1u))] = (int32_t)(b + 32 * k + lane);
+      }
+    }
   }
 }
+
 __global__ void __launch_bounds__(kMemThreads) k_cl_sort(const int64_t *counts,
                                                          const int64_t *cl_off, int64_t n,
-                                                         const int32_t *label, int32_t *mem) {
+                                                         const int32_t *label, const int32_t *flag,
+                                                         const int64_t *pos, int32_t *mem,
+                                                         Huge huge) {
   pdl_wait();
-  __shared__ int32_t s_mem[kMemMax];
+  __shared__ uint32_t s_mem[kMemMax + kMemMax / 8];
   __shared__ int s_list[2][kMemThreads], s_n[2];  // clusters for a warp, for the block
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t ncl = counts[1];
-  for (int64_t c0 = (int64_t)blockIdx.x * kMemThreads; c0 < ncl;
-       c0 += (int64_t)gridDim.x * kMemThreads) {
+  const int64_t ncl = counts[1], nh = (int64_t)*huge.count;
+  // clusters b, b + gridDim, b + 2 gridDim, ... to block b
+  for (int64_t t0 = 0; blockIdx.x + gridDim.x * t0 < ncl; t0 += kMemThreads) {
     if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t c = c0 + threadIdx.x;
+    const int64_t c = blockIdx.x + gridDim.x * (t0 + threadIdx.x);
     if (c < ncl) {
       const int64_t o = cl_off[c];
       const int m = (int)(cl_off[c + 1] - o);
@@ -286,33 +348,43 @@ __global__ void __launch_bounds__(kMemThreads) k_cl_sort(const int64_t *counts,
 #pragma unroll
         for (int k = 0; k < kMemSmall; ++k)
           if (k < m) mem[o + k] = v[k];
-      } else {
-        const int q = m > 32;
+      } else if (m <= kMemMax) {
+        const int q = m > 32 * kItems;
         s_list[q][atomicAdd(&s_n[q], 1)] = threadIdx.x;
       }
     }
     __syncthreads();
     for (int q = w; q < s_n[0]; q += kMemThreads / 32) {
-      const int64_t d = c0 + s_list[0][q], o = cl_off[d];
+      const int64_t d = blockIdx.x + gridDim.x * (t0 + s_list[0][q]), o = cl_off[d];
       const int m = (int)(cl_off[d + 1] - o);
-      const int32_t v = lane < m ? mem[o + lane] : 0x7fffffff;
-      int rank = 0;
-      for (int j = 0; j < m; ++j) rank += __shfl_sync(0xffffffffu, v, j) < v;
-      if (lane < m) mem[o + rank] = v;
+      if (m <= 32) {
+        const int32_t v = lane < m ? mem[o + lane] : 0x7fffffff;
+        int rank = 0;
+        for (int j = 0; j < m; ++j) rank += __shfl_sync(0xffffffffu, v, j) < v;
+        if (lane < m) mem[o + rank] = v;
+      } else {
+        uint32_t v[kItems];
+#pragma unroll
+        for (int k = 0; k < kItems; ++k)
+          v[k] = 32 * k + lane < m ? (uint32_t)mem[o + 32 * k + lane] : ~0u;
+        warp_sort(v);
+#pragma unroll
+        for (int k = 0; k < kItems; ++k)
+          if (kItems * lane + k < m) mem[o + kItems * lane + k] = (int32_t)v[k];
+      }
     }
     for (int q = 0; q < s_n[1]; ++q) {
-      const int64_t d = c0 + s_list[1][q], o = cl_off[d];
+      const int64_t d = blockIdx.x + gridDim.x * (t0 + s_list[1][q]), o = cl_off[d];
       const int m = (int)(cl_off[d + 1] - o);
-      if (m <= kMemMax) {
-        rank_members(mem + o, m, s_mem);
-      } else {
-        const int32_t r = mem[o];
-        __syncthreads();  // mem[o] is read before it is written
-        list_members(n, label, r, mem + o, m, s_mem);
-      }
+      for (int e = threadIdx.x; e < m; e += kMemThreads) s_mem[slot(e)] = (uint32_t)mem[o + e];
+      __syncthreads();
+      sort_words(s_mem, m);
+      for (int e = threadIdx.x; e < m; e += kMemThreads) mem[o + e] = (int32_t)s_mem[slot(e)];
+      __syncthreads();
     }
     __syncthreads();
   }
+  if (nh > 0) place_huge(n, huge, label, flag, pos, mem);
 }
 
 }  // namespace
@@ -325,6 +397,10 @@ int p3t_run_neighbours(p3t_ctx *c, const p3t_particles *p, int64_t *nb_off,
   const int64_t gc = p3t_grid(c->cand_cap, kBlock, maxb);
   int64_t *cnt = c->counters;
   int rc;
+  // (counters[28], [29]; the rows' degrees are spent when the roots are numbered;
+  // the third quarter of the flags holds the places)
+  const Huge huge{reinterpret_cast<unsigned long long *>(&cnt[28]), c->deg, c->parent};
+  int32_t *place = c->flag + 2 * c->cap;
   // ---- neighbour lists ----
   P3T_CUDA_TRY(cudaMemsetAsync(c->deg, 0, sizeof(int32_t) * (n + 1), s));
   pdl_launch(k_nb_filter, dim3((unsigned)gc), dim3(kBlock), 0, s, &cnt[9], c->cand_i, c->cand_j, c->idx, *p,
@@ -334,11 +410,11 @@ int p3t_run_neighbours(p3t_ctx *c, const p3t_particles *p, int64_t *nb_off,
   pdl_launch(k_nb_fill, dim3((unsigned)gc), dim3(kBlock), 0, s, &cnt[9], c->cand_i, c->cand_j,
              c->idx, c->cand_keep, nb_off, nb_off + n, nb_cap, c->deg, nb_idx, c->status);
   pdl_launch(k_nb_sort_rows, dim3((unsigned)g), dim3(kBlock), 0, s, n, nb_off, nb_idx, c->parent,
-             c->csize, c->cl_counts, c->status);
+             c->csize, c->cl_counts, huge.count, c->status);
   // ---- neighbour clusters ----
   pdl_launch(k_uf_union, dim3((unsigned)g), dim3(kBlock), 0, s, n, nb_off, nb_idx, c->parent, c->status);
-  pdl_launch(k_uf_label, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->parent, c->label, c->csize);
-  pdl_launch(k_cl_flags, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->label, c->csize, c->flag, c->cl_counts);
+  pdl_launch(k_uf_label, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->parent, c->label, c->csize, place);
+  pdl_launch(k_cl_flags, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->label, c->csize, c->flag, c->cl_counts, huge);
   // two packed scans: (isolated, members) and (roots, root sizes); their
   // totals in cnt[21], cnt[22]
   for (int q = 0; q < 2; ++q) {
@@ -350,9 +426,9 @@ int p3t_run_neighbours(p3t_ctx *c, const p3t_particles *p, int64_t *nb_off,
   // addresses from step to step (a step captured in a CUDA graph reads the
   // previous step's clusters there)
   pdl_launch(k_cl_scatter, dim3((unsigned)g), dim3(kBlock), 0, s, n, c->label, c->flag, c->pos,
-             &cnt[21], c->singles, c->cl_off, c->csize, c->mvals, c->cl_counts);
+             &cnt[21], c->singles, c->cl_off, place, c->mvals, c->cl_counts, huge);
   pdl_launch(k_cl_sort, dim3((unsigned)p3t_grid(n / 2 + 1, kMemThreads, c->num_sms)), dim3(kMemThreads), 0,
-             s, c->cl_counts, c->cl_off, n, c->label, c->mvals);
+             s, c->cl_counts, c->cl_off, n, c->label, c->flag, c->pos, c->mvals, huge);
   // filter, fill, sort_rows, uf_union, uf_label, flags, scatter, sort
   p3t_note_launches(8);
   c->cl_mem = c->mvals;

@@ -1,6 +1,7 @@
 // Device-wide primitives of libp3t: exclusive scan and stable LSD radix sort.
 // Element counts are read from device memory so that a whole soft step can be
 // enqueued (and captured in a CUDA graph) without reading sizes on the host.
+#include "block_sort.cuh"
 #include "p3t_internal.cuh"
 
 namespace {
@@ -369,7 +370,6 @@ radix_downsweep(const uint64_t *keys, const int32_t *vals, uint64_t *okeys,
 // buckets' blocks (three of 512 threads an SM beat two, and blocks of 256 with
 // buckets of 2,048: 339, 348, 346 us).  Keys of 32 bits or less keep the radix
 // passes (cut-off bins of 377,740: 40 against 76 us).
-constexpr int kItems = 8;                 // a thread's run of sorted keys
 constexpr int kBlockSortMax = 1024 * kItems;
 static_assert(kBlockSortMax == P3T_SORT_BLOCK, "one block's sort");
 constexpr int kLocalThreads = 512;
@@ -390,16 +390,7 @@ struct SortWork {
 __device__ __forceinline__ bool pair_less(uint64_t ka, int32_t va, uint64_t kb, int32_t vb) {
   return ka < kb || (ka == kb && va < vb);
 }
-// shared-memory slot of entry i (a word skipped every eight: a thread's runs
-// start in different banks)
-__device__ __forceinline__ int slot(int i) { return i + (i >> 3); }
 constexpr size_t sort_smem(int max) { return (size_t)(max + max / 8) * 12; }
-
-__device__ __forceinline__ void sort2(uint64_t &a, uint64_t &b) {
-  const uint64_t x = a < b ? a : b;
-  b = a < b ? b : a;
-  a = x;
-}
 
 // One 64-bit word per entry: the leading bits of its key (kb bits, taken
 // relative to the smallest possible one), as much of its value (vb bits) as
@@ -421,91 +412,6 @@ struct WordSpec {
     return u << kPlace | (uint64_t)place;
   }
 };
-
-// the words [0, n) in shared memory sorted by the block: eight a thread by an
-// odd-even merge network, up to 256 a warp by bitonic merges in registers
-// (no barrier), then merge rounds through shared memory, each thread taking
-// the eight outputs that its merge-path search gives it
-__device__ void sort_words(uint64_t *sk, int n) {
-  const int i0 = threadIdx.x * kItems, lane = threadIdx.x & 31;
-  const bool in = i0 < n;
-  uint64_t k[kItems];
-  if ((int)(threadIdx.x & ~31u) * kItems < n) {  // the warp holds entries
-#pragma unroll
-    for (int q = 0; q < kItems; ++q) k[q] = i0 + q < n ? sk[slot(i0 + q)] : ~0ull;
-    // Batcher's odd-even merge sort of eight
-#pragma unroll
-    for (int p = 1; p < kItems; p <<= 1)
-#pragma unroll
-      for (int h = p; h > 0; h >>= 1)
-#pragma unroll
-        for (int j = h % p; j + h < kItems; j += 2 * h)
-#pragma unroll
-          for (int i = 0; i < h; ++i)
-            if (j + i + h < kItems && (j + i) / (2 * p) == (j + i + h) / (2 * p))
-              sort2(k[j + i], k[j + i + h]);
-    // runs of L lanes -> runs of 2 L lanes: the second run taken backwards,
-    // then half-cleaners across lanes and within the thread
-#pragma unroll
-    for (int L = 1; L < 32; L <<= 1) {
-      uint64_t o[kItems];
-#pragma unroll
-      for (int q = 0; q < kItems; ++q)
-        o[q] = __shfl_xor_sync(0xffffffffu, k[kItems - 1 - q], 2 * L - 1);
-      const bool up = (lane & L) != 0;
-#pragma unroll
-      for (int q = 0; q < kItems; ++q) k[q] = (k[q] < o[q]) != up ? k[q] : o[q];
-#pragma unroll
-      for (int h = L >> 1; h > 0; h >>= 1) {
-        const bool hi = (lane & h) != 0;
-#pragma unroll
-        for (int q = 0; q < kItems; ++q) {
-          const uint64_t x = __shfl_xor_sync(0xffffffffu, k[q], h);
-          k[q] = (k[q] < x) != hi ? k[q] : x;
-        }
-      }
-#pragma unroll
-      for (int h = kItems / 2; h > 0; h >>= 1)
-#pragma unroll
-        for (int q = 0; q < kItems; ++q)
-          if (!(q & h)) sort2(k[q], k[q + h]);
-    }
-#pragma unroll
-    for (int q = 0; q < kItems; ++q)
-      if (i0 + q < n) sk[slot(i0 + q)] = k[q];
-  }
-  __syncthreads();
-  for (int w = 32 * kItems; w < n; w <<= 1) {
-    if (in) {
-      const int base = i0 & ~(2 * w - 1), diag = i0 - base;
-      const int a1 = min(base + w, n), b1 = min(base + 2 * w, n);
-      int lo = max(0, diag - (b1 - a1)), hi = min(diag, a1 - base);
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (sk[slot(base + mid)] < sk[slot(a1 + diag - 1 - mid)]) lo = mid + 1; else hi = mid;
-      }
-      int ia = base + lo, ib = a1 + diag - lo;
-      uint64_t ka = ia < a1 ? sk[slot(ia)] : ~0ull, kb = ib < b1 ? sk[slot(ib)] : ~0ull;
-#pragma unroll
-      for (int q = 0; q < kItems; ++q) {
-        const bool ta = ka <= kb;  // words are distinct but for the filler
-        k[q] = ta ? ka : kb;
-        ia += ta;
-        ib += !ta;
-        const int nx = ta ? ia : ib;
-        const uint64_t nk = nx < (ta ? a1 : b1) ? sk[slot(nx)] : ~0ull;
-        if (ta) ka = nk; else kb = nk;
-      }
-    }
-    __syncthreads();
-    if (in) {
-#pragma unroll
-      for (int q = 0; q < kItems; ++q)
-        if (i0 + q < n) sk[slot(i0 + q)] = k[q];
-    }
-    __syncthreads();
-  }
-}
 
 // entries [0, n) of (sk, sv) sorted by (key, value) in merge rounds: the plain
 // form for entries that sort_words cannot tell apart
