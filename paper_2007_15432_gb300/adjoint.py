@@ -25,7 +25,9 @@ kernels:
   * states are checkpointed every ``checkpoint`` steps; the backward pass
     recomputes each segment forward from its checkpoint, up to its last drift.
     The last segment, which the backward pass takes first, is kept by the
-    forward pass (the memory that one recomputed segment takes).
+    forward pass and given up once it is swept: no more than a recomputed
+    segment's memory, but held from the forward pass on (by each of several
+    rollouts in one graph).
 
 Positions and velocities are (3, n) float64 CUDA tensors (rows x, y, z).
 """
@@ -137,12 +139,11 @@ class SoftKDK:
             P.p3t_kick(self.ctx, st, self.acc, h)
 
     # ---- sweeps --------------------------------------------------------------
-    def forward(self, x0, v0, m, r_out, r_search=None):
-        """Returns (x_N, v_N, tape); the tape holds the checkpoints.  The tree
-        force needs the frozen search radii as well (``r_search``)."""
-        return self._forward(x0, v0, m, r_out, r_search, True)
-
-    def _forward(self, x0, v0, m, r_out, r_search, keep_last: bool):
+    def forward(self, x0, v0, m, r_out, r_search=None, keep_last: bool = True):
+        """Returns (x_N, v_N, tape); the tape holds the checkpoints and, with
+        ``keep_last``, the last segment's states (without: the backward pass
+        recomputes them; for a forward sweep alone, or to save memory).  The
+        tree force needs the frozen search radii as well (``r_search``)."""
         if self.force == "tree":
             if r_search is None:
                 raise ValueError("the tree force needs r_search")
@@ -169,7 +170,8 @@ class SoftKDK:
                           vN=V.clone())
 
     def backward(self, tape, lam_x, lam_v):
-        """Adjoints (dL/dx_0, dL/dv_0, dL/dm) from those of (x_N, v_N)."""
+        """Adjoints (dL/dx_0, dL/dv_0, dL/dm) from those of (x_N, v_N).  Takes
+        the kept last segment from the tape (a second sweep recomputes it)."""
         dt, h = self.params.dt_soft, 0.5 * self.params.dt_soft
         m, r_out = tape["m"], tape["r_out"]
         lx = lam_x.detach().clone().contiguous()
@@ -180,8 +182,8 @@ class SoftKDK:
         for k0, Xc, Vc, clc in reversed(tape["checkpoints"]):
             k1 = min(self.steps, k0 + self.checkpoint)
             keep = []
-            if k1 == self.steps and tape["last"] is not None:
-                keep = tape["last"]
+            if k1 == self.steps and tape.get("last") is not None:
+                keep = tape.pop("last")
             elif clc is not None:
                 # the checkpoint's force and clusters, as in the forward sweep
                 X, V = Xc.clone(), Vc.clone()
@@ -209,8 +211,9 @@ class SoftKDK:
 
 class _KDK(torch.autograd.Function):
     @staticmethod
-    def forward(ctx, x0, v0, m, r_out, runner, r_search):
-        xN, vN, tape = runner._forward(x0, v0, m, r_out, r_search, any(ctx.needs_input_grad))
+    def forward(ctx, x0, v0, m, r_out, runner, r_search, graph):
+        xN, vN, tape = runner.forward(x0, v0, m, r_out, r_search,
+                                      graph and any(ctx.needs_input_grad))
         ctx.runner, ctx.tape = runner, tape
         return xN, vN
 
@@ -219,12 +222,12 @@ class _KDK(torch.autograd.Function):
         r = ctx.runner
         z = torch.zeros(3, r.n, dtype=torch.float64, device=r.dev)
         gx0, gv0, gm = r.backward(ctx.tape, z if gx is None else gx, z if gv is None else gv)
-        return gx0, gv0, gm, None, None, None
+        return gx0, gv0, gm, None, None, None, None
 
 
 def soft_kdk(x0, v0, m, r_out, runner: SoftKDK, r_search=None):
     """(x_N, v_N) of the rollout, differentiable in x0, v0 and m (radii frozen)."""
-    return _KDK.apply(x0, v0, m, r_out, runner, r_search)
+    return _KDK.apply(x0, v0, m, r_out, runner, r_search, torch.is_grad_enabled())
 
 
 def cutoffs(params: P.Params, x0, v0, m, device: int = 0, with_search: bool = False):
