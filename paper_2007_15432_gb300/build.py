@@ -24,7 +24,7 @@ SOURCES = ["primitives.cu", "tree.cu", "walk.cu", "neighbours.cu", "hard.cu", "c
            "noalloc.cu", "adjoint.cu", "direct.cu", "hermite_adj.cu"]
 NO_FMA = {"tree.cu", "neighbours.cu", "hard.cu", "ctx.cu", "noalloc.cu", "hermite_adj.cu"}
 # FP32 subnormals flushed to zero (the all-pairs kernels' FP32 operands are
-# far from 2^-126; rsqrtf then needs no subnormal handling)
+# far from 2^-126)
 FTZ = {"direct.cu"}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

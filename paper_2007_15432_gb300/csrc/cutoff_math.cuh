@@ -4,11 +4,12 @@
 
 #include "p3t_internal.cuh"
 
-// 1 / sqrt(x) and x^(-1/4) from the 20-bit seed (one rounding more than the
-// last at most; the rsqrt_seed range, otherwise out of line): with e = 1 - x y^2
-// (|e| <= 2^-18), y (1 + e / 2 + 3/8 e^2), the rest below 2^-55; with e = 1 - x z^4
-// (|e| <= 2^-16), z (1 + e / 4 + 5/32 e^2 + 15/128 e^3), the rest below 2^-67.  4
-// and 8 FP64 instructions, where rsqrt() takes 5 to 6 and sqrt() 9.
+// 1 / sqrt(x) and x^(-1/4) from the 20-bit seed y by the binomial series (one
+// rounding more than the last at most; the seed's range and bound are
+// rsqrt_seed's, otherwise out of line): y (1 + e / 2 + 3/8 e^2) with e = 1 - x y^2;
+// z (1 + e / 4 + 5/32 e^2 + 15/128 e^3) with z = y times the seed of y^(-1/2) and
+// e = 1 - x z^4 (|e| < 2^-17), the rest below 2^-71.  5 and 8 FP64 instructions.
+// rsqrt() for inv_sqrt: the radii of 1e6 bodies 205 -> 209 us.
 __device__ __forceinline__ bool seed_range(double x) {
   return (unsigned)((__double2hiint(x) >> 20) - 512) < 1024u;
 }
@@ -51,8 +52,9 @@ __device__ __forceinline__ float2 cut_scale(double Rmin, double lmin, double lma
 // nb / (2 span) ln(R^2 / Rmin^2) decides it first when no integer lies within
 // its error bound of the estimate: the squares cut to 24 bits, their quotient's
 // two roundings and logf's last place leave the logarithm within 3.6e-7 + 1.2e-7
-// of itself, the scale's and the products' roundings are 3e-7 relative; the
-// bound is twice that.  (One particle in a thousand is left at 377 bins over a
+// of itself (2.4e-7 of the scale after the half), the scale's and the products'
+// roundings are 3e-7 relative; the bound is 1.7 times the one and 3.3 times the
+// other.  (One particle in a thousand is left at 377 bins over a
 // factor e; a bound ten times wider sent a warp in four through the FP64
 // logarithm.)  Otherwise the FP64 expression is evaluated.
 static __device__ __noinline__ int cut_bin_fp64(double R2, double Rmin, double Rmax, double lmin,
@@ -76,8 +78,8 @@ __device__ __forceinline__ int cut_bin(double R2, float2 sc, double Rmin, double
 }
 
 // x^(1/3) for x >= 0: the inverse cube root z = x^(-1/3) from an FP32 seed
-// (relative error below 5e-7), corrected once: with e = 1 - x z^3, z (1 + e / 3 +
-// 2/9 e^2), the rest below 2^-60; then x^(1/3) = x z^2.  Inputs outside the
+// (relative error below 5e-7), corrected once by the binomial series: with e = 1 -
+// x z^3, z (1 + e / 3 + 2/9 e^2), the rest below 2^-60; then x^(1/3) = x z^2.  Inputs outside the
 // seed's range take cbrt.  Conversions by integer operations (an FP64 one
 // takes the FP64 pipe).
 static __device__ __noinline__ double cbrt_rare(double x) { return cbrt(x); }

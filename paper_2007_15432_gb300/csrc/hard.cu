@@ -1446,8 +1446,8 @@ constexpr int64_t kEBlocks = 152 * 4 * 8;  // blocks asked for: eight waves of f
 // with 1 / r from the 20-bit seed.  Sources are staged by tile, a tile's sum
 // in FP32 (FP64) per target, the tiles' sums in float-float (FP64).  Measured
 // (one scalar target a thread over all sources before): mixed N = 1e5 11,640 ->
-// 2,790 us, 1e4 703 -> 69; FP64 N = 1e4 10,950 -> 1,330.  (rsqrtf's subnormal
-// scaling on every pair: 3,490 and 72.)
+// 2,790 us, 1e4 703 -> 69; FP64 N = 1e4 10,950 -> 1,330.  (With rsqrtf
+// for rsqrt_normal: 3,490 and 72.)
 template <bool MIXED>
 __global__ void __launch_bounds__(kEThreads) k_energy(p3t_particles p, p3t_params prm, int tiles,
                                                       int chunk, double *part) {

@@ -48,15 +48,16 @@ __device__ __forceinline__ FF ff_div(FF a, FF b) {
   return ff_fast(q1, r.h / b.h);
 }
 
-// 1 / sqrt(r2): the FP32 estimate and one Newton step y (3 - r2 y^2) / 2 with
-// the residual 1 - r2 y^2 formed in float-float
-// rsqrtf of a normal number (the same bits): without flushing, rsqrtf adds a
-// comparison and two multiplications that only a subnormal needs
+// rsqrtf of a normal number (the same bits for every one of them) in one
+// instruction: energy of 1e5 bodies 3,490 -> 2,790 us
 __device__ __forceinline__ float rsqrt_normal(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+
+// 1 / sqrt(r2): the FP32 estimate and one Newton step y (3 - r2 y^2) / 2 with
+// the residual 1 - r2 y^2 formed in float-float
 __device__ __forceinline__ FF ff_rsqrt(FF r2) {
   const float y = rsqrtf(r2.h);
   const float p = y * y;
@@ -70,13 +71,14 @@ __device__ __forceinline__ FF ff_rsqrt(FF r2) {
 // On this part an FP64 warp instruction costs 64 cycles of its sub-partition
 // (76 with all four busy), the 20-bit reciprocal square root seed 8 on
 // another pipe.  With y the seed and e = 1 - x y^2 (|e| <= 2^-19, measured
-// over all leading mantissas), x^(-3/2) = y^3 (1 - e)^(-3/2) = y^3 (1 + 3/2 e +
-// 15/8 e^2 + O(2.2 e^3)): the rest is below 2^-55, so the result carries only
-// its last rounding and y^3's, and takes 6 FP64 instructions where rsqrt()
-// cubed takes 7 to 8 and three more roundings.  Outside 2^-511 <= x < 2^513 the
-// seed is rsqrt() itself (0 for x = 0), out of line: inlined, the compiler
-// predicates its FP64 instructions into every use, and predicated-off ones
-// still take the pipe.
+// over all leading mantissas), the binomial series x^(-3/2) = y^3 (1 - e)^(-3/2) =
+// y^3 (1 + 3/2 e + 15/8 e^2 + O(2.2 e^3)) leaves a rest below 2^-55, so the result
+// carries little but its last rounding and y^3's, from 6 FP64 instructions (FP64
+// ring force of 1e5 bodies, with this and a lane a source, 4,790 -> 2,700 us);
+// likewise x^(-1/2) = y (1 + e / 2 + 3/8 e^2), the rest below 2^-58, from 5.
+// Outside 2^-511 <= x < 2^513 the seed is rsqrt() itself (0 for x = 0), out of
+// line: inlined, the compiler predicates its FP64 instructions into every use, and
+// predicated-off ones still take the pipe.
 static __device__ __noinline__ double rsqrt_rare(double x) {
   return __double_as_longlong(x) == 0 ? 0.0 : rsqrt(x);
 }

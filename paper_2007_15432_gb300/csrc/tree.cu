@@ -164,8 +164,8 @@ __global__ void k_cut_segbins(SegView sv, int vran_bins, const unsigned long lon
 
 // What bounds the cut-offs from some 1e5 particles on is the FP64 pipe (19 cycles
 // of an SM a warp instruction): 23 FP64 instructions a particle in k_cut_u2 and
-// some 40 in k_cut_final, where library roots, a division and the bounds'
-// logarithms took 56 and 57 and, a thread, 120 more.  Measured at N = 377,740:
+// some 40 in k_cut_final, the roots from seeds and the bounds' logarithms once.
+// Measured, with CUDA's roots and the logarithms a thread, and now, at N = 377,740:
 // k_cut_u2 108 -> 27 us, k_cut_final 52 -> 33, k_cut_range 18 -> 14, the whole 213
 // -> 104; below, the launches: N = 1,000 43 -> 32 us, 1e5 92 -> 52, 1e6 378 -> 205.
 // |u|^2 and the radial bin of every particle (kept for k_cut_final); (bin,

@@ -793,11 +793,10 @@ __global__ void __launch_bounds__(kWarps * 32, U == 1 ? kManyBlocks : kFewBlocks
 // chunk, so the host may choose it by the size of the system.  A batch whose
 // entries are all beyond every target's cut-off reach (decided in FP32 with a
 // margin) skips the changeover and the candidate test; the factor K = 1
-// would leave the same bits.  16 FP64 instructions a far pair, 31 a near one,
-// 37 a node (21, 33 and 42 with one lane a target, rsqrt() and 0.6-0.9 of the
-// lanes in use): N = 1e5 ring, theta 0.5, 4,790 -> 2,700 us a
-// walk (93 % of the FP64 pipe's instruction rate); 3 to 5 blocks an SM and
-// chunks of 4 or 8 within 2 %.
+// would leave the same bits.  16 FP64 instructions a far pair, 30 a near one,
+// 37 a node, every lane in use (with rsqrt() and one lane a target 0.6-0.9 of
+// them): N = 1e5 ring, theta 0.5, 4,790 -> 2,700 us a walk (93 % of the FP64 pipe's
+// instruction rate); 3 to 5 blocks an SM and chunks of 4 or 8 within 2 %.
 constexpr int kChunk = 8;
 constexpr int kWalk64Blocks = 4;
 struct Targets64 {
