@@ -9,6 +9,7 @@
 #include "p3t_internal.cuh"
 
 int64_t p3t_walk_warps(int num_sms, int64_t n);
+int64_t p3t_walk_stack(int64_t n);
 int p3t_walk_blocks_per_sm();
 
 static std::atomic<long long> g_launches{0};
@@ -16,7 +17,6 @@ void p3t_note_launches(int64_t k) { g_launches.fetch_add(k, std::memory_order_re
 
 namespace {
 
-constexpr int64_t kStackCap = 8192;  // walk stack entries per warp
 
 struct DeviceGuard {
   int prev = -1;
@@ -116,7 +116,7 @@ int reserve(p3t_ctx *c, int64_t n, int64_t cand_cap) {
   c->node_cap = NC;
   c->cand_cap = cand_cap;
   c->walk_warps = p3t_walk_warps(c->num_sms, N);
-  c->stack_cap = kStackCap < NC ? kStackCap : NC;  // a walk pushes a node at most once
+  c->stack_cap = p3t_walk_stack(N);
   c->radix_hist_cap = p3t_radix_hist_entries(N > NC ? N : NC);
   bool ok = true;
   ok &= dalloc(c->keys, N) && dalloc(c->keys_alt, N) && dalloc(c->idx, N) && dalloc(c->idx_alt, N);

@@ -1477,12 +1477,24 @@ int p3t_run_soft_force(p3t_ctx *c, const p3t_particles *p, double *ax,
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }
 
-// persistent walk warps for a context of up to n particles: 6 blocks per SM,
-// fewer for small systems: a block for every 4 particles (the FP64 walks take
+// entries of a walk's stack in a context of up to n particles: all that can stand
+// there.  A warp pops the deepest 32 and pushes their children in the same order,
+// so the stack's levels ascend: a level's nodes are opened only when all deeper
+// ones are among the popped, so at most 8 x 32 entries of a level stand there (the
+// first two levels 8 and 64), and as disjoint subtrees no more than the particles.
+// (Disks of 1e3 to 1e6 bodies reach 70 to 464.)
+int64_t p3t_walk_stack(int64_t n) {
+  return std::min<int64_t>(n, 8 + 64 + 256 * (P3T_BITS - 2));
+}
+
+// persistent walk warps for a context of up to n particles: the most blocks per SM
+// of the kernels that take it (a program may hold many small contexts: 5,000 bodies
+// 122 -> 55 MB each), fewer still below: a block for every 4 particles (the FP64 walks take
 // single targets there; with a block for every 256, 1,000 particles in FP64
 // ran on 4 SMs: 2,535 us at theta = 0, 105 now; mixed 1e5 ring 338 -> 253)
 int64_t p3t_walk_warps(int num_sms, int64_t n) {
-  int64_t blocks = (int64_t)num_sms * p3t_walk_blocks_per_sm();
+  const bool small = n <= (int64_t)kFewTargets * num_sms;
+  int64_t blocks = (int64_t)num_sms * (small ? std::max(kWalk64Blocks, kFewBlocks) : kManyBlocks);
   const int64_t want = n / 4 + 1;
   if (want < blocks) blocks = want;
   return blocks * kWarps;
