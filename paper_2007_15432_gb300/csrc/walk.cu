@@ -737,20 +737,24 @@ __global__ void __launch_bounds__(kWarps * 32, U == 1 ? kManyBlocks : kFewBlocks
   int32_t *stack = a.stack + ((int64_t)blockIdx.x * kWarps + w) * a.stack_cap;
   const int64_t nleaf = *a.d_nleaf;
   const int64_t round_limit = *a.d_nnode + 2;  // a node is pushed at most once per walk
+  const int64_t paired = max((int64_t)0, nleaf - (int64_t)gridDim.x * kWarps);
   unsigned npp = 0, npn = 0;
 
   for (;;) {
-    // work unit u: the first 32 targets of target group u, then, once all of
-    // those are taken, the rest of group u - nleaf (empty for a group of at
-    // most 32): units of at most 32 targets keep the warps' finishing times
-    // close, and the rests, mostly small, are left for the end (against a
-    // group's rest right after its first 32: N = 3e5 463 -> 441 us, 1e5 254 ->
-    // 250, 1e6 the same)
+    // work unit u: the first 32 targets of a target group or the rest of it
+    // (empty for a group of at most 32): units of at most 32 targets keep the
+    // warps' finishing times close.  A group's rest follows its first 32, which
+    // meet much the same nodes, but for the last groups, as many as there are
+    // warps: all their first 32, then their rests, mostly small, so that the end
+    // has small units.  Force, rests at once / all at the end / this, wide disk: N =
+    // 2e5 307 / 321 / 286 us, 3e5 456 / 434 / 430, 6e5 729 / 756 / 710, 1e6 1,243 /
+    // 1,218 / 1,202; ring 1e5 330 / 248 / 240
     int64_t u = 0;
     if (lane == 0) u = atomicAdd(reinterpret_cast<unsigned long long *>(a.cursor), 1ull);
     u = __shfl_sync(0xffffffffu, u, 0);
-    const bool rest = u >= nleaf;
-    const int64_t g = rest ? u - nleaf : u;
+    const int64_t v = u - 2 * paired;
+    const bool rest = v < 0 ? (u & 1) : v >= nleaf - paired;
+    const int64_t g = v < 0 ? u >> 1 : (rest ? v - nleaf + 2 * paired : v + paired);
     if (g >= nleaf) break;
     if (*(volatile int32_t *)&a.st->code != 0) break;
     const TreeNode &G = a.node[a.leaf_list[g]];
