@@ -23,8 +23,9 @@
 // matter and every run gives the same bits.
 //
 // Bound by the FP64 pipe like the context's kernels, whose arithmetic it shares
-// (cutoff_math.cuh); the range's logarithms and each bin's v_ran are formed once,
-// by the last block of the kernel before, where every thread formed them:
+// (cutoff_math.cuh); the range's logarithms and (with few bins) each bin's v_ran
+// are formed once, by the last block of the kernel before, where every thread
+// formed them:
 // N = 1,000 61 -> 47 us, 1e5 106 -> 45, 1e6 623 -> 208.
 #include <math.h>
 
@@ -168,11 +169,18 @@ __device__ __forceinline__ void nz_add128(unsigned long long *lo, unsigned long 
   if (a_hi + carry) atomicAdd(hi, a_hi + carry);
 }
 
+// v_ran of a bin, from its 128-bit sum in FP64: hi 2^-24 + lo 2^-88
+__device__ __forceinline__ double nz_vran(const unsigned long long *sc, int k) {
+  const double sum = (double)__ldcg(&sc[2 + kMaxBins + k]) * 5.9604644775390625e-08 +
+                     (double)__ldcg(&sc[2 + k]) * 3.2311742677852644e-27;
+  return sqrt(sum / (double)__ldcg(&sc[2 + 2 * kMaxBins + k]));
+}
+
 // random velocity u = v - sqrt(G M_* / |x|) phi_hat, |u|^2 summed per bin
 // (per block in shared memory first when the bins fit)
 __global__ void nz_bins(int64_t n, const double *x, const double *y,
                         const double *z, const double *vx, const double *vy,
-                        const double *vz, double smu, int nb,
+                        const double *vz, double smu, int nb, bool by_bin,
                         unsigned long long *sc) {
   extern __shared__ unsigned long long s_w[];
   const bool shared = nb <= kSharedBins;
@@ -207,22 +215,17 @@ __global__ void nz_bins(int64_t n, const double *x, const double *y,
       }
     }
   }
-  if (!nz_last(&sc[kExtra + 1])) return;
-  // v_ran of every bin, the 128-bit sum to FP64: hi 2^-24 + lo 2^-88
-  for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-    const double sum = (double)__ldcg(&g_hi[k]) * 5.9604644775390625e-08 +
-                       (double)__ldcg(&g_lo[k]) * 3.2311742677852644e-27;
-    const double vr = sqrt(sum / (double)__ldcg(&g_cnt[k]));
-    g_lo[k] = (unsigned long long)__double_as_longlong(vr);
-  }
+  if (!by_bin || !nz_last(&sc[kExtra + 1])) return;
+  for (int k = threadIdx.x; k < nb; k += blockDim.x)
+    g_lo[k] = (unsigned long long)__double_as_longlong(nz_vran(sc, k));
 }
 
 // r_out = max(R~cut,0 r_Hill, R~cut,1 v_ran dt), r_search = R~s,0 r_out + R~s,1 v_ran dt
 __global__ void nz_final(int64_t n, const double *x, const double *y,
                          const double *z, const double *vx, const double *vy,
                          const double *vz, const double *m, p3t_params prm, double imu,
-                         double i3ms, int nb, const unsigned long long *sc, double *r_out,
-                         double *r_search) {
+                         double i3ms, int nb, bool by_bin, const unsigned long long *sc,
+                         double *r_out, double *r_search) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const double R2 = x[i] * x[i] + y[i] * y[i], r2 = __fma_rn(z[i], z[i], R2);
@@ -231,7 +234,8 @@ __global__ void nz_final(int64_t n, const double *x, const double *y,
     const double alpha = __fma_rn(-v2, imu, 2.0 * ir);  // 1/a, vis-viva
     const double a = alpha > 0.0 ? 1.0 / alpha : r2 * ir;
     const double rhill = cbrt_pos(m[i] * i3ms) * a;
-    const double vr = __longlong_as_double((long long)sc[2 + nz_bin(R2, sc, nb)]);
+    const int k = nz_bin(R2, sc, nb);
+    const double vr = by_bin ? __longlong_as_double((long long)sc[2 + k]) : nz_vran(sc, k);
     const double ro = prm.cutoff_mode == P3T_CUT_HILL_VRAN
                           ? fmax(prm.rcut0 * rhill, prm.rcut1 * vr * prm.dt_soft)
                           : prm.rcut0 * rhill;
@@ -274,13 +278,18 @@ extern "C" int p3t_cutoffs_noalloc(const p3t_params *prm, p3t_particles *p,
   if (g > (int64_t)sms * P3T_NSM_BLOCKS) g = (int64_t)sms * P3T_NSM_BLOCKS;
   if (g < 1) g = 1;
   const double mu = prm->G * prm->m_star;
+  // v_ran once a bin, by the last block of nz_bins, or by every particle for itself:
+  // one block's roots and divisions take their turns, the particles' run on every SM
+  // (by bin / by particle: N = 1e3 with 4,096 bins 73 / 31 us, 1e5 with 256 43 / 44,
+  // 3e5 with 2,048 120 / 115, 1e6 with 1,000 228 / 262)
+  const bool by_bin = n >= 256 * (int64_t)nb;
   nz_clear<<<4, kBlock, 0, s>>>(sc, nb);
   nz_range<<<(unsigned)g, kBlock, 0, s>>>(n, p->x, p->y, nb, sc);
   const size_t smem = nb <= kSharedBins ? 3 * sizeof(unsigned long long) * nb : 0;
   nz_bins<<<(unsigned)g, kBlock, smem, s>>>(n, p->x, p->y, p->z, p->vx, p->vy, p->vz,
-                                            sqrt(mu), nb, sc);
+                                            sqrt(mu), nb, by_bin, sc);
   nz_final<<<(unsigned)g, kBlock, 0, s>>>(n, p->x, p->y, p->z, p->vx, p->vy, p->vz,
-                                          p->m, *prm, 1.0 / mu, 1.0 / (3.0 * prm->m_star), nb, sc,
-                                          p->r_out, p->r_search);
+                                          p->m, *prm, 1.0 / mu, 1.0 / (3.0 * prm->m_star), nb, by_bin,
+                                          sc, p->r_out, p->r_search);
   return cudaGetLastError() == cudaSuccess ? P3T_OK : P3T_ERR_CUDA;
 }
