@@ -49,8 +49,8 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # DRAM bytes (read + write) of one k_walk launch on the N = 10^6 wide disk,
 # group size 64, from a single-pass ncu capture of this kernel
-# (dram__bytes_read.sum 110.27 MB + dram__bytes_write.sum 23.07 MB)
-WALK_TRAFFIC_1E6 = 133.34e6
+# (dram__bytes_read.sum 79.19 MB + dram__bytes_write.sum 16.49 MB)
+WALK_TRAFFIC_1E6 = 95.68e6
 
 
 def parse():

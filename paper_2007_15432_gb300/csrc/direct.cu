@@ -8,10 +8,10 @@
 // the pair arithmetic's type; a block is 8 warps over 64 targets (two per
 // lane); each warp takes one eighth of the block's source range and stages
 // it 32 sources at a time in its own shared-memory slots (one broadcast load
-// per 4-vector, shared by the lane's two targets).  A grid column (blockIdx.y) is one split of the sources; each
-// block adds its 8 warps in order and writes its per-target sums to
-// part[(split * C + c) * n + k]; the last block of a target tile to finish
-// adds the splits in order: the result does not depend on scheduling.
+// per 4-vector, shared by the lane's two targets).  A grid column (blockIdx.y) is
+// one split of the sources; each block adds its 8 warps in order and writes its
+// per-target sums to part[(split * C + c) * n + k]; the last block of a target tile
+// to finish adds the splits in order: the result does not depend on scheduling.
 //
 // Far sources: with the particles in no spatial order a source is inside the
 // cut-off reach of some target of a warp about once in a thousand times (ring
@@ -23,10 +23,15 @@
 // in full at once, as long as near pairs are met); in FP64, where a vote costs
 // little beside a pair, each source is voted on.  What bounds the kernels is
 // the FP32 (FP64) pipe: a packed instruction holds it two cycles (73 % active at
-// N = 50,000).  Measured per call, FP32: force N = 1e4 150 -> 125 us, 5e4 2,550
-// -> 1,670, VJP 242 -> 199, 4,663 -> 3,352; FP64: force N = 8,191 3,000 -> 2,130,
-// VJP N = 1e4 8,984 -> 7,370.  Four targets a lane: 1,590 us at 5e4, 128 at 1e4
-// and 50 instead of 45 at 1,000 (fewer, longer blocks): two kept.
+// N = 50,000).  Measured per call, FP32: force N = 1e4 124 -> 95 us, 5e4 2,518
+// -> 1,630, VJP 210 -> 165, 4,624 -> 3,300; FP64: force N = 8,191 2,960 -> 2,100,
+// VJP N = 1e4 8,940 -> 7,290.  Where most pairs are near (several neighbours a body,
+// whose clusters percolate) the form costs: N = 1e4 124 -> 157 us, VJP 210 -> 293
+// (a warp's first chunk of two taken twice), 5e4 2,518 -> 2,526 and 4,624 -> 4,994.  A
+// first guess from 512 pairs a block makes that 127 and 225, but 95 -> 99 and 165 ->
+// 168 where few are near; votes within a chunk cost the far form 8 to 12 %.  Four
+// targets a lane: 1,590 us at 5e4, 128 at 1e4 and 50 instead of 45 at 1,000 (fewer,
+// longer blocks): two kept.
 //
 // Precision: FP64 throughout, or (MIXED) float-float positions whose
 // difference (hi_k - hi_j) + (lo_k - lo_j) carries the relative coordinate
